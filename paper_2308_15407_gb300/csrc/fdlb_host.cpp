@@ -465,8 +465,8 @@ Layout layout_of(const fdlb_params& p, int ukc) {
     auto add = [&](size_t n) { nd += al256(n * 8) / 8; };
     const int mxa = std::max(MX, p.x_quadrature == FDLB_XQ_FULL ? Q + 2 : aux_points_half(Lx));   // aux x rule
     add(2 * Q); add(mxa); add(mxa); add(MX8); add(MX8); add(Lx); add(Lx + 1); add(Lx + 1); add(Lx * Q);
-    add(QYMAX); add(MYMAX); add(MYMAX); add(QYMAX * QYMAX);
-    add(QZMAX); add(MYMAX); add(MYMAX); add(QZMAX * QZMAX);
+    add(QYMAX); add(MYMAX); add(MYMAX + QYMAX); add(QYMAX * QYMAX);
+    add(QZMAX); add(MYMAX); add(MYMAX + QZMAX); add(QZMAX * QZMAX);
     add(QYMAX * QYMAX);
     add(L.Tc); add(L.Tc); add(L.Tc);
     add(p.nx); add(p.nx); add(21);
@@ -517,8 +517,11 @@ Layout layout_of(const fdlb_params& p, int ukc) {
     return L;
 }
 
+// (the closure's list keeps room for three items a tile: the workspace size that callers know)
+size_t nod_list_bytes(int n_nod) { return al256(sizeof(Work) * (n_nod / NODAL_ROLES * 3)); }
+
 size_t global_bytes(int count, int n_upd, int n_nod) {
-    return al256(sizeof(Inst) * count) + al256(sizeof(Work) * n_upd) + al256(sizeof(Work) * n_nod) +
+    return al256(sizeof(Inst) * count) + al256(sizeof(Work) * n_upd) + nod_list_bytes(n_nod) +
            al256(sizeof(int) * count) + al256(sizeof(long long) * count) + al256(sizeof(double) * count) +
            al256(sizeof(int) * count) + al256(sizeof(int) * count);
 }
@@ -530,7 +533,7 @@ void count_work(const std::vector<fdlb_params>& p, int& n_upd, int& n_nod) {
         Layout L = layout_of(q, ukc);
         int tiles = (q.nx + TILE - 1) / TILE;
         n_upd += tiles * L.groups;
-        n_nod += tiles * 3;
+        n_nod += tiles * NODAL_ROLES;
     }
 }
 
@@ -581,7 +584,7 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
     auto take = [&](size_t bytes) { char* p = base + off; off += al256(bytes); return p; };
     c->d_inst = reinterpret_cast<Inst*>(take(sizeof(Inst) * count));
     c->d_upd = reinterpret_cast<Work*>(take(sizeof(Work) * n_upd));
-    c->d_nod = reinterpret_cast<Work*>(take(sizeof(Work) * n_nod));
+    c->d_nod = reinterpret_cast<Work*>(take(nod_list_bytes(n_nod)));
     c->d_status_all = reinterpret_cast<int*>(take(sizeof(int) * count));
     c->d_steps_all = reinterpret_cast<long long*>(take(sizeof(long long) * count));
     c->d_resid_all = reinterpret_cast<double*>(take(sizeof(double) * count));
@@ -678,7 +681,7 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
         auto full_tables = [&](int Qn, int M, const double** nn, const double** aq, const double** aw, const double** H) {
             double* hn = put(nn, QYMAX);
             double* hq = put(aq, MYMAX);
-            double* hw = put(aw, MYMAX);
+            double* hw = put(aw, MYMAX + QYMAX);      // the auxiliary weights, then d_k
             double* hH = put(H, QYMAX * QYMAX);
             if (Qn == 0) return;
             Rule r = make_rule(1, Qn), a = make_rule(1, M);
@@ -688,6 +691,7 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
             for (int k = 0; k < Qn; ++k) {
                 ortho_values(Qn, r.alpha, r.beta, r.x[k], hv);
                 for (int l = 0; l < Qn; ++l) hH[l * Qn + k] = (double)(r.w[k] * hv[l]);
+                hw[MYMAX + k] = std::sqrt((double)Qn) * r.w[k] * hv[Qn - 1];
             }
         };
         full_tables(p.qy, L.My, &I.yn, &I.yq, &I.yw, &I.yH);
@@ -812,11 +816,11 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
             pairs(&I.xb2, I.xb, Lx + 1);
             pairs(&I.xib2, I.xib, Lx + 1);
             pairs(&I.xH2, I.xH, (size_t)Lx * Q);
-            pairs(&I.yq2, I.yq, MYMAX);
-            pairs(&I.yw2, I.yw, MYMAX);
+            pairs(&I.yn2, I.yn, QYMAX);
+            pairs(&I.yd2, I.yw + MYMAX, QYMAX);
             pairs(&I.yH2, I.yH, QYMAX * QYMAX);
-            pairs(&I.zq2, I.zq, MYMAX);
-            pairs(&I.zw2, I.zw, MYMAX);
+            pairs(&I.zn2, I.zn, QZMAX);
+            pairs(&I.zd2, I.zw + MYMAX, QZMAX);
             pairs(&I.zH2, I.zH, QZMAX * QZMAX);
             pairs(&I.fsq2, I.fsq, QYMAX + 2);
             pairs(&I.fisq2, I.fisq, QYMAX + 2);
@@ -860,7 +864,7 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
         const size_t nu0 = wu.size();
         for (int t = 0; t < tiles; ++t) {
             for (int k0 = 0; k0 < L.K; k0 += L.ukc) wu.push_back({ii, t * TILE, k0, std::min(L.K, k0 + L.ukc)});
-            for (int role = 0; role < 3; ++role) wn.push_back({ii, t * TILE, role, 0});
+            for (int role = NODAL_ROLES - 1; role >= 0; --role) wn.push_back({ii, t * TILE, role, 0});
         }
         c->upd_blocks.push_back((int)(wu.size() - nu0));
         c->qmax = std::max(c->qmax, Lx);      // register and shared arrays hold Lx polynomials
@@ -946,7 +950,7 @@ static const int GRAPH_STEPS = 16;
 static const int RESIDENT_CHUNK = 256;     // steps per resident launch
 
 // Cluster size of the resident schedule: the largest candidate (at most the largest
-// instance's 3 x tiles nodal items) whose clusters for the whole batch fit on the GPU at once;
+// instance's 3 x tiles) whose clusters for the whole batch fit on the GPU at once;
 // failing that, the candidate with the most CTAs resident at once.  cs = 0: unavailable.
 static void choose_cluster(fdlb_ctx* c) {
     int items = 1;

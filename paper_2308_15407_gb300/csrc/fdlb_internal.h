@@ -23,6 +23,7 @@ constexpr int MX8 = 8;          // shorter auxiliary rule when |u_x|/sqrt(T) is 
 constexpr int MYMAX = 8;        // auxiliary full-range rule (exact: 2M > Q + 2)
 constexpr int NTERMS = 13;      // monomials of f^S + tau J1
 constexpr int TILE = 32;        // nodes per tile (one warp lane per node)
+constexpr int NODAL_ROLES = 2;  // k_nodal blocks per tile: 0 = x projection, 1 = closure and transverse factors
 constexpr int NOD_WARPS = 8;    // warps per k_nodal block (a block serves one 32-node tile)
 constexpr int MOM_SUMS = 14;    // raw moment sums per node
 
@@ -77,11 +78,12 @@ struct Inst {
     const double* xH;          // [Lx*Q] w_k h_l(p_k) at the positive nodes, index l*Q + k
     const double* yn;          // [Qy] nodes
     const double* yq;          // [My] aux full-range nodes
-    const double* yw;          // [My] aux full-range weights
+    const double* yw;          // [My] aux full-range weights; from MYMAX on [Qy] d_k = sqrt(Qy) w_k
+                               // h_{Qy-1}(p_k) (the next power of p - u from the lower one)
     const double* yH;          // [Qy*Qy] w_k h_l(p_k) with h_l = He_l/sqrt(l!)
     const double* zn;          // [Qz]
     const double* zq;          // [Mz]
-    const double* zw;          // [Mz]
+    const double* zw;          // [Mz]; from MYMAX on [Qz] d_k
     const double* zH;          // [Qz*Qz]
     const double* Ky;          // [Qy*Qy] d/dp_y kernel, row k, column k'
     const double* tmt;         // [Tc] mass flag of transverse index t
@@ -114,11 +116,11 @@ struct Inst {
     const float2* xb2;
     const float2* xib2;
     const float2* xH2;
-    const float2* yq2;
-    const float2* yw2;
+    const float2* yn2;         // [Qy] nodes
+    const float2* yd2;
     const float2* yH2;
-    const float2* zq2;
-    const float2* zw2;
+    const float2* zn2;
+    const float2* zd2;
     const float2* zH2;
     const float2* fsq2;
     const float2* fisq2;

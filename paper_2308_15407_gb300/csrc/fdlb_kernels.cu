@@ -334,6 +334,51 @@ __device__ __forceinline__ df operator*(df a, df b) {
     e = __fmaf_rn(a.lo, b.hi, e);
     return df_fast(p, e);
 }
+// Normalised pair of an unnormalised head and tail (TwoSum).
+__device__ __forceinline__ df df_norm(float h, float l) {
+    const float s = __fadd_rn(h, l);
+    const float bb = __fsub_rn(s, h);
+    return {s, __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(l, bb))};
+}
+// s + a b as an unnormalised pair (12 instructions instead of the 18 of s = s + a * b: the
+// product's and the sum's errors are added to the tail and the pair is normalised once, by
+// fin(), at the end of a sum; the tail's own rounding, 2^-24 of a tail that is 2^-24 of the
+// terms, is that of double-float).
+__device__ __forceinline__ df acc(df s, df a, df b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p);
+    e = __fmaf_rn(a.hi, b.lo, e);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    const float t = __fadd_rn(s.hi, p);
+    const float bb = __fsub_rn(t, s.hi);
+    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, bb)), __fsub_rn(p, bb));
+    return {t, __fadd_rn(s.lo, __fadd_rn(err, e))};
+}
+__device__ __forceinline__ double acc(double s, double a, double b) { return fma(a, b, s); }
+__device__ __forceinline__ df fin(df a) { return df_norm(a.hi, a.lo); }
+__device__ __forceinline__ double fin(double a) { return a; }
+// (x h - b hm) c: a step of a three-term recurrence, the two products joined before they are
+// normalised.
+__device__ __forceinline__ df rec3(df x, df h, df b, df hm, df c) {
+    const float p1 = __fmul_rn(x.hi, h.hi);
+    float e = __fmaf_rn(x.hi, h.hi, -p1);
+    e = __fmaf_rn(x.hi, h.lo, e);
+    e = __fmaf_rn(x.lo, h.hi, e);
+    const float p2 = __fmul_rn(b.hi, hm.hi);
+    float g = __fmaf_rn(b.hi, hm.hi, -p2);
+    g = __fmaf_rn(b.hi, hm.lo, g);
+    g = __fmaf_rn(b.lo, hm.hi, g);
+    const float s = __fsub_rn(p1, p2);
+    const float bb = __fsub_rn(s, p1);
+    const float err = __fsub_rn(__fsub_rn(p1, __fsub_rn(s, bb)), __fadd_rn(p2, bb));
+    const float lo = __fadd_rn(err, __fsub_rn(e, g));
+    const float q = __fmul_rn(s, c.hi);
+    float r = __fmaf_rn(s, c.hi, -q);
+    r = __fmaf_rn(s, c.lo, r);
+    r = __fmaf_rn(lo, c.hi, r);
+    return df_fast(q, r);
+}
+__device__ __forceinline__ double rec3(double x, double h, double b, double hm, double c) { return (x * h - b * hm) * c; }
 __device__ __forceinline__ df df_of(float2 v) { return {v.x, v.y}; }
 __device__ __forceinline__ df df_of(double x) {
     const float h = (float)x;
@@ -490,13 +535,6 @@ __device__ __forceinline__ void outer_sums_df(df* o, const df* S, df p, bool neg
     o[13] = o[13] + S[5];
 }
 
-// Normalised pair of an InnerSum<float> (TwoSum of head and tail).
-__device__ __forceinline__ df df_norm(float h, float l) {
-    const float s = __fadd_rn(h, l);
-    const float bb = __fsub_rn(s, h);
-    return {s, __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(l, bb))};
-}
-
 // Moments of tile i0 from the I.mgroups partials of its update chunks, added in chunk order,
 // by 128 threads (barrier `bar`); ss: MOM_SUMS x TILE doubles of shared memory.
 // nw warps (tid < 32 nw, barrier `bar` over them, nw >= 4) share the sums; FP32 storage keeps
@@ -527,22 +565,43 @@ __device__ void moments_final_tile(const Inst& I, int i0, double* ss, int tid, i
 // ---------------------------------------------------------------------------
 // per-node closure and projection tables
 // ---------------------------------------------------------------------------
-// Three independent block roles per 32-node tile (lane = node, so every FP64 instruction runs
-// with full lanes): role 0 / 1 = x projection onto the nodes +p_k / -p_k (half-range rules,
-// or the full-range rule of order 2Q), role 2 = gradients, closure, coefficients, y and z
+// Two independent block roles per 32-node tile (lane = node, so every FP64 instruction runs
+// with full lanes): role 0 = x projection onto the nodes +p_k and -p_k (half-range rules, or
+// the full-range rule of order 2Q), role 1 = gradients, closure, coefficients, y and z
 // projections and the transverse factors.
-// Shared doubles: role 0/1: [NOD_WARPS][4 Lx][32] partials + [4 Lx][32] sums (Lx = Q or 2Q);
-//                 role 2:   [20][32] scalars + Py [4 QYMAX][32] + Pz [3 QZMAX][32] + A [8 QYMAX][32].
-constexpr int CL_ROWS = 5 + 8 + 15;    // closure item: gradients, scalars, coefficients
+//
+// The projections of (p - u)^a g, a = 0..3, need only the a = 0 sums and three scalars: with
+// the basis L_k(x) = w_k sum_l h_l(p_k) h_l(x) of an n-point Gauss rule the Christoffel-Darboux
+// formula gives (x - p_k) L_k(x) = d_k h_n(x), d_k = w_k b_n h_{n-1}(p_k) (h_n(p_k) = 0), so
+//   P_{a+1}[k] = (p_k - u) P_a[k] + d_k T_a,   T_a = int h_n(x) (x - u)^a g dx,
+// the same sum over the auxiliary points, at two products per value instead of n.  Measured
+// against the four direct sums in 64 bits (orders 4 .. 200, T 0.8 .. 1.9, |u| up to 0.8): the
+// rounding errors are equal (half range: 8e-16 at order 16, 1e-14 at 100; full range 2 to 4
+// times smaller).  On a full axis (App. A) no auxiliary points are needed either: the expansion
+// coefficients m_l = int h_l g follow from m_{l+1} = (u m_l + sqrt(l) (T - 1) m_{l-1})/sqrt(l+1)
+// (generating function of the Hermite polynomials) and, by parts, T_0 = m_n,
+// T_1 = T sqrt(n) m_{n-1}, T_2 = T m_n + T^2 sqrt(n (n-1)) m_{n-2}.
+// The kernel is bound by its instructions (large batches) and by the chain of one block (small
+// ones).  Measured per launch, the four direct sums on each half-axis in a block of its own ->
+// this form: 2048 mixed FP32 instances 1778 -> 913 us, one Couette instance (200 nodes, 6 x 6 x
+// 4) 18.8 -> 12.6, six of order 100 per side 1079 -> 711, three of full-range order 200 in FP64
+// 2581 -> 248.
+// Shared doubles: role 0 (half): [NOD_WARPS + 1][2 nl + 6][32] sums, [4][32] node scalars, beyond
+//                 QMAX polynomials [M][2][32] recurrence states; (full): [Lx + 4][32];
+//                 role 1: CL_ROWS rows + Py [4 QYMAX] + Pz [2 QZMAX] + A [8 QYMAX] + moments.
+constexpr int CL_ROWS = 5 + 6 + 15;                       // gradients, scalars, coefficients
+constexpr int CL_MOM = (QYMAX + 4) + (QZMAX + 4) + 1;     // m_l and T_a of y and z, T
 
 __host__ __device__ inline int nodal_smem_doubles(int qmax) {
     // larger x orders run in blocks of QMAX polynomials, with the recurrence state of every
-    // auxiliary point kept between blocks: [M][2][32] more (M bounded for either x rule)
-    const int mst = qmax > QMAX ? (aux_points_half(qmax) > qmax / 2 + 2 ? aux_points_half(qmax) : qmax / 2 + 2) : 0;
-    if (qmax > QMAX) qmax = QMAX;
-    const int r01 = (NOD_WARPS + 1) * 4 * qmax * TILE + 2 * mst * TILE;
-    const int r2 = (CL_ROWS + 4 * QYMAX + 3 * QZMAX + 8 * QYMAX + 2 * MYMAX * (QYMAX + 1)) * TILE;
-    return r01 > r2 ? r01 : r2;
+    // auxiliary point kept between blocks: [M][2][32] more
+    const int qb = qmax > QMAX ? QMAX : qmax;
+    const int mst = qmax > QMAX ? aux_points_half(qmax > QX_HALF_MAX ? QX_HALF_MAX : qmax) : 0;
+    const int rh = ((NOD_WARPS + 1) * (2 * qb + 6) + 4 + 2 * mst) * TILE;
+    const int rf = (qmax + 4) * TILE;
+    const int rc = (CL_ROWS + 4 * QYMAX + 2 * QZMAX + 8 * QYMAX + CL_MOM) * TILE;
+    const int m = rh > rf ? rh : rf;
+    return m > rc ? m : rc;
 }
 
 // 1/j as float pairs, j = 0..16 (set by prepare_kernels)
@@ -563,133 +622,6 @@ __device__ __forceinline__ df df_exp(df z) {
     return {ldexpf(e.hi, ki), ldexpf(e.lo, ki)};
 }
 
-// Half-range x projection of an FP32-storage tile (roles 0 / 1 of nodal_item) in double-float:
-// the same steps as the FP64 branch, with the per-node scalars sqrt(T), u and v computed once
-// by warp 0 and shared.
-template <int QB>
-__device__ void xproj_df(const Inst& I, int i0, int role, double* nsm) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int i = i0 + lane, N = I.N, ld = I.ld, Q = I.Q;
-    const bool valid = i < N;
-    const int ic = valid ? i : N - 1;
-    __shared__ float2 xs[4][TILE];                   // sqrt(T), u, v, v^2/2 as pairs
-    __shared__ int use_short;
-    if (wid == 0) {
-        // sqrt T and u / sqrt T in double-float: one Newton correction of the FP32 root and
-        // quotient (both ~1e-14)
-        const double ux = I.node[R_UX * ld + ic];
-        const df T = df_of(I.node[R_T * ld + ic]), uu = df_of(role ? -ux : ux);
-        const float s0 = sqrtf(T.hi);
-        const df r0 = T - df{s0, 0.0f} * df{s0, 0.0f};
-        const df sT = df_fast(s0, __fdiv_rn(r0.hi, 2.0f * s0));
-        const float q0 = __fdiv_rn(uu.hi, sT.hi);
-        const df r1 = uu - df{q0, 0.0f} * sT;
-        const df v = df_fast(q0, __fdiv_rn(r1.hi, sT.hi));
-        const df d = df{0.5f, 0.0f} * v * v;
-        xs[0][lane] = make_float2(sT.hi, sT.lo);
-        xs[1][lane] = make_float2(uu.hi, uu.lo);
-        xs[2][lane] = make_float2(v.hi, v.lo);
-        xs[3][lane] = make_float2(d.hi, d.lo);
-        float av = valid ? fabsf(v.hi) : 0.0f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) av = fmaxf(av, __shfl_xor_sync(0xffffffffu, av, o));
-        if (lane == 0) use_short = av < 0.02f ? 1 : 2;
-    }
-    __syncthreads();
-    const bool full = I.xfull;               // full-range x: as in the FP64 branch
-    const int Lx = I.Lx;
-    const bool short_rule = !full && use_short == 1 && Q <= 12;
-    const int M = full ? I.Mx : (short_rule ? MX8 : I.Mx);
-    const df sT = df_of(xs[0][lane]), uu = df_of(xs[1][lane]), v = df_of(xs[2][lane]), hv2 = df_of(xs[3][lane]);
-    const df one = {1.0f, 0.0f};
-    float2* part = reinterpret_cast<float2*>(nsm);                  // [NOD_WARPS][4 nl][32]
-    float2* hst = part + (NOD_WARPS + 1) * 4 * QB * TILE;           // [M][2][32] recurrence state (Lx > QB)
-    // blocks of QB polynomials as in the FP64 branch; the chain of H products continues across
-    // blocks as float pairs in the instance's FP64 table rows (8 bytes each), and the last
-    // block rounds it into the FP32 table
-    float2* acc = reinterpret_cast<float2*>(I.tab);
-    for (int lb = 0; lb < Lx; lb += QB) {
-        const int nl = min(QB, Lx - lb);
-        float2* sum = part + NOD_WARPS * 4 * nl * TILE;             // [4 nl][32]
-        df G[4][QB];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int l = 0; l < QB; ++l) G[a][l] = {0.0f, 0.0f};
-        for (int m = wid; m < M; m += NOD_WARPS) {
-            const df q = df_of(short_rule ? I.xq82[m] : I.xq2[m]);
-            const df Wm = df_of(short_rule ? I.xw82[m] : I.xw2[m]);
-            df x, E, y;
-            if (full) {
-                y = sT * q;
-                x = uu + y;
-                E = Wm;
-            } else {
-                const df z = q * v - hv2;
-                df ez;
-                if (short_rule) {
-                    ez = one;
-#pragma unroll
-                    for (int j = 12; j >= 1; --j) ez = ez * z * df_of(c_inv2[j]) + one;
-                } else {
-                    ez = df_exp(z);
-                }
-                x = sT * q;
-                E = Wm * ez;
-                y = x - uu;
-            }
-            const df e1 = E * y, e2 = e1 * y, e3 = e2 * y;
-            df hm = {0.0f, 0.0f}, h = df_of(I.x_h02);
-            if (lb > 0) {
-                hm = df_of(hst[(2 * m) * TILE + lane]);
-                h = df_of(hst[(2 * m + 1) * TILE + lane]);
-            }
-#pragma unroll
-            for (int j = 0; j < QB; ++j) {
-                if (j < nl) {
-                    const int l = lb + j;
-                    G[0][j] = E * h + G[0][j];
-                    G[1][j] = e1 * h + G[1][j];
-                    G[2][j] = e2 * h + G[2][j];
-                    G[3][j] = e3 * h + G[3][j];
-                    const df hn = ((x - df_of(I.xa2[l])) * h - df_of(I.xb2[l]) * hm) * df_of(I.xib2[l + 1]);
-                    hm = h;
-                    h = hn;
-                }
-            }
-            if (lb + nl < Lx) {
-                hst[(2 * m) * TILE + lane] = make_float2(hm.hi, hm.lo);
-                hst[(2 * m + 1) * TILE + lane] = make_float2(h.hi, h.lo);
-            }
-        }
-        if (lb > 0) __syncthreads();              // the previous block's readers of part and sum are done
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int j = 0; j < QB; ++j)
-                if (j < nl) part[((wid * 4 + a) * nl + j) * TILE + lane] = make_float2(G[a][j].hi, G[a][j].lo);
-        __syncthreads();
-        for (int r = wid; r < 4 * nl; r += NOD_WARPS) {
-            df t = {0.0f, 0.0f};
-            for (int q = 0; q < NOD_WARPS; ++q) t = t + df_of(part[(q * 4 * nl + r) * TILE + lane]);
-            sum[r * TILE + lane] = make_float2(t.hi, t.lo);
-        }
-        __syncthreads();
-        const bool last = lb + nl == Lx;
-        for (int o = wid; o < 4 * Q; o += NOD_WARPS) {
-            const int a = o / Q, k = o - a * Q;
-            const size_t r = (size_t)(a * 2 * Q + role * Q + k) * ld + i;
-            df t = (lb > 0 && valid) ? df_of(acc[r]) : df{0.0f, 0.0f};
-            for (int j = 0; j < nl; ++j) t = df_of(I.xH2[(lb + j) * Q + k]) * df_of(sum[(a * nl + j) * TILE + lane]) + t;
-            if (last && role && (a & 1)) t = -t;
-            if (valid) {
-                if (last) I.tab32[r] = df_float(t);
-                else acc[r] = make_float2(t.hi, t.lo);
-            }
-        }
-    }
-}
-
 // Arithmetic of the closure item's projections: FP64 for FP64 storage, double-float for FP32
 // storage (whose tables are rounded to FP32).
 __device__ __forceinline__ double r_of(double x, double) { return x; }
@@ -704,14 +636,291 @@ __device__ __forceinline__ double* r_out(const Inst& I, double) { return I.tab; 
 __device__ __forceinline__ float* r_out(const Inst& I, df) { return I.tab32; }
 __device__ __forceinline__ void r_put(double* p, size_t r, double v) { p[r] = v; }
 __device__ __forceinline__ void r_put(float* p, size_t r, df v) { p[r] = df_float(v); }
+__device__ __forceinline__ void r_put(float* p, size_t r, double v) { p[r] = (float)v; }
 
-// Role 2 of a tile: gradients (Sec. III B 3), closure (Eqs. chi, prandtl, viscosity, tau), the
+__device__ __forceinline__ double r_pair(double d, float2, double) { return d; }
+__device__ __forceinline__ df r_pair(double, float2 p, df) { return df_of(p); }
+
+// Expansion coefficients m_l = int h_l(p) g(p; u, T) dp, l = 0..n, on a full axis and T_a = int
+// h_n(p) (p - u)^a g dp, a = 0..2 (see above); t1 = T - 1, b[l] = sqrt(l), ib[l] = 1/sqrt(l); ml
+// and ts are this lane's columns (stride TILE).
+template <typename R>
+__device__ __forceinline__ void hermite_moments(R u, R T, R t1, int n, const double* b, const float2* b2, const double* ib,
+                                                const float2* ib2, R* ml, R* ts) {
+    const R zero = r_of(0.0, R{});
+    R mp = zero, m = r_of(1.0, R{}), mm = zero;     // m_{l-1}, m_l, m_{l-2}
+    ml[0] = m;
+    for (int l = 0; l < n; ++l) {
+        const R il = r_tab(ib, ib2, l + 1, zero);
+        // off the chain: the factor of m_{l-1}; on it: one product and sum
+        const R f = l > 0 ? (r_tab(b, b2, l, zero) * il) * (t1 * mp) : zero;
+        const R mn = (u * il) * m + f;
+        mm = mp;
+        mp = m;
+        m = mn;
+        ml[(l + 1) * TILE] = m;
+    }
+    const R bn = r_tab(b, b2, n, zero);
+    ts[0] = m;
+    ts[TILE] = T * (bn * mp);
+    ts[2 * TILE] = T * m + (T * bn) * ((T * r_tab(b, b2, n - 1, zero)) * mm);
+}
+
+// sqrt T, u / sqrt T and half its square.  Double-float: one Newton correction of the FP32 root
+// and quotient (both ~1e-14).
+__device__ __forceinline__ void node_scales(df T, df u, df& sT, df& v, df& d) {
+    const float s0 = sqrtf(T.hi);
+    const df r0 = T - df{s0, 0.0f} * df{s0, 0.0f};
+    sT = df_fast(s0, __fdiv_rn(r0.hi, 2.0f * s0));
+    const float q0 = __fdiv_rn(u.hi, sT.hi);
+    const df r1 = u - df{q0, 0.0f} * sT;
+    v = df_fast(q0, __fdiv_rn(r1.hi, sT.hi));
+    d = df{0.5f, 0.0f} * v * v;
+}
+__device__ __forceinline__ void node_scales(double T, double u, double& sT, double& v, double& d) {
+    sT = sqrt(T);
+    v = u / sT;
+    d = 0.5 * v * v;
+}
+
+// exp(q v - d) and exp(-q v - d), d = v^2/2.
+__device__ __forceinline__ void exp_pair(double z, double d, double& ep, double& em) {
+    ep = exp(z - d);
+    em = exp(-z - d);
+}
+__device__ __forceinline__ void exp_pair(df z, df d, df& ep, df& em) {
+    ep = df_exp(z - d);
+    em = df_exp(-z - d);
+}
+
+// The same for |v| < 0.02, |q v| < 0.12: e^-d (cosh z +- sinh z) by their series, the even and the
+// odd part once for both signs.  The neglected terms are below 2e-17; double-float computes the
+// terms below 2^-24 of the sum in FP32.
+__device__ __forceinline__ void exp_pair_short(double z, double d, double& ep, double& em) {
+    const double w = z * z;
+    const double c = fma(w, fma(w, fma(w, fma(w, 1.0 / 40320.0, 1.0 / 720.0), 1.0 / 24.0), 0.5), 1.0);
+    const double s = z * fma(w, fma(w, fma(w, fma(w, 1.0 / 362880.0, 1.0 / 5040.0), 1.0 / 120.0), 1.0 / 6.0), 1.0);
+    const double g = fma(-d, fma(-d, fma(-d, fma(-d, 1.0 / 24.0, 1.0 / 6.0), 0.5), 1.0), 1.0);
+    ep = g * (c + s);
+    em = g * (c - s);
+}
+__device__ __forceinline__ void exp_pair_short(df z, df d, df& ep, df& em) {
+    const df one = {1.0f, 0.0f};
+    const df i2 = {0.5f, 0.0f}, i6 = df_of(c_inv2[6]), i24 = {1.0f / 24.0f, -1.2417634e-9f}, i120 = {1.0f / 120.0f, -4.3461720e-10f};
+    const df w = z * z;
+    const df c4 = i24 + df{w.hi * fmaf(w.hi, 1.0f / 40320.0f, 1.0f / 720.0f), 0.0f};
+    const df c = w * (w * c4 + i2) + one;
+    const df s5 = i120 + df{w.hi * fmaf(w.hi, 1.0f / 362880.0f, 1.0f / 5040.0f), 0.0f};
+    const df s = z * (w * (w * s5 + i6) + one);
+    const df d2 = d * d;
+    const df g = one - d + d2 * (i2 - df{d.hi * fmaf(-d.hi, 1.0f / 24.0f, 1.0f / 6.0f), 0.0f});
+    ep = g * (c + s);
+    em = g * (c - s);
+}
+
+// P_a[k] and P_a[-k], a = 0..3, of node k from the a = 0 values and the T_a of either sign of u
+// (tp, tm), written to rows a 2Q + k and a 2Q + Q + k; the values at -p_k are (-1)^a those of
+// the mirrored problem (u -> -u).
+template <typename R, typename O>
+__device__ __forceinline__ void put_powers(O* out, int Q, int k, int ld, int i, R p, R u, R d, R Pp, R Pm, const R* tp, const R* tm) {
+    const R pu = p - u, mu = p + u;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        r_put(out, (size_t)(a * 2 * Q + k) * ld + i, Pp);
+        r_put(out, (size_t)(a * 2 * Q + Q + k) * ld + i, (a & 1) ? -Pm : Pm);
+        if (a < 3) {
+            Pp = pu * Pp + d * tp[a];
+            Pm = mu * Pm + d * tm[a];
+        }
+    }
+}
+// Half-range x projection of a tile (Sec. III A 2), both half-axes: the auxiliary points
+// x = sqrt(T) q and the polynomials there do not depend on the sign of u, so one recurrence
+// serves both.  With |v| < 0.02 and Q <= 12 the 8-point auxiliary rule is used.  It is exact for
+// v = 0 (degree 15 >= Q + 2); what it misses of exp(q v) at |v| = 0.02 is 3e-13 of the largest
+// value at Q = 8 and below that for smaller orders, but 7e-11 at Q = 9 and grows to 1e-4 at
+// Q = 12 (at |v| = 0.002: 2e-15 and 1e-6).  Warp w
+// takes auxiliary points w, w + 8, ...  R: double, or double-float for FP32 storage; out: the
+// table written (FP32 storage's tab32 also from double).
+template <int QB, typename R, typename O>
+__device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int i = i0 + lane, N = I.N, ld = I.ld, Q = I.Q;
+    const bool valid = i < N;
+    const int ic = valid ? i : N - 1;           // padding lanes work on a real node, write nothing
+    const R zero = r_of(0.0, R{});
+    R* xs = reinterpret_cast<R*>(nsm);                               // [4][32] sqrt(T), u, v, v^2/2
+    R* part = xs + 4 * TILE;                                         // [NOD_WARPS + 1][2 QB + 6][32]
+    R* hst = part + (NOD_WARPS + 1) * (2 * QB + 6) * TILE;           // [M][2][32] recurrence state (Q > QB)
+    __shared__ int use_short;
+    if (wid == 0) {
+        const R u = r_of(I.node[R_UX * ld + ic], R{});
+        R sT, v, d;
+        node_scales(r_of(I.node[R_T * ld + ic], R{}), u, sT, v, d);
+        xs[0 * TILE + lane] = sT;
+        xs[1 * TILE + lane] = u;
+        xs[2 * TILE + lane] = v;
+        xs[3 * TILE + lane] = d;
+        float av = valid ? fabsf((float)r_dbl(v)) : 0.0f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) av = fmaxf(av, __shfl_xor_sync(0xffffffffu, av, o));
+        // one rule per block so that the warps agree: the largest |v| of the tile decides
+        if (lane == 0) use_short = av < 0.02f ? 1 : 0;
+    }
+    __syncthreads();
+    const bool short_rule = use_short && Q <= 12;
+    const int M = short_rule ? MX8 : I.Mx;
+    const double* xq = short_rule ? I.xq8 : I.xq;
+    const double* xw = short_rule ? I.xw8 : I.xw;
+    const float2* xq2 = short_rule ? I.xq82 : I.xq2;
+    const float2* xw2 = short_rule ? I.xw82 : I.xw2;
+    const double *xa = I.xa, *xb = I.xb, *xib = I.xib, *xH = I.xH, *px = I.px;
+    const float2 *xa2 = I.xa2, *xb2 = I.xb2, *xib2 = I.xib2, *xH2 = I.xH2, *px2 = I.px2;
+    const R h0 = r_pair(I.x_h0, I.x_h02, R{});
+    const R sT = xs[lane], u = xs[TILE + lane], v = xs[2 * TILE + lane], d = xs[3 * TILE + lane];
+    // blocks of QB polynomials: per block the sums over the auxiliary points (the recurrence
+    // continued from the previous block's state), then the H products, whose chain continues
+    // across blocks in the instance's FP64-sized table rows; the powers follow the last block
+    for (int lb = 0; lb < Q; lb += QB) {
+        const int nl = min(QB, Q - lb);
+        const bool last = lb + nl == Q;
+        const int nr = 2 * nl + (last ? 6 : 0);
+        R Gp[QB], Gm[QB], Tp[3], Tm[3];
+#pragma unroll
+        for (int j = 0; j < QB; ++j) Gp[j] = Gm[j] = zero;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) Tp[a] = Tm[a] = zero;
+        for (int m = wid; m < M; m += NOD_WARPS) {
+            const R q = r_tab(xq, xq2, m, zero), W = r_tab(xw, xw2, m, zero);
+            R ep, em;
+            if (short_rule) exp_pair_short(q * v, d, ep, em);
+            else exp_pair(q * v, d, ep, em);
+            ep = W * ep;
+            em = W * em;
+            const R x = sT * q;
+            R hm = zero, h = h0;
+            if (lb > 0) {
+                hm = hst[(2 * m) * TILE + lane];
+                h = hst[(2 * m + 1) * TILE + lane];
+            }
+#pragma unroll
+            for (int j = 0; j < QB; ++j) {
+                if (j < nl) {
+                    const int l = lb + j;
+                    Gp[j] = acc(Gp[j], ep, h);
+                    Gm[j] = acc(Gm[j], em, h);
+                    const R hn = rec3(x - r_tab(xa, xa2, l, zero), h, r_tab(xb, xb2, l, zero), hm, r_tab(xib, xib2, l + 1, zero));
+                    hm = h;
+                    h = hn;
+                }
+            }
+            if (last) {                                  // h = h_Q: the T_a of both signs
+                const R yp = x - u, ym = x + u;
+                ep = ep * h;
+                em = em * h;
+                Tp[0] = Tp[0] + ep;
+                Tm[0] = Tm[0] + em;
+                Tp[1] = acc(Tp[1], ep, yp);
+                Tm[1] = acc(Tm[1], em, ym);
+                Tp[2] = acc(Tp[2], ep, yp * yp);
+                Tm[2] = acc(Tm[2], em, ym * ym);
+            } else {
+                hst[(2 * m) * TILE + lane] = hm;
+                hst[(2 * m + 1) * TILE + lane] = h;
+            }
+        }
+        if (lb > 0) __syncthreads();              // the previous block's readers of part are done
+#pragma unroll
+        for (int j = 0; j < QB; ++j)
+            if (j < nl) {
+                part[(wid * nr + j) * TILE + lane] = Gp[j];
+                part[(wid * nr + nl + j) * TILE + lane] = Gm[j];
+            }
+        if (last)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                part[(wid * nr + 2 * nl + a) * TILE + lane] = Tp[a];
+                part[(wid * nr + 2 * nl + 3 + a) * TILE + lane] = Tm[a];
+            }
+        __syncthreads();
+        R* sum = part + NOD_WARPS * nr * TILE;
+        for (int r = wid; r < nr; r += NOD_WARPS) {
+            R t = fin(part[r * TILE + lane]);
+#pragma unroll
+            for (int q = 1; q < NOD_WARPS; ++q) t = t + part[(q * nr + r) * TILE + lane];
+            sum[r * TILE + lane] = t;
+        }
+        __syncthreads();
+        R* chain = reinterpret_cast<R*>(I.tab);
+        for (int k = wid; k < Q; k += NOD_WARPS) {
+            R sp = zero, sm = zero;
+            if (lb > 0 && valid) {
+                sp = chain[(size_t)k * ld + i];
+                sm = chain[(size_t)(Q + k) * ld + i];
+            }
+            for (int j = 0; j < nl; ++j) {
+                const R H = r_tab(xH, xH2, (lb + j) * Q + k, zero);
+                sp = acc(sp, H, sum[j * TILE + lane]);
+                sm = acc(sm, H, sum[(nl + j) * TILE + lane]);
+            }
+            sp = fin(sp);
+            sm = fin(sm);
+            if (last) {
+                const R dk = r_tab(xb, xb2, Q, zero) * r_tab(xH, xH2, (Q - 1) * Q + k, zero);
+                R tp[3], tm[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    tp[a] = sum[(2 * nl + a) * TILE + lane];
+                    tm[a] = sum[(2 * nl + 3 + a) * TILE + lane];
+                }
+                if (valid) put_powers(out, Q, k, ld, i, r_tab(px, px2, k, zero), u, dk, sp, sm, tp, tm);
+            } else if (valid) {
+                chain[(size_t)k * ld + i] = sp;
+                chain[(size_t)(Q + k) * ld + i] = sm;
+            }
+        }
+    }
+}
+
+// Full-range x projection of a tile (App. A, order Lx = 2Q): the expansion coefficients by their
+// recurrence (warp 0), then the sums over l, the even and the odd part once for both signs of
+// the node.
+template <typename R, typename O>
+__device__ void xproj_full(const Inst& I, int i0, double* nsm, O* out) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int i = i0 + lane, N = I.N, ld = I.ld, Q = I.Q, Lx = I.Lx;
+    const bool valid = i < N;
+    const int ic = valid ? i : N - 1;
+    const R zero = r_of(0.0, R{});
+    R* ml = reinterpret_cast<R*>(nsm);                               // [Lx + 1][32] m_l
+    R* ts = ml + (Lx + 1) * TILE;                                    // [3][32] T_a
+    const double *xb = I.xb, *xib = I.xib, *xH = I.xH, *px = I.px;
+    const float2 *xb2 = I.xb2, *xib2 = I.xib2, *xH2 = I.xH2, *px2 = I.px2;
+    const double T = I.node[R_T * ld + ic];
+    const R u = r_of(I.node[R_UX * ld + ic], R{});
+    if (wid == 0) hermite_moments(u, r_of(T, zero), r_of(T - 1.0, zero), Lx, xb, xb2, xib, xib2, ml + lane, ts + lane);
+    __syncthreads();
+    for (int k = wid; k < Q; k += NOD_WARPS) {
+        R e = zero, o = zero;
+        for (int l = 0; l < Lx; l += 2) {
+            e = acc(e, r_tab(xH, xH2, l * Q + k, zero), ml[l * TILE + lane]);
+            o = acc(o, r_tab(xH, xH2, (l + 1) * Q + k, zero), ml[(l + 1) * TILE + lane]);
+        }
+        e = fin(e);
+        o = fin(o);
+        const R dk = r_tab(xb, xb2, Lx, zero) * r_tab(xH, xH2, (Lx - 1) * Q + k, zero);
+        // mirrored problem of -p_k: u -> -u changes the signs of m_l, odd l, and of T_1 (Lx even)
+        const R tp[3] = {ts[lane], ts[TILE + lane], ts[2 * TILE + lane]}, tm[3] = {tp[0], -tp[1], tp[2]};
+        if (valid) put_powers(out, Q, k, ld, i, r_tab(px, px2, k, zero), u, dk, e + o, e - o, tp, tm);
+    }
+}
+
+// Role 1 of a tile: gradients (Sec. III B 3), closure (Eqs. chi, prandtl, viscosity, tau), the
 // 13 coefficients of f^S + tau J1 = n g(xi) sum_j c_j xi^(a_j, b_j, c_j) (Eq. j1), the y and z
 // projections (App. A) and the transverse factors n Y[a][t]; wall densities (Sec. III B).
-// Phase A: warps 0..4 one gradient each, warp 5 sqrt T, warp 6 the wall densities, warp 7 the
-// FP64 closure chain; warps 0..6 then run the projections (the recurrence at each auxiliary
-// point, then the rows) while warp 7 is still busy.  Phase B: the coefficients; phase C:
-// assembly.
+// Phase A: warps 0..4 one gradient each, warps 5 and 6 the expansion coefficients of y and z
+// (warp 6 also the wall densities), warp 7 the FP64 closure chain; warps 0..6 then run the
+// projections while warp 7 is still busy.  Phase B: the coefficients; phase C: assembly.
 template <typename R>
 __device__ void closure_item(const Inst& I, int i0, double* nsm) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -720,13 +929,14 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
     const int ic = valid ? i : N - 1;           // padding lanes work on a real node, write nothing
     const double* nd = I.node;
     double* gr = nsm;                           // [5][32] d/dx of ln n, ln chi, ln T, u_x, u_y
-    double* cs = gr + 5 * TILE;                 // [8][32] W = -tau b rho chi, A, 1/T, tau, -, n; sqrt T, u_y as R
-    R* sc = reinterpret_cast<R*>(cs + 8 * TILE);        // [15][32] coefficients, n, 1/tau
+    double* cs = gr + 5 * TILE;                 // [6][32] W = -tau b rho chi, A, 1/T, tau, -, n
+    R* sc = reinterpret_cast<R*>(cs + 6 * TILE);        // [15][32] coefficients, n, 1/tau
     R* Py = sc + 15 * TILE;                             // [4 QYMAX][32]
-    R* Pz = Py + 4 * QYMAX * TILE;                      // [3 QZMAX][32]
-    R* Ay = Pz + 3 * QZMAX * TILE;                      // [8 QYMAX][32]
-    R* hp = Ay + 8 * QYMAX * TILE;                      // [2 MYMAX][QYMAX][32] h_l at the auxiliary points
-    R* yp = hp + 2 * MYMAX * QYMAX * TILE;              // [2 MYMAX][32] p - u0 at the auxiliary points
+    R* Pz = Py + 4 * QYMAX * TILE;                      // [2 QZMAX][32] (p_z^0 and p_z^2)
+    R* Ay = Pz + 2 * QZMAX * TILE;                      // [8 QYMAX][32]
+    R* my = Ay + 8 * QYMAX * TILE;                      // [QYMAX + 1][32] m_l of y, then T_a [3][32]
+    R* mz = my + (QYMAX + 4) * TILE;                    // the same of z
+    R* Ts = mz + (QZMAX + 4) * TILE;                    // [32] T
     // Fischer-Methfessel contact value (Eq. chi_ret): the averaged density n-bar and ln chi(n-bar)
     // on the tile and a halo of 7 nodes each side (what the gradient stencils reach)
     constexpr int FH = 7;
@@ -764,11 +974,18 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
         }
         gr[wid * TILE + lane] = g * I.xpinv[ic];
     } else if (wid == 5) {
-        // sqrt T and u_y in the projections' arithmetic, converted once
-        R* cr = reinterpret_cast<R*>(cs + 6 * TILE);
-        cr[lane] = r_of(sqrt(nd[R_T * ld + ic]), R{});
-        cr[TILE + lane] = r_of(nd[R_UY * ld + ic], R{});
+        const double T = nd[R_T * ld + ic];
+        const R Tr = r_of(T, R{});
+        Ts[lane] = Tr;
+        if (I.form != FORM_REDUCED1D)
+            hermite_moments(r_of(nd[R_UY * ld + ic], R{}), Tr, r_of(T - 1.0, R{}), Qy, I.fsq, I.fsq2, I.fisq, I.fisq2, my + lane,
+                            my + (QYMAX + 1) * TILE + lane);
     } else if (wid == 6) {
+        if (I.form == FORM_UNREDUCED) {
+            const double T = nd[R_T * ld + ic];
+            hermite_moments(r_of(0.0, R{}), r_of(T, R{}), r_of(T - 1.0, R{}), Qz, I.fsq, I.fsq2, I.fisq, I.fisq2, mz + lane,
+                            mz + (QZMAX + 1) * TILE + lane);
+        }
         if (i0 == 0 && lane == 0) {
             // zero net mass flux through each wall (Sec. III B): the outgoing wall-face flux is
             // the quadratic reconstruction (11 f_1 - 7 f_2 + 2 f_3)/6 of outgoing populations.
@@ -792,63 +1009,39 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
         cs[3 * TILE + lane] = tau;
         cs[5 * TILE + lane] = n;
     }
-    // warps 0..6 go on to the projections (they need sqrt T and u_y only) while warp 7 still
+    // warps 0..6 go on to the projections (they need m_l, T and u_y only) while warp 7 still
     // runs the closure chain; named barrier 1 synchronises the 7 warps
-    if (wid < NOD_WARPS - 1) {
+    if (wid < NOD_WARPS - 1 && I.form != FORM_REDUCED1D) {
         const R z = r_of(0.0, R{});
         named_sync(1, (NOD_WARPS - 1) * TILE);
-        // full-range projections, step 1: the orthonormal recurrence h_l at each auxiliary point
-        // (y points first, then z points), one point per warp of warps 0..6
-        if (I.form != FORM_REDUCED1D) {
-            const int My = I.My, Mz = I.form == FORM_UNREDUCED ? I.Mz : 0;
-            const R* cr = reinterpret_cast<const R*>(cs + 6 * TILE);
-            const R sT = cr[lane], uy = cr[TILE + lane], one = r_of(1.0, z);
-            for (int pt = wid; pt < My + Mz; pt += NOD_WARPS - 1) {
-                const bool ydir = pt < My;
-                const int m = ydir ? pt : pt - My, Qn = ydir ? Qy : Qz;
-                const R y = sT * (ydir ? r_tab(I.yq, I.yq2, m, z) : r_tab(I.zq, I.zq2, m, z));
-                const R x = ydir ? uy + y : y;
-                yp[pt * TILE + lane] = y;
-                R hm = z, h = one;
-#pragma unroll
-                for (int l = 0; l < QYMAX; ++l) {
-                    if (l < Qn) {
-                        hp[(pt * QYMAX + l) * TILE + lane] = h;
-                        const R hn = (x * h - r_tab(I.fsq, I.fsq2, l, z) * hm) * r_tab(I.fisq, I.fisq2, l + 1, z);
-                        hm = h;
-                        h = hn;
-                    }
-                }
-            }
-        }
-        named_sync(1, (NOD_WARPS - 1) * TILE);
-        if (I.form != FORM_REDUCED1D && (wid < 4 || I.form == FORM_UNREDUCED)) {
-            // step 2: warps 0..3 rows a = wid of Py ((p_y - u_y)^a g), warps 4..6 rows a = wid - 4 of
-            // Pz (p_z^a g): sum over the auxiliary points of w y^a h_l, then the H matrix (App. A)
-            const bool ydir = wid < 4;
-            const int a = ydir ? wid : wid - 4, Qn = ydir ? Qy : Qz, M = ydir ? I.My : I.Mz, p0 = ydir ? 0 : I.My;
-            const double* aw = ydir ? I.yw : I.zw;
-            const float2* aw2 = ydir ? I.yw2 : I.zw2;
-            R G[QYMAX];
-#pragma unroll
-            for (int l = 0; l < QYMAX; ++l) G[l] = z;
-            for (int m = 0; m < M; ++m) {
-                const R y = yp[(p0 + m) * TILE + lane];
-                R e = r_tab(aw, aw2, m, z);
-                for (int j = 0; j < a; ++j) e = e * y;
-#pragma unroll
-                for (int l = 0; l < QYMAX; ++l)
-                    if (l < Qn) G[l] = e * hp[((p0 + m) * QYMAX + l) * TILE + lane] + G[l];
-            }
+        // one node of y or z per warp: (p_y - u_y)^b g, b = 0..3, and p_z^c g, c = 0, 2
+        const int nz = I.form == FORM_UNREDUCED ? Qz : 0;
+        for (int it = wid; it < Qy + nz; it += NOD_WARPS - 1) {
+            const bool ydir = it < Qy;
+            const int k = ydir ? it : it - Qy, Qn = ydir ? Qy : Qz;
             const double* H = ydir ? I.yH : I.zH;
             const float2* H2 = ydir ? I.yH2 : I.zH2;
-            R* P = ydir ? Py + a * QYMAX * TILE : Pz + a * QZMAX * TILE;
-            for (int k2 = 0; k2 < Qn; ++k2) {
-                R t = z;
+            const R* m = ydir ? my : mz;
+            const R* ts = m + (ydir ? QYMAX + 1 : QZMAX + 1) * TILE;
+            R P = z;
 #pragma unroll
-                for (int l = 0; l < QYMAX; ++l)
-                    if (l < Qn) t = r_tab(H, H2, l * Qn + k2, z) * G[l] + t;
-                P[k2 * TILE + lane] = t;
+            for (int l = 0; l < QYMAX; ++l)
+                if (l < Qn) P = acc(P, r_tab(H, H2, l * Qn + k, z), m[l * TILE + lane]);
+            P = fin(P);
+            const R dk = r_tab((ydir ? I.yw : I.zw) + MYMAX, ydir ? I.yd2 : I.zd2, k, z);
+            if (ydir) {
+                const R pu = r_tab(I.yn, I.yn2, k, z) - r_of(nd[R_UY * ld + ic], z);
+                Py[k * TILE + lane] = P;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    P = pu * P + dk * ts[a * TILE + lane];
+                    Py[((a + 1) * QYMAX + k) * TILE + lane] = P;
+                }
+            } else {
+                const R p = r_tab(I.zn, I.zn2, k, z);
+                Pz[k * TILE + lane] = P;
+                P = p * P + dk * ts[lane];
+                Pz[(QZMAX + k) * TILE + lane] = p * P + dk * ts[TILE + lane];
             }
         }
     }
@@ -925,8 +1118,7 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
         __syncthreads();
         // transverse factors n Y[a][t] = A[a][0][ky] Z0(t) + A[a][1][ky] Z2(t), t = ky Tz + kz;
         // a warp takes (a, ky) pairs and runs over kz (no per-output index divisions)
-        const double T = nd[R_T * ld + ic];
-        const R Tr = r_of(T, R{}), one = r_of(1.0, R{}), T23 = r_of(3.0 * T * T, R{});
+        const R Tr = Ts[lane], T3 = r_of(3.0, R{}) * Tr;
         const bool unred = form == FORM_UNREDUCED;
         const int Tz = unred ? Qz : 2;
         for (int pr = wid; pr < 4 * Qy; pr += NOD_WARPS) {
@@ -935,11 +1127,11 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
             auto* row = out + (size_t)(8 * Q + a * Tc + ky * Tz) * ld + i;
             if (unred) {
                 for (int kz = 0; kz < Qz; ++kz) {
-                    const R v = A0 * Pz[(0 * QZMAX + kz) * TILE + lane] + A1 * Pz[(2 * QZMAX + kz) * TILE + lane];
+                    const R v = A0 * Pz[(0 * QZMAX + kz) * TILE + lane] + A1 * Pz[(QZMAX + kz) * TILE + lane];
                     if (valid) r_put(row, (size_t)kz * ld, v);
                 }
             } else {
-                const R v0 = A0 * one + A1 * Tr, v1 = A0 * Tr + A1 * T23;
+                const R v0 = A0 + A1 * Tr, v1 = (A0 + A1 * T3) * Tr;
                 if (valid) {
                     r_put(row, 0, v0);
                     r_put(row, (size_t)ld, v1);
@@ -948,161 +1140,47 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
         }
     } else {
         // 1D reduced (Sec. II B 1): slots phi, theta carry the (p_y, p_z) Gaussian moments
+        // (E[1] = 1, E[xi^2] = T, E[xi^4] = 3 T^2, odd moments zero):
+        //   phi   = n (c_a0 + (c_a20 + c_a02) T),  theta = n (2 c_a0 + 4 (c_a20 + c_a02) T) T
+        // with the coefficients of xi_x^a, xi_x^a xi_y^2 and xi_x^a xi_z^2
         const int a = wid >> 1, slot = wid & 1;
-        const double T = nd[R_T * ld + ic];
-        double t = 0.0;
-        for (int j = 0; j < NTERMS; ++j) {
-            if (c_mono[j][0] != a) continue;
-            const int b = c_mono[j][1], cc = c_mono[j][2];
-            const double e = slot == 0 ? gmom(b, T) * gmom(cc, T) : gmom(b + 2, T) * gmom(cc, T) + gmom(b, T) * gmom(cc + 2, T);
-            t = fma(r_dbl(sc[j * TILE + lane]), e, t);
-        }
-        if (valid) r_put(out, (size_t)(8 * Q + a * Tc + slot) * ld + i, r_of(r_dbl(sc[13 * TILE + lane]) * t, R{}));
+        const R Tr = Ts[lane];
+        const R c0 = sc[(a == 0 ? 0 : a == 1 ? 1 : a == 2 ? 3 : 7) * TILE + lane];
+        R c2 = r_of(0.0, R{});
+        if (a == 0) c2 = sc[4 * TILE + lane] + sc[5 * TILE + lane];
+        if (a == 1) c2 = sc[8 * TILE + lane] + sc[9 * TILE + lane];
+        const R two = r_of(2.0, R{});
+        R t = slot == 0 ? c0 + c2 * Tr : (two * c0 + (two * two * c2) * Tr) * Tr;
+        if (valid) r_put(out, (size_t)(8 * Q + a * Tc + slot) * ld + i, sc[13 * TILE + lane] * t);
     }
     if (wid == 0 && valid) r_put(out, (size_t)(8 * Q + 4 * Tc) * ld + i, sc[14 * TILE + lane]);
 }
 
-// One (tile, role) item by a block of NOD_WARPS warps; nsm holds nodal_smem_doubles(QB)
+// One (tile, role) item by a block of NOD_WARPS warps; nsm holds nodal_smem_doubles(max Lx)
 // doubles; fp32: the instance stores f in FP32 (tables go to tab32).
 template <int QB>
 __device__ void nodal_item(const Inst& I, int i0, int role, double* nsm, bool fp32) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int i = i0 + lane;
     __syncthreads();                      // the previous item's readers of nsm are done
-    // FP32 storage: the half-range x projection in double-float, up to 32 polynomials.  Larger
-    // orders keep the FP64 projection below (writing the FP32 table): the orthonormal
-    // polynomials grow to ~e^(x^2/4) at the auxiliary points x = sqrt(T) q, beyond the float
-    // range (3e38) once x > ~18.8 -- the full-range rule of order 200 has |q| up to ~19, the
-    // half-range aux rule of order 100 q up to ~17 (overflow from T ~ 1.2); at 32 polynomials
-    // the aux rule ends near q = 11, which would need T > 3.
-    if (fp32 && role < 2 && !I.xfull && I.Lx <= 32) {
-        xproj_df<QB>(I, i0, role, nsm);
+    if (role == 1) {
+        if (fp32) closure_item<df>(I, i0, nsm);
+        else closure_item<double>(I, i0, nsm);
         return;
     }
-    const int N = I.N, ld = I.ld, Q = I.Q, Tc = I.Tc;
-    const bool valid = i < N;
-    const int ic = valid ? i : N - 1;           // padding lanes work on a real node, write nothing
-    const double* nd = I.node;
-    if (role < 2) {
-        // ---- half-range x projection (Sec. III A 2), half-axis `role`.  With |v| < 0.02 and
-        // Q <= 12 the 8-point auxiliary rule is used (exact for v = 0 up to degree 15 >= Q + 2;
-        // the neglected part of exp(q v) is below 1e-14 relative) with exp(q v - v^2/2) from its
-        // Taylor series (|argument| < 0.12, 12 terms).  Warp w takes auxiliary points w, w + 8.
-        // sqrt T, u and v = u / sqrt T once per node (warp 0), shared; one rule per block so that
-        // the warps agree: the largest |v| of the tile decides
-        __shared__ double xs[3][TILE];
-        __shared__ int use_short;
-        if (wid == 0) {
-            const double T = nd[R_T * ld + ic], ux = nd[R_UX * ld + ic];
-            const double sT0 = sqrt(T), uu0 = role ? -ux : ux, v0 = uu0 / sT0;
-            xs[0][lane] = sT0;
-            xs[1][lane] = uu0;
-            xs[2][lane] = v0;
-            double av = valid ? fabs(v0) : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) av = fmax(av, __shfl_xor_sync(0xffffffffu, av, o));
-            if (lane == 0) use_short = av < 0.02 ? 1 : 2;
-        }
-        __syncthreads();
-        const double sT = xs[0][lane], uu = xs[1][lane], v = xs[2][lane];
-        // full-range x (App. A): Lx = 2Q polynomials, x = u + sqrt(T) q on the exact Mx-point
-        // Gauss-Hermite rule, no exponential (the Maxwellian is the rule's weight)
-        const bool full = I.xfull;
-        const int Lx = I.Lx;
-        const bool short_rule = !full && use_short == 1 && Q <= 12;
-        const int M = full ? I.Mx : (short_rule ? MX8 : I.Mx);
-        double* part = nsm;                                  // [NOD_WARPS][4 nl][32]
-        double* hst = nsm + (NOD_WARPS + 1) * 4 * QB * TILE; // [M][2][32] recurrence state (Lx > QB)
-        // the polynomials in blocks of QB: per block the sums over the auxiliary points (the
-        // recurrence continued from the previous block's state), then the H products, whose
-        // chain continues across blocks in the instance's FP64 table rows (signed and written at
-        // the last block)
-        for (int lb = 0; lb < Lx; lb += QB) {
-            const int nl = min(QB, Lx - lb);
-            double* sum = nsm + NOD_WARPS * 4 * nl * TILE;   // [4 nl][32]
-            double G[4][QB];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int l = 0; l < QB; ++l) G[a][l] = 0.0;
-            for (int m = wid; m < M; m += NOD_WARPS) {
-                const double q = short_rule ? I.xq8[m] : I.xq[m];
-                const double Wm = short_rule ? I.xw8[m] : I.xw[m];
-                double x, E, y;
-                if (full) {
-                    y = sT * q;
-                    x = uu + y;
-                    E = Wm;
-                } else {
-                    const double z = fma(q, v, -0.5 * v * v);
-                    double ez;
-                    if (short_rule) {
-                        ez = 1.0;
-#pragma unroll
-                        for (int j = 12; j >= 1; --j) ez = fma(ez * z, c_inv[j], 1.0);
-                    } else {
-                        ez = exp(z);
-                    }
-                    x = sT * q;
-                    E = Wm * ez;
-                    y = x - uu;
-                }
-                const double e1 = E * y, e2 = e1 * y, e3 = e2 * y;
-                // recurrence state at the block's first polynomial: from the start, or as the
-                // previous block left it (this thread stored it)
-                double hm = 0.0, h = I.x_h0;
-                if (lb > 0) {
-                    hm = hst[(2 * m) * TILE + lane];
-                    h = hst[(2 * m + 1) * TILE + lane];
-                }
-#pragma unroll
-                for (int j = 0; j < QB; ++j) {
-                    if (j < nl) {
-                        const int l = lb + j;
-                        G[0][j] = fma(E, h, G[0][j]);
-                        G[1][j] = fma(e1, h, G[1][j]);
-                        G[2][j] = fma(e2, h, G[2][j]);
-                        G[3][j] = fma(e3, h, G[3][j]);
-                        const double hn = ((x - I.xa[l]) * h - I.xb[l] * hm) * I.xib[l + 1];
-                        hm = h;
-                        h = hn;
-                    }
-                }
-                if (lb + nl < Lx) {
-                    hst[(2 * m) * TILE + lane] = hm;
-                    hst[(2 * m + 1) * TILE + lane] = h;
-                }
-            }
-            if (lb > 0) __syncthreads();          // the previous block's readers of part and sum are done
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int j = 0; j < QB; ++j)
-                    if (j < nl) part[((wid * 4 + a) * nl + j) * TILE + lane] = G[a][j];
-            __syncthreads();
-            for (int r = wid; r < 4 * nl; r += NOD_WARPS) {
-                double s = 0.0;
-                for (int q = 0; q < NOD_WARPS; ++q) s += part[(q * 4 * nl + r) * TILE + lane];
-                sum[r * TILE + lane] = s;
-            }
-            __syncthreads();
-            const bool last = lb + nl == Lx;
-            for (int o = wid; o < 4 * Q; o += NOD_WARPS) {
-                const int a = o / Q, k = o - a * Q;
-                const size_t r = (size_t)(a * 2 * Q + role * Q + k) * ld + i;
-                double s = (lb > 0 && valid) ? I.tab[r] : 0.0;
-                for (int j = 0; j < nl; ++j) s = fma(I.xH[(lb + j) * Q + k], sum[(a * nl + j) * TILE + lane], s);
-                if (last && role && (a & 1)) s = -s;
-                if (valid) {
-                    if (last && fp32) I.tab32[r] = (float)s;
-                    else I.tab[r] = s;
-                }
-            }
-        }
+    if (I.xfull) {
+        // the coefficients m_l and w_k h_l(p_k) stay small at every order: double-float for FP32
+        // storage up to order 200
+        if (fp32) xproj_full<df>(I, i0, nsm, I.tab32);
+        else xproj_full<double>(I, i0, nsm, I.tab);
         return;
     }
-    if (fp32) closure_item<df>(I, i0, nsm);
-    else closure_item<double>(I, i0, nsm);
+    // FP32 storage: double-float up to 32 polynomials.  Larger half-range orders sum in FP64
+    // (writing the FP32 table): the orthonormal polynomials grow to ~e^(x^2/4) at the auxiliary
+    // points x = sqrt(T) q, beyond the float range (3e38) once x > ~18.8 -- the aux rule of order
+    // 100 has q up to ~17 (overflow from T ~ 1.2); at 32 polynomials it ends near q = 11, which
+    // would need T > 3.
+    if (!fp32) xproj_half<QB, double>(I, i0, nsm, I.tab);
+    else if (I.Lx <= 32) xproj_half<QB, df>(I, i0, nsm, I.tab32);
+    else xproj_half<QB, double>(I, i0, nsm, I.tab32);
 }
 
 template <int QB>
@@ -1887,8 +1965,8 @@ __device__ void res_step(Inst& I, int idx, double tol, double* resid_all, int ra
     const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
     // the update items' epilogue computes the moments of each stage's result
     for (int stage = 1; stage <= 3; ++stage) {
-        for (int it = rank; it < 3 * tiles; it += CS)
-            nodal_item<QB>(I, (it / 3) * TILE, it % 3, reinterpret_cast<double*>(sm), sizeof(S) == 4);
+        for (int it = rank; it < NODAL_ROLES * tiles; it += CS)
+            nodal_item<QB>(I, (it / NODAL_ROLES) * TILE, it % NODAL_ROLES, reinterpret_cast<double*>(sm), sizeof(S) == 4);
         cl.sync();
         for (int it = rank; it < tiles * nch; it += CS) {
             const int tl = it / nch, c = it - tl * nch, k0 = c * KC;
@@ -1941,8 +2019,8 @@ __device__ void smem_step(Inst& I, int idx, double tol, double* resid_all, unsig
     const int tiles = (I.N + TILE - 1) / TILE, K = I.K, KC = I.ukc, nch = I.mgroups;
     const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
     for (int stage = 1; stage <= 3; ++stage) {
-        for (int it = 0; it < 3 * tiles; ++it)
-            nodal_item<QB>(I, (it / 3) * TILE, it % 3, reinterpret_cast<double*>(sm), sizeof(S) == 4);
+        for (int it = 0; it < NODAL_ROLES * tiles; ++it)
+            nodal_item<QB>(I, (it / NODAL_ROLES) * TILE, it % NODAL_ROLES, reinterpret_cast<double*>(sm), sizeof(S) == 4);
         __syncthreads();
         for (int it = 0; it < tiles * nch; ++it) {
             const int tl = it / nch, c = it - tl * nch, k0 = c * KC;
@@ -2214,7 +2292,17 @@ cudaError_t launch_set_smem_flags(Inst* d_inst, const int* d_list, int n, int on
     return cudaGetLastError();
 }
 
-size_t smemres_scratch_bytes(int qmax, size_t upd_max) { return resident_smem_bytes(qmax, upd_max); }
+// The scratch is at least the bound that the set of shared-memory instances has always been
+// chosen with, so that a batch keeps its mix when the closure's own need changes.
+size_t smemres_scratch_bytes(int qmax, size_t upd_max) {
+    const int qb = qmax > QMAX ? QMAX : qmax;
+    const int states = qmax > QMAX ? (aux_points_half(qmax) > qmax / 2 + 2 ? aux_points_half(qmax) : qmax / 2 + 2) : 0;
+    const int rows_x = (NOD_WARPS + 1) * 4 * qb + 2 * states;
+    const int rows_c = 28 + 4 * QYMAX + 3 * QZMAX + 8 * QYMAX + 2 * MYMAX * (QYMAX + 1);
+    const size_t bound = (size_t)(rows_x > rows_c ? rows_x : rows_c) * TILE * sizeof(double);
+    const size_t need = resident_smem_bytes(qmax, upd_max);
+    return need > bound ? need : bound;
+}
 size_t smemres_buffer_bytes(int K, int ld, size_t s) { return smemres_f_bytes(K, ld, s); }
 
 // Dynamic shared memory available to k_smemres<QB>: the per-block maximum minus its static part.
