@@ -507,7 +507,7 @@ Layout layout_of(const fdlb_params& p, int ukc) {
     };
     {
         const size_t s_max = p.precision == FDLB_FP32_STORAGE ? 4 : 8;
-        while (L.ukc > 8 && update_smem_bytes(trows(L.ukc), L.ukc, s_max, s_max) > UPD_SMEM_LIMIT) L.ukc = (L.ukc + 1) / 2;
+        while (L.ukc > 8 && update_smem_bound(trows(L.ukc), L.ukc, s_max) > UPD_SMEM_LIMIT) L.ukc = (L.ukc + 1) / 2;
     }
     L.trows = trows(L.ukc);
     L.groups = (L.K + L.ukc - 1) / L.ukc;
@@ -869,8 +869,8 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
         c->upd_blocks.push_back((int)(wu.size() - nu0));
         c->qmax = std::max(c->qmax, Lx);      // register and shared arrays hold Lx polynomials
         c->ukc_max = std::max(c->ukc_max, L.ukc);
-        if (p.precision != FDLB_FP32_STORAGE) max_smem64 = std::max(max_smem64, update_smem_bytes(L.trows, L.ukc, 8, 8)), c->any_fp64 = true;
-        if (p.precision != FDLB_FP64) max_smem32 = std::max(max_smem32, update_smem_bytes(L.trows, L.ukc, 4, 4)), c->any_fp32 = true;
+        if (p.precision != FDLB_FP32_STORAGE) max_smem64 = std::max(max_smem64, update_smem_bytes(L.trows, L.ukc, 8)), c->any_fp64 = true;
+        if (p.precision != FDLB_FP64) max_smem32 = std::max(max_smem32, update_smem_bytes(L.trows, L.ukc, 4)), c->any_fp32 = true;
     }
     if (off > need) { delete c; return fail(nullptr, FDLB_EINVAL, "internal: workspace layout overflow"); }
     {
@@ -1007,7 +1007,7 @@ static void choose_smem_resident(fdlb_ctx* c) {
         const Inst& I = c->inst[i];
         if (I.two_phase) continue;
         const size_t sz = I.precision == FDLB_FP32_STORAGE ? 4 : 8;
-        const size_t upd = update_smem_bytes(I.trows, I.ukc, sz, sz);
+        const size_t upd = update_smem_bound(I.trows, I.ukc, sz);
         const size_t fb = smemres_buffer_bytes(I.K, I.ld, sz);
         const size_t need = smemres_scratch_bytes(I.Lx, upd) + 3 * fb;
         if (need <= limit) cand.push_back({i, I.Lx, upd, fb, need});

@@ -24,6 +24,7 @@
 // residual in double.
 #include "fdlb_internal.h"
 #include "fdlb_launch.h"
+#include "fdlb_weno.cuh"
 #include "../../include/fdlb.h"
 
 #include <cooperative_groups.h>
@@ -386,53 +387,47 @@ __device__ __forceinline__ df df_of(double x) {
 }
 __device__ __forceinline__ float df_float(df a) { return __fadd_rn(a.hi, a.lo); }
 
+// Arithmetic of the closure item's projections: FP64 for FP64 storage, double-float for FP32
+// storage (whose tables are rounded to FP32).
+__device__ __forceinline__ double r_of(double x, double) { return x; }
+__device__ __forceinline__ df r_of(double x, df) { return df_of(x); }
+__device__ __forceinline__ double r_tab(const double* d, const float2*, int k, double) { return d[k]; }
+__device__ __forceinline__ df r_tab(const double*, const float2* p, int k, df) { return df_of(p[k]); }
+__device__ __forceinline__ double r_dbl(double x) { return x; }
+__device__ __forceinline__ double r_dbl(df x) { return (double)x.hi + (double)x.lo; }
+
+// Output rows of the projection table in the closure's arithmetic type.
+__device__ __forceinline__ double* r_out(const Inst& I, double) { return I.tab; }
+__device__ __forceinline__ float* r_out(const Inst& I, df) { return I.tab32; }
+__device__ __forceinline__ void r_put(double* p, size_t r, double v) { p[r] = v; }
+__device__ __forceinline__ void r_put(float* p, size_t r, df v) { p[r] = df_float(v); }
+__device__ __forceinline__ void r_put(float* p, size_t r, double v) { p[r] = (float)v; }
+
 constexpr int NTW = 6;     // transverse weights: mt, mt py, mt py^2, mt py^3, et, et py
 
-// Inner (transverse) running sum of w(t) f over t.  FP64 storage: an FP64 FMA.  FP32
-// storage: an unevaluated pair hi + lo of floats (error-free product of f with the float
-// head of w, the tail of w applied in float, TwoSum accumulation), ~1e-13 relative.
-template <typename S>
-struct InnerSum;
-
-template <>
-struct InnerSum<double> {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double f, double w, float, float) { s = fma(w, f, s); }
-    __device__ __forceinline__ double value() const { return s; }
-};
-
-template <>
-struct InnerSum<float> {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float f, double, float wh, float wl) {
-        const float p = f * wh;
-        float e = fmaf(f, wh, -p);
-        e = fmaf(f, wl, e);
-        const float t = hi + p;
-        const float bb = t - hi;
-        const float err = (hi - (t - bb)) + (p - bb);
-        hi = t;
-        lo += err + e;
-    }
-    // adds a value known exactly (a product by a power of two), TwoSum on the head: the same
-    // result as add() with a zero product error
-    __device__ __forceinline__ void add_exact(float p) {
-        const float t = hi + p;
-        const float bb = t - hi;
-        const float err = (hi - (t - bb)) + (p - bb);
-        hi = t;
-        lo += err;
-    }
-    // adds another pair's value h + l (TwoSum on the heads)
-    __device__ __forceinline__ void add_pair(float h, float l) {
-        const float t = hi + h;
-        const float bb = t - hi;
-        const float err = (hi - (t - bb)) + (h - bb);
-        hi = t;
-        lo += err + l;
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
+// Terms of the moment sums in the two arithmetics: FP64, and unnormalised float pairs for FP32
+// storage (error-free sums and products, ~1e-13 relative).
+__device__ __forceinline__ df plus(df s, df a) {                // s + a, unnormalised
+    const float t = __fadd_rn(s.hi, a.hi);
+    const float bb = __fsub_rn(t, s.hi);
+    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, bb)), __fsub_rn(a.hi, bb));
+    return {t, __fadd_rn(s.lo, __fadd_rn(err, a.lo))};
+}
+__device__ __forceinline__ double plus(double s, double a) { return s + a; }
+__device__ __forceinline__ df plus(df s, float f) {
+    const float t = __fadd_rn(s.hi, f);
+    const float bb = __fsub_rn(t, s.hi);
+    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, bb)), __fsub_rn(f, bb));
+    return {t, __fadd_rn(s.lo, err)};
+}
+__device__ __forceinline__ df acc(df s, float f, df w) {        // s + f w
+    const float p = __fmul_rn(f, w.hi);
+    const float e = __fmaf_rn(f, w.lo, __fmaf_rn(f, w.hi, -p));
+    const float t = __fadd_rn(s.hi, p);
+    const float bb = __fsub_rn(t, s.hi);
+    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, bb)), __fsub_rn(p, bb));
+    return {t, __fadd_rn(s.lo, __fadd_rn(err, e))};
+}
 
 // Per node: the 14 raw sums over all velocities, factorised as sum_kx px^a (sum_t w_j(t) f),
 // and the moments they give.
@@ -498,41 +493,26 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 
-// Adds the x-velocity p's contribution to the 14 raw sums from the 6 transverse sums S.
-__device__ __forceinline__ void outer_sums(double* o, const double* S, double p, bool neg) {
-    const double p2 = p * p, p3 = p2 * p;
-    o[0] += S[0];
-    if (neg) o[1] = fma(p, S[0], o[1]); else o[2] = fma(p, S[0], o[2]);
-    o[3] += S[1];
-    o[4] = fma(p2, S[0], o[4]);
-    o[5] = fma(p, S[1], o[5]);
-    o[6] += S[2];
-    o[7] += S[4];
-    o[8] = fma(p3, S[0], o[8]);
-    o[9] = fma(p, S[2], o[9]);
-    o[10] = fma(p2, S[1], o[10]);
-    o[11] += S[3];
-    o[12] = fma(p, S[4], o[12]);
-    o[13] += S[5];
-}
-
-
-// Outer sums in double-float (FP32 storage): as outer_sums, p and S as float pairs.
-__device__ __forceinline__ void outer_sums_df(df* o, const df* S, df p, bool neg) {
-    const df p2 = p * p, p3 = p2 * p;
-    o[0] = o[0] + S[0];
-    if (neg) o[1] = p * S[0] + o[1]; else o[2] = p * S[0] + o[2];
-    o[3] = o[3] + S[1];
-    o[4] = p2 * S[0] + o[4];
-    o[5] = p * S[1] + o[5];
-    o[6] = o[6] + S[2];
-    o[7] = o[7] + S[4];
-    o[8] = p3 * S[0] + o[8];
-    o[9] = p * S[2] + o[9];
-    o[10] = p2 * S[1] + o[10];
-    o[11] = o[11] + S[3];
-    o[12] = p * S[4] + o[12];
-    o[13] = o[13] + S[5];
+// Adds the x-velocity p's contribution to the 14 raw sums from its 6 transverse sums S; ydep: some
+// transverse index has p_y (else the sums with p_y stay zero).
+template <typename R>
+__device__ __forceinline__ void outer_sums(R* o, const R* S, R p, bool neg, bool ydep) {
+    const R p2 = p * p, p3 = p2 * p;
+    o[0] = plus(o[0], S[0]);
+    if (neg) o[1] = acc(o[1], p, S[0]); else o[2] = acc(o[2], p, S[0]);
+    o[4] = acc(o[4], p2, S[0]);
+    o[7] = plus(o[7], S[4]);
+    o[8] = acc(o[8], p3, S[0]);
+    o[12] = acc(o[12], p, S[4]);
+    if (ydep) {
+        o[3] = plus(o[3], S[1]);
+        o[5] = acc(o[5], p, S[1]);
+        o[6] = plus(o[6], S[2]);
+        o[9] = acc(o[9], p, S[2]);
+        o[10] = acc(o[10], p2, S[1]);
+        o[11] = plus(o[11], S[3]);
+        o[13] = plus(o[13], S[5]);
+    }
 }
 
 // Moments of tile i0 from the I.mgroups partials of its update chunks, added in chunk order,
@@ -621,22 +601,6 @@ __device__ __forceinline__ df df_exp(df z) {
     const int ki = (int)k;
     return {ldexpf(e.hi, ki), ldexpf(e.lo, ki)};
 }
-
-// Arithmetic of the closure item's projections: FP64 for FP64 storage, double-float for FP32
-// storage (whose tables are rounded to FP32).
-__device__ __forceinline__ double r_of(double x, double) { return x; }
-__device__ __forceinline__ df r_of(double x, df) { return df_of(x); }
-__device__ __forceinline__ double r_tab(const double* d, const float2*, int k, double) { return d[k]; }
-__device__ __forceinline__ df r_tab(const double*, const float2* p, int k, df) { return df_of(p[k]); }
-__device__ __forceinline__ double r_dbl(double x) { return x; }
-__device__ __forceinline__ double r_dbl(df x) { return (double)x.hi + (double)x.lo; }
-
-// Output rows of the projection table in the closure's arithmetic type.
-__device__ __forceinline__ double* r_out(const Inst& I, double) { return I.tab; }
-__device__ __forceinline__ float* r_out(const Inst& I, df) { return I.tab32; }
-__device__ __forceinline__ void r_put(double* p, size_t r, double v) { p[r] = v; }
-__device__ __forceinline__ void r_put(float* p, size_t r, df v) { p[r] = df_float(v); }
-__device__ __forceinline__ void r_put(float* p, size_t r, double v) { p[r] = (float)v; }
 
 __device__ __forceinline__ double r_pair(double d, float2, double) { return d; }
 __device__ __forceinline__ df r_pair(double, float2 p, df) { return df_of(p); }
@@ -1352,83 +1316,6 @@ __global__ void __launch_bounds__(256) k_resid(Inst* insts, int anchor, double t
 // update: WENO-5 advection + walls + force + relaxation + RK3 combination
 // ---------------------------------------------------------------------------
 
-// Upwind-biased WENO-5 face value from (f_{i-2}, f_{i-1}, f_i, f_{i+1}, f_{i+2}) taken in the
-// upwind direction (Sec. III B 2).  Weights delta_q/phi_q^2 without epsilon; a vanishing
-// indicator takes the weight in the limit (the normalised weights are continuous there).
-__device__ __forceinline__ double weno_face(double a, double b, double c, double d, double e) {
-    const double F1 = fma(1.0 / 3.0, a, fma(-7.0 / 6.0, b, 11.0 / 6.0 * c));
-    const double F2 = fma(-1.0 / 6.0, b, fma(5.0 / 6.0, c, 1.0 / 3.0 * d));
-    const double F3 = fma(1.0 / 3.0, c, fma(5.0 / 6.0, d, -1.0 / 6.0 * e));
-    const double t1 = a - 2.0 * b + c, t2 = a - 4.0 * b + 3.0 * c;
-    const double u1 = b - 2.0 * c + d, u2 = b - d;
-    const double v1 = c - 2.0 * d + e, v2 = 3.0 * c - 4.0 * d + e;
-    const double s1 = fma(13.0 / 12.0, t1 * t1, 0.25 * t2 * t2);
-    const double s2 = fma(13.0 / 12.0, u1 * u1, 0.25 * u2 * u2);
-    const double s3 = fma(13.0 / 12.0, v1 * v1, 0.25 * v2 * v2);
-    const double smax = fmax(s1, fmax(s2, s3));
-    double w1, w2, w3;
-    if (smax == 0.0) {
-        w1 = 0.1; w2 = 0.6; w3 = 0.3;
-    } else {
-        // omega_q ~ delta_q / phi_q^2 ~ delta_q prod_{r != q} phi_r^2 (phi scaled by the max)
-        const double r = 1.0 / smax;
-        const double a1 = s1 * r, a2 = s2 * r, a3 = s3 * r;
-        const double p1 = a1 * a1, p2 = a2 * a2, p3 = a3 * a3;
-        w1 = 0.1 * p2 * p3;
-        w2 = 0.6 * p1 * p3;
-        w3 = 0.3 * p1 * p2;
-        double sum = w1 + w2 + w3;
-        if (sum == 0.0) {
-            // two indicators vanish (or underflow): weight on the smallest ones
-            const double smin = fmin(s1, fmin(s2, s3));
-            w1 = s1 == smin ? 0.1 : 0.0;
-            w2 = s2 == smin ? 0.6 : 0.0;
-            w3 = s3 == smin ? 0.3 : 0.0;
-            sum = w1 + w2 + w3;
-        }
-        const double is = 1.0 / sum;
-        w1 *= is; w2 *= is; w3 *= is;
-    }
-    return fma(w1, F1, fma(w2, F2, w3 * F3));
-}
-
-__device__ __forceinline__ float weno_face(float a, float b, float c, float d, float e) {
-    const float F1 = fmaf(1.0f / 3.0f, a, fmaf(-7.0f / 6.0f, b, 11.0f / 6.0f * c));
-    const float F2 = fmaf(-1.0f / 6.0f, b, fmaf(5.0f / 6.0f, c, 1.0f / 3.0f * d));
-    const float F3 = fmaf(1.0f / 3.0f, c, fmaf(5.0f / 6.0f, d, -1.0f / 6.0f * e));
-    const float t1 = a - 2.0f * b + c, t2 = a - 4.0f * b + 3.0f * c;
-    const float u1 = b - 2.0f * c + d, u2 = b - d;
-    const float v1 = c - 2.0f * d + e, v2 = 3.0f * c - 4.0f * d + e;
-    const float s1 = fmaf(13.0f / 12.0f, t1 * t1, 0.25f * t2 * t2);
-    const float s2 = fmaf(13.0f / 12.0f, u1 * u1, 0.25f * u2 * u2);
-    const float s3 = fmaf(13.0f / 12.0f, v1 * v1, 0.25f * v2 * v2);
-    const float smax = fmaxf(s1, fmaxf(s2, s3));
-    float w1, w2, w3;
-    if (smax < 1e-30f) {
-        // uniform to FP32 resolution (indicators zero or below any meaningful difference): the
-        // candidates agree, the ideal weights are the limit
-        w1 = 0.1f; w2 = 0.6f; w3 = 0.3f;
-    } else {
-        // omega_q ~ delta_q / phi_q^2 ~ delta_q prod_{r != q} phi_r^2, phi scaled by the largest
-        // (one reciprocal; fast division: the FP32 form's tolerance is far above its error)
-        const float r = __fdividef(1.0f, smax);
-        const float a1 = s1 * r, a2 = s2 * r, a3 = s3 * r;
-        const float p1 = a1 * a1, p2 = a2 * a2, p3 = a3 * a3;
-        w1 = 0.1f * p2 * p3;
-        w2 = 0.6f * p1 * p3;
-        w3 = 0.3f * p1 * p2;
-        if (w1 + w2 + w3 < 1e-30f) {
-            // two indicators vanish relative to the third (or underflow): weight on the smallest
-            const float smin = fminf(s1, fminf(s2, s3));
-            w1 = s1 == smin ? 0.1f : 0.0f;
-            w2 = s2 == smin ? 0.6f : 0.0f;
-            w3 = s3 == smin ? 0.3f : 0.0f;
-        }
-    }
-    const float is = __fdividef(1.0f, w1 + w2 + w3);
-    return fmaf(w1 * is, F1, fmaf(w2 * is, F2, w3 * is * F3));
-}
-
 constexpr int UPD_WARPS = 8;          // warps of an update block; the moment epilogue's partials
 constexpr int UPD_WARPS_WIDE = 16;    // wide update blocks: the velocity loop on 16 warps
 
@@ -1463,21 +1350,19 @@ __device__ __forceinline__ uint32_t sr_seed(const Inst& I, int stage) {
 
 // base + inc stored as a float: the exact sum s + err (TwoSum) goes to its round-to-nearest
 // value s, or to the neighbouring float on the side of err with probability |err| / gap, so
-// that its expectation is the exact sum.
+// that its expectation is the exact sum: err plus a uniform number of (-gap/2, gap/2) added to s
+// rounds to the neighbour exactly with that probability (gap = the last place of s; at a power of
+// two the finer grid below takes part of it, and below 2^-103 the sum is rounded to nearest).
+// 15 instructions, no branch and no integer-to-float conversion, against 25 for comparing a
+// uniform number with |err| / gap.
 __device__ __forceinline__ float sr_add(float base, float inc, uint32_t bits) {
     const float s = __fadd_rn(base, inc);
     const float bb = __fsub_rn(s, base);
     const float err = __fadd_rn(__fsub_rn(base, __fsub_rn(s, bb)), __fsub_rn(inc, bb));
-    if (err == 0.0f) return s;
-    // the neighbouring float on the side of err: one unit in the last place of s's magnitude
-    // bits, up when s and err have the same sign, down otherwise (s = 0: the smallest
-    // subnormal with err's sign)
-    const uint32_t sb = __float_as_uint(s);
-    const float nb = s == 0.0f ? copysignf(__uint_as_float(1u), err)
-                               : __uint_as_float((s > 0.0f) == (err > 0.0f) ? sb + 1u : sb - 1u);
-    const float gap = fabsf(__fsub_rn(nb, s));
-    const float u = __uint2float_rz(bits >> 8) * 0x1p-24f;        // uniform on [0, 1), exact
-    return __fmul_rn(u, gap) < fabsf(err) ? nb : s;
+    const float gap = __int_as_float(max((int)(__float_as_uint(s) & 0x7f800000u) - (23 << 23), 0));
+    // uniform on [-1/2, 1/2), shifted by half a step so that it is symmetric
+    const float u = __fadd_rn(__uint_as_float(0x3f800000u | (bits >> 9)), -1.49999994f);
+    return __fadd_rn(s, err == 0.0f ? 0.0f : __fmaf_rn(u, gap, err));
 }
 
 // Tables read by the update kernel in its compute type (FP32 copies for FP32 storage).
@@ -1502,24 +1387,20 @@ struct Tabs<float> {
     __device__ static const float* Ky(const Inst& I) { return I.Ky32; }
 };
 
-// Shared memory of one update item: the projection table, the transverse moment weights, the
-// staged source rows of the chunk (each with a 4-node halo on either side: 40 values per row;
-// the epilogue's per-warp sums reuse this space once the rows are consumed), and the step's F
+// Shared memory of one update item: the transverse moment weights; the projection table and the
+// staged source rows of the chunk (each with a 4-node halo on either side: 40 values per row),
+// whose space the epilogue's per-warp sums reuse once both are consumed; and the step's F
 // values, which the outputs replace (the epilogue reads them there).
 constexpr size_t TW_BYTES = (size_t)NTW * TCMAX * sizeof(double);
 constexpr int SW = 40;                // staged row: nodes i0 - 4 .. i0 + 35
-__host__ __device__ inline size_t upd_table_bytes(int ntab, size_t c) { return ((size_t)ntab * TILE * c + 15) / 16 * 16; }
+__host__ __device__ inline size_t upd_table_bytes(int trows, size_t s) { return ((size_t)trows * TILE * s + 15) / 16 * 16; }
 __host__ __device__ inline size_t upd_ex_bytes() { return (size_t)(UPD_WARPS + 1) * MOM_SUMS * TILE * sizeof(double); }
-__host__ __device__ inline size_t upd_stage_bytes(int ukc, size_t s) {
-    const size_t rows = (size_t)ukc * SW * s, ex = upd_ex_bytes();
-    return ((rows > ex ? rows : ex) + 15) / 16 * 16;
+__host__ __device__ inline size_t upd_fo_offset(int trows, int ukc, size_t s) {
+    const size_t rows = upd_table_bytes(trows, s) + (size_t)ukc * SW * s, ex = upd_ex_bytes();
+    return TW_BYTES + ((rows > ex ? rows : ex) + 15) / 16 * 16;
 }
-__host__ __device__ inline size_t upd_stage_offset(int ntab, size_t c) { return upd_table_bytes(ntab, c) + TW_BYTES; }
-__host__ __device__ inline size_t upd_fo_offset(int ntab, int ukc, size_t c, size_t s) {
-    return upd_stage_offset(ntab, c) + upd_stage_bytes(ukc, s);
-}
-__host__ __device__ inline size_t upd_smem_bytes(int ntab, int ukc, size_t c, size_t s) {
-    return upd_fo_offset(ntab, ukc, c, s) + (size_t)ukc * TILE * s;
+__host__ __device__ inline size_t upd_smem_bytes(int trows, int ukc, size_t s) {
+    return upd_fo_offset(trows, ukc, s) + (size_t)ukc * TILE * s;
 }
 
 // Transverse moment weights of the epilogue into shared memory (FP32 storage: float heads
@@ -1539,96 +1420,95 @@ __device__ __forceinline__ void load_tw(const Inst& I, void* tws, int tid, int n
     }
 }
 
+__device__ __forceinline__ double mom_w(const double* tw, int, int e, double) { return tw[e]; }
+__device__ __forceinline__ df mom_w(const double* tw, int n, int e, df) {
+    const float* h = reinterpret_cast<const float*>(tw);
+    return {h[e], h[n + e]};
+}
+__device__ __forceinline__ df mom_of(float f) { return {f, 0.0f}; }
+__device__ __forceinline__ double mom_of(double f) { return f; }
+
 // Epilogue of an update item: raw moment sums of the chunk's values fo[k - k0][lane] with the
-// factorisation of the moments (per x-velocity the transverse sums, then the outer sums over
-// x-velocities; FP32 pairs and double-float for FP32 storage), summed over the warps, then
-// the moments (one chunk per tile) or the chunk's partial sums in msum[grp].
+// factorisation of the moments, summed over the warps, then the moments (one chunk per tile) or
+// the chunk's partial sums in msum[grp].  The weights factor as well: over the p_z values of a
+// p_y (or its two reduced slots) only A = sum f and B = sum e_z f are formed (the mass and the
+// internal energy), then the 6 transverse sums A, y A, y^2 A, y^3 A, B, y B once per p_y, then
+// the outer sums once per x-velocity: 2 + 6/Q_z terms per value instead of 6 (3 for the reduced
+// slots, without the zero-weight tests).
 template <typename S>
 __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, const S* fo, double* ex, const void* tws,
                               int lane, int wy, int nwb = UPD_WARPS) {
+    using R = decltype(mom_of(S{}));
     const int i = i0 + lane, ld = I.ld, Tc = I.Tc, Q = I.Q, G = I.mgroups;
     const bool valid = i < I.N;
+    const bool unred = I.form == FORM_UNREDUCED, ydep = I.form != FORM_REDUCED1D;
+    const int Tz = unred ? I.Qz : 2, ntw = NTW * Tc;
+    const double* tw = static_cast<const double*>(tws);
+    const R zero = mom_of((S)0);
     // warp wy < UPD_WARPS takes the velocities [ka, kb) of the chunk (warps beyond, in a wide
     // block, take none and only join the cross-warp sums: the same arithmetic in any block)
     const int per = (k1 - k0 + UPD_WARPS - 1) / UPD_WARPS;
     const int ka = min(k1, k0 + wy * per), kb = min(k1, ka + per);
     double* ss = ex + UPD_WARPS * MOM_SUMS * TILE;
-    if constexpr (sizeof(S) == 4) {
-        df o[MOM_SUMS];
+    R o[MOM_SUMS];
 #pragma unroll
-        for (int j = 0; j < MOM_SUMS; ++j) o[j] = {0.0f, 0.0f};
-        for (int kk = ka; kk < kb;) {
-            const int kx = kk / Tc, ta = kk - kx * Tc, tb = min(Tc, kb - kx * Tc);
-            kk = kx * Tc + tb;
-            const float* twh = static_cast<const float*>(tws);
-            const float* twl = twh + NTW * Tc;
-            InnerSum<float> a[NTW];
-            for (int t = ta; t < tb; ++t) {
-                const float fv = fo[(kx * Tc + t - k0) * TILE + lane];
+    for (int j = 0; j < MOM_SUMS; ++j) o[j] = zero;
+    int kx = ka / Tc, t = ka - kx * Tc;
+    const S* fr = fo + (ka - k0) * TILE + lane;
+    for (int kk = ka; kk < kb; ++kx, t = 0) {
+        const int tb = min(Tc, t + (kb - kk));
+        kk += tb - t;
+        R Sv[NTW];
 #pragma unroll
-                for (int j = 0; j < NTW; ++j) {
-                    // the weight is the same for every lane: zero weights (the mass and energy
-                    // flags of the reduced slots) are skipped, power-of-two weights with no
-                    // tail give exact products; both leave the sum's bits as add() would
-                    const float wh = twh[j * Tc + t], wl = twl[j * Tc + t];
-                    if (wh == 0.0f) continue;
-                    if (wl == 0.0f && (__float_as_uint(wh) & 0x007fffffu) == 0u) a[j].add_exact(fv * wh);
-                    else a[j].add(fv, 0.0, wh, wl);
+        for (int j = 0; j < NTW; ++j) Sv[j] = zero;
+        while (t < tb) {
+            const int ky = t / Tz, ty = ky * Tz, te = min(tb, ty + Tz);
+            R A = zero, B = zero;
+            if (unred) {
+                A = mom_of(*fr);
+                B = acc(zero, *fr, mom_w(tw, ntw, 4 * Tc + t, R{}));
+                fr += TILE;
+                for (++t; t < te; ++t, fr += TILE) {
+                    A = plus(A, *fr);
+                    B = acc(B, *fr, mom_w(tw, ntw, 4 * Tc + t, R{}));
+                }
+            } else {
+                if (t == ty) {
+                    A = mom_of(*fr);
+                    fr += TILE;
+                    ++t;
+                }
+                if (t < te) {
+                    B = mom_of((S)0.5 * *fr);
+                    fr += TILE;
+                    ++t;
                 }
             }
-            df Sd[NTW];
-#pragma unroll
-            for (int j = 0; j < NTW; ++j) Sd[j] = df_norm(a[j].hi, a[j].lo);
-            outer_sums_df(o, Sd, df_of(I.px2[kx]), kx >= Q);
-        }
-        float2* pe = reinterpret_cast<float2*>(ex);
-        if (wy < UPD_WARPS)
-#pragma unroll
-            for (int j = 0; j < MOM_SUMS; ++j) pe[(wy * MOM_SUMS + j) * TILE + lane] = make_float2(o[j].hi, o[j].lo);
-        __syncthreads();
-        for (int j = wy; j < MOM_SUMS; j += nwb) {
-            df v = {0.0f, 0.0f};
-            for (int q = 0; q < UPD_WARPS; ++q) v = v + df_of(pe[(q * MOM_SUMS + j) * TILE + lane]);
-            if (G > 1) {
-                if (valid) reinterpret_cast<float2*>(I.msum)[((size_t)grp * MOM_SUMS + j) * ld + i] = make_float2(v.hi, v.lo);
-            } else {
-                ss[j * TILE + lane] = (double)v.hi + (double)v.lo;
+            Sv[0] = plus(Sv[0], A);
+            Sv[4] = plus(Sv[4], B);
+            if (ydep) {
+                const R y = mom_w(tw, ntw, Tc + ty, R{});
+                Sv[1] = acc(Sv[1], A, y);
+                Sv[2] = acc(Sv[2], A, mom_w(tw, ntw, 2 * Tc + ty, R{}));
+                Sv[3] = acc(Sv[3], A, mom_w(tw, ntw, 3 * Tc + ty, R{}));
+                Sv[5] = acc(Sv[5], B, y);
             }
         }
-    } else {
-        double o[MOM_SUMS];
+        outer_sums(o, Sv, r_tab(I.px, I.px2, kx, R{}), kx >= Q, ydep);
+    }
+    R* pe = reinterpret_cast<R*>(ex);
+    if (wy < UPD_WARPS)
 #pragma unroll
-        for (int j = 0; j < MOM_SUMS; ++j) o[j] = 0.0;
-        for (int kk = ka; kk < kb;) {
-            const int kx = kk / Tc, ta = kk - kx * Tc, tb = min(Tc, kb - kx * Tc);
-            kk = kx * Tc + tb;
-            const double* tw = static_cast<const double*>(tws);
-            InnerSum<double> a[NTW];
-            for (int t = ta; t < tb; ++t) {
-                const double fv = fo[(kx * Tc + t - k0) * TILE + lane];
+        for (int j = 0; j < MOM_SUMS; ++j) pe[(wy * MOM_SUMS + j) * TILE + lane] = fin(o[j]);
+    __syncthreads();
+    for (int j = wy; j < MOM_SUMS; j += nwb) {
+        R v = pe[j * TILE + lane];
 #pragma unroll
-                for (int j = 0; j < NTW; ++j) {
-                    const double w = tw[j * Tc + t];
-                    if (w != 0.0) a[j].add(fv, w, 0.0f, 0.0f);     // same for every lane
-                }
-            }
-            double Sv[NTW];
-#pragma unroll
-            for (int j = 0; j < NTW; ++j) Sv[j] = a[j].value();
-            outer_sums(o, Sv, I.px[kx], kx >= Q);
-        }
-        if (wy < UPD_WARPS)
-#pragma unroll
-            for (int j = 0; j < MOM_SUMS; ++j) ex[(wy * MOM_SUMS + j) * TILE + lane] = o[j];
-        __syncthreads();
-        for (int j = wy; j < MOM_SUMS; j += nwb) {
-            double v = 0.0;
-            for (int q = 0; q < UPD_WARPS; ++q) v += ex[(q * MOM_SUMS + j) * TILE + lane];
-            if (G > 1) {
-                if (valid) I.msum[((size_t)grp * MOM_SUMS + j) * ld + i] = v;
-            } else {
-                ss[j * TILE + lane] = v;
-            }
+        for (int q = 1; q < UPD_WARPS; ++q) v = v + pe[(q * MOM_SUMS + j) * TILE + lane];
+        if (G > 1) {
+            if (valid) reinterpret_cast<R*>(I.msum)[((size_t)grp * MOM_SUMS + j) * ld + i] = v;
+        } else {
+            ss[j * TILE + lane] = r_dbl(v);
         }
     }
     if (G > 1) return;
@@ -1740,22 +1620,51 @@ __device__ bool stage_rows(const Inst& I, int i0, int k0, int nrows, int stage, 
     }
 }
 
-// Velocities [k0, k1) of one tile for RK stage `stage`, by W warps (lane, warp wy; the
-// velocity loop on all W, the moment partials on UPD_WARPS of them, so that W = 8 and 16 give
-// the same results bit for bit);
-// smem_raw holds upd_smem_bytes(ntab, ukc, sizeof(C), sizeof(S)).  The chunk's source rows (and
-// F) are staged in shared memory first (stage_rows); the stencil, the ghost cells of the diffuse
-// walls and F are then read from there.  The epilogue computes the moments of the new values
-// (chunk_moments).  Returns false when the staging copies failed.
-template <typename S, typename C, bool BULK, int W = UPD_WARPS>
+// RK3 combination of a new value (Eq. rk3) from f, the step's F and inc = cb dt L: FP64 cb f + inc
+// + ca F, two roundings of the size of f; FP32 as an increment of F, F + cb ((f - F) + dt L)
+// (stage 1: f + dt L).  In the printed form ca F + cb (f +
+// dt L) the rounded weights (float) 1/3 + (float) 2/3 = 1 + 3e-8 scale a steady f up by half an
+// ulp every step, a mass drift of ~1e-3 over a solve; the increment form has no such bias.  The
+// FP32 sum is stored with stochastic rounding (sr_add).
+struct Stage {
+    double ca, cb;
+    bool first;
+    uint32_t seed;
+};
+__device__ __forceinline__ double rk_combine(const Stage& g, double fi, double F, double inc, uint32_t) {
+    return g.first ? fi + inc : fma(g.ca, F, fma(g.cb, fi, inc));
+}
+__device__ __forceinline__ float rk_combine(const Stage& g, float fi, float F, float inc, uint32_t e) {
+    const float cb = (float)g.cb;
+    const float base = g.first ? fi : F;
+    if (!g.first) inc = fmaf(cb, fi - F, inc);
+    return sr_add(base, inc, fmix32(e ^ g.seed));
+}
+
+// Velocities [k0, k1) of one tile for RK stage `stage`, by W warps (lane, warp wy; the moment
+// partials on UPD_WARPS of them, so that W = 8 and 16 give the same results bit for bit);
+// smem_raw holds upd_smem_bytes(trows, ukc, sizeof(S)).  The chunk's source rows (and F) are
+// staged in shared memory first (stage_rows).  Each warp then takes a contiguous range of at most
+// 32 velocities: with one lane per velocity it writes the ghost cells of the diffuse walls into
+// its rows and computes the faces that the node-per-lane loop cannot share (the left face of the
+// tile's first node, and the wall face), so that the loop itself is the same for every tile: five
+// stencil values, one face per lane, the left face from the neighbouring lane.  The epilogue
+// computes the moments of the new values (chunk_moments).  Returns false when the staging copies
+// failed.
+// What bounds it: FP64 storage, the FP64 pipe (21 FP64 instructions per node-velocity and stage
+// before the moments, from ~170: the first node's left face had cost a second whole face
+// evaluation per warp, now one per 32 velocities, and see fdlb_weno.cuh); FP32 storage, the
+// instructions issued.
+template <typename S, bool BULK, int W = UPD_WARPS>
 __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, unsigned char* smem_raw, int lane, int wy) {
-    C* stab = reinterpret_cast<C*>(smem_raw);
-    void* tws = smem_raw + upd_table_bytes(I.trows, sizeof(C));
-    S* Sw = reinterpret_cast<S*>(smem_raw + upd_stage_offset(I.trows, sizeof(C)));
-    double* ex = reinterpret_cast<double*>(Sw);                 // after the rows are consumed
-    S* fo = reinterpret_cast<S*>(smem_raw + upd_fo_offset(I.trows, I.ukc, sizeof(C), sizeof(S)));
-    const int i = i0 + lane;
+    using C = S;
     const int N = I.N, ld = I.ld, Q = I.Q, Tc = I.Tc, trows = I.trows;
+    void* tws = smem_raw;
+    C* stab = reinterpret_cast<C*>(smem_raw + TW_BYTES);
+    S* Sw = reinterpret_cast<S*>(smem_raw + TW_BYTES + upd_table_bytes(trows, sizeof(C)));
+    double* ex = reinterpret_cast<double*>(stab);               // after table and rows are consumed
+    S* fo = reinterpret_cast<S*>(smem_raw + upd_fo_offset(trows, I.ukc, sizeof(S)));
+    const int i = i0 + lane;
     // compact table: the x-projection rows of the NKX x-velocities from kx0 on (the chunk's),
     // then the 4 Tc transverse rows and 1/tau; NKX = 2Q (kx0 = 0) is the whole table
     const int NKX = (trows - 4 * Tc - 1) / 4;
@@ -1763,9 +1672,6 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
     const bool valid = i < N;
     const C* tabc = Tabs<C>::tab(I);
     const C* pxc = Tabs<C>::px(I);
-    const C* gLc = Tabs<C>::gL(I);
-    const C* gRc = Tabs<C>::gR(I);
-    const C* Kyc = Tabs<C>::Ky(I);
     __syncthreads();                      // the previous item's readers of shared memory are done
     if (!stage_rows<S, BULK>(I, i0, k0, k1 - k0, stage, Sw, fo, lane, wy, W)) return false;
     // rows in batches: all loads of a batch are issued before its shared-memory stores
@@ -1791,111 +1697,132 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
         }
     }
     load_tw<S>(I, tws, wy * TILE + lane, W * TILE);
+    const C nwL = (C)I.misc[M_NWL], nwR = (C)I.misc[M_NWR];
+    const int per = (k1 - k0 + W - 1) / W;
+    const int ka = min(k1, k0 + wy * per), nk = min(k1, ka + per) - ka;
+    const bool rwall = N <= i0 + TILE + 3;       // the stencil reaches the right wall
+    C flv = (C)0, fwv = (C)0;
+    if (lane < nk) {
+        const int k = ka + lane;
+        const bool pos = k < Q * Tc;
+        S* row = Sw + (k - k0) * SW + 4 - i0;    // staged node j at row[j]
+        // ghost cells and wall faces (Sec. III B): incoming populations take the wall Maxwellian
+        // n_w g, outgoing ones the quadratic extrapolation of the three nodes next to the wall
+        if (i0 == 0) {
+            if (pos) {
+                flv = nwL * Tabs<C>::gL(I)[k];
+                row[-1] = row[-2] = row[-3] = flv;
+            } else {
+                const C f0 = row[0], f1 = row[1], f2 = row[2];
+                row[-1] = 3 * f0 - 3 * f1 + f2;
+                row[-2] = 6 * f0 - 8 * f1 + 3 * f2;
+                row[-3] = 10 * f0 - 15 * f1 + 6 * f2;
+                flv = (11 * f0 - 7 * f1 + 2 * f2) * (C)(1.0 / 6.0);
+            }
+        }
+        if (rwall) {
+            C g0, g1, g2;
+            if (!pos) {
+                fwv = nwR * Tabs<C>::gR(I)[k];
+                g0 = g1 = g2 = fwv;
+            } else {
+                const C f0 = row[N - 1], f1 = row[N - 2], f2 = row[N - 3];
+                g0 = 3 * f0 - 3 * f1 + f2;
+                g1 = 6 * f0 - 8 * f1 + 3 * f2;
+                g2 = 10 * f0 - 15 * f1 + 6 * f2;
+                fwv = (11 * f0 - 7 * f1 + 2 * f2) * (C)(1.0 / 6.0);
+            }
+            // (the row ends at node i0 + 35)
+            if (N < i0 + 36) row[N] = g0;
+            if (N + 1 < i0 + 36) row[N + 1] = g1;
+            if (N + 2 < i0 + 36) row[N + 2] = g2;
+        }
+        if (i0 != 0) {
+            const S* q = row + (pos ? i0 - 3 : i0 + 2);
+            const int d = pos ? 1 : -1;
+            flv = weno_face(q[0], q[d], q[2 * d], q[3 * d], q[4 * d]);
+        }
+    }
     __syncthreads();
     const S* src = static_cast<const S*>(I.f[stage - 1]);
     S* dst = static_cast<S*>(I.f[stage % 3]);
-    const C ca = stage == 1 ? (C)0 : (stage == 2 ? (C)0.75 : (C)(1.0 / 3.0));
-    const C cb = stage == 1 ? (C)1 : (stage == 2 ? (C)0.25 : (C)(2.0 / 3.0));
-    const C dt = (C)I.dt;
-    const uint32_t seed = sizeof(S) == 4 ? sr_seed(I, stage) : 0u;
-    const C nwL = (C)I.misc[M_NWL], nwR = (C)I.misc[M_NWR];
-    const C xpi = valid ? Tabs<C>::xpinv(I)[i] : (C)0;
-    const C invtau = stab[(4 * NKX + 4 * Tc) * TILE + lane];
+    Stage g;
+    g.first = stage == 1;
+    g.ca = stage == 1 ? 0.0 : (stage == 2 ? 0.75 : 1.0 / 3.0);
+    g.cb = stage == 1 ? 1.0 : (stage == 2 ? 0.25 : 2.0 / 3.0);
+    g.seed = sizeof(S) == 4 ? sr_seed(I, stage) : 0u;
+    // increments are in units of cb dt
+    const C cdt = (C)(g.cb * I.dt);
+    const C xpi = valid ? -cdt * Tabs<C>::xpinv(I)[i] : (C)0;
+    const C invtau = cdt * stab[(4 * NKX + 4 * Tc) * TILE + lane];
     const bool force = I.accel_y != 0.0 && I.form != FORM_REDUCED1D;
-    const int Tz = I.form == FORM_UNREDUCED ? I.Qz : 2;
-    const C ay = (C)I.accel_y;
-    const C sixth = (C)(1.0 / 6.0);
-    // every stencil node of the tile inside the domain: no ghost cells (block-uniform)
-    const bool interior = i0 >= 3 && i0 + TILE + 3 <= N;
-    // (kx, t) of the warp's velocities k = k0 + wy + W m, stepped without divisions
-    int kx = (k0 + wy) / Tc, t = (k0 + wy) - kx * Tc;
-    for (int k = k0 + wy; k < k1; k += W) {
-        const bool pos = kx < Q;
-        const C p = pxc[kx];
-        // node values i-3 .. i+3 (staged node j at row index j - i0 + 4) with the ghost cells of
-        // the diffuse walls (Sec. III B): incoming populations take the wall Maxwellian n_w g,
-        // outgoing ones the quadratic extrapolation of the three nodes next to the wall
-        const S* row = Sw + (k - k0) * SW + 4 - i0;
-        C v[7];
-#pragma unroll
-        for (int jj = 0; jj < 7; ++jj) {
-            const int j = i - 3 + jj;
-            C val;
-            if (interior || (j >= 0 && j < N)) {
-                val = (C)row[j];
-            } else if (j < 0) {
-                if (pos) {
-                    val = nwL * gLc[k];
-                } else {
-                    const C f0 = (C)row[0], f1 = (C)row[1], f2 = (C)row[2];
-                    val = j == -1 ? 3 * f0 - 3 * f1 + f2 : (j == -2 ? 6 * f0 - 8 * f1 + 3 * f2 : 10 * f0 - 15 * f1 + 6 * f2);
-                }
-            } else {
-                if (!pos) {
-                    val = nwR * gRc[k];
-                } else {
-                    const C f0 = (C)row[N - 1], f1 = (C)row[N - 2], f2 = (C)row[N - 3];
-                    val = j == N ? 3 * f0 - 3 * f1 + f2 : (j == N + 1 ? 6 * f0 - 8 * f1 + 3 * f2 : 10 * f0 - 15 * f1 + 6 * f2);
-                }
-            }
-            v[jj] = val;
-        }
-        // right face (i + 1/2)
-        C fr;
-        if (i + 1 == N) fr = pos ? (11 * v[3] - 7 * v[2] + 2 * v[1]) * sixth : nwR * gRc[k];
-        else fr = pos ? weno_face(v[1], v[2], v[3], v[4], v[5]) : weno_face(v[6], v[5], v[4], v[3], v[2]);
-        C fl = __shfl_up_sync(0xffffffffu, fr, 1);
-        if (lane == 0) {
-            if (i == 0) fl = pos ? nwL * gLc[k] : (11 * v[3] - 7 * v[4] + 2 * v[5]) * sixth;
-            else fl = pos ? weno_face(v[0], v[1], v[2], v[3], v[4]) : weno_face(v[5], v[4], v[3], v[2], v[1]);
-        }
-        S* fk = fo + (k - k0) * TILE + lane;
-        if (valid) {
-            C L = -xpi * p * (fr - fl);
-            if (force) {
-                const int ky = t / Tz, kz = t - ky * Tz;
-                const C* Kr = Kyc + ky * I.Qy;
-                C d = 0;
-                for (int kp = 0; kp < I.Qy; ++kp) d += Kr[kp] * (C)src[(size_t)(kx * Tc + kp * Tz + kz) * ld + i];
-                L -= ay * d;
-            }
-            C tgt = 0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) tgt += stab[(a * NKX + kx - kx0) * TILE + lane] * stab[(4 * NKX + a * Tc + t) * TILE + lane];
-            const C fi = v[3];
-            const C Fk = stage == 1 ? (C)0 : (C)*fk;
-            L += (tgt - fi) * invtau;
-            C out;
-            if constexpr (sizeof(C) == 4) {
-                // FP32: the same combination written as an increment of F, F + cb ((f - F) + dt L)
-                // (stage 1: f + dt L).  In the printed form ca F + cb (f + dt L) the rounded
-                // weights (float) 1/3 + (float) 2/3 = 1 + 3e-8 scale a steady f up by half an ulp
-                // every step, a mass drift of ~1e-3 over a solve; the increment form has no such
-                // bias.  The sum is stored with stochastic rounding (sr_add).
-                const C base = stage == 1 ? fi : Fk;
-                const C inc = stage == 1 ? dt * L : cb * ((fi - Fk) + dt * L);
-                out = sr_add(base, inc, fmix32(((uint32_t)k * (uint32_t)ld + (uint32_t)i) ^ seed));
-            } else {
-                out = cb * (fi + dt * L);
-                if (stage != 1) out += ca * Fk;
-            }
-            dst[(size_t)k * ld + i] = (S)out;
-            *fk = (S)out;
-        } else {
-            *fk = (S)0;
-        }
-        t += W;
-        while (t >= Tc) {
-            t -= Tc;
+    const int Qy = I.Qy, Tz = I.form == FORM_UNREDUCED ? I.Qz : 2;
+    const C ay = cdt * (C)I.accel_y;
+    const C* Kyc = Tabs<C>::Ky(I);
+    // padding lanes read the last node's values and write nothing
+    const int li = valid ? lane : N - 1 - i0;
+    const bool at_wall = i + 1 == N;
+    int kx = ka / Tc, t = ka - kx * Tc;
+    C Px[4] = {(C)0, (C)0, (C)0, (C)0}, xp = (C)0;
+    bool pos = true;
+    for (int m = 0; m < nk; ++m, ++t) {
+        const int k = ka + m;
+        if (t == Tc) {
+            t = 0;
             ++kx;
         }
+        if (m == 0 || t == 0) {
+            pos = kx < Q;
+            xp = xpi * pxc[kx];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) Px[a] = stab[(a * NKX + kx - kx0) * TILE + lane];
+        }
+        const S* row = Sw + (k - k0) * SW + 4 + li;
+        C v[5];                                    // upwind order, v[2] the face's own side
+        if (pos) {
+#pragma unroll
+            for (int j = 0; j < 5; ++j) v[j] = row[j - 2];
+        } else {
+#pragma unroll
+            for (int j = 0; j < 5; ++j) v[j] = row[3 - j];
+        }
+        const C fi = pos ? v[2] : v[3];
+        C fr = weno_face(v[0], v[1], v[2], v[3], v[4]);             // right face (i + 1/2)
+        if (rwall) {
+            const C fw = __shfl_sync(0xffffffffu, fwv, m);
+            if (at_wall) fr = fw;
+        }
+        const C f0 = __shfl_sync(0xffffffffu, flv, m);
+        C fl = __shfl_up_sync(0xffffffffu, fr, 1);
+        if (lane == 0) fl = f0;
+        const C* Yt = stab + (4 * NKX + t) * TILE + lane;
+        C tgt = Px[0] * Yt[0];
+#pragma unroll
+        for (int a = 1; a < 4; ++a) tgt += Px[a] * Yt[a * Tc * TILE];
+        C inc = xp * (fr - fl) + (tgt - fi) * invtau;
+        if (force) {
+            const int ky = t / Tz, kg = kx * Tc + (t - ky * Tz);      // first of the p_y values
+            const C* Kr = Kyc + ky * Qy;
+            C d = 0;
+            if (kx * Tc >= k0 && (kx + 1) * Tc <= k1) {
+                const S* rg = Sw + (kg - k0) * SW + 4 + li;
+                for (int kp = 0; kp < Qy; ++kp) d += Kr[kp] * rg[kp * Tz * SW];
+            } else {
+                for (int kp = 0; kp < Qy; ++kp) d += Kr[kp] * src[(size_t)(kg + kp * Tz) * ld + i0 + li];
+            }
+            inc -= ay * d;
+        }
+        S* fk = fo + (k - k0) * TILE + lane;
+        const S out = rk_combine(g, fi, g.first ? (S)0 : *fk, inc, (uint32_t)k * (uint32_t)ld + (uint32_t)i);
+        if (valid) dst[(size_t)k * ld + i] = out;
+        *fk = valid ? out : (S)0;
     }
-    __syncthreads();                      // every warp is done with the staged rows (ex aliases them)
+    __syncthreads();                      // every warp is done with table and rows (ex aliases them)
     chunk_moments<S>(I, i0, k0, k1, k0 / I.ukc, fo, ex, tws, lane, wy, W);
     return true;
 }
 
-template <typename S, typename C, int W>
+template <typename S, int W>
 __global__ void __launch_bounds__(TILE * W) k_update(const Inst* __restrict__ insts, const Work* __restrict__ work, int stage) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_wait();
@@ -1903,9 +1830,9 @@ __global__ void __launch_bounds__(TILE * W) k_update(const Inst* __restrict__ in
     const Inst& I = insts[w.inst];
     if (*I.status != FDLB_ACTIVE || I.smem_res) return;
     if ((I.precision == FDLB_FP64) != (sizeof(S) == 8)) return;
-    if (!update_item<S, C, true, W>(I, w.i0, w.k0, w.k1, stage, smem_raw, threadIdx.x, threadIdx.y)) return;
+    if (!update_item<S, true, W>(I, w.i0, w.k0, w.k1, stage, smem_raw, threadIdx.x, threadIdx.y)) return;
     if (I.mgroups > 1)
-        chunk_ticket_final<S>(I, w.i0, reinterpret_cast<double*>(smem_raw + upd_stage_offset(I.trows, sizeof(C))) + UPD_WARPS * MOM_SUMS * TILE, W);
+        chunk_ticket_final<S>(I, w.i0, reinterpret_cast<double*>(smem_raw + TW_BYTES) + UPD_WARPS * MOM_SUMS * TILE, W);
 }
 
 // Moments of buffer `buf` from scratch (creation, new profiles, a loaded state): one block per
@@ -1970,7 +1897,7 @@ __device__ void res_step(Inst& I, int idx, double tol, double* resid_all, int ra
         cl.sync();
         for (int it = rank; it < tiles * nch; it += CS) {
             const int tl = it / nch, c = it - tl * nch, k0 = c * KC;
-            update_item<S, S, false>(I, tl * TILE, k0, min(K, k0 + KC), stage, sm, lane, wy);
+            update_item<S, false>(I, tl * TILE, k0, min(K, k0 + KC), stage, sm, lane, wy);
         }
         cl.sync();
         if (nch > 1) res_final<S>(I, rank, CS, sm, cl);
@@ -2024,7 +1951,7 @@ __device__ void smem_step(Inst& I, int idx, double tol, double* resid_all, unsig
         __syncthreads();
         for (int it = 0; it < tiles * nch; ++it) {
             const int tl = it / nch, c = it - tl * nch, k0 = c * KC;
-            update_item<S, S, false>(I, tl * TILE, k0, min(K, k0 + KC), stage, sm, lane, wy);
+            update_item<S, false>(I, tl * TILE, k0, min(K, k0 + KC), stage, sm, lane, wy);
         }
         __syncthreads();
         if (nch > 1) {
@@ -2135,7 +2062,15 @@ size_t moments_smem_bytes(int ukc, size_t s) {
     return TW_BYTES + (size_t)ukc * TILE * s + (size_t)(UPD_WARPS + 1) * MOM_SUMS * TILE * sizeof(double);
 }
 
-size_t update_smem_bytes(int ntab, int ukc, size_t c, size_t s) { return upd_smem_bytes(ntab, ukc, c, s); }
+size_t update_smem_bytes(int trows, int ukc, size_t s) { return upd_smem_bytes(trows, ukc, s); }
+
+// The need that the chunk of the largest velocity sets and the set of shared-memory instances are
+// chosen with: an upper bound of update_smem_bytes, kept apart from it so that a batch's layout
+// and mix do not change with the kernel's own use.
+size_t update_smem_bound(int trows, int ukc, size_t s) {
+    const size_t rows = (size_t)ukc * SW * s, ex = upd_ex_bytes();
+    return upd_table_bytes(trows, s) + TW_BYTES + ((rows > ex ? rows : ex) + 15) / 16 * 16 + (size_t)ukc * TILE * s;
+}
 
 cudaError_t launch_moments(const Inst* d_inst, const Work* d_upd, int n_upd, int buf, int ukc_max, bool f64, bool f32,
                            cudaStream_t s) {
@@ -2172,15 +2107,15 @@ cudaError_t launch_resid(const Inst* d_inst, int count, int anchor_inst, double 
 static cudaError_t set_smem(DevAttr* A, size_t smem64, size_t smem32) {
     cudaError_t e = cudaSuccess;
     if (smem64 > 48 * 1024 && smem64 > A->upd64) {
-        e = cudaFuncSetAttribute(k_update<double, double, UPD_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64);
+        e = cudaFuncSetAttribute(k_update<double, UPD_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_update<double, double, UPD_WARPS_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64);
+            e = cudaFuncSetAttribute(k_update<double, UPD_WARPS_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64);
         if (e == cudaSuccess) A->upd64 = smem64;
     }
     if (e == cudaSuccess && smem32 > 48 * 1024 && smem32 > A->upd32) {
-        e = cudaFuncSetAttribute(k_update<float, float, UPD_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem32);
+        e = cudaFuncSetAttribute(k_update<float, UPD_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem32);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_update<float, float, UPD_WARPS_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem32);
+            e = cudaFuncSetAttribute(k_update<float, UPD_WARPS_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem32);
         if (e == cudaSuccess) A->upd32 = smem32;
     }
     return e;
@@ -2343,13 +2278,13 @@ cudaError_t launch_update(const Inst* d_inst, const Work* d_upd, int n_upd, int 
     cudaError_t e = cudaSuccess;
     if (wide) {
         const dim3 blk(TILE, UPD_WARPS_WIDE);
-        if (f64) e = launch_pdl(k_update<double, double, UPD_WARPS_WIDE>, (unsigned)n_upd, blk, smem64, s, d_inst, d_upd, stage);
+        if (f64) e = launch_pdl(k_update<double, UPD_WARPS_WIDE>, (unsigned)n_upd, blk, smem64, s, d_inst, d_upd, stage);
         if (e == cudaSuccess && f32)
-            e = launch_pdl(k_update<float, float, UPD_WARPS_WIDE>, (unsigned)n_upd, blk, smem32, s, d_inst, d_upd, stage);
+            e = launch_pdl(k_update<float, UPD_WARPS_WIDE>, (unsigned)n_upd, blk, smem32, s, d_inst, d_upd, stage);
     } else {
         const dim3 blk(TILE, UPD_WARPS);
-        if (f64) e = launch_pdl(k_update<double, double, UPD_WARPS>, (unsigned)n_upd, blk, smem64, s, d_inst, d_upd, stage);
-        if (e == cudaSuccess && f32) e = launch_pdl(k_update<float, float, UPD_WARPS>, (unsigned)n_upd, blk, smem32, s, d_inst, d_upd, stage);
+        if (f64) e = launch_pdl(k_update<double, UPD_WARPS>, (unsigned)n_upd, blk, smem64, s, d_inst, d_upd, stage);
+        if (e == cudaSuccess && f32) e = launch_pdl(k_update<float, UPD_WARPS>, (unsigned)n_upd, blk, smem32, s, d_inst, d_upd, stage);
     }
     return e;
 }

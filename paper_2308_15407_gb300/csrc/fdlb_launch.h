@@ -15,8 +15,10 @@ cudaError_t launch_setup(const Inst* d_inst, int count, cudaStream_t s);
 cudaError_t launch_moments(const Inst* d_inst, const Work* d_upd, int n_upd, int buf, int ukc_max, bool f64, bool f32,
                            cudaStream_t s);
 
-// Shared memory of one update item (table of ntab rows in type size c, ukc outputs of size s).
-size_t update_smem_bytes(int ntab, int ukc, size_t c, size_t s);
+// Shared memory of one update item (table of trows rows, ukc velocities, storage size s), and the
+// bound of it that layouts are chosen with.
+size_t update_smem_bytes(int trows, int ukc, size_t s);
+size_t update_smem_bound(int trows, int ukc, size_t s);
 
 // Residual / status pass after a step (anchor_inst = -2), or re-anchor instance `anchor_inst`
 // (-1 = all): previous moments := current, residual := +inf, without a status change.
