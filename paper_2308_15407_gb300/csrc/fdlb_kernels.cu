@@ -306,180 +306,73 @@ __global__ void k_profiles(Inst* insts, int inst) {
 // ---------------------------------------------------------------------------
 // moments
 // ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
-// double-float arithmetic (unevaluated float pairs hi + lo, ~2^-46 relative) for the
-// projections of FP32-storage instances: their tables are rounded to FP32, and FP32 FMAs run
-// 64 times faster than FP64 FMAs on this GPU.  Error-free transformations (TwoSum, FMA
-// products, Dekker's fast two-sum) use the _rn intrinsics so that no contraction changes them.
-// ---------------------------------------------------------------------------
-struct df {
-    float hi, lo;
-};
-
-__device__ __forceinline__ df df_fast(float a, float b) {      // |a| >= |b|
-    const float s = __fadd_rn(a, b);
-    return {s, __fadd_rn(b, __fsub_rn(a, s))};
-}
-__device__ __forceinline__ df operator+(df a, df b) {
-    const float s = __fadd_rn(a.hi, b.hi);
-    const float bb = __fsub_rn(s, a.hi);
-    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
-    return df_fast(s, __fadd_rn(e, __fadd_rn(a.lo, b.lo)));
-}
-__device__ __forceinline__ df operator-(df a) { return {-a.hi, -a.lo}; }
-__device__ __forceinline__ df operator-(df a, df b) { return a + (-b); }
-__device__ __forceinline__ df operator*(df a, df b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = __fmaf_rn(a.hi, b.hi, -p);
-    e = __fmaf_rn(a.hi, b.lo, e);
-    e = __fmaf_rn(a.lo, b.hi, e);
-    return df_fast(p, e);
-}
-// Normalised pair of an unnormalised head and tail (TwoSum).
-__device__ __forceinline__ df df_norm(float h, float l) {
-    const float s = __fadd_rn(h, l);
-    const float bb = __fsub_rn(s, h);
-    return {s, __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(l, bb))};
-}
-// s + a b as an unnormalised pair (12 instructions instead of the 18 of s = s + a * b: the
-// product's and the sum's errors are added to the tail and the pair is normalised once, by
-// fin(), at the end of a sum; the tail's own rounding, 2^-24 of a tail that is 2^-24 of the
-// terms, is that of double-float).
-__device__ __forceinline__ df acc(df s, df a, df b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = __fmaf_rn(a.hi, b.hi, -p);
-    e = __fmaf_rn(a.hi, b.lo, e);
-    e = __fmaf_rn(a.lo, b.hi, e);
-    const float t = __fadd_rn(s.hi, p);
-    const float bb = __fsub_rn(t, s.hi);
-    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, bb)), __fsub_rn(p, bb));
-    return {t, __fadd_rn(s.lo, __fadd_rn(err, e))};
-}
-__device__ __forceinline__ double acc(double s, double a, double b) { return fma(a, b, s); }
-__device__ __forceinline__ df fin(df a) { return df_norm(a.hi, a.lo); }
-__device__ __forceinline__ double fin(double a) { return a; }
-// (x h - b hm) c: a step of a three-term recurrence, the two products joined before they are
-// normalised.
-__device__ __forceinline__ df rec3(df x, df h, df b, df hm, df c) {
-    const float p1 = __fmul_rn(x.hi, h.hi);
-    float e = __fmaf_rn(x.hi, h.hi, -p1);
-    e = __fmaf_rn(x.hi, h.lo, e);
-    e = __fmaf_rn(x.lo, h.hi, e);
-    const float p2 = __fmul_rn(b.hi, hm.hi);
-    float g = __fmaf_rn(b.hi, hm.hi, -p2);
-    g = __fmaf_rn(b.hi, hm.lo, g);
-    g = __fmaf_rn(b.lo, hm.hi, g);
-    const float s = __fsub_rn(p1, p2);
-    const float bb = __fsub_rn(s, p1);
-    const float err = __fsub_rn(__fsub_rn(p1, __fsub_rn(s, bb)), __fadd_rn(p2, bb));
-    const float lo = __fadd_rn(err, __fsub_rn(e, g));
-    const float q = __fmul_rn(s, c.hi);
-    float r = __fmaf_rn(s, c.hi, -q);
-    r = __fmaf_rn(s, c.lo, r);
-    r = __fmaf_rn(lo, c.hi, r);
-    return df_fast(q, r);
-}
-__device__ __forceinline__ double rec3(double x, double h, double b, double hm, double c) { return (x * h - b * hm) * c; }
-__device__ __forceinline__ df df_of(float2 v) { return {v.x, v.y}; }
-__device__ __forceinline__ df df_of(double x) {
-    const float h = (float)x;
-    return {h, (float)(x - (double)h)};
-}
-__device__ __forceinline__ float df_float(df a) { return __fadd_rn(a.hi, a.lo); }
-
-// Arithmetic of the closure item's projections: FP64 for FP64 storage, double-float for FP32
-// storage (whose tables are rounded to FP32).
-__device__ __forceinline__ double r_of(double x, double) { return x; }
-__device__ __forceinline__ df r_of(double x, df) { return df_of(x); }
-__device__ __forceinline__ double r_tab(const double* d, const float2*, int k, double) { return d[k]; }
-__device__ __forceinline__ df r_tab(const double*, const float2* p, int k, df) { return df_of(p[k]); }
-__device__ __forceinline__ double r_dbl(double x) { return x; }
-__device__ __forceinline__ double r_dbl(df x) { return (double)x.hi + (double)x.lo; }
+// Arithmetic R of the per-node work: FP64 for FP64 storage, double-float for FP32 storage (whose
+// tables are rounded to FP32).
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ df shfl_xor(df v, int o) { return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)}; }
 
 // Output rows of the projection table in the closure's arithmetic type.
 __device__ __forceinline__ double* r_out(const Inst& I, double) { return I.tab; }
 __device__ __forceinline__ float* r_out(const Inst& I, df) { return I.tab32; }
-__device__ __forceinline__ void r_put(double* p, size_t r, double v) { p[r] = v; }
-__device__ __forceinline__ void r_put(float* p, size_t r, df v) { p[r] = df_float(v); }
-__device__ __forceinline__ void r_put(float* p, size_t r, double v) { p[r] = (float)v; }
 
 constexpr int NTW = 6;     // transverse weights: mt, mt py, mt py^2, mt py^3, et, et py
-
-// Terms of the moment sums in the two arithmetics: FP64, and unnormalised float pairs for FP32
-// storage (error-free sums and products, ~1e-13 relative).
-__device__ __forceinline__ df plus(df s, df a) {                // s + a, unnormalised
-    const float t = __fadd_rn(s.hi, a.hi);
-    const float bb = __fsub_rn(t, s.hi);
-    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, bb)), __fsub_rn(a.hi, bb));
-    return {t, __fadd_rn(s.lo, __fadd_rn(err, a.lo))};
-}
-__device__ __forceinline__ double plus(double s, double a) { return s + a; }
-__device__ __forceinline__ df plus(df s, float f) {
-    const float t = __fadd_rn(s.hi, f);
-    const float bb = __fsub_rn(t, s.hi);
-    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, bb)), __fsub_rn(f, bb));
-    return {t, __fadd_rn(s.lo, err)};
-}
-__device__ __forceinline__ df acc(df s, float f, df w) {        // s + f w
-    const float p = __fmul_rn(f, w.hi);
-    const float e = __fmaf_rn(f, w.lo, __fmaf_rn(f, w.hi, -p));
-    const float t = __fadd_rn(s.hi, p);
-    const float bb = __fsub_rn(t, s.hi);
-    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, bb)), __fsub_rn(p, bb));
-    return {t, __fadd_rn(s.lo, __fadd_rn(err, e))};
-}
 
 // Per node: the 14 raw sums over all velocities, factorised as sum_kx px^a (sum_t w_j(t) f),
 // and the moments they give.
 
-// Temperature from the raw sums (the same operations wherever it is needed).
-__device__ __forceinline__ double sums_temperature(double n, double s1, double s2, double s3, double s4, double s6,
-                                                   double s7) {
-    const double ux = (s1 + s2) / n, uy = s3 / n;
-    const double Pxx = s4 - n * ux * ux, Pyy = s6 - n * uy * uy;
-    const double E = 0.5 * (Pxx + Pyy) + s7;
-    return E / (1.5 * n);
+template <typename R>
+__device__ __forceinline__ R chi_of(R eta) {
+    const R om = r_c(1.0, R{}) - eta;
+    return r_div(r_c(2.0, R{}) - eta, r_c(2.0, R{}) * om * om * om);
 }
 
 // Moments of the nodes of tile i0 from the raw sums ss[MOM_SUMS][TILE], by 128 threads: warp 0
-// writes the primitive rows, warps 1..3 ln n, ln T and ln chi(eta0 n) (independent FP64
-// chains on different schedulers).
-__device__ void finalize_tile(const Inst& I, int i0, const double* ss, int tid) {
+// writes the primitive rows, warps 1..3 ln n, ln T and ln chi(eta0 n) (independent chains on
+// different schedulers).  FP32 storage finalises its double-float sums in double-float: in FP64
+// this took 362 FP64 instructions per tile, 45 % of the FP64 pipe's time on large batches.
+template <typename R>
+__device__ void finalize_tile(const Inst& I, int i0, const R* ss, int tid) {
     const int lane = tid & 31, g = tid >> 5, i = i0 + lane;
     if (i >= I.N) return;
     const int ld = I.ld;
     double* nd = I.node;
-    double s[MOM_SUMS];
+    R s[MOM_SUMS];
 #pragma unroll
     for (int j = 0; j < MOM_SUMS; ++j) s[j] = ss[j * TILE + lane];
-    const double n = s[0];
+    const R n = s[0], half = r_c(0.5, R{}), two = r_c(2.0, R{}), three = r_c(3.0, R{});
     if (g == 1) {
-        nd[R_LNN * ld + i] = log(n);
-    } else if (g == 2) {
-        nd[R_LNT * ld + i] = log(sums_temperature(n, s[1], s[2], s[3], s[4], s[6], s[7]));
+        nd[R_LNN * ld + i] = r_dbl(r_log(n));
     } else if (g == 3) {
-        nd[R_LNCHI * ld + i] = log(chi_cs(I.eta0 * n));
+        nd[R_LNCHI * ld + i] = r_dbl(r_log(chi_of(r_of(I.eta0, R{}) * n)));
     } else {
-        const double sx = s[1] + s[2];
-        const double ux = sx / n, uy = s[3] / n;
-        const double Pxx = s[4] - n * ux * ux, Pxy = s[5] - n * ux * uy;
-        const double T = sums_temperature(n, s[1], s[2], s[3], s[4], s[6], s[7]);
-        const double cx3 = s[8] - 3.0 * ux * s[4] + 2.0 * n * ux * ux * ux;
-        const double cxyy = s[9] - 2.0 * uy * s[5] - ux * s[6] + 2.0 * n * ux * uy * uy;
-        const double cxxy = s[10] - 2.0 * ux * s[5] - uy * s[4] + 2.0 * n * ux * ux * uy;
-        const double cy3 = s[11] - 3.0 * uy * s[6] + 2.0 * n * uy * uy * uy;
-        const double qx = 0.5 * (cx3 + cxyy) + (s[12] - ux * s[7]);
-        const double qy = 0.5 * (cy3 + cxxy) + (s[13] - uy * s[7]);
-        nd[R_N * ld + i] = n;
-        nd[R_UX * ld + i] = ux;
-        nd[R_UY * ld + i] = uy;
-        nd[R_T * ld + i] = T;
-        nd[R_QX * ld + i] = qx;
-        nd[R_QY * ld + i] = qy;
-        nd[R_PXX * ld + i] = Pxx;
-        nd[R_PXY * ld + i] = Pxy;
-        nd[R_SNEG * ld + i] = s[1];
-        nd[R_SPOS * ld + i] = s[2];
+        // n times the thermal energy, without a division: T = (n E)/(1.5 n^2)
+        const R sx = s[1] + s[2];
+        const R nE = half * ((n * s[4] - sx * sx) + (n * s[6] - s[3] * s[3])) + n * s[7];
+        const R T = r_div(nE, r_c(1.5, R{}) * (n * n));
+        if (g == 2) {
+            nd[R_LNT * ld + i] = r_dbl(r_log(T));
+            return;
+        }
+        const R ux = r_div(sx, n), uy = r_div(s[3], n);
+        const R ux2 = ux * ux, uy2 = uy * uy, n2 = two * n;
+        const R Pxx = s[4] - n * ux2, Pxy = s[5] - n * (ux * uy);
+        // third-order sums about the mean: s8 - 3 ux s4 + 2 n ux^3 and so on
+        const R cx3 = s[8] + ux * (n2 * ux2 - three * s[4]);
+        const R cxyy = s[9] - two * (uy * s[5]) + ux * (n2 * uy2 - s[6]);
+        const R cxxy = s[10] - two * (ux * s[5]) + uy * (n2 * ux2 - s[4]);
+        const R cy3 = s[11] + uy * (n2 * uy2 - three * s[6]);
+        const R qx = half * (cx3 + cxyy) + (s[12] - ux * s[7]);
+        const R qy = half * (cy3 + cxxy) + (s[13] - uy * s[7]);
+        nd[R_N * ld + i] = r_dbl(n);
+        nd[R_UX * ld + i] = r_dbl(ux);
+        nd[R_UY * ld + i] = r_dbl(uy);
+        nd[R_T * ld + i] = r_dbl(T);
+        nd[R_QX * ld + i] = r_dbl(qx);
+        nd[R_QY * ld + i] = r_dbl(qy);
+        nd[R_PXX * ld + i] = r_dbl(Pxx);
+        nd[R_PXY * ld + i] = r_dbl(Pxy);
+        nd[R_SNEG * ld + i] = r_dbl(s[1]);
+        nd[R_SPOS * ld + i] = r_dbl(s[2]);
     }
 }
 
@@ -515,31 +408,33 @@ __device__ __forceinline__ void outer_sums(R* o, const R* S, R p, bool neg, bool
     }
 }
 
-// Moments of tile i0 from the I.mgroups partials of its update chunks, added in chunk order,
-// by 128 threads (barrier `bar`); ss: MOM_SUMS x TILE doubles of shared memory.
-// nw warps (tid < 32 nw, barrier `bar` over them, nw >= 4) share the sums; FP32 storage keeps
-// the partials as float pairs and adds them in double-float, FP64 storage in FP64.
+__device__ __forceinline__ double mom_of(double f) { return f; }
+__device__ __forceinline__ df mom_of(float f) { return {f, 0.0f}; }
+template <typename S>
+using MomR = decltype(mom_of(S{}));      // arithmetic of the moment sums of storage type S
+__device__ __forceinline__ double ld_cg(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ df ld_cg(const df* p) { return df_of(__ldcg(reinterpret_cast<const float2*>(p))); }
+
+// Moments of tile i0 from the I.mgroups partials of its update chunks, added in chunk order, by
+// nw warps (tid < 32 nw, barrier `bar` over them, nw >= 4); ss: MOM_SUMS x TILE values of shared
+// memory.
 template <typename S>
 __device__ void moments_final_tile(const Inst& I, int i0, double* ss, int tid, int nw, int bar) {
+    using R = MomR<S>;
     const int lane = tid & 31, g = tid >> 5, i = i0 + lane;
     const int ld = I.ld, G = I.mgroups;
+    R* rs = reinterpret_cast<R*>(ss);
     named_sync(bar, 32 * nw);             // the previous item's readers of `ss` are done
     for (int j = g; j < MOM_SUMS; j += nw) {
-        double v = 0.0;
+        R a = mom_of((S)0);
         if (i < I.N) {
-            if constexpr (sizeof(S) == 4) {
-                const float2* ms = reinterpret_cast<const float2*>(I.msum);
-                df a = {0.0f, 0.0f};
-                for (int q = 0; q < G; ++q) a = a + df_of(__ldcg(ms + ((size_t)q * MOM_SUMS + j) * ld + i));
-                v = (double)a.hi + (double)a.lo;
-            } else {
-                for (int q = 0; q < G; ++q) v += __ldcg(I.msum + ((size_t)q * MOM_SUMS + j) * ld + i);
-            }
+            const R* ms = reinterpret_cast<const R*>(I.msum);
+            for (int q = 0; q < G; ++q) a = a + ld_cg(ms + ((size_t)q * MOM_SUMS + j) * ld + i);
         }
-        ss[j * TILE + lane] = v;
+        rs[j * TILE + lane] = a;
     }
     named_sync(bar, 32 * nw);
-    if (tid < 128) finalize_tile(I, i0, ss, tid);
+    if (tid < 128) finalize_tile<R>(I, i0, rs, tid);
 }
 
 // ---------------------------------------------------------------------------
@@ -569,7 +464,7 @@ __device__ void moments_final_tile(const Inst& I, int i0, double* ss, int tid, i
 // Shared doubles: role 0 (half): [NOD_WARPS + 1][2 nl + 6][32] sums, [4][32] node scalars, beyond
 //                 QMAX polynomials [M][2][32] recurrence states; (full): [Lx + 4][32];
 //                 role 1: CL_ROWS rows + Py [4 QYMAX] + Pz [2 QZMAX] + A [8 QYMAX] + moments.
-constexpr int CL_ROWS = 5 + 6 + 15;                       // gradients, scalars, coefficients
+constexpr int CL_ROWS = 5 + 8 + 14;                       // gradients, scalars, coefficients and n
 constexpr int CL_MOM = (QYMAX + 4) + (QZMAX + 4) + 1;     // m_l and T_a of y and z, T
 
 __host__ __device__ inline int nodal_smem_doubles(int qmax) {
@@ -602,17 +497,14 @@ __device__ __forceinline__ df df_exp(df z) {
     return {ldexpf(e.hi, ki), ldexpf(e.lo, ki)};
 }
 
-__device__ __forceinline__ double r_pair(double d, float2, double) { return d; }
-__device__ __forceinline__ df r_pair(double, float2 p, df) { return df_of(p); }
-
 // Expansion coefficients m_l = int h_l(p) g(p; u, T) dp, l = 0..n, on a full axis and T_a = int
-// h_n(p) (p - u)^a g dp, a = 0..2 (see above); t1 = T - 1, b[l] = sqrt(l), ib[l] = 1/sqrt(l); ml
-// and ts are this lane's columns (stride TILE).
+// h_n(p) (p - u)^a g dp, a = 0..2 (see above); b[l] = sqrt(l), ib[l] = 1/sqrt(l); ml and ts are this
+// lane's columns (stride TILE).
 template <typename R>
-__device__ __forceinline__ void hermite_moments(R u, R T, R t1, int n, const double* b, const float2* b2, const double* ib,
+__device__ __forceinline__ void hermite_moments(R u, R T, int n, const double* b, const float2* b2, const double* ib,
                                                 const float2* ib2, R* ml, R* ts) {
-    const R zero = r_of(0.0, R{});
-    R mp = zero, m = r_of(1.0, R{}), mm = zero;     // m_{l-1}, m_l, m_{l-2}
+    const R zero = r_c(0.0, R{}), one = r_c(1.0, R{}), t1 = T - one;
+    R mp = zero, m = one, mm = zero;                // m_{l-1}, m_l, m_{l-2}
     ml[0] = m;
     for (int l = 0; l < n; ++l) {
         const R il = r_tab(ib, ib2, l + 1, zero);
@@ -628,23 +520,6 @@ __device__ __forceinline__ void hermite_moments(R u, R T, R t1, int n, const dou
     ts[0] = m;
     ts[TILE] = T * (bn * mp);
     ts[2 * TILE] = T * m + (T * bn) * ((T * r_tab(b, b2, n - 1, zero)) * mm);
-}
-
-// sqrt T, u / sqrt T and half its square.  Double-float: one Newton correction of the FP32 root
-// and quotient (both ~1e-14).
-__device__ __forceinline__ void node_scales(df T, df u, df& sT, df& v, df& d) {
-    const float s0 = sqrtf(T.hi);
-    const df r0 = T - df{s0, 0.0f} * df{s0, 0.0f};
-    sT = df_fast(s0, __fdiv_rn(r0.hi, 2.0f * s0));
-    const float q0 = __fdiv_rn(u.hi, sT.hi);
-    const df r1 = u - df{q0, 0.0f} * sT;
-    v = df_fast(q0, __fdiv_rn(r1.hi, sT.hi));
-    d = df{0.5f, 0.0f} * v * v;
-}
-__device__ __forceinline__ void node_scales(double T, double u, double& sT, double& v, double& d) {
-    sT = sqrt(T);
-    v = u / sT;
-    d = 0.5 * v * v;
 }
 
 // exp(q v - d) and exp(-q v - d), d = v^2/2.
@@ -698,6 +573,9 @@ __device__ __forceinline__ void put_powers(O* out, int Q, int k, int ld, int i, 
         }
     }
 }
+__device__ __forceinline__ float to_float(double x) { return (float)x; }
+__device__ __forceinline__ float to_float(df x) { return x.hi; }
+
 // Half-range x projection of a tile (Sec. III A 2), both half-axes: the auxiliary points
 // x = sqrt(T) q and the polynomials there do not depend on the sign of u, so one recurrence
 // serves both.  With |v| < 0.02 and Q <= 12 the 8-point auxiliary rule is used.  It is exact for
@@ -719,13 +597,13 @@ __device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out) {
     __shared__ int use_short;
     if (wid == 0) {
         const R u = r_of(I.node[R_UX * ld + ic], R{});
-        R sT, v, d;
-        node_scales(r_of(I.node[R_T * ld + ic], R{}), u, sT, v, d);
+        const R sT = r_sqrt(r_of(I.node[R_T * ld + ic], R{}));
+        const R v = r_div(u, sT), d = r_c(0.5, R{}) * v * v;
         xs[0 * TILE + lane] = sT;
         xs[1 * TILE + lane] = u;
         xs[2 * TILE + lane] = v;
         xs[3 * TILE + lane] = d;
-        float av = valid ? fabsf((float)r_dbl(v)) : 0.0f;
+        float av = valid ? fabsf(to_float(v)) : 0.0f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) av = fmaxf(av, __shfl_xor_sync(0xffffffffu, av, o));
         // one rule per block so that the warps agree: the largest |v| of the tile decides
@@ -862,7 +740,7 @@ __device__ void xproj_full(const Inst& I, int i0, double* nsm, O* out) {
     const float2 *xb2 = I.xb2, *xib2 = I.xib2, *xH2 = I.xH2, *px2 = I.px2;
     const double T = I.node[R_T * ld + ic];
     const R u = r_of(I.node[R_UX * ld + ic], R{});
-    if (wid == 0) hermite_moments(u, r_of(T, zero), r_of(T - 1.0, zero), Lx, xb, xb2, xib, xib2, ml + lane, ts + lane);
+    if (wid == 0) hermite_moments(u, r_of(T, zero), Lx, xb, xb2, xib, xib2, ml + lane, ts + lane);
     __syncthreads();
     for (int k = wid; k < Q; k += NOD_WARPS) {
         R e = zero, o = zero;
@@ -882,9 +760,10 @@ __device__ void xproj_full(const Inst& I, int i0, double* nsm, O* out) {
 // Role 1 of a tile: gradients (Sec. III B 3), closure (Eqs. chi, prandtl, viscosity, tau), the
 // 13 coefficients of f^S + tau J1 = n g(xi) sum_j c_j xi^(a_j, b_j, c_j) (Eq. j1), the y and z
 // projections (App. A) and the transverse factors n Y[a][t]; wall densities (Sec. III B).
-// Phase A: warps 0..4 one gradient each, warps 5 and 6 the expansion coefficients of y and z
-// (warp 6 also the wall densities), warp 7 the FP64 closure chain; warps 0..6 then run the
-// projections while warp 7 is still busy.  Phase B: the coefficients; phase C: assembly.
+// Phase A: warps 0..4 one gradient each (warp 3 also the expansion coefficients of z, warp 4 the
+// wall densities), warp 5 the expansion coefficients of y, warps 6 and 7 the closure's factors of
+// n and T and of chi, kept apart so that neither chain waits for the other; warps 0..6 then run
+// the projections while warp 7 is still busy.  Phase B: the coefficients; phase C: assembly.
 template <typename R>
 __device__ void closure_item(const Inst& I, int i0, double* nsm) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -892,10 +771,10 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
     const bool valid = i < N;
     const int ic = valid ? i : N - 1;           // padding lanes work on a real node, write nothing
     const double* nd = I.node;
-    double* gr = nsm;                           // [5][32] d/dx of ln n, ln chi, ln T, u_x, u_y
-    double* cs = gr + 5 * TILE;                 // [6][32] W = -tau b rho chi, A, 1/T, tau, -, n
-    R* sc = reinterpret_cast<R*>(cs + 6 * TILE);        // [15][32] coefficients, n, 1/tau
-    R* Py = sc + 15 * TILE;                             // [4 QYMAX][32]
+    R* gr = reinterpret_cast<R*>(nsm);                  // [5][32] d/dx of ln n, ln chi, ln T, u_x, u_y
+    R* cs = gr + 5 * TILE;                              // [8][32] closure scalars
+    R* sc = cs + 8 * TILE;                              // [14][32] coefficients, n
+    R* Py = sc + 14 * TILE;                             // [4 QYMAX][32]
     R* Pz = Py + 4 * QYMAX * TILE;                      // [2 QZMAX][32] (p_z^0 and p_z^2)
     R* Ay = Pz + 2 * QZMAX * TILE;                      // [8 QYMAX][32]
     R* my = Ay + 8 * QYMAX * TILE;                      // [QYMAX + 1][32] m_l of y, then T_a [3][32]
@@ -904,30 +783,36 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
     // Fischer-Methfessel contact value (Eq. chi_ret): the averaged density n-bar and ln chi(n-bar)
     // on the tile and a halo of 7 nodes each side (what the gradient stencils reach)
     constexpr int FH = 7;
-    __shared__ double fm_nbar[TILE + 2 * FH], fm_lnchi[TILE + 2 * FH];
+    __shared__ __align__(8) unsigned char fm_raw[2 * (TILE + 2 * FH) * 8];
+    R* fm_nbar = reinterpret_cast<R*>(fm_raw);
+    double* fm_lnchi = reinterpret_cast<double*>(fm_raw) + TILE + 2 * FH;
     const bool fm = I.chi_model == FDLB_CHI_RET_FM;
     const int h0 = i0 - FH;
+    const R zero = r_c(0.0, R{}), one = r_c(1.0, R{});
     if (fm) {
         for (int h = wid; h < TILE + 2 * FH; h += NOD_WARPS) {
             const int j = h0 + h;
-            double v = 0.0;
+            R v = zero;
             if (j >= 0 && j < N)
-                for (int e = I.fm_ptr[j] + lane; e < I.fm_ptr[j + 1]; e += 32) v = fma(I.fm_w[e], nd[R_N * ld + I.fm_col[e]], v);
+                for (int e = I.fm_ptr[j] + lane; e < I.fm_ptr[j + 1]; e += 32)
+                    v = acc(v, r_of(I.fm_w[e], R{}), r_of(nd[R_N * ld + I.fm_col[e]], R{}));
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) fm_nbar[h] = v;
+            for (int o = 16; o > 0; o >>= 1) v = plus(v, shfl_xor(v, o));
+            if (lane == 0) fm_nbar[h] = fin(v);
         }
         __syncthreads();
         if (threadIdx.x < TILE + 2 * FH) {
             const int j = h0 + threadIdx.x;
-            fm_lnchi[threadIdx.x] = (j >= 0 && j < N) ? log(chi_cs(I.eta0 * fm_nbar[threadIdx.x])) : 0.0;
+            fm_lnchi[threadIdx.x] = (j >= 0 && j < N) ? r_dbl(r_log(chi_of(r_of(I.eta0, R{}) * fm_nbar[threadIdx.x]))) : 0.0;
         }
         __syncthreads();
     }
     if (wid < 5) {
+        // the gradients stay FP64 for either storage: differences of nearly equal numbers
         const int row = wid == 0 ? R_LNN : (wid == 1 ? R_LNCHI : (wid == 2 ? R_LNT : (wid == 3 ? R_UX : R_UY)));
         const double cen[7] = {-1.0 / 60.0, 3.0 / 20.0, -0.75, 0.0, 0.75, -3.0 / 20.0, 1.0 / 60.0};
         double g = 0.0;
+#pragma unroll
         for (int j = 0; j < 7; ++j) {
             int idx;
             double wj;
@@ -936,42 +821,48 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
             else { idx = ic - 3 + j; wj = cen[j]; }
             g = fma(wj, (fm && wid == 1) ? fm_lnchi[idx - h0] : nd[row * ld + idx], g);
         }
-        gr[wid * TILE + lane] = g * I.xpinv[ic];
+        gr[wid * TILE + lane] = r_of(g * I.xpinv[ic], R{});
+        if (wid == 3 && I.form == FORM_UNREDUCED)
+            hermite_moments(zero, r_of(nd[R_T * ld + ic], R{}), Qz, I.fsq, I.fsq2, I.fisq, I.fisq2, mz + lane,
+                            mz + (QZMAX + 1) * TILE + lane);
+        if (wid == 4 && i0 == 0 && lane < 2) {
+            // zero net mass flux through each wall (Sec. III B): the outgoing wall-face flux is
+            // the quadratic reconstruction (11 f_1 - 7 f_2 + 2 f_3)/6 of outgoing populations
+            // (lane 0 the left wall, lane 1 the right one)
+            const double* sr = nd + (lane ? R_SPOS * ld + N - 1 : R_SNEG * ld);
+            const int st = lane ? -1 : 1;
+            const double o = (11.0 * sr[0] - 7.0 * sr[st] + 2.0 * sr[2 * st]) / 6.0;
+            I.misc[lane ? M_NWR : M_NWL] = -o / I.misc[lane ? M_INR : M_INL];
+        }
     } else if (wid == 5) {
-        const double T = nd[R_T * ld + ic];
-        const R Tr = r_of(T, R{});
-        Ts[lane] = Tr;
+        const R T = r_of(nd[R_T * ld + ic], R{});
+        Ts[lane] = T;
         if (I.form != FORM_REDUCED1D)
-            hermite_moments(r_of(nd[R_UY * ld + ic], R{}), Tr, r_of(T - 1.0, R{}), Qy, I.fsq, I.fsq2, I.fisq, I.fisq2, my + lane,
+            hermite_moments(r_of(nd[R_UY * ld + ic], R{}), T, Qy, I.fsq, I.fsq2, I.fisq, I.fisq2, my + lane,
                             my + (QYMAX + 1) * TILE + lane);
     } else if (wid == 6) {
-        if (I.form == FORM_UNREDUCED) {
-            const double T = nd[R_T * ld + ic];
-            hermite_moments(r_of(0.0, R{}), r_of(T, R{}), r_of(T - 1.0, R{}), Qz, I.fsq, I.fsq2, I.fisq, I.fisq2, mz + lane,
-                            mz + (QZMAX + 1) * TILE + lane);
-        }
-        if (i0 == 0 && lane == 0) {
-            // zero net mass flux through each wall (Sec. III B): the outgoing wall-face flux is
-            // the quadratic reconstruction (11 f_1 - 7 f_2 + 2 f_3)/6 of outgoing populations.
-            const double oL = (11.0 * nd[R_SNEG * ld + 0] - 7.0 * nd[R_SNEG * ld + 1] + 2.0 * nd[R_SNEG * ld + 2]) / 6.0;
-            const double oR = (11.0 * nd[R_SPOS * ld + N - 1] - 7.0 * nd[R_SPOS * ld + N - 2] + 2.0 * nd[R_SPOS * ld + N - 3]) / 6.0;
-            I.misc[M_NWL] = -oL / I.misc[M_INL];
-            I.misc[M_NWR] = -oR / I.misc[M_INR];
-        }
+        // the factors of n and T alone: tau = mu/(n T) = mu0c X g, g = sqrt T/(T n)
+        const R n = r_of(nd[R_N * ld + ic], R{}), T = r_of(nd[R_T * ld + ic], R{});
+        const R iT = r_div(one, T), in = r_div(one, n), sT = r_sqrt(T);
+        cs[0 * TILE + lane] = (iT * in) * sT;                             // g
+        cs[1 * TILE + lane] = iT;
+        cs[2 * TILE + lane] = (r_c(0.2, R{}) * in) * (iT * iT);
+        cs[3 * TILE + lane] = n * sT;                                     // 1/g
+        sc[13 * TILE + lane] = n;
     } else {
-        const double k_mu = (4.0 / 25.0) * (1.0 + 12.0 / CUDART_PI);
-        const double k_pd = (9.0 / 25.0) * (1.0 + 32.0 / (9.0 * CUDART_PI));
-        const double n = nd[R_N * ld + ic], T = nd[R_T * ld + ic];
-        const double eta = I.eta0 * n, chi = chi_cs(fm ? I.eta0 * fm_nbar[ic - h0] : eta), br = 4.0 * eta, brc = br * chi;
-        const double Pr = (2.0 / 3.0) * (1.0 + 0.8 * brc + k_mu * brc * brc) / (1.0 + 1.2 * brc + k_pd * brc * brc);
-        const double iT = 1.0 / T, in = 1.0 / n;
-        // tau = mu/(n T) = mu0c X sqrt T / (T n), W = -tau b rho chi
-        const double tau = I.mu0c * (1.0 / chi + 0.8 * br + k_mu * br * br * chi) * iT * in * sqrt(T);
-        cs[0 * TILE + lane] = -tau * brc;
-        cs[1 * TILE + lane] = (1.0 - Pr) * 0.2 * iT * iT * in;
-        cs[2 * TILE + lane] = iT;
-        cs[3 * TILE + lane] = tau;
-        cs[5 * TILE + lane] = n;
+        // the factors of chi: X = 1/chi + 0.8 b rho + k_mu (b rho)^2 chi, Pr, b rho chi
+        const R k_mu = r_c((4.0 / 25.0) * (1.0 + 12.0 / CUDART_PI), R{});
+        const R k_pd = r_c((9.0 / 25.0) * (1.0 + 32.0 / (9.0 * CUDART_PI)), R{});
+        const R n = r_of(nd[R_N * ld + ic], R{}), e0 = r_of(I.eta0, R{});
+        const R eta = e0 * n, ec = fm ? e0 * fm_nbar[ic - h0] : eta;
+        const R om = one - ec, den = r_c(2.0, R{}) * om * om * om, num = r_c(2.0, R{}) - ec;
+        const R chi = r_div(num, den), br = r_c(4.0, R{}) * eta, brc = br * chi, brc2 = brc * brc;
+        const R Pr = r_div(r_c(2.0 / 3.0, R{}) * (one + r_c(0.8, R{}) * brc + k_mu * brc2),
+                           one + r_c(1.2, R{}) * brc + k_pd * brc2);
+        const R X = r_of(I.mu0c, R{}) * (r_div(den, num) + r_c(0.8, R{}) * br + k_mu * br * brc);
+        cs[4 * TILE + lane] = -(X * brc);                                 // W = -tau b rho chi = this times g
+        cs[5 * TILE + lane] = one - Pr;
+        cs[6 * TILE + lane] = X;
     }
     // warps 0..6 go on to the projections (they need m_l, T and u_y only) while warp 7 still
     // runs the closure chain; named barrier 1 synchronises the 7 warps
@@ -1010,53 +901,52 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
         }
     }
     __syncthreads();
+    auto* out = r_out(I, R{});
     {
-        // coefficients: warp w computes a few, reading only what they need
-        const R z = r_of(0.0, R{});
-        const double* W = cs + 0 * TILE;
-        const double* A = cs + 1 * TILE;
-        const double* iT = cs + 2 * TILE;
+        // coefficients: warp w computes a few, reading only what they need; warp 6 also 1/tau
+        const R W = cs[4 * TILE + lane] * cs[0 * TILE + lane], A = cs[5 * TILE + lane] * cs[2 * TILE + lane];
+        const R iT = cs[1 * TILE + lane];
+        const R qx = r_of(nd[R_QX * ld + ic], R{}), qy = r_of(nd[R_QY * ld + ic], R{});
         switch (wid) {
-            case 0:
-                sc[0 * TILE + lane] = r_of(1.0 - W[lane] * gr[3 * TILE + lane], z);
-                sc[13 * TILE + lane] = r_of(cs[5 * TILE + lane], z);
-                break;
+            case 0: sc[0 * TILE + lane] = one - W * gr[3 * TILE + lane]; break;
             case 1: {
-                const double Gr = 2.0 * gr[0 * TILE + lane] + gr[1 * TILE + lane] + gr[2 * TILE + lane];
-                sc[1 * TILE + lane] = r_of(-5.0 * A[lane] * nd[R_QX * ld + ic] + W[lane] * (Gr - 1.5 * gr[2 * TILE + lane]), z);
+                // 2 d ln n + d ln chi + d ln T - 1.5 d ln T
+                const R Gr = r_c(2.0, R{}) * gr[0 * TILE + lane] + gr[1 * TILE + lane] - r_c(0.5, R{}) * gr[2 * TILE + lane];
+                sc[1 * TILE + lane] = W * Gr - r_c(5.0, R{}) * (A * qx);
                 break;
             }
             case 2:
-                sc[2 * TILE + lane] = r_of(-5.0 * A[lane] * nd[R_QY * ld + ic], z);
-                sc[6 * TILE + lane] = I.j1_shear ? r_of(W[lane] * 0.4 * gr[4 * TILE + lane] * iT[lane], z) : z;
+                sc[2 * TILE + lane] = -(r_c(5.0, R{}) * (A * qy));
+                sc[6 * TILE + lane] = I.j1_shear ? (W * r_c(0.4, R{})) * (gr[4 * TILE + lane] * iT) : zero;
                 break;
             case 3: {
-                const double u = W[lane] * gr[3 * TILE + lane] * iT[lane];
-                sc[3 * TILE + lane] = r_of(0.6 * u, z);
-                sc[4 * TILE + lane] = r_of(0.2 * u, z);
-                sc[5 * TILE + lane] = sc[4 * TILE + lane];
+                const R u = (W * gr[3 * TILE + lane]) * iT, c = r_c(0.2, R{}) * u;
+                sc[3 * TILE + lane] = r_c(0.6, R{}) * u;
+                sc[4 * TILE + lane] = c;
+                sc[5 * TILE + lane] = c;
                 break;
             }
             case 4: {
-                const R c3 = r_of(A[lane] * nd[R_QX * ld + ic] * iT[lane] + W[lane] * 0.3 * gr[2 * TILE + lane] * iT[lane], z);
+                const R c3 = (A * qx + r_c(0.3, R{}) * (W * gr[2 * TILE + lane])) * iT;
                 sc[7 * TILE + lane] = c3;
                 sc[8 * TILE + lane] = c3;
                 sc[9 * TILE + lane] = c3;
                 break;
             }
             case 5: {
-                const R cy = r_of(A[lane] * nd[R_QY * ld + ic] * iT[lane], z);
+                const R cy = (A * qy) * iT;
                 sc[10 * TILE + lane] = cy;
                 sc[11 * TILE + lane] = cy;
                 sc[12 * TILE + lane] = cy;
                 break;
             }
-            case 6: sc[14 * TILE + lane] = r_of(1.0 / cs[3 * TILE + lane], z); break;
+            case 6:
+                if (valid) r_put(out, (size_t)(8 * Q + 4 * Tc) * ld + i, r_div(cs[3 * TILE + lane], cs[6 * TILE + lane]));
+                break;
             default: break;
         }
     }
     __syncthreads();
-    auto* out = r_out(I, R{});
     const int form = I.form;
     if (form != FORM_REDUCED1D) {
         // A[a][c'][ky] = n sum over the monomials (a, b, c = 2 c') of coef * Py[b][ky]; with the
@@ -1117,7 +1007,6 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
         R t = slot == 0 ? c0 + c2 * Tr : (two * c0 + (two * two * c2) * Tr) * Tr;
         if (valid) r_put(out, (size_t)(8 * Q + a * Tc + slot) * ld + i, sc[13 * TILE + lane] * t);
     }
-    if (wid == 0 && valid) r_put(out, (size_t)(8 * Q + 4 * Tc) * ld + i, sc[14 * TILE + lane]);
 }
 
 // One (tile, role) item by a block of NOD_WARPS warps; nsm holds nodal_smem_doubles(max Lx)
@@ -1425,9 +1314,6 @@ __device__ __forceinline__ df mom_w(const double* tw, int n, int e, df) {
     const float* h = reinterpret_cast<const float*>(tw);
     return {h[e], h[n + e]};
 }
-__device__ __forceinline__ df mom_of(float f) { return {f, 0.0f}; }
-__device__ __forceinline__ double mom_of(double f) { return f; }
-
 // Epilogue of an update item: raw moment sums of the chunk's values fo[k - k0][lane] with the
 // factorisation of the moments, summed over the warps, then the moments (one chunk per tile) or
 // the chunk's partial sums in msum[grp].  The weights factor as well: over the p_z values of a
@@ -1438,7 +1324,7 @@ __device__ __forceinline__ double mom_of(double f) { return f; }
 template <typename S>
 __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, const S* fo, double* ex, const void* tws,
                               int lane, int wy, int nwb = UPD_WARPS) {
-    using R = decltype(mom_of(S{}));
+    using R = MomR<S>;
     const int i = i0 + lane, ld = I.ld, Tc = I.Tc, Q = I.Q, G = I.mgroups;
     const bool valid = i < I.N;
     const bool unred = I.form == FORM_UNREDUCED, ydep = I.form != FORM_REDUCED1D;
@@ -1449,7 +1335,8 @@ __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, co
     // block, take none and only join the cross-warp sums: the same arithmetic in any block)
     const int per = (k1 - k0 + UPD_WARPS - 1) / UPD_WARPS;
     const int ka = min(k1, k0 + wy * per), kb = min(k1, ka + per);
-    double* ss = ex + UPD_WARPS * MOM_SUMS * TILE;
+    R* pe = reinterpret_cast<R*>(ex);
+    R* ss = pe + UPD_WARPS * MOM_SUMS * TILE;
     R o[MOM_SUMS];
 #pragma unroll
     for (int j = 0; j < MOM_SUMS; ++j) o[j] = zero;
@@ -1496,7 +1383,6 @@ __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, co
         }
         outer_sums(o, Sv, r_tab(I.px, I.px2, kx, R{}), kx >= Q, ydep);
     }
-    R* pe = reinterpret_cast<R*>(ex);
     if (wy < UPD_WARPS)
 #pragma unroll
         for (int j = 0; j < MOM_SUMS; ++j) pe[(wy * MOM_SUMS + j) * TILE + lane] = fin(o[j]);
@@ -1508,13 +1394,13 @@ __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, co
         if (G > 1) {
             if (valid) reinterpret_cast<R*>(I.msum)[((size_t)grp * MOM_SUMS + j) * ld + i] = v;
         } else {
-            ss[j * TILE + lane] = r_dbl(v);
+            ss[j * TILE + lane] = v;
         }
     }
     if (G > 1) return;
     __syncthreads();
     const int tid = wy * TILE + lane;
-    if (tid < 128) finalize_tile(I, i0, ss, tid);
+    if (tid < 128) finalize_tile<R>(I, i0, ss, tid);
 }
 
 // Tiled schedule, tiles split into several chunks: the last chunk block of the tile to arrive
