@@ -140,7 +140,8 @@ struct Inst {
     int* status;
     long long* steps;
 };
-// Projection table layout per node i (column i of a row-major [ntab][ld] array):
+// Projection table layout: [tile][ntab][TILE], so that a tile's table (and each group of its rows) is
+// one contiguous block (bulk copies); per node (column of the tile):
 //   rows 0 .. 8Q-1          : Px[a][kx], a = 0..3, kx = 0..2Q-1   (row a*2Q + kx)
 //   rows 8Q .. 8Q+4Tc-1     : n * Y[a][t]                         (row 8Q + a*Tc + t)
 //   row  8Q+4Tc             : 1/tau

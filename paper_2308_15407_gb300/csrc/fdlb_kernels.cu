@@ -40,6 +40,9 @@ __constant__ double c_inv[13] = {0.0, 1.0, 1.0 / 2, 1.0 / 3, 1.0 / 4, 1.0 / 5, 1
 __constant__ int c_mono[NTERMS][3] = {{0, 0, 0}, {1, 0, 0}, {0, 1, 0}, {2, 0, 0}, {0, 2, 0}, {0, 0, 2}, {1, 1, 0},
                                       {3, 0, 0}, {1, 2, 0}, {1, 0, 2}, {2, 1, 0}, {0, 3, 0}, {0, 1, 2}};
 
+// Column `lane` of tile i0's projection table (rows TILE apart).
+__device__ __forceinline__ size_t tab_col(const Inst& I, int i0, int lane) { return (size_t)(i0 / TILE) * I.ntab * TILE + lane; }
+
 __device__ __forceinline__ double chi_cs(double eta) {
     const double om = 1.0 - eta;
     return (2.0 - eta) / (2.0 * om * om * om);
@@ -282,9 +285,10 @@ __global__ void k_profiles(Inst* insts, int inst) {
     c[0] = 1.0;
     for (int i = threadIdx.x; i < I.N; i += blockDim.x) {
         const double n = I.node[R_N * ld + i], uy = I.node[R_UY * ld + i], T = I.node[R_T * ld + i];
-        proj_x(I, 0.0, T, 0, I.tab + i, ld);
-        proj_x(I, 0.0, T, 1, I.tab + i, ld);
-        build_Y(I, c, uy, T, n, I.tab + 8 * Q * ld + i, ld);
+        double* col = I.tab + tab_col(I, i / TILE * TILE, i % TILE);
+        proj_x(I, 0.0, T, 0, col, TILE);
+        proj_x(I, 0.0, T, 1, col, TILE);
+        build_Y(I, c, uy, T, n, col + 8 * Q * TILE, TILE);
     }
     __syncthreads();
     S* F = static_cast<S*>(I.f[0]);
@@ -292,8 +296,10 @@ __global__ void k_profiles(Inst* insts, int inst) {
         const int kx = k / Tc, t = k - kx * Tc;
         for (int i = threadIdx.x; i < ld; i += blockDim.x) {
             double v = 0.0;
-            if (i < I.N)
-                for (int a = 0; a < 4; ++a) v = fma(I.tab[(a * 2 * Q + kx) * ld + i], I.tab[(8 * Q + a * Tc + t) * ld + i], v);
+            if (i < I.N) {
+                const double* col = I.tab + tab_col(I, i / TILE * TILE, i % TILE);
+                for (int a = 0; a < 4; ++a) v = fma(col[(a * 2 * Q + kx) * TILE], col[(8 * Q + a * Tc + t) * TILE], v);
+            }
             F[(size_t)k * ld + i] = (S)v;
         }
     }
@@ -311,9 +317,9 @@ __global__ void k_profiles(Inst* insts, int inst) {
 __device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ df shfl_xor(df v, int o) { return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)}; }
 
-// Output rows of the projection table in the closure's arithmetic type.
-__device__ __forceinline__ double* r_out(const Inst& I, double) { return I.tab; }
-__device__ __forceinline__ float* r_out(const Inst& I, df) { return I.tab32; }
+// Projection table outputs in the closure's arithmetic type.
+__device__ __forceinline__ double* r_out(const Inst& I, int i0, int lane, double) { return I.tab + tab_col(I, i0, lane); }
+__device__ __forceinline__ float* r_out(const Inst& I, int i0, int lane, df) { return I.tab32 + tab_col(I, i0, lane); }
 
 constexpr int NTW = 6;     // transverse weights: mt, mt py, mt py^2, mt py^3, et, et py
 
@@ -382,31 +388,29 @@ __device__ void finalize_tile(const Inst& I, int i0, const R* ss, int tid) {
 // for a kernel launched without the attribute).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// The instance's record, copied into shared memory by the whole block (ends with a barrier).  The
+// record and the work list are written at creation, before any stepping kernel is launched, so
+// this runs before pdl_wait and overlaps the predecessor's end; the two fields that kernels
+// change (precision, smem_res) are read again after it.  A block otherwise meets one L2 round trip
+// per line of the record that its code touches first.
+__device__ __forceinline__ void load_inst(const Inst* src, Inst* dst, int tid, int n) {
+    static_assert(sizeof(Inst) % 8 == 0, "copied in 8-byte words");
+    for (int w = tid; w < (int)(sizeof(Inst) / 8); w += n)
+        reinterpret_cast<unsigned long long*>(dst)[w] = reinterpret_cast<const unsigned long long*>(src)[w];
+    __syncthreads();
+}
+
+// After the predecessor: does this launch step the instance (active, of this storage, not with the
+// shared-memory-resident kernel)?  g: the record in global memory, I: its copy.
+__device__ __forceinline__ bool runs_now(const Inst& g, const Inst& I, bool fp64) {
+    pdl_wait();
+    const int st = *(volatile int*)I.status, res = *(const volatile int*)&g.smem_res, pr = *(const volatile int*)&g.precision;
+    return st == FDLB_ACTIVE && !res && (pr == FDLB_FP64) == fp64;
+}
+
 // Named barrier over `n` threads (moment finalisation runs on 128-thread parts of a block).
 __device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
-
-// Adds the x-velocity p's contribution to the 14 raw sums from its 6 transverse sums S; ydep: some
-// transverse index has p_y (else the sums with p_y stay zero).
-template <typename R>
-__device__ __forceinline__ void outer_sums(R* o, const R* S, R p, bool neg, bool ydep) {
-    const R p2 = p * p, p3 = p2 * p;
-    o[0] = plus(o[0], S[0]);
-    if (neg) o[1] = acc(o[1], p, S[0]); else o[2] = acc(o[2], p, S[0]);
-    o[4] = acc(o[4], p2, S[0]);
-    o[7] = plus(o[7], S[4]);
-    o[8] = acc(o[8], p3, S[0]);
-    o[12] = acc(o[12], p, S[4]);
-    if (ydep) {
-        o[3] = plus(o[3], S[1]);
-        o[5] = acc(o[5], p, S[1]);
-        o[6] = plus(o[6], S[2]);
-        o[9] = acc(o[9], p, S[2]);
-        o[10] = acc(o[10], p2, S[1]);
-        o[11] = plus(o[11], S[3]);
-        o[13] = plus(o[13], S[5]);
-    }
-}
 
 __device__ __forceinline__ double mom_of(double f) { return f; }
 __device__ __forceinline__ df mom_of(float f) { return {f, 0.0f}; }
@@ -428,8 +432,17 @@ __device__ void moments_final_tile(const Inst& I, int i0, double* ss, int tid, i
     for (int j = g; j < MOM_SUMS; j += nw) {
         R a = mom_of((S)0);
         if (i < I.N) {
-            const R* ms = reinterpret_cast<const R*>(I.msum);
-            for (int q = 0; q < G; ++q) a = a + ld_cg(ms + ((size_t)q * MOM_SUMS + j) * ld + i);
+            // (loads of a batch in flight together: each is a round trip to L2)
+            const R* ms = reinterpret_cast<const R*>(I.msum) + (size_t)j * ld + i;
+            constexpr int B = 6;
+            for (int q = 0; q < G; q += B) {
+                R b[B];
+#pragma unroll
+                for (int e = 0; e < B; ++e) b[e] = q + e < G ? ld_cg(ms + (size_t)(q + e) * MOM_SUMS * ld) : mom_of((S)0);
+#pragma unroll
+                for (int e = 0; e < B; ++e)
+                    if (q + e < G) a = a + b[e];
+            }
         }
         rs[j * TILE + lane] = a;
     }
@@ -561,12 +574,12 @@ __device__ __forceinline__ void exp_pair_short(df z, df d, df& ep, df& em) {
 // (tp, tm), written to rows a 2Q + k and a 2Q + Q + k; the values at -p_k are (-1)^a those of
 // the mirrored problem (u -> -u).
 template <typename R, typename O>
-__device__ __forceinline__ void put_powers(O* out, int Q, int k, int ld, int i, R p, R u, R d, R Pp, R Pm, const R* tp, const R* tm) {
+__device__ __forceinline__ void put_powers(O* out, int Q, int k, R p, R u, R d, R Pp, R Pm, const R* tp, const R* tm) {
     const R pu = p - u, mu = p + u;
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
-        r_put(out, (size_t)(a * 2 * Q + k) * ld + i, Pp);
-        r_put(out, (size_t)(a * 2 * Q + Q + k) * ld + i, (a & 1) ? -Pm : Pm);
+        r_put(out, (a * 2 * Q + k) * TILE, Pp);
+        r_put(out, (a * 2 * Q + Q + k) * TILE, (a & 1) ? -Pm : Pm);
         if (a < 3) {
             Pp = pu * Pp + d * tp[a];
             Pm = mu * Pm + d * tm[a];
@@ -693,12 +706,12 @@ __device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out) {
             sum[r * TILE + lane] = t;
         }
         __syncthreads();
-        R* chain = reinterpret_cast<R*>(I.tab);
+        R* chain = reinterpret_cast<R*>(I.tab) + tab_col(I, i0, lane);
         for (int k = wid; k < Q; k += NOD_WARPS) {
             R sp = zero, sm = zero;
             if (lb > 0 && valid) {
-                sp = chain[(size_t)k * ld + i];
-                sm = chain[(size_t)(Q + k) * ld + i];
+                sp = chain[k * TILE];
+                sm = chain[(Q + k) * TILE];
             }
             for (int j = 0; j < nl; ++j) {
                 const R H = r_tab(xH, xH2, (lb + j) * Q + k, zero);
@@ -715,10 +728,10 @@ __device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out) {
                     tp[a] = sum[(2 * nl + a) * TILE + lane];
                     tm[a] = sum[(2 * nl + 3 + a) * TILE + lane];
                 }
-                if (valid) put_powers(out, Q, k, ld, i, r_tab(px, px2, k, zero), u, dk, sp, sm, tp, tm);
+                if (valid) put_powers(out, Q, k, r_tab(px, px2, k, zero), u, dk, sp, sm, tp, tm);
             } else if (valid) {
-                chain[(size_t)k * ld + i] = sp;
-                chain[(size_t)(Q + k) * ld + i] = sm;
+                chain[k * TILE] = sp;
+                chain[(Q + k) * TILE] = sm;
             }
         }
     }
@@ -753,7 +766,7 @@ __device__ void xproj_full(const Inst& I, int i0, double* nsm, O* out) {
         const R dk = r_tab(xb, xb2, Lx, zero) * r_tab(xH, xH2, (Lx - 1) * Q + k, zero);
         // mirrored problem of -p_k: u -> -u changes the signs of m_l, odd l, and of T_1 (Lx even)
         const R tp[3] = {ts[lane], ts[TILE + lane], ts[2 * TILE + lane]}, tm[3] = {tp[0], -tp[1], tp[2]};
-        if (valid) put_powers(out, Q, k, ld, i, r_tab(px, px2, k, zero), u, dk, e + o, e - o, tp, tm);
+        if (valid) put_powers(out, Q, k, r_tab(px, px2, k, zero), u, dk, e + o, e - o, tp, tm);
     }
 }
 
@@ -901,7 +914,7 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
         }
     }
     __syncthreads();
-    auto* out = r_out(I, R{});
+    auto* out = r_out(I, i0, lane, R{});
     {
         // coefficients: warp w computes a few, reading only what they need; warp 6 also 1/tau
         const R W = cs[4 * TILE + lane] * cs[0 * TILE + lane], A = cs[5 * TILE + lane] * cs[2 * TILE + lane];
@@ -941,7 +954,7 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
                 break;
             }
             case 6:
-                if (valid) r_put(out, (size_t)(8 * Q + 4 * Tc) * ld + i, r_div(cs[3 * TILE + lane], cs[6 * TILE + lane]));
+                if (valid) r_put(out, (8 * Q + 4 * Tc) * TILE, r_div(cs[3 * TILE + lane], cs[6 * TILE + lane]));
                 break;
             default: break;
         }
@@ -978,17 +991,17 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
         for (int pr = wid; pr < 4 * Qy; pr += NOD_WARPS) {
             const int a = pr / Qy, ky = pr - a * Qy;
             const R A0 = Ay[((2 * a) * Qy + ky) * TILE + lane], A1 = Ay[((2 * a + 1) * Qy + ky) * TILE + lane];
-            auto* row = out + (size_t)(8 * Q + a * Tc + ky * Tz) * ld + i;
+            auto* row = out + (8 * Q + a * Tc + ky * Tz) * TILE;
             if (unred) {
                 for (int kz = 0; kz < Qz; ++kz) {
                     const R v = A0 * Pz[(0 * QZMAX + kz) * TILE + lane] + A1 * Pz[(QZMAX + kz) * TILE + lane];
-                    if (valid) r_put(row, (size_t)kz * ld, v);
+                    if (valid) r_put(row, kz * TILE, v);
                 }
             } else {
                 const R v0 = A0 + A1 * Tr, v1 = (A0 + A1 * T3) * Tr;
                 if (valid) {
                     r_put(row, 0, v0);
-                    r_put(row, (size_t)ld, v1);
+                    r_put(row, TILE, v1);
                 }
             }
         }
@@ -1005,14 +1018,39 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
         if (a == 1) c2 = sc[8 * TILE + lane] + sc[9 * TILE + lane];
         const R two = r_of(2.0, R{});
         R t = slot == 0 ? c0 + c2 * Tr : (two * c0 + (two * two * c2) * Tr) * Tr;
-        if (valid) r_put(out, (size_t)(8 * Q + a * Tc + slot) * ld + i, sc[13 * TILE + lane] * t);
+        if (valid) r_put(out, (8 * Q + a * Tc + slot) * TILE, sc[13 * TILE + lane] * t);
     }
+}
+
+// The read-only tables of role `role` (at most 16 KB of them) into L1, one load per 128-byte line,
+// before the predecessor has finished: the loops that read them would else wait for L2 once per
+// line, one after the other.
+__device__ __forceinline__ void warm_lines(const void* from, size_t bytes, int tid, int n) {
+    const char* a = static_cast<const char*>(from);
+    const int lines = (int)((bytes < 16384 ? bytes : 16384) + 127) / 128;
+    for (int l = tid; l < lines; l += n) {
+        unsigned x;
+        asm volatile("ld.global.b32 %0, [%1];" : "=r"(x) : "l"(a + l * 128));
+    }
+}
+__device__ __forceinline__ void warm_tables(const Inst& I, int role, int tid, int n) {
+    const bool f32 = I.precision == FDLB_FP32_STORAGE;
+    const char *b, *e;
+    if (role == 0) {
+        b = f32 ? (const char*)I.xq2 : (const char*)I.px;
+        e = f32 ? (const char*)I.yn2 : (const char*)I.yn;
+    } else {
+        b = f32 ? (const char*)I.yn2 : (const char*)I.yn;
+        e = f32 ? (const char*)I.px2 : (const char*)I.Ky;
+    }
+    warm_lines(b, e - b, tid, n);
 }
 
 // One (tile, role) item by a block of NOD_WARPS warps; nsm holds nodal_smem_doubles(max Lx)
 // doubles; fp32: the instance stores f in FP32 (tables go to tab32).
 template <int QB>
 __device__ void nodal_item(const Inst& I, int i0, int role, double* nsm, bool fp32) {
+    const int lane = threadIdx.x & 31;
     __syncthreads();                      // the previous item's readers of nsm are done
     if (role == 1) {
         if (fp32) closure_item<df>(I, i0, nsm);
@@ -1022,8 +1060,8 @@ __device__ void nodal_item(const Inst& I, int i0, int role, double* nsm, bool fp
     if (I.xfull) {
         // the coefficients m_l and w_k h_l(p_k) stay small at every order: double-float for FP32
         // storage up to order 200
-        if (fp32) xproj_full<df>(I, i0, nsm, I.tab32);
-        else xproj_full<double>(I, i0, nsm, I.tab);
+        if (fp32) xproj_full<df>(I, i0, nsm, r_out(I, i0, lane, df{}));
+        else xproj_full<double>(I, i0, nsm, r_out(I, i0, lane, 0.0));
         return;
     }
     // FP32 storage: double-float up to 32 polynomials.  Larger half-range orders sum in FP64
@@ -1031,19 +1069,23 @@ __device__ void nodal_item(const Inst& I, int i0, int role, double* nsm, bool fp
     // points x = sqrt(T) q, beyond the float range (3e38) once x > ~18.8 -- the aux rule of order
     // 100 has q up to ~17 (overflow from T ~ 1.2); at 32 polynomials it ends near q = 11, which
     // would need T > 3.
-    if (!fp32) xproj_half<QB, double>(I, i0, nsm, I.tab);
-    else if (I.Lx <= 32) xproj_half<QB, df>(I, i0, nsm, I.tab32);
-    else xproj_half<QB, double>(I, i0, nsm, I.tab32);
+    if (!fp32) xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, 0.0));
+    else if (I.Lx <= 32) xproj_half<QB, df>(I, i0, nsm, r_out(I, i0, lane, df{}));
+    else xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, df{}));
 }
 
 template <int QB>
-__global__ void __launch_bounds__(TILE * NOD_WARPS) k_nodal(const Inst* __restrict__ insts, const Work* __restrict__ work) {
+__global__ void __launch_bounds__(TILE * NOD_WARPS, QB == 8 ? 3 : 1) k_nodal(const Inst* __restrict__ insts, const Work* __restrict__ work) {
     extern __shared__ __align__(16) double nsm[];
-    pdl_wait();
+    __shared__ Inst I;
     const Work w = work[blockIdx.x];
-    const Inst& I = insts[w.inst];
-    if (*I.status != FDLB_ACTIVE || I.smem_res) return;
-    nodal_item<QB>(I, w.i0, w.k0, nsm, I.precision == FDLB_FP32_STORAGE);
+    load_inst(insts + w.inst, &I, threadIdx.x, TILE * NOD_WARPS);
+    warm_tables(I, w.k0, threadIdx.x, TILE * NOD_WARPS);
+    pdl_wait();
+    const Inst& g = insts[w.inst];
+    const int st = *(volatile int*)I.status, res = *(const volatile int*)&g.smem_res, pr = *(const volatile int*)&g.precision;
+    if (st != FDLB_ACTIVE || res) return;
+    nodal_item<QB>(I, w.i0, w.k0, nsm, pr == FDLB_FP32_STORAGE);
 }
 
 // ---------------------------------------------------------------------------
@@ -1292,8 +1334,9 @@ __host__ __device__ inline size_t upd_smem_bytes(int trows, int ukc, size_t s) {
     return upd_fo_offset(trows, ukc, s) + (size_t)ukc * TILE * s;
 }
 
-// Transverse moment weights of the epilogue into shared memory (FP32 storage: float heads
-// and tails, FP64: doubles), by the whole block.
+// Transverse moment weights of the epilogue into shared memory (FP32 storage: float heads and, from
+// TWL on, tails; FP64: doubles), by the whole block.
+constexpr int TWL = NTW * TCMAX;
 template <typename S>
 __device__ __forceinline__ void load_tw(const Inst& I, void* tws, int tid, int nthreads) {
     const int n = NTW * I.Tc;
@@ -1301,7 +1344,7 @@ __device__ __forceinline__ void load_tw(const Inst& I, void* tws, int tid, int n
         float* h = static_cast<float*>(tws);
         for (int e = tid; e < n; e += nthreads) {
             h[e] = I.twh[e];
-            h[n + e] = I.twl[e];
+            h[TWL + e] = I.twl[e];
         }
     } else {
         double* d = static_cast<double*>(tws);
@@ -1309,92 +1352,152 @@ __device__ __forceinline__ void load_tw(const Inst& I, void* tws, int tid, int n
     }
 }
 
-__device__ __forceinline__ double mom_w(const double* tw, int, int e, double) { return tw[e]; }
-__device__ __forceinline__ df mom_w(const double* tw, int n, int e, df) {
+__device__ __forceinline__ double mom_w(const double* tw, int e, double) { return tw[e]; }
+__device__ __forceinline__ df mom_w(const double* tw, int e, df) {
     const float* h = reinterpret_cast<const float*>(tw);
-    return {h[e], h[n + e]};
+    return {h[e], h[TWL + e]};
 }
-// Epilogue of an update item: raw moment sums of the chunk's values fo[k - k0][lane] with the
-// factorisation of the moments, summed over the warps, then the moments (one chunk per tile) or
-// the chunk's partial sums in msum[grp].  The weights factor as well: over the p_z values of a
-// p_y (or its two reduced slots) only A = sum f and B = sum e_z f are formed (the mass and the
-// internal energy), then the 6 transverse sums A, y A, y^2 A, y^3 A, B, y B once per p_y, then
-// the outer sums once per x-velocity: 2 + 6/Q_z terms per value instead of 6 (3 for the reduced
-// slots, without the zero-weight tests).
+
+// The 6 transverse sums of the velocities t in [t, tb) of one x-velocity, values *fr, TILE apart.
+// The weights factor: over the p_z values of a p_y (or its two reduced slots) only A = sum f and
+// B = sum e_z f are formed (the mass and the internal energy), then A, y A, y^2 A, y^3 A, B, y B
+// once per p_y: 2 + 6/Q_z terms per value instead of 6 (3 for the reduced slots).
+template <typename S, typename R>
+__device__ __forceinline__ void transverse_sums(const double* tw, int Tc, int Tz, bool unred, bool ydep, int t, int tb,
+                                                const S* fr, R* Sv) {
+    const R zero = mom_of((S)0);
+#pragma unroll
+    for (int j = 0; j < NTW; ++j) Sv[j] = zero;
+    int ty = t / Tz * Tz;                       // first index of t's p_y
+    for (; t < tb; ty += Tz) {
+        const int te = min(tb, ty + Tz);
+        R A = zero, B = zero;
+        if (unred) {
+            A = mom_of(*fr);
+            B = acc(zero, *fr, mom_w(tw, 4 * Tc + t, R{}));
+            fr += TILE;
+            for (++t; t < te; ++t, fr += TILE) {
+                A = plus(A, *fr);
+                B = acc(B, *fr, mom_w(tw, 4 * Tc + t, R{}));
+            }
+        } else {
+            if (t == ty) {
+                A = mom_of(*fr);
+                fr += TILE;
+                ++t;
+            }
+            if (t < te) {
+                B = mom_of((S)0.5 * *fr);
+                fr += TILE;
+                ++t;
+            }
+        }
+        Sv[0] = plus(Sv[0], A);
+        Sv[4] = plus(Sv[4], B);
+        if (ydep) {
+            const R y = mom_w(tw, Tc + ty, R{});
+            Sv[1] = acc(Sv[1], A, y);
+            Sv[2] = acc(Sv[2], A, mom_w(tw, 2 * Tc + ty, R{}));
+            Sv[3] = acc(Sv[3], A, mom_w(tw, 3 * Tc + ty, R{}));
+            Sv[5] = acc(Sv[5], B, y);
+        }
+    }
+}
+
+// Epilogue of an update item: the 14 raw moment sums of the chunk's values fo[k - k0][lane],
+// then the moments (one chunk per tile) or the chunk's partial sums in msum[grp].
+// The chunk is cut into pieces of at most one x-velocity's length (whole x-velocities when there
+// are at least UPD_WARPS of them, else an eighth of the chunk); a warp forms the transverse sums of
+// a piece, one slot of shared memory per x-velocity it touches (at most two).  Then each warp
+// adds one or two of the 14 sums over the slots, times the power of p_x.  Against 14 sums per warp
+// and a sum over the warps this takes 14 terms per slot once instead of per warp.  The pieces and
+// the order of the slots depend on the chunk alone, not on the number of warps.
+// Shared space ex: [2 UPD_WARPS][NTW][TILE] slots, [MOM_SUMS][TILE] sums, [2 UPD_WARPS][4] powers.
+constexpr unsigned long long MOM_S = 0x54312042101000ull;       // transverse sum of raw sum j (hex digit j)
+constexpr unsigned long long MOM_P = 0x01021300120110ull;       // power of p_x of raw sum j
 template <typename S>
 __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, const S* fo, double* ex, const void* tws,
                               int lane, int wy, int nwb = UPD_WARPS) {
     using R = MomR<S>;
-    const int i = i0 + lane, ld = I.ld, Tc = I.Tc, Q = I.Q, G = I.mgroups;
+    const int i = i0 + lane, ld = I.ld, Tc = I.Tc, Q = I.Q, G = I.mgroups, nk = k1 - k0;
     const bool valid = i < I.N;
     const bool unred = I.form == FORM_UNREDUCED, ydep = I.form != FORM_REDUCED1D;
-    const int Tz = unred ? I.Qz : 2, ntw = NTW * Tc;
+    const int Tz = unred ? I.Qz : 2;
     const double* tw = static_cast<const double*>(tws);
-    const R zero = mom_of((S)0);
-    // warp wy < UPD_WARPS takes the velocities [ka, kb) of the chunk (warps beyond, in a wide
-    // block, take none and only join the cross-warp sums: the same arithmetic in any block)
-    const int per = (k1 - k0 + UPD_WARPS - 1) / UPD_WARPS;
-    const int ka = min(k1, k0 + wy * per), kb = min(k1, ka + per);
-    R* pe = reinterpret_cast<R*>(ex);
-    R* ss = pe + UPD_WARPS * MOM_SUMS * TILE;
-    R o[MOM_SUMS];
+    R* sl = reinterpret_cast<R*>(ex);
+    R* ss = sl + 2 * UPD_WARPS * NTW * TILE;
+    R* pw = ss + MOM_SUMS * TILE;
+    const int kx0 = k0 / Tc, t0 = k0 - kx0 * Tc;
+    const int len = (t0 == 0 && nk >= UPD_WARPS * Tc && nk % Tc == 0) ? Tc : min(Tc, (nk + UPD_WARPS - 1) / UPD_WARPS);
+    R v[2] = {mom_of((S)0), mom_of((S)0)};
+    // (kx, t) of the first velocity of piece q0 (for the sums) and of this warp's piece
+    int kxs = kx0, ts = t0;
+    for (int q0 = 0; q0 * len < nk; q0 += UPD_WARPS) {
+        if (q0) __syncthreads();          // the slots' readers are done
+        const int a = (q0 + wy) * len;
+        if (wy < UPD_WARPS && a < nk) {
+            int t = t0 + a, kx = kx0 + t / Tc;
+            t -= (kx - kx0) * Tc;
+            const int n = min(len, nk - a), n0 = min(n, Tc - t);
+            const S* fr = fo + a * TILE + lane;
+            for (int seg = 0; seg < 2; ++seg) {
+                const int ta = seg ? 0 : t, tb = seg ? n - n0 : t + n0;
+                if (ta < tb) {
+                    R Sv[NTW];
+                    transverse_sums(tw, Tc, Tz, unred, ydep, ta, tb, fr + (seg ? n0 * TILE : 0), Sv);
+                    const int slot = 2 * wy + seg;
 #pragma unroll
-    for (int j = 0; j < MOM_SUMS; ++j) o[j] = zero;
-    int kx = ka / Tc, t = ka - kx * Tc;
-    const S* fr = fo + (ka - k0) * TILE + lane;
-    for (int kk = ka; kk < kb; ++kx, t = 0) {
-        const int tb = min(Tc, t + (kb - kk));
-        kk += tb - t;
-        R Sv[NTW];
-#pragma unroll
-        for (int j = 0; j < NTW; ++j) Sv[j] = zero;
-        while (t < tb) {
-            const int ky = t / Tz, ty = ky * Tz, te = min(tb, ty + Tz);
-            R A = zero, B = zero;
-            if (unred) {
-                A = mom_of(*fr);
-                B = acc(zero, *fr, mom_w(tw, ntw, 4 * Tc + t, R{}));
-                fr += TILE;
-                for (++t; t < te; ++t, fr += TILE) {
-                    A = plus(A, *fr);
-                    B = acc(B, *fr, mom_w(tw, ntw, 4 * Tc + t, R{}));
+                    for (int j = 0; j < NTW; ++j) sl[(slot * NTW + j) * TILE + lane] = fin(Sv[j]);
+                    if (lane == 0) {
+                        const R p = r_tab(I.px, I.px2, kx + seg, R{}), p2 = p * p;
+                        pw[slot * 4 + 1] = p;
+                        pw[slot * 4 + 2] = p2;
+                        pw[slot * 4 + 3] = p2 * p;
+                    }
                 }
-            } else {
-                if (t == ty) {
-                    A = mom_of(*fr);
-                    fr += TILE;
-                    ++t;
-                }
-                if (t < te) {
-                    B = mom_of((S)0.5 * *fr);
-                    fr += TILE;
-                    ++t;
-                }
-            }
-            Sv[0] = plus(Sv[0], A);
-            Sv[4] = plus(Sv[4], B);
-            if (ydep) {
-                const R y = mom_w(tw, ntw, Tc + ty, R{});
-                Sv[1] = acc(Sv[1], A, y);
-                Sv[2] = acc(Sv[2], A, mom_w(tw, ntw, 2 * Tc + ty, R{}));
-                Sv[3] = acc(Sv[3], A, mom_w(tw, ntw, 3 * Tc + ty, R{}));
-                Sv[5] = acc(Sv[5], B, y);
             }
         }
-        outer_sums(o, Sv, r_tab(I.px, I.px2, kx, R{}), kx >= Q, ydep);
+        __syncthreads();
+        int kx = kxs, t = ts;
+        for (int r = 0; r < UPD_WARPS && (q0 + r) * len < nk; ++r) {
+            const int n = min(len, nk - (q0 + r) * len);
+            const int segs = t + n > Tc ? 2 : 1;
+            for (int seg = 0; seg < segs; ++seg) {
+                const int slot = 2 * r + seg;
+                const bool neg = kx + seg >= Q;
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    const int j = wy + o * nwb;
+                    if (j < MOM_SUMS) {
+                        const int b = (int)(MOM_S >> (4 * j)) & 15, e = (int)(MOM_P >> (4 * j)) & 15;
+                        // raw sums 1 and 2: the momentum of the negative and of the positive x-velocities
+                        const bool skip = (!ydep && b != 0 && b != 4) || (j == 1 && !neg) || (j == 2 && neg);
+                        if (!skip) {
+                            const R x = sl[(slot * NTW + b) * TILE + lane];
+                            v[o] = e == 0 ? plus(v[o], x) : acc(v[o], pw[slot * 4 + e], x);
+                        }
+                    }
+                }
+            }
+            t += n;
+            if (t >= Tc) {
+                t -= Tc;
+                ++kx;
+            }
+        }
+        kxs = kx;
+        ts = t;
     }
-    if (wy < UPD_WARPS)
 #pragma unroll
-        for (int j = 0; j < MOM_SUMS; ++j) pe[(wy * MOM_SUMS + j) * TILE + lane] = fin(o[j]);
-    __syncthreads();
-    for (int j = wy; j < MOM_SUMS; j += nwb) {
-        R v = pe[j * TILE + lane];
-#pragma unroll
-        for (int q = 1; q < UPD_WARPS; ++q) v = v + pe[(q * MOM_SUMS + j) * TILE + lane];
-        if (G > 1) {
-            if (valid) reinterpret_cast<R*>(I.msum)[((size_t)grp * MOM_SUMS + j) * ld + i] = v;
-        } else {
-            ss[j * TILE + lane] = v;
+    for (int o = 0; o < 2; ++o) {
+        const int j = wy + o * nwb;
+        if (j < MOM_SUMS) {
+            const R x = fin(v[o]);
+            if (G > 1) {
+                if (valid) reinterpret_cast<R*>(I.msum)[((size_t)grp * MOM_SUMS + j) * ld + i] = x;
+            } else {
+                ss[j * TILE + lane] = x;
+            }
         }
     }
     if (G > 1) return;
@@ -1448,39 +1551,63 @@ __device__ __forceinline__ bool mbar_poll(uint64_t* bar, uint32_t parity) {
 
 constexpr long COPY_WAIT_POLLS = 2000000;      // ~2 s at the suspend hint
 
-// Rows [k0, k0 + nrows) of one tile into shared memory: the source stage's values of nodes
-// i0 - 4 .. i0 + 35 (clipped to the row) into Sw[r][0..SW), and, with F, the step's values of
-// nodes i0 .. i0 + 31 into Fo[r][0..TILE).  BULK: one cp.async.bulk per row, all of the block's
-// rows in flight at once, completion counted in bytes on an mbarrier (the tiled schedule);
-// otherwise plain loads (the resident schedule).  Both leave the same values in shared memory.
-// Window bounds are multiples of 4 nodes, so every bulk copy starts on a 16-byte boundary and
-// moves a multiple of 16 bytes.  Returns false if the copies did not complete within the wait
-// limit (the instance is then marked FDLB_FAILED_COPY).
+// What an update item reads, into shared memory: rows [k0, k0 + nrows) of one tile -- the source
+// stage's values of nodes i0 - 4 .. i0 + 35 (clipped to the row) into Sw[r][0..SW), and, beyond
+// stage 1, the step's values of nodes i0 .. i0 + 31 into Fo[r][0..TILE) --, the compact projection
+// table (rows of the NKX x-velocities from kx0 on, then the 4 Tc transverse rows and 1/tau) and the
+// moment weights.  BULK: cp.async.bulk copies, one per row, one to five for the table, issued by
+// the lanes of all warps and in flight together, completion counted in bytes on an mbarrier (the
+// tiled schedule); otherwise plain loads (the resident schedules).  Both leave the same values in
+// shared memory.  Window bounds are multiples of 4 nodes, so every bulk copy starts on a 16-byte
+// boundary and moves a multiple of 16 bytes.  Returns false if the copies did not complete within
+// the wait limit (the instance is then marked FDLB_FAILED_COPY).
 template <typename S, bool BULK>
-__device__ bool stage_rows(const Inst& I, int i0, int k0, int nrows, int stage, S* Sw, S* Fo, int lane, int wy,
-                           int nwb = UPD_WARPS) {
-    const int ld = I.ld;
+__device__ bool stage_item(const Inst& I, int i0, int k0, int nrows, int stage, int NKX, int kx0, S* Sw, S* Fo, S* stab,
+                           void* tws, int lane, int wy, int nwb) {
+    const int ld = I.ld, Q2 = 2 * I.Q, Tc = I.Tc;
     const int lo = max(0, i0 - 4), hi = min(ld, i0 + 36);
     const int off = lo - (i0 - 4);
     const S* src = static_cast<const S*>(I.f[stage - 1]);
     const S* F = static_cast<const S*>(I.f[0]);
     const bool withF = stage != 1;
+    const S* tab = Tabs<S>::tab(I) + tab_col(I, i0, 0);
+    const int nx = min(NKX, Q2 - kx0);                  // (the last chunk's x-velocities may be fewer)
+    const int trest = 4 * Tc + 1;
+    const int tid = wy * TILE + lane;
     if constexpr (BULK) {
         __shared__ __align__(8) uint64_t bar;
         const uint32_t rowbytes = (uint32_t)(hi - lo) * sizeof(S), fbytes = TILE * sizeof(S);
-        const int tid = wy * TILE + lane;
+        const uint32_t rb = TILE * sizeof(S);           // a table row
+        const bool whole = NKX == Q2;
+        const uint32_t twb = ((uint32_t)(NTW * Tc) * (sizeof(S) == 4 ? 4 : 8) + 15) / 16 * 16;   // (tables are padded to 256 B)
         if (tid == 0) {
             mbar_init(&bar, 1);
-            mbar_expect_tx(&bar, (uint32_t)nrows * (rowbytes + (withF ? fbytes : 0u)));
+            mbar_expect_tx(&bar, (uint32_t)nrows * (rowbytes + (withF ? fbytes : 0u)) + (4 * nx + trest) * rb + (sizeof(S) == 4 ? 2 : 1) * twb);
         }
         // earlier generic accesses of this shared memory come before the copies' writes
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (lane == 0)
-            for (int r = wy; r < nrows; r += nwb) {
+        // copy 0 .. 6: table and weights, then the rows; lane-major so that every warp issues a share
+        for (int c = lane * nwb + wy; c < 7 + nrows; c += TILE * nwb) {
+            if (c >= 7) {
+                const int r = c - 7;
                 bulk_g2s(Sw + r * SW + off, src + (size_t)(k0 + r) * ld + lo, rowbytes, &bar);
                 if (withF) bulk_g2s(Fo + r * TILE, F + (size_t)(k0 + r) * ld + i0, fbytes, &bar);
+            } else if (c < 4) {
+                if (whole) {
+                    if (c == 0) bulk_g2s(stab, tab, (4 * nx + trest) * rb, &bar);
+                } else {
+                    bulk_g2s(stab + c * NKX * TILE, tab + (c * Q2 + kx0) * TILE, nx * rb, &bar);
+                }
+            } else if (c == 4) {
+                if (!whole) bulk_g2s(stab + 4 * NKX * TILE, tab + 4 * Q2 * TILE, trest * rb, &bar);
+            } else if constexpr (sizeof(S) == 4) {
+                if (c == 5) bulk_g2s(tws, I.twh, twb, &bar);
+                else bulk_g2s(static_cast<float*>(tws) + TWL, I.twl, twb, &bar);
+            } else {
+                if (c == 5) bulk_g2s(tws, I.tw, twb, &bar);
             }
+        }
         bool ok = false;
         for (long it = 0; it < COPY_WAIT_POLLS && !ok; ++it) ok = mbar_poll(&bar, 0);
         if (__syncthreads_or(!ok)) {          // the same decision in every thread of the block
@@ -1501,6 +1628,10 @@ __device__ bool stage_rows(const Inst& I, int i0, int k0, int nrows, int stage, 
             for (int j = lane; j < n; j += TILE) Sw[r * SW + off + j] = row[j];
             if (withF) Fo[r * TILE + lane] = F[(size_t)(k0 + r) * ld + i0 + lane];
         }
+        for (int a = 0; a < 4; ++a)
+            for (int j = wy; j < nx; j += nwb) stab[(a * NKX + j) * TILE + lane] = tab[(a * Q2 + kx0 + j) * TILE + lane];
+        for (int r = wy; r < trest; r += nwb) stab[(4 * NKX + r) * TILE + lane] = tab[(4 * Q2 + r) * TILE + lane];
+        load_tw<S>(I, tws, tid, nwb * TILE);
         __syncthreads();
         return true;
     }
@@ -1530,11 +1661,11 @@ __device__ __forceinline__ float rk_combine(const Stage& g, float fi, float F, f
 // Velocities [k0, k1) of one tile for RK stage `stage`, by W warps (lane, warp wy; the moment
 // partials on UPD_WARPS of them, so that W = 8 and 16 give the same results bit for bit);
 // smem_raw holds upd_smem_bytes(trows, ukc, sizeof(S)).  The chunk's source rows (and F) are
-// staged in shared memory first (stage_rows).  Each warp then takes a contiguous range of at most
-// 32 velocities: with one lane per velocity it writes the ghost cells of the diffuse walls into
-// its rows and computes the faces that the node-per-lane loop cannot share (the left face of the
-// tile's first node, and the wall face), so that the loop itself is the same for every tile: five
-// stencil values, one face per lane, the left face from the neighbouring lane.  The epilogue
+// staged in shared memory first (stage_item).  Then, with one thread per velocity, the ghost cells
+// of the diffuse walls are written into the rows and the faces computed that a node-per-lane loop
+// cannot share (the left face of the tile's first node, and the wall face), so that the loop
+// itself is the same for every tile: a contiguous range of velocities per warp, five stencil
+// values, one face per lane, the left face from the neighbouring lane.  The epilogue
 // computes the moments of the new values (chunk_moments).  Returns false when the staging copies
 // failed.
 // What bounds it: FP64 storage, the FP64 pipe (21 FP64 instructions per node-velocity and stage
@@ -1556,42 +1687,18 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
     const int NKX = (trows - 4 * Tc - 1) / 4;
     const int kx0 = NKX == 2 * Q ? 0 : k0 / Tc;
     const bool valid = i < N;
-    const C* tabc = Tabs<C>::tab(I);
     const C* pxc = Tabs<C>::px(I);
     __syncthreads();                      // the previous item's readers of shared memory are done
-    if (!stage_rows<S, BULK>(I, i0, k0, k1 - k0, stage, Sw, fo, lane, wy, W)) return false;
-    // rows in batches: all loads of a batch are issued before its shared-memory stores
-    constexpr int TB = 16;
-    for (int r0 = wy; r0 < trows; r0 += W * TB) {
-        C tmp[TB];
-#pragma unroll
-        for (int b = 0; b < TB; ++b) {
-            const int r = r0 + b * W;
-            int gr = -1;                              // row of the instance's table
-            if (r < 4 * NKX) {
-                const int a = r / NKX, kx = kx0 + (r - a * NKX);
-                if (kx < 2 * Q) gr = a * 2 * Q + kx;
-            } else if (r < trows) {
-                gr = 8 * Q + (r - 4 * NKX);
-            }
-            tmp[b] = (valid && gr >= 0) ? tabc[(size_t)gr * ld + i] : (C)0;
-        }
-#pragma unroll
-        for (int b = 0; b < TB; ++b) {
-            const int r = r0 + b * W;
-            if (r < trows) stab[r * TILE + lane] = tmp[b];
-        }
-    }
-    load_tw<S>(I, tws, wy * TILE + lane, W * TILE);
+    if (!stage_item<S, BULK>(I, i0, k0, k1 - k0, stage, NKX, kx0, Sw, fo, stab, tws, lane, wy, W)) return false;
     const C nwL = (C)I.misc[M_NWL], nwR = (C)I.misc[M_NWR];
-    const int per = (k1 - k0 + W - 1) / W;
-    const int ka = min(k1, k0 + wy * per), nk = min(k1, ka + per) - ka;
     const bool rwall = N <= i0 + TILE + 3;       // the stencil reaches the right wall
-    C flv = (C)0, fwv = (C)0;
-    if (lane < nk) {
-        const int k = ka + lane;
+    // one thread per velocity; the left face goes into the row's first value and the wall face into
+    // its last one (nodes i0 - 4 and i0 + 35, which no stencil reads)
+    for (int r = wy * TILE + lane; r < k1 - k0; r += W * TILE) {
+        const int k = k0 + r;
         const bool pos = k < Q * Tc;
-        S* row = Sw + (k - k0) * SW + 4 - i0;    // staged node j at row[j]
+        S* row = Sw + r * SW + 4 - i0;           // staged node j at row[j]
+        C flv;
         // ghost cells and wall faces (Sec. III B): incoming populations take the wall Maxwellian
         // n_w g, outgoing ones the quadratic extrapolation of the three nodes next to the wall
         if (i0 == 0) {
@@ -1607,7 +1714,7 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
             }
         }
         if (rwall) {
-            C g0, g1, g2;
+            C g0, g1, g2, fwv;
             if (!pos) {
                 fwv = nwR * Tabs<C>::gR(I)[k];
                 g0 = g1 = g2 = fwv;
@@ -1618,17 +1725,21 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
                 g2 = 10 * f0 - 15 * f1 + 6 * f2;
                 fwv = (11 * f0 - 7 * f1 + 2 * f2) * (C)(1.0 / 6.0);
             }
-            // (the row ends at node i0 + 35)
-            if (N < i0 + 36) row[N] = g0;
-            if (N + 1 < i0 + 36) row[N + 1] = g1;
-            if (N + 2 < i0 + 36) row[N + 2] = g2;
+            // (stencils end at node i0 + 34)
+            if (N < i0 + 35) row[N] = g0;
+            if (N + 1 < i0 + 35) row[N + 1] = g1;
+            if (N + 2 < i0 + 35) row[N + 2] = g2;
+            Sw[r * SW + SW - 1] = fwv;
         }
         if (i0 != 0) {
             const S* q = row + (pos ? i0 - 3 : i0 + 2);
             const int d = pos ? 1 : -1;
             flv = weno_face(q[0], q[d], q[2 * d], q[3 * d], q[4 * d]);
         }
+        Sw[r * SW] = flv;
     }
+    const int per = (k1 - k0 + W - 1) / W;
+    const int ka = min(k1, k0 + wy * per), nk = min(k1, ka + per) - ka;
     __syncthreads();
     const S* src = static_cast<const S*>(I.f[stage - 1]);
     S* dst = static_cast<S*>(I.f[stage % 3]);
@@ -1648,14 +1759,18 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
     // padding lanes read the last node's values and write nothing
     const int li = valid ? lane : N - 1 - i0;
     const bool at_wall = i + 1 == N;
-    int kx = ka / Tc, t = ka - kx * Tc;
+    int kx = ka / Tc, t = ka - kx * Tc, kz = t % Tz, ky = t / Tz;
     C Px[4] = {(C)0, (C)0, (C)0, (C)0}, xp = (C)0;
     bool pos = true;
-    for (int m = 0; m < nk; ++m, ++t) {
+    for (int m = 0; m < nk; ++m, ++t, ++kz) {
         const int k = ka + m;
         if (t == Tc) {
             t = 0;
             ++kx;
+            ky = kz = 0;
+        } else if (kz == Tz) {
+            kz = 0;
+            ++ky;
         }
         if (m == 0 || t == 0) {
             pos = kx < Q;
@@ -1674,20 +1789,16 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
         }
         const C fi = pos ? v[2] : v[3];
         C fr = weno_face(v[0], v[1], v[2], v[3], v[4]);             // right face (i + 1/2)
-        if (rwall) {
-            const C fw = __shfl_sync(0xffffffffu, fwv, m);
-            if (at_wall) fr = fw;
-        }
-        const C f0 = __shfl_sync(0xffffffffu, flv, m);
+        if (at_wall) fr = row[SW - 5 - li];
         C fl = __shfl_up_sync(0xffffffffu, fr, 1);
-        if (lane == 0) fl = f0;
+        if (lane == 0) fl = row[-4 - li];
         const C* Yt = stab + (4 * NKX + t) * TILE + lane;
         C tgt = Px[0] * Yt[0];
 #pragma unroll
         for (int a = 1; a < 4; ++a) tgt += Px[a] * Yt[a * Tc * TILE];
         C inc = xp * (fr - fl) + (tgt - fi) * invtau;
         if (force) {
-            const int ky = t / Tz, kg = kx * Tc + (t - ky * Tz);      // first of the p_y values
+            const int kg = kx * Tc + kz;               // first of the p_y values
             const C* Kr = Kyc + ky * Qy;
             C d = 0;
             if (kx * Tc >= k0 && (kx + 1) * Tc <= k1) {
@@ -1711,14 +1822,13 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
 template <typename S, int W>
 __global__ void __launch_bounds__(TILE * W) k_update(const Inst* __restrict__ insts, const Work* __restrict__ work, int stage) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_wait();
+    __shared__ Inst I;
     const Work w = work[blockIdx.x];
-    const Inst& I = insts[w.inst];
-    if (*I.status != FDLB_ACTIVE || I.smem_res) return;
-    if ((I.precision == FDLB_FP64) != (sizeof(S) == 8)) return;
+    load_inst(insts + w.inst, &I, threadIdx.y * TILE + threadIdx.x, W * TILE);
+    if (!runs_now(insts[w.inst], I, sizeof(S) == 8)) return;
     if (!update_item<S, true, W>(I, w.i0, w.k0, w.k1, stage, smem_raw, threadIdx.x, threadIdx.y)) return;
     if (I.mgroups > 1)
-        chunk_ticket_final<S>(I, w.i0, reinterpret_cast<double*>(smem_raw + TW_BYTES) + UPD_WARPS * MOM_SUMS * TILE, W);
+        chunk_ticket_final<S>(I, w.i0, reinterpret_cast<double*>(smem_raw + TW_BYTES), W);
 }
 
 // Moments of buffer `buf` from scratch (creation, new profiles, a loaded state): one block per
@@ -1741,7 +1851,7 @@ __global__ void __launch_bounds__(TILE * UPD_WARPS) k_moments(const Inst* __rest
     load_tw<S>(I, tws, wy * TILE + lane, UPD_WARPS * TILE);
     __syncthreads();
     chunk_moments<S>(I, w.i0, w.k0, w.k1, w.k0 / I.ukc, fo, ex, tws, lane, wy);
-    if (I.mgroups > 1) chunk_ticket_final<S>(I, w.i0, ex + UPD_WARPS * MOM_SUMS * TILE);
+    if (I.mgroups > 1) chunk_ticket_final<S>(I, w.i0, ex);
 }
 
 // ---------------------------------------------------------------------------
