@@ -414,6 +414,8 @@ __device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sy
 
 __device__ __forceinline__ double mom_of(double f) { return f; }
 __device__ __forceinline__ df mom_of(float f) { return {f, 0.0f}; }
+__device__ __forceinline__ double mom_zero(double) { return 0.0; }
+__device__ __forceinline__ df mom_zero(df) { return {0.0f, 0.0f}; }
 template <typename S>
 using MomR = decltype(mom_of(S{}));      // arithmetic of the moment sums of storage type S
 __device__ __forceinline__ double ld_cg(const double* p) { return __ldcg(p); }
@@ -1408,16 +1410,50 @@ __device__ __forceinline__ void transverse_sums(const double* tw, int Tc, int Tz
 // then the moments (one chunk per tile) or the chunk's partial sums in msum[grp].
 // The chunk is cut into pieces of at most one x-velocity's length (whole x-velocities when there
 // are at least UPD_WARPS of them, else an eighth of the chunk); a warp forms the transverse sums of
-// a piece, one slot of shared memory per x-velocity it touches (at most two).  Then each warp
-// adds one or two of the 14 sums over the slots, times the power of p_x.  Against 14 sums per warp
-// and a sum over the warps this takes 14 terms per slot once instead of per warp.  The pieces and
-// the order of the slots depend on the chunk alone, not on the number of warps.
+// a piece, one slot of shared memory per x-velocity it touches (at most two).  Then warps 0..5 add
+// the 14 sums over the slots, times the power of p_x, each the sums that share a transverse sum
+// (a value is read once, and the code has no index tables: those took as many instructions as the
+// sums).  Against 14 sums per warp and a sum over the warps this takes 14 terms per slot once
+// instead of per warp.  The pieces and the order of the slots depend on the chunk alone, not on
+// the number of warps.
 // Shared space ex: [2 UPD_WARPS][NTW][TILE] slots, [MOM_SUMS][TILE] sums, [2 UPD_WARPS][4] powers.
-constexpr unsigned long long MOM_S = 0x54312042101000ull;       // transverse sum of raw sum j (hex digit j)
-constexpr unsigned long long MOM_P = 0x01021300120110ull;       // power of p_x of raw sum j
+
+// Adds over the slots of up to UPD_WARPS pieces (sl: this lane's column), to v[0..n): x-velocity power E_j times transverse sum
+// B (E_j < 0: none).  SIGN: v[0] takes the negative x-velocities, v[1] the positive ones.
+struct Slots {
+    int kx, t, Q, Tc, len, nk, q0;
+};
+template <typename R, int B, int E0, int E1 = -1, int E2 = -1, bool SIGN = false>
+__device__ __forceinline__ void add_slots(const Slots& g, const R* sl, const R* pw, R* v) {
+    int kx = g.kx, t = g.t;
+    const R* x = sl + B * TILE;
+    for (int r = 0, a = g.q0 * g.len; r < UPD_WARPS && a < g.nk; ++r, a += g.len, x += 2 * NTW * TILE, pw += 8) {
+        const int n = min(g.len, g.nk - a);
+        t += n;
+        for (int seg = 0; seg < 2; ++seg) {
+            if (seg && t <= g.Tc) break;
+            const R xs = x[seg * NTW * TILE];
+            const R* ps = pw + 4 * seg;
+            if (SIGN) {
+                const R y = acc(mom_zero(R{}), ps[1], xs);
+                if (kx + seg >= g.Q) v[0] = plus(v[0], y);
+                else v[1] = plus(v[1], y);
+            } else {
+                v[0] = E0 == 0 ? plus(v[0], xs) : acc(v[0], ps[E0], xs);
+                if (E1 >= 0) v[1] = acc(v[1], ps[E1 < 0 ? 0 : E1], xs);
+                if (E2 >= 0) v[2] = acc(v[2], ps[E2 < 0 ? 0 : E2], xs);
+            }
+        }
+        if (t >= g.Tc) {
+            t -= g.Tc;
+            ++kx;
+        }
+    }
+}
+
 template <typename S>
 __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, const S* fo, double* ex, const void* tws,
-                              int lane, int wy, int nwb = UPD_WARPS) {
+                              int lane, int wy) {
     using R = MomR<S>;
     const int i = i0 + lane, ld = I.ld, Tc = I.Tc, Q = I.Q, G = I.mgroups, nk = k1 - k0;
     const bool valid = i < I.N;
@@ -1429,9 +1465,8 @@ __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, co
     R* pw = ss + MOM_SUMS * TILE;
     const int kx0 = k0 / Tc, t0 = k0 - kx0 * Tc;
     const int len = (t0 == 0 && nk >= UPD_WARPS * Tc && nk % Tc == 0) ? Tc : min(Tc, (nk + UPD_WARPS - 1) / UPD_WARPS);
-    R v[2] = {mom_of((S)0), mom_of((S)0)};
-    // (kx, t) of the first velocity of piece q0 (for the sums) and of this warp's piece
-    int kxs = kx0, ts = t0;
+    R v[3] = {mom_of((S)0), mom_of((S)0), mom_of((S)0)};
+    Slots g = {kx0, t0, Q, Tc, len, nk, 0};           // kx, t: of the first velocity of piece q0
     for (int q0 = 0; q0 * len < nk; q0 += UPD_WARPS) {
         if (q0) __syncthreads();          // the slots' readers are done
         const int a = (q0 + wy) * len;
@@ -1458,45 +1493,41 @@ __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, co
             }
         }
         __syncthreads();
-        int kx = kxs, t = ts;
-        for (int r = 0; r < UPD_WARPS && (q0 + r) * len < nk; ++r) {
-            const int n = min(len, nk - (q0 + r) * len);
-            const int segs = t + n > Tc ? 2 : 1;
-            for (int seg = 0; seg < segs; ++seg) {
-                const int slot = 2 * r + seg;
-                const bool neg = kx + seg >= Q;
-#pragma unroll
-                for (int o = 0; o < 2; ++o) {
-                    const int j = wy + o * nwb;
-                    if (j < MOM_SUMS) {
-                        const int b = (int)(MOM_S >> (4 * j)) & 15, e = (int)(MOM_P >> (4 * j)) & 15;
-                        // raw sums 1 and 2: the momentum of the negative and of the positive x-velocities
-                        const bool skip = (!ydep && b != 0 && b != 4) || (j == 1 && !neg) || (j == 2 && neg);
-                        if (!skip) {
-                            const R x = sl[(slot * NTW + b) * TILE + lane];
-                            v[o] = e == 0 ? plus(v[o], x) : acc(v[o], pw[slot * 4 + e], x);
-                        }
-                    }
+        g.q0 = q0;
+        switch (wy) {
+            case 0: add_slots<R, 0, 0, 2, 3>(g, sl + lane, pw, v); break;                 // raw sums 0, 4, 8
+            case 1: add_slots<R, 0, 1, 1, -1, true>(g, sl + lane, pw, v); break;          // 1, 2
+            case 2: if (ydep) add_slots<R, 1, 0, 1, 2>(g, sl + lane, pw, v); break;       // 3, 5, 10
+            case 3: if (ydep) add_slots<R, 2, 0, 1>(g, sl + lane, pw, v); break;          // 6, 9
+            case 4: add_slots<R, 4, 0, 1>(g, sl + lane, pw, v); break;                    // 7, 12
+            case 5:
+                if (ydep) {
+                    add_slots<R, 3, 0>(g, sl + lane, pw, v);                              // 11
+                    add_slots<R, 5, 0>(g, sl + lane, pw, v + 1);                          // 13
                 }
-            }
-            t += n;
-            if (t >= Tc) {
-                t -= Tc;
-                ++kx;
-            }
+                break;
+            default: break;
         }
-        kxs = kx;
-        ts = t;
+        if (q0 + UPD_WARPS < (nk + len - 1) / len) {
+            const int t = g.t + UPD_WARPS * len;
+            g.kx += t / Tc;
+            g.t = t % Tc;
+        }
     }
+    const int j0 = wy == 0 ? 0 : wy == 1 ? 1 : wy == 2 ? 3 : wy == 3 ? 6 : wy == 4 ? 7 : 11;
+    const int j1 = wy == 0 ? 4 : wy == 1 ? 2 : wy == 2 ? 5 : wy == 3 ? 9 : wy == 4 ? 12 : 13;
+    const int j2 = wy == 0 ? 8 : wy == 2 ? 10 : -1;
+    if (wy < 6) {
 #pragma unroll
-    for (int o = 0; o < 2; ++o) {
-        const int j = wy + o * nwb;
-        if (j < MOM_SUMS) {
-            const R x = fin(v[o]);
-            if (G > 1) {
-                if (valid) reinterpret_cast<R*>(I.msum)[((size_t)grp * MOM_SUMS + j) * ld + i] = x;
-            } else {
-                ss[j * TILE + lane] = x;
+        for (int o = 0; o < 3; ++o) {
+            const int j = o == 0 ? j0 : (o == 1 ? j1 : j2);
+            if (j >= 0) {
+                const R x = fin(v[o]);
+                if (G > 1) {
+                    if (valid) reinterpret_cast<R*>(I.msum)[((size_t)grp * MOM_SUMS + j) * ld + i] = x;
+                } else {
+                    ss[j * TILE + lane] = x;
+                }
             }
         }
     }
@@ -1541,6 +1572,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                  :: "r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
+// 16 bytes from global src to shared dst (both 16-byte aligned), asynchronously
+__device__ __forceinline__ void cp16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
 // Phase `parity` of bar complete?  Each poll may suspend the thread for up to ~1 us.
 __device__ __forceinline__ bool mbar_poll(uint64_t* bar, uint32_t parity) {
     uint32_t done;
@@ -1555,11 +1591,12 @@ constexpr long COPY_WAIT_POLLS = 2000000;      // ~2 s at the suspend hint
 // stage's values of nodes i0 - 4 .. i0 + 35 (clipped to the row) into Sw[r][0..SW), and, beyond
 // stage 1, the step's values of nodes i0 .. i0 + 31 into Fo[r][0..TILE) --, the compact projection
 // table (rows of the NKX x-velocities from kx0 on, then the 4 Tc transverse rows and 1/tau) and the
-// moment weights.  BULK: cp.async.bulk copies, one per row, one to five for the table, issued by
-// the lanes of all warps and in flight together, completion counted in bytes on an mbarrier (the
-// tiled schedule); otherwise plain loads (the resident schedules).  Both leave the same values in
-// shared memory.  Window bounds are multiples of 4 nodes, so every bulk copy starts on a 16-byte
-// boundary and moves a multiple of 16 bytes.  Returns false if the copies did not complete within
+// moment weights.  BULK (the tiled schedule): the table and the weights as cp.async.bulk copies (one
+// to five and two, their completion counted in bytes on an mbarrier), the rows as 16-byte cp.async
+// copies, all in flight together; a row is too short for a bulk copy of its own, whose operands go
+// through uniform registers one lane at a time.  Otherwise (the resident schedules) plain loads.
+// Both leave the same values in shared memory.  Window bounds are multiples of 4 nodes, so every
+// copy starts on a 16-byte boundary.  Returns false if the bulk copies did not complete within
 // the wait limit (the instance is then marked FDLB_FAILED_COPY).
 template <typename S, bool BULK>
 __device__ bool stage_item(const Inst& I, int i0, int k0, int nrows, int stage, int NKX, int kx0, S* Sw, S* Fo, S* stab,
@@ -1576,24 +1613,20 @@ __device__ bool stage_item(const Inst& I, int i0, int k0, int nrows, int stage, 
     const int tid = wy * TILE + lane;
     if constexpr (BULK) {
         __shared__ __align__(8) uint64_t bar;
-        const uint32_t rowbytes = (uint32_t)(hi - lo) * sizeof(S), fbytes = TILE * sizeof(S);
         const uint32_t rb = TILE * sizeof(S);           // a table row
         const bool whole = NKX == Q2;
         const uint32_t twb = ((uint32_t)(NTW * Tc) * (sizeof(S) == 4 ? 4 : 8) + 15) / 16 * 16;   // (tables are padded to 256 B)
         if (tid == 0) {
             mbar_init(&bar, 1);
-            mbar_expect_tx(&bar, (uint32_t)nrows * (rowbytes + (withF ? fbytes : 0u)) + (4 * nx + trest) * rb + (sizeof(S) == 4 ? 2 : 1) * twb);
+            mbar_expect_tx(&bar, (4 * nx + trest) * rb + (sizeof(S) == 4 ? 2 : 1) * twb);
         }
         // earlier generic accesses of this shared memory come before the copies' writes
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        // copy 0 .. 6: table and weights, then the rows; lane-major so that every warp issues a share
-        for (int c = lane * nwb + wy; c < 7 + nrows; c += TILE * nwb) {
-            if (c >= 7) {
-                const int r = c - 7;
-                bulk_g2s(Sw + r * SW + off, src + (size_t)(k0 + r) * ld + lo, rowbytes, &bar);
-                if (withF) bulk_g2s(Fo + r * TILE, F + (size_t)(k0 + r) * ld + i0, fbytes, &bar);
-            } else if (c < 4) {
+        // table and weights: lane 0 of the first warps
+        if (lane == 0 && wy < 7) {
+            const int c = wy;
+            if (c < 4) {
                 if (whole) {
                     if (c == 0) bulk_g2s(stab, tab, (4 * nx + trest) * rb, &bar);
                 } else {
@@ -1608,7 +1641,28 @@ __device__ bool stage_item(const Inst& I, int i0, int k0, int nrows, int stage, 
                 if (c == 5) bulk_g2s(tws, I.tw, twb, &bar);
             }
         }
-        bool ok = false;
+        // rows: 16 lanes each, 16 bytes per copy
+        {
+            constexpr int V = 16 / sizeof(S);
+            const int nv = (hi - lo) / V;
+            const S* g = src + (size_t)(k0 + (tid >> 4)) * ld + lo + (tid & 15) * V;
+            const S* gf = F + (size_t)(k0 + (tid >> 4)) * ld + i0 + (tid & 15) * V;
+            S* d = Sw + (tid >> 4) * SW + off + (tid & 15) * V;
+            S* df_ = Fo + (tid >> 4) * TILE + (tid & 15) * V;
+            const int dr = nwb * 2;                     // rows per pass of the block
+            for (int r = tid >> 4; r < nrows; r += dr) {
+                if ((tid & 15) < nv) cp16(d, g);
+                if (sizeof(S) == 8 && (tid & 15) + 16 < nv) cp16(d + 16 * V, g + 16 * V);
+                if (withF && (tid & 15) < TILE / V) cp16(df_, gf);
+                g += (size_t)dr * ld;
+                gf += (size_t)dr * ld;
+                d += dr * SW;
+                df_ += dr * TILE;
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        }
+        // warp 0 polls, the others wait at the barrier
+        bool ok = wy != 0;
         for (long it = 0; it < COPY_WAIT_POLLS && !ok; ++it) ok = mbar_poll(&bar, 0);
         if (__syncthreads_or(!ok)) {          // the same decision in every thread of the block
             if (tid == 0) atomicExch(I.status, FDLB_FAILED_COPY);
@@ -1656,6 +1710,63 @@ __device__ __forceinline__ float rk_combine(const Stage& g, float fi, float F, f
     const float base = g.first ? fi : F;
     if (!g.first) inc = fmaf(cb, fi - F, inc);
     return sr_add(base, inc, fmix32(e ^ g.seed));
+}
+
+// What a lane (node) carries through its warp's velocities; the pointers are stepped from one
+// velocity to the next.
+template <typename S>
+struct Lane {
+    bool valid, at_wall;
+    int lane, ld, TcS;
+    S xp, invtau, Px[4];       // -cb dt p/(x' ds), cb dt/tau, the x projections of this p
+    const S* row;              // staged row at this node
+    const S* wall;             // staged row: [0] left face of the tile's first node, [SW - 1] wall face
+    const S* Y;                // transverse factors n Y[a][t], a TcS apart
+    S* fo;
+    S* dst;
+    uint32_t elem;             // k ld + i, for the stochastic rounding
+};
+template <typename S>
+struct Force {
+    const S* f;                // values of this x-velocity's velocities t, `stride` apart
+    const S* K;
+    int stride, Qy, Tz;
+    S ay;
+};
+
+// n velocities t, t + 1, ... of one x-velocity; POS: p_x > 0.
+template <typename S, bool POS, bool FORCE>
+__device__ __forceinline__ void update_run(const Stage& g, Lane<S>& c, const Force<S>& fc, int t, int n) {
+    for (int m = 0; m < n; ++m) {
+        // right face (i + 1/2) from the five upwind nodes
+        const S* r = c.row;
+        const S fi = r[0];
+        S fr = POS ? weno_face(r[-2], r[-1], fi, r[1], r[2]) : weno_face(r[3], r[2], r[1], fi, r[-1]);
+        if (c.at_wall) fr = c.wall[SW - 1];
+        S fl = __shfl_up_sync(0xffffffffu, fr, 1);
+        if (c.lane == 0) fl = c.wall[0];
+        S tgt = c.Px[0] * c.Y[0];
+#pragma unroll
+        for (int a = 1; a < 4; ++a) tgt += c.Px[a] * c.Y[a * c.TcS];
+        S inc = c.xp * (fr - fl) + (tgt - fi) * c.invtau;
+        if (FORCE) {
+            const int ky = (t + m) / fc.Tz, kz = (t + m) - ky * fc.Tz;
+            const S* Kr = fc.K + ky * fc.Qy;
+            const S* q = fc.f + (size_t)kz * fc.stride;
+            S d = (S)0;
+            for (int kp = 0; kp < fc.Qy; ++kp, q += (size_t)fc.Tz * fc.stride) d += Kr[kp] * *q;
+            inc -= fc.ay * d;
+        }
+        const S out = rk_combine(g, fi, g.first ? (S)0 : *c.fo, inc, c.elem);
+        if (c.valid) *c.dst = out;
+        *c.fo = c.valid ? out : (S)0;
+        c.row += SW;
+        c.wall += SW;
+        c.Y += TILE;
+        c.fo += TILE;
+        c.dst += c.ld;
+        c.elem += (uint32_t)c.ld;
+    }
 }
 
 // Velocities [k0, k1) of one tile for RK stage `stage`, by W warps (lane, warp wy; the moment
@@ -1758,64 +1869,47 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
     const C* Kyc = Tabs<C>::Ky(I);
     // padding lanes read the last node's values and write nothing
     const int li = valid ? lane : N - 1 - i0;
-    const bool at_wall = i + 1 == N;
-    int kx = ka / Tc, t = ka - kx * Tc, kz = t % Tz, ky = t / Tz;
-    C Px[4] = {(C)0, (C)0, (C)0, (C)0}, xp = (C)0;
-    bool pos = true;
-    for (int m = 0; m < nk; ++m, ++t, ++kz) {
-        const int k = ka + m;
-        if (t == Tc) {
-            t = 0;
-            ++kx;
-            ky = kz = 0;
-        } else if (kz == Tz) {
-            kz = 0;
-            ++ky;
-        }
-        if (m == 0 || t == 0) {
-            pos = kx < Q;
-            xp = xpi * pxc[kx];
+    Lane<S> c;
+    c.valid = valid;
+    c.at_wall = i + 1 == N;
+    c.lane = lane;
+    c.ld = ld;
+    c.TcS = Tc * TILE;
+    c.invtau = invtau;
+    c.row = Sw + (ka - k0) * SW + 4 + li;
+    c.wall = Sw + (ka - k0) * SW;
+    c.fo = fo + (ka - k0) * TILE + lane;
+    c.dst = dst + (size_t)ka * ld + i;
+    c.elem = (uint32_t)ka * (uint32_t)ld + (uint32_t)i;
+    int kx = ka / Tc, t = ka - kx * Tc;
+    for (int left = nk; left > 0; ++kx) {
+        const int nt = min(left, Tc - t);
+        c.xp = xpi * pxc[kx];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) Px[a] = stab[(a * NKX + kx - kx0) * TILE + lane];
-        }
-        const S* row = Sw + (k - k0) * SW + 4 + li;
-        C v[5];                                    // upwind order, v[2] the face's own side
-        if (pos) {
-#pragma unroll
-            for (int j = 0; j < 5; ++j) v[j] = row[j - 2];
-        } else {
-#pragma unroll
-            for (int j = 0; j < 5; ++j) v[j] = row[3 - j];
-        }
-        const C fi = pos ? v[2] : v[3];
-        C fr = weno_face(v[0], v[1], v[2], v[3], v[4]);             // right face (i + 1/2)
-        if (at_wall) fr = row[SW - 5 - li];
-        C fl = __shfl_up_sync(0xffffffffu, fr, 1);
-        if (lane == 0) fl = row[-4 - li];
-        const C* Yt = stab + (4 * NKX + t) * TILE + lane;
-        C tgt = Px[0] * Yt[0];
-#pragma unroll
-        for (int a = 1; a < 4; ++a) tgt += Px[a] * Yt[a * Tc * TILE];
-        C inc = xp * (fr - fl) + (tgt - fi) * invtau;
+        for (int a = 0; a < 4; ++a) c.Px[a] = stab[(a * NKX + kx - kx0) * TILE + lane];
+        c.Y = stab + (4 * NKX + t) * TILE + lane;
+        Force<S> fc;
         if (force) {
-            const int kg = kx * Tc + kz;               // first of the p_y values
-            const C* Kr = Kyc + ky * Qy;
-            C d = 0;
-            if (kx * Tc >= k0 && (kx + 1) * Tc <= k1) {
-                const S* rg = Sw + (kg - k0) * SW + 4 + li;
-                for (int kp = 0; kp < Qy; ++kp) d += Kr[kp] * rg[kp * Tz * SW];
-            } else {
-                for (int kp = 0; kp < Qy; ++kp) d += Kr[kp] * src[(size_t)(kg + kp * Tz) * ld + i0 + li];
-            }
-            inc -= ay * d;
+            // the rows of this x-velocity's other p_y: staged if the chunk has them all
+            const bool in = kx * Tc >= k0 && (kx + 1) * Tc <= k1;
+            fc.f = in ? Sw + (kx * Tc - k0) * SW + 4 + li : src + (size_t)kx * Tc * ld + i0 + li;
+            fc.stride = in ? SW : ld;
+            fc.K = Kyc;
+            fc.ay = ay;
+            fc.Qy = Qy;
+            fc.Tz = Tz;
+            if (kx < Q) update_run<S, true, true>(g, c, fc, t, nt);
+            else update_run<S, false, true>(g, c, fc, t, nt);
+        } else if (kx < Q) {
+            update_run<S, true, false>(g, c, fc, t, nt);
+        } else {
+            update_run<S, false, false>(g, c, fc, t, nt);
         }
-        S* fk = fo + (k - k0) * TILE + lane;
-        const S out = rk_combine(g, fi, g.first ? (S)0 : *fk, inc, (uint32_t)k * (uint32_t)ld + (uint32_t)i);
-        if (valid) dst[(size_t)k * ld + i] = out;
-        *fk = valid ? out : (S)0;
+        left -= nt;
+        t = 0;
     }
     __syncthreads();                      // every warp is done with table and rows (ex aliases them)
-    chunk_moments<S>(I, i0, k0, k1, k0 / I.ukc, fo, ex, tws, lane, wy, W);
+    chunk_moments<S>(I, i0, k0, k1, k0 / I.ukc, fo, ex, tws, lane, wy);
     return true;
 }
 
