@@ -10,11 +10,19 @@
 // K = 16 per instruction) by one thread, accumulated in tensor memory, completed through an
 // mbarrier and read back with tcgen05.ld (thread t of the 128-thread block owns TMEM lane t).
 //
-// Forward: one block per 128-point tile, weights converted to BF16 in shared memory, the
+// Forward: one block per 128-point tile, the weights' BF16 images copied into shared memory, the
 // activation tile chained through one shared buffer.  Backward (training): per tile,
 // dW_l = H_{l-1}^T dZ_l and dH_{l-1} = dZ_l W_l^T as tcgen05 GEMMs; each block writes its
 // gradient to its own slot of a partial buffer, and the Adam kernel adds the slots in block
-// order (deterministic) before the update.  This network has no counterpart in the paper.
+// order (deterministic) before the update and refreshes the BF16 images.  This network has no
+// counterpart in the paper.
+//
+// What bounds a tile: the activation functions and the staging of operands between the GEMMs
+// (the tensor pipe is busy for under 1 %).  So a block has 16 warps: tensor memory lane quarter
+// w % 4 (a warp reaches no other) and column quarter w / 4, one point and 32 columns per thread;
+// operands whose 8 consecutive columns belong to one thread are stored 16 bytes at a time; the
+// pre-activations go to global memory with the point fastest, so that a warp writes and reads
+// whole lines.
 #include "../../include/fdlb.h"
 
 #include <cuda_bf16.h>
@@ -37,6 +45,7 @@ constexpr int OW4 = OB3 + NH, OB4 = OW4 + NH * NH;
 constexpr int OW5 = OB4 + NH, OB5 = OW5 + NH * NOUT;
 constexpr int NPARAM = OB5 + NOUT;                 // 53776
 constexpr int TILE = 128;
+constexpr int THREADS = 512;                       // 16 warps: 4 lane quarters x 4 column quarters
 constexpr int WAIT_LIMIT = 4000000;                // bounded mbarrier wait
 
 __host__ __device__ constexpr int woff(int l) { return l == 1 ? OW1 : l == 2 ? OW2 : l == 3 ? OW3 : l == 4 ? OW4 : OW5; }
@@ -117,18 +126,30 @@ __device__ __forceinline__ void tmem_free(uint32_t tmem, int cols) {
 }
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float z) {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+// GELU and its derivative from one error function.
+__device__ __forceinline__ float gelu_both(float z, float& grad) {
+    const float phi = 1.0f + erff(z * 0.70710678118654752f);
+    grad = 0.5f * phi + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+    return 0.5f * z * phi;
 }
 
 __device__ __forceinline__ void put_bf16(unsigned char* base, int off, float v) {
     *reinterpret_cast<__nv_bfloat16*>(base + off) = __float2bfloat16_rn(v);
 }
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+// 8 consecutive columns of one row (one 16-byte line of a core matrix)
+__device__ __forceinline__ void put8(unsigned char* base, int off, const float* v) {
+    *reinterpret_cast<uint4*>(base + off) = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+}
 
 // ------------------------------------------------------------------------------ packed weights
 // The BF16 core-matrix images of the weights that the forward and backward kernels use as
-// GEMM operands, written once per call from the FP32 master copy (k_mlp_pack) and copied into
-// each block's shared memory with bulk asynchronous copies.
+// GEMM operands.  They belong to the handle's state like the FP32 master copy: written whenever
+// that is (initialisation, set_params, the Adam update), and copied into each block's shared
+// memory with bulk asynchronous copies.
 constexpr int PK_FWD = 106496;                 // W1t, W2t..W4t, W5t (the forward's first bytes)
 constexpr int PK_BWD = 102400;                 // W2n..W4n, W5n (the backward's first bytes)
 constexpr int PK_BYTES = PK_FWD + PK_BWD;
@@ -152,31 +173,35 @@ __device__ bool load_packed(unsigned char* dst, const unsigned char* src, int by
     return __syncthreads_and(wait_bar(cbar, 0) ? 1 : 0) != 0;
 }
 
-__global__ void k_mlp_pack(const float* __restrict__ prm, unsigned char* __restrict__ pk) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+// BF16 images of parameter e (value v): forward operands B = W_l^T (rows: outputs, K = inputs);
+// backward B = W_l (rows: inputs, K = outputs) for l >= 2; byte offsets as in the kernels'
+// shared-memory layouts.  Biases have none.
+__device__ __forceinline__ void pack_param(unsigned char* pk, int e, float v) {
     unsigned char* fw = pk;
     unsigned char* bw = pk + PK_FWD;
-    // forward operands B = W_l^T (rows: outputs, K = inputs); backward B = W_l (rows: inputs,
-    // K = outputs) for l >= 2; byte offsets as in the kernels' shared-memory layouts
     if (e < OB1) {
-        const int k = e / NH, n = e % NH;
-        put_bf16(fw, cm(n, k, NIN), prm[e]);
+        put_bf16(fw, cm(e % NH, e / NH, NIN), v);
     } else {
         for (int l = 2; l <= 4; ++l) {
             const int q = e - woff(l);
             if (q >= 0 && q < NH * NH) {
                 const int a = q / NH, b = q % NH;
-                put_bf16(fw + 4096 + (l - 2) * 32768, cm(b, a, NH), prm[e]);
-                put_bf16(bw + (l - 2) * 32768, cm(a, b, NH), prm[e]);
+                put_bf16(fw + 4096 + (l - 2) * 32768, cm(b, a, NH), v);
+                put_bf16(bw + (l - 2) * 32768, cm(a, b, NH), v);
             }
         }
         const int q = e - OW5;
         if (q >= 0 && q < NH * NOUT) {
             const int a = q / NOUT, b = q % NOUT;
-            put_bf16(fw + 4096 + 3 * 32768, cm(b, a, NH), prm[e]);
-            put_bf16(bw + 3 * 32768, cm(a, b, NOUT), prm[e]);
+            put_bf16(fw + 4096 + 3 * 32768, cm(b, a, NH), v);
+            put_bf16(bw + 3 * 32768, cm(a, b, NOUT), v);
         }
     }
+}
+
+__global__ void k_mlp_pack(const float* __restrict__ prm, unsigned char* __restrict__ pk) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < NPARAM) pack_param(pk, e, prm[e]);
 }
 
 // ------------------------------------------------------------------------------ forward
@@ -184,30 +209,44 @@ __global__ void k_mlp_pack(const float* __restrict__ prm, unsigned char* __restr
 constexpr int F_W1 = 0, F_W2 = 4096, F_W3 = F_W2 + 32768, F_W4 = F_W3 + 32768, F_W5 = F_W4 + 32768;
 constexpr int F_A = F_W5 + 4096, F_BIAS = F_A + 32768, F_BYTES = F_BIAS + 4 * 4 * NH + 4 * NOUT;
 
-__global__ void __launch_bounds__(TILE) k_mlp_fwd(const float* __restrict__ prm, const unsigned char* __restrict__ pk,
-                                                  const float* __restrict__ X, int P, float* __restrict__ pred,
-                                                  float* __restrict__ Zs, int* err) {
+// Pre-activations kept for the backward pass, point fastest: Zs[tile][layer][column][point], the last
+// tile with its own number of points.
+__device__ __forceinline__ float* z_row(float* Zs, int row) { return Zs + (size_t)blockIdx.x * (4 * NH * TILE) + row; }
+__device__ __forceinline__ int z_stride(int P) { return min(TILE, P - (int)blockIdx.x * TILE); }
+
+__global__ void __launch_bounds__(THREADS) k_mlp_fwd(const float* __restrict__ prm, const unsigned char* __restrict__ pk,
+                                                     const float* __restrict__ X, int P, float* __restrict__ pred,
+                                                     float* __restrict__ Zs, int* err) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(8) uint64_t bar, cbar;
     __shared__ uint32_t tslot;
-    const int tid = threadIdx.x;
-    const int p = blockIdx.x * TILE + tid;
+    const int tid = threadIdx.x, wid = tid >> 5;
+    const int row = (wid & 3) * 32 + (tid & 31), cg = (wid >> 2) * 32;   // this thread's point and columns
+    const int p = blockIdx.x * TILE + row;
     const bool valid = p < P;
+    float* z = z_row(Zs, row);
+    const int zs = z_stride(P);
     if (tid < 32) tmem_alloc(&tslot, NH);
-    // weights as B operands (N = outputs x K = inputs): the packed BF16 image, biases
-    static_assert(F_A == PK_FWD, "packed forward image = the weight region of shared memory");
-    bool ok = load_packed(sm, pk, PK_FWD, &cbar);
+    // input tile (K = 16): four features per thread
+    {
+        const int r = tid >> 2, k = (tid & 3) * 4, q = blockIdx.x * TILE + r;
+        float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (q < P)
+            for (int j = 0; j < 4; ++j) x[j] = X[(size_t)q * NIN + k + j];
+        *reinterpret_cast<uint2*>(sm + F_A + cm(r, k, NIN)) = make_uint2(pack2(x[0], x[1]), pack2(x[2], x[3]));
+    }
     float* bias = reinterpret_cast<float*>(sm + F_BIAS);
-    for (int e = tid; e < 4 * NH + NOUT; e += TILE) bias[e] = e < 4 * NH ? prm[boff(e / NH + 1) + e % NH] : prm[OB5 + e - 4 * NH];
-    // input tile (K = 16)
-    for (int k = 0; k < NIN; ++k) put_bf16(sm + F_A, cm(tid, k, NIN), valid ? X[(size_t)p * NIN + k] : 0.0f);
+    for (int e = tid; e < 4 * NH + NOUT; e += THREADS) bias[e] = e < 4 * NH ? prm[boff(e / NH + 1) + e % NH] : prm[OB5 + e - 4 * NH];
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(saddr(&bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // weights as B operands (N = outputs x K = inputs): the packed BF16 image, biases
+    static_assert(F_A == PK_FWD, "packed forward image = the weight region of shared memory");
+    bool ok = load_packed(sm, pk, PK_FWD, &cbar);
     sync_for_mma();
     const uint32_t tmem = tslot;
-    const uint32_t lane_addr = tmem + ((uint32_t)((tid >> 5) * 32) << 16);
+    const uint32_t lane_addr = tmem + ((uint32_t)((wid & 3) * 32) << 16);
     for (int l = 1; l <= 5 && ok; ++l) {
         const int K = l == 1 ? NIN : NH, N = l == 5 ? NOUT : NH;
         const unsigned char* W = sm + (l == 1 ? F_W1 : l == 2 ? F_W2 : l == 3 ? F_W3 : l == 4 ? F_W4 : F_W5);
@@ -219,19 +258,23 @@ __global__ void __launch_bounds__(TILE) k_mlp_fwd(const float* __restrict__ prm,
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!ok) break;                      // uniform across the block
         const float* bl = bias + (l - 1) * NH;
-        for (int c0 = 0; c0 < N; c0 += 32) {
+        if (cg < N) {                        // layer 5: the first column quarter only
             float v[32];
-            tmem_ld32(lane_addr + c0, v);    // 32 columns (all inside the 128 allocated)
-            const int cn = N - c0 < 32 ? N - c0 : 32;
-            for (int j = 0; j < cn; ++j) {
-                const int c = c0 + j;
-                const float z = v[j] + bl[c];
-                if (l < 5) {
-                    if (Zs && valid) Zs[(size_t)p * 4 * NH + (l - 1) * NH + c] = z;
-                    put_bf16(sm + F_A, cm(tid, c, NH), gelu(z));
-                } else if (c < NUSED && valid) {
-                    pred[(size_t)p * NUSED + c] = z;
+            tmem_ld32(lane_addr + cg, v);    // 32 columns (all inside the 128 allocated)
+            if (l < 5) {
+#pragma unroll
+                for (int c = 0; c < 32; c += 8) {
+                    float h[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float x = v[c + j] + bl[cg + c + j];
+                        if (Zs && valid) z[((l - 1) * NH + cg + c + j) * zs] = x;
+                        h[j] = gelu(x);
+                    }
+                    put8(sm + F_A, cm(row, cg + c, NH), h);
                 }
+            } else if (valid) {
+                for (int c = 0; c < NUSED; ++c) pred[(size_t)p * NUSED + c] = v[c] + bl[c];
             }
         }
         sync_for_mma();
@@ -248,61 +291,76 @@ __global__ void __launch_bounds__(TILE) k_mlp_fwd(const float* __restrict__ prm,
 constexpr int B_W2 = 0, B_W3 = 32768, B_W4 = 65536, B_W5 = 98304, B_A = B_W5 + 4096, B_B = B_A + 32768, B_C = B_B + 32768;
 constexpr int B_BYTES = B_C + 32768;
 
-__global__ void __launch_bounds__(TILE) k_mlp_bwd(const unsigned char* __restrict__ pk, const float* __restrict__ X,
-                                                  const float* __restrict__ Y, int P, const float* __restrict__ pred,
-                                                  const float* __restrict__ Zs, float* __restrict__ gpart,
-                                                  float* __restrict__ lpart, int* err) {
+__global__ void __launch_bounds__(THREADS) k_mlp_bwd(const unsigned char* __restrict__ pk, const float* __restrict__ X,
+                                                     const float* __restrict__ Y, int P, const float* __restrict__ pred,
+                                                     float* __restrict__ Zs, float* __restrict__ gpart,
+                                                     float* __restrict__ lpart, int* err) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(8) uint64_t bar, cbar;
     __shared__ uint32_t tslot;
     __shared__ float red[TILE / 32];
-    const int tid = threadIdx.x;
-    const int p = blockIdx.x * TILE + tid;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    const int row = (wid & 3) * 32 + lane, cg = (wid >> 2) * 32;         // this thread's point and columns
+    const int p = blockIdx.x * TILE + row;
     const bool valid = p < P;
     float* g = gpart + (size_t)blockIdx.x * NPARAM;
+    const float* z = z_row(Zs, row);
+    const int zs = z_stride(P);
     if (tid < 32) tmem_alloc(&tslot, 2 * NH);
-    // weights as B operands of the dH GEMMs (N = inputs x K = outputs): the packed BF16 image
-    static_assert(B_A == PK_BWD, "packed backward image = the weight region of shared memory");
-    bool ok = load_packed(sm, pk + PK_FWD, PK_BWD, &cbar);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(saddr(&bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // dZ_5 = dL/dpred on the used outputs; loss partial
-    float d[NH];
+    // weights as B operands of the dH GEMMs (N = inputs x K = outputs): the packed BF16 image
+    static_assert(B_A == PK_BWD, "packed backward image = the weight region of shared memory");
+    bool ok = load_packed(sm, pk + PK_FWD, PK_BWD, &cbar);
+    // dZ_5 = dL/dpred on the used outputs (columns 0..2 of the first column quarter); loss partial
+    float d[32];
     float sq = 0.0f;
 #pragma unroll
-    for (int j = 0; j < NH; ++j) d[j] = 0.0f;
-    if (valid)
+    for (int j = 0; j < 32; ++j) d[j] = 0.0f;
+    if (valid && cg == 0)
+#pragma unroll
         for (int j = 0; j < NUSED; ++j) {
             const float df = pred[(size_t)p * NUSED + j] - Y[(size_t)p * NUSED + j];
             sq += df * df;
             d[j] = 2.0f * df / (float)(NUSED * P);
         }
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if ((tid & 31) == 0) red[tid >> 5] = sq;
+    if (cg == 0 && lane == 0) red[wid & 3] = sq;
     sync_for_mma();
     if (tid == 0) lpart[blockIdx.x] = red[0] + red[1] + red[2] + red[3];
     const uint32_t tmem = tslot;
-    const uint32_t lane_addr = tmem + ((uint32_t)((tid >> 5) * 32) << 16);
+    const uint32_t lane_addr = tmem + ((uint32_t)((wid & 3) * 32) << 16);
     uint32_t phase = 0;
     for (int l = 5; l >= 1 && ok; --l) {
         const int N = l == 5 ? NOUT : NH;          // outputs of layer l
         // operands: dW GEMM  A = H_{l-1}^T (rows: inputs), B = dZ^T (rows: outputs), K = points;
         //           layer 1: A = dZ_1^T (rows: outputs), B = X^T (rows: inputs).
         //           dH GEMM  A = dZ (rows: points, K = outputs), B = W_l natural (rows: inputs).
+        float dg[32];                              // GELU'(Z_{l-1}) of this thread's columns
         if (l >= 2) {
-            for (int c = 0; c < NH; ++c) {
-                const float z = valid ? Zs[(size_t)p * 4 * NH + (l - 2) * NH + c] : 0.0f;
-                put_bf16(sm + B_A, cm(c, tid, TILE), valid ? gelu(z) : 0.0f);
+#pragma unroll
+            for (int c = 0; c < 32; ++c) {
+                const float h = gelu_both(valid ? z[((l - 2) * NH + cg + c) * zs] : 0.0f, dg[c]);
+                put_bf16(sm + B_A, cm(cg + c, row, TILE), valid ? h : 0.0f);
+                if (!valid) dg[c] = 0.0f;
             }
-            for (int j = 0; j < N; ++j) {
-                put_bf16(sm + B_B, cm(j, tid, TILE), d[j]);
-                put_bf16(sm + B_C, cm(tid, j, N), d[j]);
+            if (cg < N) {
+                const int n = N < 32 ? N : 32;
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (j < n) put_bf16(sm + B_B, cm(cg + j, row, TILE), d[j]);
+#pragma unroll
+                for (int j = 0; j < 32; j += 8)
+                    if (j < n) put8(sm + B_C, cm(row, cg + j, N), d + j);
             }
         } else {
-            for (int j = 0; j < NH; ++j) put_bf16(sm + B_A, cm(j, tid, TILE), d[j]);
-            for (int k = 0; k < NIN; ++k) put_bf16(sm + B_B, cm(k, tid, TILE), valid ? X[(size_t)p * NIN + k] : 0.0f);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) put_bf16(sm + B_A, cm(cg + j, row, TILE), d[j]);
+            // X^T: four features per thread
+            for (int k = (wid >> 2) * 4; k < (wid >> 2) * 4 + 4; ++k)
+                put_bf16(sm + B_B, cm(k, row, TILE), valid ? X[(size_t)p * NIN + k] : 0.0f);
         }
         sync_for_mma();
         if (tid == 0) {
@@ -314,38 +372,47 @@ __global__ void __launch_bounds__(TILE) k_mlp_bwd(const unsigned char* __restric
         phase ^= 1;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!ok) break;                      // uniform across the block
-        // weight gradient: row tid of the dW accumulator
+        // weight gradient: row `row`, columns from cg, of the dW accumulator
         const int NW = l >= 2 ? N : NIN;
-        for (int c0 = 0; c0 < NW; c0 += 32) {
-            float v[32];
-            tmem_ld32(lane_addr + c0, v);        // 32 columns inside the dW accumulator's 128
-            const int cn = NW - c0 < 32 ? NW - c0 : 32;
-            for (int j = 0; j < cn; ++j) {
-                const int c = c0 + j;
-                if (l >= 2) g[woff(l) + tid * N + c] = v[j];          // dW_l[in = tid][out = c]
-                else g[OW1 + c * NH + tid] = v[j];                    // dW_1[in = c][out = tid]
+        float v[32];
+        if (cg < NW) {
+            tmem_ld32(lane_addr + cg, v);        // 32 columns inside the dW accumulator's 128
+            if (l == 1) {
+#pragma unroll
+                for (int j = 0; j < NIN; ++j) g[OW1 + j * NH + row] = v[j];            // dW_1[in = j][out = row]
+            } else {
+                // dW_l[in = row][out = cg + j], 16 bytes at a time (woff(l) and N are multiples of 4)
+                float4* o = reinterpret_cast<float4*>(g + woff(l) + row * N + cg);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (4 * j < NW) o[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             }
         }
-        // bias gradient: column sums of dZ_l over the tile's points
+        // bias gradient: column sums of dZ_l over the tile's points, four threads per column
         {
             const unsigned char* src = sm + (l >= 2 ? B_B : B_A);
-            if (tid < N) {
-                float s = 0.0f;
-                for (int q = 0; q < TILE; ++q) s += __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(src + cm(tid, q, TILE)));
-                g[boff(l) + tid] = s;
-            }
+            const int col = tid >> 2, part = tid & 3;
+            float s = 0.0f;
+            if (col < N)
+                for (int q = part * 32; q < part * 32 + 32; q += 8) {
+                    const uint4 w = *reinterpret_cast<const uint4*>(src + cm(col, q, TILE));
+                    const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x[j]));
+                        s += f.x;
+                        s += f.y;
+                    }
+                }
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (part == 0 && col < N) g[boff(l) + col] = s;
         }
         if (l >= 2) {
             // dH_{l-1} (row = point), then dZ_{l-1} = dH * GELU'(Z_{l-1})
-            for (int c0 = 0; c0 < NH; c0 += 32) {
-                float v[32];
-                tmem_ld32(lane_addr + NH + c0, v);
+            tmem_ld32(lane_addr + NH + cg, v);
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float z = valid ? Zs[(size_t)p * 4 * NH + (l - 2) * NH + c0 + j] : 0.0f;
-                    d[c0 + j] = valid ? v[j] * gelu_grad(z) : 0.0f;
-                }
-            }
+            for (int j = 0; j < 32; ++j) d[j] = v[j] * dg[j];
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
@@ -359,18 +426,28 @@ __global__ void __launch_bounds__(TILE) k_mlp_bwd(const unsigned char* __restric
 
 // ------------------------------------------------------------------------------ Adam
 __global__ void k_mlp_adam(float* prm, float* m, float* v, const float* gpart, int nblk, float lr, float b1t, float b2t,
-                           float* gout) {
+                           float* gout, unsigned char* pk) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= NPARAM) return;
     float gsum = 0.0f;
-    for (int b = 0; b < nblk; ++b) gsum += gpart[(size_t)b * NPARAM + q];
+    // (in block order; the loads of a batch in flight together)
+    constexpr int B = 16;
+    for (int b = 0; b < nblk; b += B) {
+        float x[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) x[j] = b + j < nblk ? gpart[(size_t)(b + j) * NPARAM + q] : 0.0f;
+#pragma unroll
+        for (int j = 0; j < B; ++j) gsum += x[j];
+    }
     if (gout) gout[q] = gsum;
     if (lr == 0.0f) return;
     const float mq = 0.9f * m[q] + 0.1f * gsum;
     const float vq = 0.999f * v[q] + 0.001f * gsum * gsum;
     m[q] = mq;
     v[q] = vq;
-    prm[q] -= lr * (mq / (1.0f - b1t)) / (sqrtf(vq / (1.0f - b2t)) + 1e-8f);
+    const float w = prm[q] - lr * (mq / (1.0f - b1t)) / (sqrtf(vq / (1.0f - b2t)) + 1e-8f);
+    prm[q] = w;
+    pack_param(pk, q, w);
 }
 
 // Glorot-uniform weights from a counter-based hash (splitmix64 of seed and index), zero biases;
@@ -476,6 +553,7 @@ extern "C" int fdlb_mlp_create(fdlb_mlp** out, void* dev_ws, size_t bytes, int32
     if (!rc) rc = mlp_cuda(h, cudaFuncSetAttribute(k_mlp_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, B_BYTES), "attributes");
     if (!rc) {
         k_mlp_init<<<(NPARAM + 255) / 256, 256, 0, h->stream>>>(h->prm, h->m, h->v, (unsigned long long)seed);
+        k_mlp_pack<<<(NPARAM + 255) / 256, 256, 0, h->stream>>>(h->prm, h->pk);
         rc = mlp_cuda(h, cudaGetLastError(), "init kernel");
     }
     if (!rc) rc = mlp_cuda(h, cudaMemsetAsync(h->err, 0, sizeof(int), h->stream), "clear");
@@ -499,6 +577,10 @@ extern "C" int fdlb_mlp_set_params(fdlb_mlp* h, const float* host) {
     int rc = mlp_cuda(h, cudaMemcpyAsync(h->prm, host, sizeof(float) * NPARAM, cudaMemcpyHostToDevice, h->stream), "copy");
     if (!rc) rc = mlp_cuda(h, cudaMemsetAsync(h->m, 0, sizeof(float) * NPARAM, h->stream), "clear");
     if (!rc) rc = mlp_cuda(h, cudaMemsetAsync(h->v, 0, sizeof(float) * NPARAM, h->stream), "clear");
+    if (!rc) {
+        k_mlp_pack<<<(NPARAM + 255) / 256, 256, 0, h->stream>>>(h->prm, h->pk);
+        rc = mlp_cuda(h, cudaGetLastError(), "pack kernel");
+    }
     if (!rc) rc = mlp_cuda(h, cudaStreamSynchronize(h->stream), "synchronize");
     h->t = 0;
     return rc;
@@ -515,8 +597,7 @@ static int check_err(fdlb_mlp* h) {
 extern "C" int fdlb_mlp_predict(fdlb_mlp* h, const float* dev_x, int32_t points, float* dev_y) {
     if (!h || !dev_x || !dev_y || points < 1) return mlp_fail(h, FDLB_EINVAL, "fdlb_mlp_predict: bad arguments");
     const int nblk = (points + TILE - 1) / TILE;
-    k_mlp_pack<<<(NPARAM + 255) / 256, 256, 0, h->stream>>>(h->prm, h->pk);
-    k_mlp_fwd<<<nblk, TILE, F_BYTES, h->stream>>>(h->prm, h->pk, dev_x, points, dev_y, nullptr, h->err);
+    k_mlp_fwd<<<nblk, THREADS, F_BYTES, h->stream>>>(h->prm, h->pk, dev_x, points, dev_y, nullptr, h->err);
     int rc = mlp_cuda(h, cudaGetLastError(), "forward kernel");
     if (!rc) rc = check_err(h);
     return rc;
@@ -527,13 +608,12 @@ extern "C" int fdlb_mlp_train_step(fdlb_mlp* h, const float* dev_x, const float*
     if (!h || !dev_x || !dev_y || points < 1 || points > h->max_points || !(lr >= 0.0f))
         return mlp_fail(h, FDLB_EINVAL, "fdlb_mlp_train_step: bad arguments (points must be <= max_points)");
     const int nblk = (points + TILE - 1) / TILE;
-    k_mlp_pack<<<(NPARAM + 255) / 256, 256, 0, h->stream>>>(h->prm, h->pk);
-    k_mlp_fwd<<<nblk, TILE, F_BYTES, h->stream>>>(h->prm, h->pk, dev_x, points, h->pred, h->Zs, h->err);
-    k_mlp_bwd<<<nblk, TILE, B_BYTES, h->stream>>>(h->pk, dev_x, dev_y, points, h->pred, h->Zs, h->gpart, h->lpart, h->err);
+    k_mlp_fwd<<<nblk, THREADS, F_BYTES, h->stream>>>(h->prm, h->pk, dev_x, points, h->pred, h->Zs, h->err);
+    k_mlp_bwd<<<nblk, THREADS, B_BYTES, h->stream>>>(h->pk, dev_x, dev_y, points, h->pred, h->Zs, h->gpart, h->lpart, h->err);
     if (lr > 0.0f) h->t += 1;
     const float b1t = lr > 0.0f ? (float)std::pow(0.9, (double)h->t) : 0.0f;
     const float b2t = lr > 0.0f ? (float)std::pow(0.999, (double)h->t) : 0.0f;
-    k_mlp_adam<<<(NPARAM + 255) / 256, 256, 0, h->stream>>>(h->prm, h->m, h->v, h->gpart, nblk, lr, b1t, b2t, dev_grad);
+    k_mlp_adam<<<(NPARAM + 255) / 256, 256, 0, h->stream>>>(h->prm, h->m, h->v, h->gpart, nblk, lr, b1t, b2t, dev_grad, h->pk);
     int rc = mlp_cuda(h, cudaGetLastError(), "training kernels");
     if (!rc && host_loss) {
         std::vector<float> lp(nblk);
