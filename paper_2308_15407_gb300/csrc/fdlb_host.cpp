@@ -69,6 +69,7 @@ struct fdlb_ctx {
     // than SMs it would run in waves
     int n_sms = 0;
     std::vector<int> upd_blocks;      // update work items of each instance
+    std::vector<int> upd_first, nod_first;   // its first items in d_upd and d_nod
     bool upd_wide = false;            // in use: fdlb_step keeps the choice made at creation (all
     bool upd_wide_all = false;        // instances active); fdlb_run re-chooses at each status check
     // CUDA graph of GRAPH_STEPS steps for one freeze tolerance and update width (replayed by
@@ -862,6 +863,8 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
 
         int tiles = (N + TILE - 1) / TILE;
         const size_t nu0 = wu.size();
+        c->upd_first.push_back((int)nu0);
+        c->nod_first.push_back((int)wn.size());
         for (int t = 0; t < tiles; ++t) {
             for (int k0 = 0; k0 < L.K; k0 += L.ukc) wu.push_back({ii, t * TILE, k0, std::min(L.K, k0 + L.ukc)});
             for (int role = NODAL_ROLES - 1; role >= 0; --role) wn.push_back({ii, t * TILE, role, 0});
@@ -917,6 +920,7 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
     if (!rc) rc = cuda_check(c, prepare_kernels(c->smem_upd_f64, c->smem_upd_f32, c->qmax), "kernel attributes");
     if (!rc) choose_cluster(c);
     if (!rc) rc = cuda_check(c, launch_setup(c->d_inst, count, s), "setup kernel");
+    if (!rc) rc = cuda_check(c, launch_profiles(c->d_inst, c->d_nod, n_nod, c->qmax, s), "setup kernel");
     if (!rc) rc = cuda_check(c, launch_moments(c->d_inst, c->d_upd, n_upd, 0, c->ukc_max, c->any_fp64, c->any_fp32, s), "moments kernel");
     if (!rc) rc = cuda_check(c, launch_resid(c->d_inst, count, -1, 0.0, c->d_resid_all, s), "residual kernel");
     if (!rc) rc = cuda_check(c, cudaStreamSynchronize(s), "fdlb_create synchronize");
@@ -1301,6 +1305,12 @@ extern "C" int fdlb_moments(fdlb_ctx* c, int32_t inst, double* host_out) {
     return rc;
 }
 
+// Moments of instance `inst` from scratch (its own update items).
+static int moments_of(fdlb_ctx* c, int inst) {
+    return cuda_check(c, launch_moments(c->d_inst, c->d_upd + c->upd_first[inst], c->upd_blocks[inst], 0, c->ukc_max, c->any_fp64,
+                                        c->any_fp32, c->stream), "moments kernel");
+}
+
 extern "C" int fdlb_set_profiles(fdlb_ctx* c, int32_t inst, const double* n, const double* uy, const double* T) {
     if (!c || !n || !uy || !T) return fail(c, FDLB_EINVAL, "fdlb_set_profiles: bad arguments");
     if (inst < 0 || inst >= c->count) return fail(c, FDLB_EINVAL, "fdlb_set_profiles: instance out of range");
@@ -1315,8 +1325,9 @@ extern "C" int fdlb_set_profiles(fdlb_ctx* c, int32_t inst, const double* n, con
     }
     if (I.form == FORM_REDUCED1D) for (int i = 0; i < I.N; ++i) rows[2 * I.ld + i] = 0.0;
     int rc = cuda_check(c, cudaMemcpyAsync(I.node, rows.data(), sizeof(double) * rows.size(), cudaMemcpyHostToDevice, c->stream), "profiles upload");
-    if (!rc) rc = cuda_check(c, launch_set_profiles(c->d_inst, inst, c->stream), "profiles kernel");
-    if (!rc) rc = cuda_check(c, launch_moments(c->d_inst, c->d_upd, c->n_upd, 0, c->ukc_max, c->any_fp64, c->any_fp32, c->stream), "moments kernel");
+    const int nod = (I.N + TILE - 1) / TILE * NODAL_ROLES;
+    if (!rc) rc = cuda_check(c, launch_profiles(c->d_inst, c->d_nod + c->nod_first[inst], nod, c->qmax, c->stream), "profiles kernel");
+    if (!rc) rc = moments_of(c, inst);
     if (!rc) rc = cuda_check(c, launch_resid(c->d_inst, c->count, inst, 0.0, c->d_resid_all, c->stream), "residual kernel");
     if (!rc) rc = cuda_check(c, cudaStreamSynchronize(c->stream), "profiles synchronize");
     return rc;
@@ -1424,7 +1435,7 @@ extern "C" int fdlb_set_state(fdlb_ctx* c, int32_t inst, const void* host, size_
         if (!rc) rc = cuda_check(c, cudaMemcpyAsync(I.misc + M_SWITCH, &swd, sizeof(swd), cudaMemcpyHostToDevice, c->stream), "state upload");
     }
     if (!rc) rc = cuda_check(c, cudaMemcpyAsync(I.f[0], static_cast<const char*>(host) + 24 + ph, need - 24 - ph, cudaMemcpyHostToDevice, c->stream), "state upload");
-    if (!rc) rc = cuda_check(c, launch_moments(c->d_inst, c->d_upd, c->n_upd, 0, c->ukc_max, c->any_fp64, c->any_fp32, c->stream), "moments kernel");
+    if (!rc) rc = moments_of(c, inst);
     if (!rc) rc = cuda_check(c, launch_resid(c->d_inst, c->count, inst, 0.0, c->d_resid_all, c->stream), "residual kernel");
     if (!rc) rc = cuda_check(c, cudaMemcpyAsync(I.steps, &st, sizeof(st), cudaMemcpyHostToDevice, c->stream), "state upload");
     if (!rc) rc = cuda_check(c, cudaStreamSynchronize(c->stream), "state synchronize");
@@ -1472,7 +1483,7 @@ int ctx_reanchor(fdlb_ctx* c, int inst) {
     static const int active = FDLB_ACTIVE;
     const Inst& I = c->inst[inst];
     int rc = cuda_check(c, cudaMemcpyAsync(I.status, &active, sizeof(int), cudaMemcpyHostToDevice, c->stream), "status reset");
-    if (!rc) rc = cuda_check(c, launch_moments(c->d_inst, c->d_upd, c->n_upd, 0, c->ukc_max, c->any_fp64, c->any_fp32, c->stream), "moments kernel");
+    if (!rc) rc = moments_of(c, inst);
     if (!rc) rc = cuda_check(c, launch_resid(c->d_inst, c->count, inst, 0.0, c->d_resid_all, c->stream), "residual kernel");
     return rc;
 }

@@ -262,53 +262,6 @@ __global__ void k_setup(Inst* insts) {
     }
 }
 
-// Projected local equilibrium from the profile rows into F (all instances when inst < 0).
-template <typename S>
-__global__ void k_profiles(Inst* insts, int inst) {
-    Inst& I = insts[inst < 0 ? blockIdx.x : inst];
-    if (I.two_phase) {
-        // a two-phase instance restarts in its FP32 phase: the FP64 launch (first in stream
-        // order) resets the phase, the FP32 launch writes f
-        if (sizeof(S) == 8) {
-            if (threadIdx.x == 0) {
-                I.precision = FDLB_FP32_STORAGE;
-                I.misc[M_SWITCH] = -1.0;
-            }
-            return;
-        }
-    } else if ((I.precision == FDLB_FP64) != (sizeof(S) == 8)) {
-        return;
-    }
-    const int ld = I.ld, Q = I.Q, Tc = I.Tc;
-    double c[NTERMS];
-    for (int j = 0; j < NTERMS; ++j) c[j] = 0.0;
-    c[0] = 1.0;
-    for (int i = threadIdx.x; i < I.N; i += blockDim.x) {
-        const double n = I.node[R_N * ld + i], uy = I.node[R_UY * ld + i], T = I.node[R_T * ld + i];
-        double* col = I.tab + tab_col(I, i / TILE * TILE, i % TILE);
-        proj_x(I, 0.0, T, 0, col, TILE);
-        proj_x(I, 0.0, T, 1, col, TILE);
-        build_Y(I, c, uy, T, n, col + 8 * Q * TILE, TILE);
-    }
-    __syncthreads();
-    S* F = static_cast<S*>(I.f[0]);
-    for (int k = 0; k < I.K; ++k) {
-        const int kx = k / Tc, t = k - kx * Tc;
-        for (int i = threadIdx.x; i < ld; i += blockDim.x) {
-            double v = 0.0;
-            if (i < I.N) {
-                const double* col = I.tab + tab_col(I, i / TILE * TILE, i % TILE);
-                for (int a = 0; a < 4; ++a) v = fma(col[(a * 2 * Q + kx) * TILE], col[(8 * Q + a * Tc + t) * TILE], v);
-            }
-            F[(size_t)k * ld + i] = (S)v;
-        }
-    }
-    if (threadIdx.x == 0) {
-        *I.status = FDLB_ACTIVE;
-        *I.steps = 0;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // moments
 // ---------------------------------------------------------------------------
@@ -1088,6 +1041,67 @@ __global__ void __launch_bounds__(TILE * NOD_WARPS, QB == 8 ? 3 : 1) k_nodal(con
     const int st = *(volatile int*)I.status, res = *(const volatile int*)&g.smem_res, pr = *(const volatile int*)&g.precision;
     if (st != FDLB_ACTIVE || res) return;
     nodal_item<QB>(I, w.i0, w.k0, nsm, pr == FDLB_FP32_STORAGE);
+}
+
+// Projected local equilibrium of the profile rows (n, u_x = 0, u_y, T) into F: one block per tile of
+// the work list's x-projection items (the other items leave at once), with the x projection of
+// the closure and the zeroth y and z projections, in FP64 for either storage; then a warp per
+// velocity writes f, whole lines at a time.  (One block per instance with a thread per node took
+// 1.0 ms for a 200-node instance of 288 velocities; this takes 20 us.)  A two-phase instance
+// restarts in its FP32 phase.
+template <int QB>
+__global__ void __launch_bounds__(TILE * NOD_WARPS) k_profiles(Inst* insts, const Work* __restrict__ work) {
+    extern __shared__ __align__(16) double nsm[];
+    __shared__ double Yz[(QYMAX + 4 + QZMAX + 4) * TILE];            // m_l and T_a of y, then of z
+    __shared__ double Yt[(QYMAX + QZMAX) * TILE];                    // P_0 of y, then of z
+    const Work w = work[blockIdx.x];
+    if (w.k0 != 0) return;
+    Inst& I = insts[w.inst];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, i0 = w.i0, i = i0 + lane, ld = I.ld, Q = I.Q, Tc = I.Tc;
+    const bool valid = i < I.N;
+    const int ic = valid ? i : I.N - 1;
+    const bool fp32 = I.two_phase || I.precision == FDLB_FP32_STORAGE;
+    double* col = I.tab + tab_col(I, i0, lane);
+    if (I.xfull) xproj_full<double>(I, i0, nsm, col);
+    else xproj_half<QB, double>(I, i0, nsm, col);
+    const double n = I.node[R_N * ld + ic], T = I.node[R_T * ld + ic];
+    const int form = I.form, Qy = I.Qy, Qz = form == FORM_UNREDUCED ? I.Qz : 0;
+    double* mz = Yz + (QYMAX + 4) * TILE;
+    if (wid == 0 && form != FORM_REDUCED1D)
+        hermite_moments(I.node[R_UY * ld + ic], T, Qy, I.fsq, I.fsq2, I.fisq, I.fisq2, Yz + lane, Yz + (QYMAX + 1) * TILE + lane);
+    if (wid == 1 && Qz)
+        hermite_moments(0.0, T, Qz, I.fsq, I.fsq2, I.fisq, I.fisq2, mz + lane, mz + (QZMAX + 1) * TILE + lane);
+    __syncthreads();
+    for (int k = wid; form != FORM_REDUCED1D && k < Qy + Qz; k += NOD_WARPS) {
+        const bool y = k < Qy;
+        const int kk = y ? k : k - Qy, Qn = y ? Qy : Qz;
+        const double *H = y ? I.yH : I.zH, *m = y ? Yz : mz;
+        double s = 0.0;
+        for (int l = 0; l < Qn; ++l) s = fma(H[l * Qn + kk], m[l * TILE + lane], s);
+        Yt[k * TILE + lane] = s;
+    }
+    __syncthreads();
+    // f = n P_0(p_x) times the transverse value (phi and theta slots carry the Gaussian's moments)
+    for (int kx = wid; kx < 2 * Q; kx += NOD_WARPS) {
+        const double px = valid ? n * col[kx * TILE] : 0.0;          // (written by this block)
+        for (int t = 0; t < Tc; ++t) {
+            double v;
+            if (form == FORM_UNREDUCED) v = px * (Yt[(t / Qz) * TILE + lane] * Yt[(Qy + t % Qz) * TILE + lane]);
+            else if (form == FORM_REDUCED2D) v = px * Yt[(t >> 1) * TILE + lane] * ((t & 1) ? T : 1.0);
+            else v = px * (t ? 2.0 * T : 1.0);
+            const size_t e = (size_t)(kx * Tc + t) * ld + i;
+            if (fp32) static_cast<float*>(I.f[0])[e] = (float)v;
+            else static_cast<double*>(I.f[0])[e] = v;
+        }
+    }
+    if (threadIdx.x == 0 && i0 == 0) {
+        if (I.two_phase) {
+            I.precision = FDLB_FP32_STORAGE;
+            I.misc[M_SWITCH] = -1.0;
+        }
+        *I.status = FDLB_ACTIVE;
+        *I.steps = 0;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1914,7 +1928,7 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
 }
 
 template <typename S, int W>
-__global__ void __launch_bounds__(TILE * W) k_update(const Inst* __restrict__ insts, const Work* __restrict__ work, int stage) {
+__global__ void __launch_bounds__(TILE * W, W == UPD_WARPS ? (sizeof(S) == 4 ? 4 : 3) : 1) k_update(const Inst* __restrict__ insts, const Work* __restrict__ work, int stage) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Inst I;
     const Work w = work[blockIdx.x];
@@ -2113,6 +2127,9 @@ static cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, dim3 bloc
 // a device keep launching.
 namespace {
 constexpr int kMaxDevices = 64;
+// Dynamic sizes above this are opted in: static and dynamic shared memory together may take 48 KB
+// without it, and the kernels' static parts are below 16 KB.
+constexpr size_t SMEM_OPTIN = 32 * 1024;
 struct DevAttr {
     bool consts = false;
     int nodal = 0;
@@ -2137,14 +2154,14 @@ cudaError_t dev_attr(DevAttr** out) {
 
 cudaError_t launch_setup(const Inst* d_inst, int count, cudaStream_t s) {
     k_setup<<<count, 128, 0, s>>>(const_cast<Inst*>(d_inst));
-    k_profiles<double><<<count, 128, 0, s>>>(const_cast<Inst*>(d_inst), -1);
-    k_profiles<float><<<count, 128, 0, s>>>(const_cast<Inst*>(d_inst), -1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_set_profiles(const Inst* d_inst, int inst, cudaStream_t s) {
-    k_profiles<double><<<1, 128, 0, s>>>(const_cast<Inst*>(d_inst), inst);
-    k_profiles<float><<<1, 128, 0, s>>>(const_cast<Inst*>(d_inst), inst);
+cudaError_t launch_profiles(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, cudaStream_t s) {
+    const size_t smem = (size_t)nodal_smem_doubles(qmax) * sizeof(double);
+    Inst* in = const_cast<Inst*>(d_inst);
+    if (qmax <= 8) k_profiles<8><<<n_nod, TILE * NOD_WARPS, smem, s>>>(in, d_nod);
+    else k_profiles<QMAX><<<n_nod, TILE * NOD_WARPS, smem, s>>>(in, d_nod);
     return cudaGetLastError();
 }
 
@@ -2169,11 +2186,11 @@ cudaError_t launch_moments(const Inst* d_inst, const Work* d_upd, int n_upd, int
         std::lock_guard<std::mutex> lk(g_attr_mu);
         DevAttr* A = nullptr;
         cudaError_t e = dev_attr(&A);
-        if (e == cudaSuccess && f64 && m64 > 48 * 1024 && m64 > A->mom64) {
+        if (e == cudaSuccess && f64 && m64 > SMEM_OPTIN && m64 > A->mom64) {
             e = cudaFuncSetAttribute(k_moments<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m64);
             if (e == cudaSuccess) A->mom64 = m64;
         }
-        if (e == cudaSuccess && f32 && m32 > 48 * 1024 && m32 > A->mom32) {
+        if (e == cudaSuccess && f32 && m32 > SMEM_OPTIN && m32 > A->mom32) {
             e = cudaFuncSetAttribute(k_moments<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m32);
             if (e == cudaSuccess) A->mom32 = m32;
         }
@@ -2196,13 +2213,13 @@ cudaError_t launch_resid(const Inst* d_inst, int count, int anchor_inst, double 
 // (the caller holds g_attr_mu)
 static cudaError_t set_smem(DevAttr* A, size_t smem64, size_t smem32) {
     cudaError_t e = cudaSuccess;
-    if (smem64 > 48 * 1024 && smem64 > A->upd64) {
+    if (smem64 > SMEM_OPTIN && smem64 > A->upd64) {
         e = cudaFuncSetAttribute(k_update<double, UPD_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_update<double, UPD_WARPS_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64);
         if (e == cudaSuccess) A->upd64 = smem64;
     }
-    if (e == cudaSuccess && smem32 > 48 * 1024 && smem32 > A->upd32) {
+    if (e == cudaSuccess && smem32 > SMEM_OPTIN && smem32 > A->upd32) {
         e = cudaFuncSetAttribute(k_update<float, UPD_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem32);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_update<float, UPD_WARPS_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem32);
@@ -2236,9 +2253,11 @@ cudaError_t prepare_kernels(size_t smem64, size_t smem32, int qmax) {
         A->consts = true;
     }
     const int smem = nodal_smem_doubles(qmax) * (int)sizeof(double);
-    if (smem > 48 * 1024 && smem > A->nodal) {
+    if ((size_t)smem > SMEM_OPTIN && smem > A->nodal) {
         cudaError_t e = cudaFuncSetAttribute(k_nodal<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k_nodal<QMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_profiles<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_profiles<QMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         A->nodal = smem;
     }

@@ -5,7 +5,7 @@
 
 namespace fdlb {
 
-// Wall Maxwellians, initial uniform equilibrium, status/steps reset, for all instances.
+// Wall Maxwellians, profile rows of the initial uniform state, status/steps reset, for all instances.
 cudaError_t launch_setup(const Inst* d_inst, int count, cudaStream_t s);
 
 // Moments of RK buffer `buf` (0 = F, 1 = A, 2 = B) of every ACTIVE instance from scratch
@@ -25,8 +25,9 @@ size_t update_smem_bound(int trows, int ukc, size_t s);
 cudaError_t launch_resid(const Inst* d_inst, int count, int anchor_inst, double freeze_tol, double* d_resid_all,
                          cudaStream_t s);
 
-// Projected local equilibrium from the profile rows (n, u_x, u_y, T) of instance `inst` into F.
-cudaError_t launch_set_profiles(const Inst* d_inst, int inst, cudaStream_t s);
+// Projected local equilibrium from the profile rows (n, u_x = 0, u_y, T) into F, for the tiles of
+// the closure items d_nod[0..n_nod); qmax as for launch_nodal.
+cudaError_t launch_profiles(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, cudaStream_t s);
 
 // Per-node closure (chi, Pr, tau, gradients, projection tables, wall densities).
 cudaError_t launch_nodal(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, cudaStream_t s);
