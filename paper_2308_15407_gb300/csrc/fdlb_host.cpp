@@ -78,6 +78,10 @@ struct fdlb_ctx {
     double graph_tol = -1.0;
     bool graph_wide = false;
     bool graph_failed = false;
+    // page-locked staging of the read calls (status, moments), made on first use: a copy to pageable
+    // memory waits for itself, and a 2D one goes row by row
+    char* pin = nullptr;
+    std::mutex pin_mu;                // one reader at a time (threads may read a context at once)
     // optional per-kernel-class event timing (fdlb_profile)
     bool prof = false;
     std::vector<cudaEvent_t> ev[KK_COUNT];
@@ -89,6 +93,7 @@ struct fdlb_ctx {
         if (ev_fork) cudaEventDestroy(ev_fork);
         if (ev_join) cudaEventDestroy(ev_join);
         if (stream2) cudaStreamDestroy(stream2);
+        if (pin) cudaFreeHost(pin);
     }
 };
 
@@ -1238,16 +1243,49 @@ extern "C" int fdlb_get_schedule_mix(const fdlb_ctx* c, int32_t* smem_resident, 
     return FDLB_OK;
 }
 
+// Page-locked staging with room for the status arrays of the batch and for the moment rows of its
+// largest instance (the caller holds pin_mu and synchronises before it lets go); null when there
+// is none to be had.
+static char* staging(fdlb_ctx* c) {
+    if (!c->pin) {
+        size_t bytes = (size_t)c->count * (sizeof(double) + sizeof(int) + sizeof(long long));
+        for (auto& I : c->inst) bytes = std::max(bytes, sizeof(double) * 8 * I.ld);
+        void* p = nullptr;
+        if (cudaMallocHost(&p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        c->pin = static_cast<char*>(p);
+    }
+    return c->pin;
+}
+
 extern "C" int fdlb_status(fdlb_ctx* c, double* residual, int32_t* status, int64_t* steps) {
     if (!c) return fail(nullptr, FDLB_EINVAL, "fdlb_status: null context");
+    const size_t n = c->count;
+    std::vector<char> own;
+    std::lock_guard<std::mutex> lk(c->pin_mu);
+    char* h = staging(c);
+    if (!h) {
+        own.resize(n * (sizeof(double) + sizeof(int) + sizeof(long long)));
+        h = own.data();
+    }
+    char *hr = h, *ht = hr + n * sizeof(double), *hs = ht + n * sizeof(long long);
     int rc = FDLB_OK;
-    if (residual && !rc) rc = cuda_check(c, cudaMemcpyAsync(residual, c->d_resid_all, sizeof(double) * c->count, cudaMemcpyDeviceToHost, c->stream), "status copy");
-    if (status && !rc) rc = cuda_check(c, cudaMemcpyAsync(status, c->d_status_all, sizeof(int) * c->count, cudaMemcpyDeviceToHost, c->stream), "status copy");
-    std::vector<long long> st(c->count);
-    if (steps && !rc) rc = cuda_check(c, cudaMemcpyAsync(st.data(), c->d_steps_all, sizeof(long long) * c->count, cudaMemcpyDeviceToHost, c->stream), "status copy");
+    if (residual && !rc) rc = cuda_check(c, cudaMemcpyAsync(hr, c->d_resid_all, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream), "status copy");
+    if (status && !rc) rc = cuda_check(c, cudaMemcpyAsync(hs, c->d_status_all, sizeof(int) * n, cudaMemcpyDeviceToHost, c->stream), "status copy");
+    if (steps && !rc) rc = cuda_check(c, cudaMemcpyAsync(ht, c->d_steps_all, sizeof(long long) * n, cudaMemcpyDeviceToHost, c->stream), "status copy");
     if (!rc) rc = cuda_check(c, cudaStreamSynchronize(c->stream), "status synchronize");
-    if (!rc && steps) for (int i = 0; i < c->count; ++i) steps[i] = st[i];
-    return rc;
+    if (rc) return rc;
+    if (residual) std::memcpy(residual, hr, sizeof(double) * n);
+    if (status) std::memcpy(status, hs, sizeof(int) * n);
+    if (steps)
+        for (size_t i = 0; i < n; ++i) {
+            long long v;
+            std::memcpy(&v, ht + i * sizeof(long long), sizeof(v));
+            steps[i] = v;
+        }
+    return FDLB_OK;
 }
 
 extern "C" int fdlb_residual(fdlb_ctx* c, double* host_out) {
@@ -1299,9 +1337,19 @@ extern "C" int fdlb_moments(fdlb_ctx* c, int32_t inst, double* host_out) {
     if (!c || !host_out) return fail(c, FDLB_EINVAL, "fdlb_moments: bad arguments");
     if (inst < 0 || inst >= c->count) return fail(c, FDLB_EINVAL, "fdlb_moments: instance out of range");
     const Inst& I = c->inst[inst];
-    int rc = cuda_check(c, cudaMemcpy2DAsync(host_out, sizeof(double) * I.N, I.node, sizeof(double) * I.ld,
-                                             sizeof(double) * I.N, 8, cudaMemcpyDeviceToHost, c->stream), "moments copy");
+    std::lock_guard<std::mutex> lk(c->pin_mu);
+    char* h = staging(c);
+    if (!h) {
+        int rc = cuda_check(c, cudaMemcpy2DAsync(host_out, sizeof(double) * I.N, I.node, sizeof(double) * I.ld,
+                                                 sizeof(double) * I.N, 8, cudaMemcpyDeviceToHost, c->stream), "moments copy");
+        if (!rc) rc = cuda_check(c, cudaStreamSynchronize(c->stream), "moments synchronize");
+        return rc;
+    }
+    // the 8 rows are contiguous on the device
+    int rc = cuda_check(c, cudaMemcpyAsync(h, I.node, sizeof(double) * 8 * I.ld, cudaMemcpyDeviceToHost, c->stream), "moments copy");
     if (!rc) rc = cuda_check(c, cudaStreamSynchronize(c->stream), "moments synchronize");
+    if (!rc)
+        for (int r = 0; r < 8; ++r) std::memcpy(host_out + (size_t)r * I.N, h + sizeof(double) * (size_t)r * I.ld, sizeof(double) * I.N);
     return rc;
 }
 

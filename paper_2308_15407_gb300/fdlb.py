@@ -273,9 +273,9 @@ class Solver:
         return self._check(self.lib.fdlb_run(self.ctx, float(tol), int(max_steps), int(check_every), float(timeout_s)))
 
     def moments(self, inst: int = 0) -> dict:
-        out = np.zeros((8, self.nx[inst]))
+        out = np.empty((8, self.nx[inst]))
         self._check(self.lib.fdlb_moments(self.ctx, inst, _dptr(out)))
-        return {k: out[j].copy() for j, k in enumerate(MOMENT_ROWS)}
+        return dict(zip(MOMENT_ROWS, out))
 
     def status(self):
         r = np.zeros(self.count)
