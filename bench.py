@@ -421,10 +421,11 @@ def run_fdlb(args):
                 "kernel_ms_per_step": {k: v[0] / PSTEPS for k, v in prof.items()},
                 "measured_over": "%d RK3 steps of the sweep after 600 start-up steps, per-launch CUDA events on the "
                                  "library's stream" % PSTEPS}
-    # launches in the timed region: per solve, 4 per instance for the reset (profiles x2,
-    # moments, residual anchor) and 7 per RK3 step of the batch (closure and update per stage,
-    # residual) until the last instance stops (fdlb_run advances in chunks of CHECK steps)
-    gpu_launches = sum(4 * s.count + 7 * CHECK * math.ceil(max(x) / CHECK) for x in steps_per_solve)
+    # launches in the timed region: per solve, 3 per instance for the reset (profiles, moments,
+    # residual anchor) and 97 per graph of 16 RK3 steps of the batch (closure and update per stage,
+    # one residual launch; the closure launches of the steps carry the other residual passes) until
+    # the last instance stops (fdlb_run advances in chunks of CHECK steps, a multiple of 16)
+    gpu_launches = sum(3 * s.count + 97 * (CHECK // 16) * math.ceil(max(x) / CHECK) for x in steps_per_solve)
 
     # ---- throughput regime: the 2048-instance mixed sweep in one batch (f > L2)
     batch = None
@@ -585,7 +586,7 @@ def run_profile_case(case, precision):
     """Small fixed workloads for ncu captures (no timing, no JSON line).
     couette1 / couette12: one instance (eta0 = 0.2, Kn = 0.5) or the whole Couette sweep;
     sweep2048: the 2048-instance mixed sweep (f 162 MB in FP32); tiled schedule: creation
-    (5 launches), 20 steps (7 launches each), 3 more steps.
+    (5 launches), 20 steps (6 launches each and one residual launch per call), 3 more steps.
     mlp: the warm-start network on 32768 points, 6 training steps and one prediction."""
     import torch
     from paper_2308_15407_gb300 import fdlb as F

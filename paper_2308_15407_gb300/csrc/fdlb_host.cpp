@@ -47,7 +47,7 @@ struct fdlb_ctx {
     double* d_resid_all = nullptr;    // count doubles (misc[M_RESID] copies)
     cudaStream_t stream = nullptr;
     size_t smem_upd_f64 = 0, smem_upd_f32 = 0;
-    bool any_fp32 = false, any_fp64 = false;
+    bool any_fp32 = false, any_fp64 = false, any_two_phase = false;
     int ukc_max = 1;
     // schedule (FDLB_SCHED_*): requested, and the one in use once chosen (0 = not yet)
     int sched_req = FDLB_SCHED_AUTO, sched = 0;
@@ -114,10 +114,11 @@ static cudaError_t prof_mark(fdlb_ctx* c, int kind) {
     return cudaEventRecord(v[c->nev[kind]++], c->stream);
 }
 
-// One TVD-RK3 step (Eq. rk3): three stages of moments -> closure -> update, then the
-// moments of the new state and the residual/status pass.  The stage-1 moments are the
-// end-of-step moments of the previous step.
-static cudaError_t step_once(fdlb_ctx* c, double freeze_tol) {
+// nsteps TVD-RK3 steps (Eq. rk3): three stages of closure -> update (whose epilogue computes the
+// moments of the stage's result), then the residual/status pass, which the first closure launch of
+// the next step carries (k_nodal) unless launches are timed or a two-phase instance may switch
+// its storage in it.
+static cudaError_t step_many(fdlb_ctx* c, int64_t nsteps, double freeze_tol) {
     cudaError_t e = cudaSuccess;
     auto guard = [&](int kind, auto&& fn) {
         if (e != cudaSuccess) return;
@@ -125,13 +126,17 @@ static cudaError_t step_once(fdlb_ctx* c, double freeze_tol) {
         if (e == cudaSuccess) e = fn();
         if (e == cudaSuccess) e = prof_mark(c, kind);
     };
-    // the update kernel's epilogue computes the moments of each stage's result
-    for (int stage = 1; stage <= 3; ++stage) {
-        guard(KK_NODAL, [&] { return launch_nodal(c->d_inst, c->d_nod, c->n_nod, c->qmax, c->stream); });
-        guard(KK_UPDATE, [&] { return launch_update(c->d_inst, c->d_upd, c->n_upd, stage, c->smem_upd_f64, c->smem_upd_f32,
-                                                    c->any_fp64, c->any_fp32, c->upd_wide, c->stream); });
+    const bool fold = !c->prof && !c->any_two_phase;
+    for (int64_t s = 0; s < nsteps && e == cudaSuccess; ++s) {
+        for (int stage = 1; stage <= 3; ++stage) {
+            const int n_resid = fold && s > 0 && stage == 1 ? c->count : 0;
+            guard(KK_NODAL, [&] { return launch_nodal(c->d_inst, c->d_nod, c->n_nod, c->qmax, n_resid, freeze_tol, c->d_resid_all, c->stream); });
+            guard(KK_UPDATE, [&] { return launch_update(c->d_inst, c->d_upd, c->n_upd, stage, c->smem_upd_f64, c->smem_upd_f32,
+                                                        c->any_fp64, c->any_fp32, c->upd_wide, c->stream); });
+        }
+        if (!fold || s + 1 == nsteps)
+            guard(KK_RESID, [&] { return launch_resid(c->d_inst, c->count, -2, freeze_tol, c->d_resid_all, c->stream); });
     }
-    guard(KK_RESID, [&] { return launch_resid(c->d_inst, c->count, -2, freeze_tol, c->d_resid_all, c->stream); });
     return e;
 }
 
@@ -614,6 +619,7 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
         I.Mx = aux_points_half(p.x_quadrature == FDLB_XQ_FULL ? 2 * p.qx_half : p.qx_half); I.My = L.My; I.Mz = L.Mz;
         I.precision = p.precision == FDLB_FP64 ? FDLB_FP64 : FDLB_FP32_STORAGE;
         I.two_phase = p.precision == FDLB_FP32_THEN_FP64;
+        c->any_two_phase |= I.two_phase != 0;
         I.j1_shear = p.j1_shear;
         I.chi_model = p.chi_model; I.ntab = L.ntab; I.trows = L.trows; I.mgroups = L.groups; I.ukc = L.ukc;
         {
@@ -1073,7 +1079,7 @@ static bool ensure_graph(fdlb_ctx* c, double tol) {
         return false;
     }
     cudaError_t e = cudaSuccess;
-    for (int s = 0; s < GRAPH_STEPS && e == cudaSuccess; ++s) e = step_once(c, tol);
+    e = step_many(c, GRAPH_STEPS, tol);
     cudaError_t e2 = cudaStreamEndCapture(c->stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess || !g) {
         if (g) cudaGraphDestroy(g);
@@ -1110,10 +1116,8 @@ static int step_tiled(fdlb_ctx* c, int64_t nsteps, double freeze_tol) {
             nsteps -= GRAPH_STEPS;
         }
     }
-    for (int64_t s = 0; s < nsteps; ++s) {
-        cudaError_t e = step_once(c, freeze_tol);
-        if (e != cudaSuccess) return cuda_check(c, e, "fdlb_step launch");
-    }
+    cudaError_t e = step_many(c, nsteps, freeze_tol);
+    if (e != cudaSuccess) return cuda_check(c, e, "fdlb_step launch");
     return FDLB_OK;
 }
 

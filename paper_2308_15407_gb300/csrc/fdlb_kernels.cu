@@ -1029,17 +1029,151 @@ __device__ void nodal_item(const Inst& I, int i0, int role, double* nsm, bool fp
     else xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, df{}));
 }
 
+// ---------------------------------------------------------------------------
+// per-step residual and status
+// ---------------------------------------------------------------------------
+// Stagnation of a two-phase instance in its FP32 phase (window rule of FDLB_FP32_THEN_FP64).
+__device__ int stagnated(Inst& I, double r, double step) {
+    if (r == 0.0) return 1;
+    double* m = I.misc;
+    if (m[M_WIN_STEP] < 0.0) {
+        m[M_WIN_STEP] = step;
+        m[M_WIN_RESID] = r;
+        return 0;
+    }
+    if (step - m[M_WIN_STEP] < FDLB_STAGNATION_WINDOW) return 0;
+    if (!(r < FDLB_STAGNATION_FACTOR * m[M_WIN_RESID])) return 1;
+    m[M_WIN_STEP] = step;
+    m[M_WIN_RESID] = r;
+    return 0;
+}
+
+// Residual, status and (two-phase) precision switch of instance I (batch index idx) after a
+// step, by a block of 256 threads; red: 7 x 256 doubles of shared memory.
+__device__ void resid_item(Inst& I, int idx, double tol, double* resid_all, double* red) {
+    const int ld = I.ld, N = I.N;
+    double* nd = I.node;
+    constexpr int RT = 256;                   // threads of the calling block
+    __shared__ double tot[7], term[4];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double s[7] = {0, 0, 0, 0, 0, 0, 0};
+    int bad_nf = 0, bad_ph = 0;
+    for (int i = threadIdx.x; i < N; i += RT) {
+        const double n = nd[R_N * ld + i], ux = nd[R_UX * ld + i], uy = nd[R_UY * ld + i], T = nd[R_T * ld + i];
+        if (!isfinite(n) || !isfinite(ux) || !isfinite(uy) || !isfinite(T)) bad_nf = 1;
+        else if (!(n > 0.0) || !(T > 0.0)) bad_ph = 1;
+        const double w = I.dxw[i];
+        const double dn = n - nd[R_PREV_N * ld + i], dT = T - nd[R_PREV_T * ld + i];
+        const double dux = ux - nd[R_PREV_UX * ld + i], duy = uy - nd[R_PREV_UY * ld + i];
+        s[0] += w * dn * dn;
+        s[1] += w * n * n;
+        s[2] += w * dT * dT;
+        s[3] += w * T * T;
+        s[4] += w * dux * dux;
+        s[5] += w * duy * duy;
+        s[6] += w * n;
+        nd[R_PREV_N * ld + i] = n;
+        nd[R_PREV_UX * ld + i] = ux;
+        nd[R_PREV_UY * ld + i] = uy;
+        nd[R_PREV_T * ld + i] = T;
+    }
+    __shared__ int flags[3];
+    __shared__ double scale;
+    if (threadIdx.x == 0) { flags[0] = 0; flags[1] = 0; flags[2] = 0; }
+#pragma unroll
+    for (int j = 0; j < 7; ++j) red[j * RT + threadIdx.x] = s[j];
+    __syncthreads();
+    if (bad_nf) atomicOr(&flags[0], 1);
+    if (bad_ph) atomicOr(&flags[1], 1);
+    // sum j over the block by warp j (independent FP64 chains on different schedulers)
+    if (wid < 7) {
+        double v = 0.0;
+#pragma unroll
+        for (int q = 0; q < RT / 32; ++q) v += red[wid * RT + q * 32 + lane];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) tot[wid] = v;
+    }
+    __syncthreads();
+    // the four terms of the residual on four warps
+    if (lane == 0 && wid < 4)
+        term[wid] = wid == 0 ? sqrt(tot[0] / tot[1]) : (wid == 1 ? sqrt(tot[2] / tot[3]) : sqrt(tot[wid + 2]));
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double r = fmax(fmax(term[0], term[1]), fmax(term[2], term[3]));
+        *I.steps += 1;
+        I.misc[M_RESID] = r;
+        resid_all[idx] = r;
+        const bool fp32 = I.precision == FDLB_FP32_STORAGE;
+        if (flags[0]) *I.status = FDLB_FAILED_NONFINITE;
+        else if (flags[1]) *I.status = FDLB_FAILED_UNPHYSICAL;
+        else if (fp32 && r == 0.0 && I.two_phase) flags[2] = 1;   // FP32 f stopped changing
+        else if (fp32 && r == 0.0 && tol > 0.0) *I.status = FDLB_STAGNATED;
+        else if (tol > 0.0 && r < tol) *I.status = FDLB_CONVERGED;
+        else if (I.two_phase && fp32) flags[2] = stagnated(I, r, (double)*I.steps);
+        scale = I.misc[M_MASS0] / tot[6];
+    }
+    __syncthreads();
+    if (!flags[2]) return;
+    // Up-cast f: floats of F -> doubles in the stage buffer A, then back into F (which holds
+    // K ld doubles in a two-phase instance; A is free between steps), times the factor that
+    // restores the channel mass of the last anchor.  The discrete scheme conserves mass, but
+    // FP32 rounding near stagnation drops the same small updates step after step and lets the
+    // mass drift, which would move the FP64 steady state.  The node rows are rescaled alike
+    // (extensive rows by the factor, ln n and ln chi(eta0 n) anew; u and T are unchanged),
+    // so the next stage sees the moments of the rescaled f.
+    const double c = scale;
+    const size_t nf = (size_t)I.K * ld;
+    const float* src = static_cast<const float*>(I.f[0]);
+    double* tmp = static_cast<double*>(I.f[1]);
+    for (size_t e = threadIdx.x; e < nf; e += blockDim.x) tmp[e] = (double)src[e] * c;
+    __syncthreads();
+    double* dst = static_cast<double*>(I.f[0]);
+    for (size_t e = threadIdx.x; e < nf; e += blockDim.x) dst[e] = tmp[e];
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        const double n = nd[R_N * ld + i] * c;
+        nd[R_N * ld + i] = n;
+        nd[R_PREV_N * ld + i] *= c;
+        nd[R_QX * ld + i] *= c;
+        nd[R_QY * ld + i] *= c;
+        nd[R_PXX * ld + i] *= c;
+        nd[R_PXY * ld + i] *= c;
+        nd[R_SNEG * ld + i] *= c;
+        nd[R_SPOS * ld + i] *= c;
+        nd[R_LNN * ld + i] = log(n);
+        nd[R_LNCHI * ld + i] = log(chi_cs(I.eta0 * n));
+    }
+    if (threadIdx.x == 0) {
+        I.precision = FDLB_FP64;
+        I.misc[M_SWITCH] = (double)*I.steps;
+    }
+}
+
+
+// The closure launch of a step's first stage can carry the residual pass of the step before it
+// (blocks from n_nod on, one per instance): both only need that step's moments, and the pass, whose
+// chain of one block takes ~5 us, no longer stands between two steps of a small batch (one Couette
+// instance 74 -> 69 us per step).  Whether the instance goes on is decided by the status that the
+// update kernels read; a closure block that still saw ACTIVE has only written tables that nothing
+// reads.  Not with two-phase instances, whose residual pass may rewrite f and the moments.
 template <int QB>
-__global__ void __launch_bounds__(TILE * NOD_WARPS, QB == 8 ? 3 : 1) k_nodal(const Inst* __restrict__ insts, const Work* __restrict__ work) {
+__global__ void __launch_bounds__(TILE * NOD_WARPS, QB == 8 ? 3 : 1) k_nodal(Inst* __restrict__ insts, const Work* __restrict__ work,
+                                                                           int n_nod, double tol, double* resid_all) {
     extern __shared__ __align__(16) double nsm[];
     __shared__ Inst I;
+    if ((int)blockIdx.x >= n_nod) {
+        pdl_wait();
+        Inst& g = insts[blockIdx.x - n_nod];
+        if (*(volatile int*)g.status == FDLB_ACTIVE && !g.smem_res) resid_item(g, blockIdx.x - n_nod, tol, resid_all, nsm);
+        return;
+    }
     const Work w = work[blockIdx.x];
     load_inst(insts + w.inst, &I, threadIdx.x, TILE * NOD_WARPS);
     warm_tables(I, w.k0, threadIdx.x, TILE * NOD_WARPS);
     pdl_wait();
     const Inst& g = insts[w.inst];
     const int st = *(volatile int*)I.status, res = *(const volatile int*)&g.smem_res, pr = *(const volatile int*)&g.precision;
-    if (st != FDLB_ACTIVE || res) return;
+    // (one decision for the block: the residual block of this launch may change the status meanwhile)
+    if (__syncthreads_or(st != FDLB_ACTIVE || res)) return;
     nodal_item<QB>(I, w.i0, w.k0, nsm, pr == FDLB_FP32_STORAGE);
 }
 
@@ -1104,127 +1238,6 @@ __global__ void __launch_bounds__(TILE * NOD_WARPS) k_profiles(Inst* insts, cons
     }
 }
 
-// ---------------------------------------------------------------------------
-// per-step residual and status
-// ---------------------------------------------------------------------------
-// Stagnation of a two-phase instance in its FP32 phase (window rule of FDLB_FP32_THEN_FP64).
-__device__ int stagnated(Inst& I, double r, double step) {
-    if (r == 0.0) return 1;
-    double* m = I.misc;
-    if (m[M_WIN_STEP] < 0.0) {
-        m[M_WIN_STEP] = step;
-        m[M_WIN_RESID] = r;
-        return 0;
-    }
-    if (step - m[M_WIN_STEP] < FDLB_STAGNATION_WINDOW) return 0;
-    if (!(r < FDLB_STAGNATION_FACTOR * m[M_WIN_RESID])) return 1;
-    m[M_WIN_STEP] = step;
-    m[M_WIN_RESID] = r;
-    return 0;
-}
-
-// Residual, status and (two-phase) precision switch of instance I (batch index idx) after a
-// step, by a block of 256 threads.
-__device__ void resid_item(Inst& I, int idx, double tol, double* resid_all) {
-    const int ld = I.ld, N = I.N;
-    double* nd = I.node;
-    constexpr int RT = 256;                   // threads of the calling block
-    __shared__ double red[7][RT];
-    __shared__ double tot[7], term[4];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double s[7] = {0, 0, 0, 0, 0, 0, 0};
-    int bad_nf = 0, bad_ph = 0;
-    for (int i = threadIdx.x; i < N; i += RT) {
-        const double n = nd[R_N * ld + i], ux = nd[R_UX * ld + i], uy = nd[R_UY * ld + i], T = nd[R_T * ld + i];
-        if (!isfinite(n) || !isfinite(ux) || !isfinite(uy) || !isfinite(T)) bad_nf = 1;
-        else if (!(n > 0.0) || !(T > 0.0)) bad_ph = 1;
-        const double w = I.dxw[i];
-        const double dn = n - nd[R_PREV_N * ld + i], dT = T - nd[R_PREV_T * ld + i];
-        const double dux = ux - nd[R_PREV_UX * ld + i], duy = uy - nd[R_PREV_UY * ld + i];
-        s[0] += w * dn * dn;
-        s[1] += w * n * n;
-        s[2] += w * dT * dT;
-        s[3] += w * T * T;
-        s[4] += w * dux * dux;
-        s[5] += w * duy * duy;
-        s[6] += w * n;
-        nd[R_PREV_N * ld + i] = n;
-        nd[R_PREV_UX * ld + i] = ux;
-        nd[R_PREV_UY * ld + i] = uy;
-        nd[R_PREV_T * ld + i] = T;
-    }
-    __shared__ int flags[3];
-    __shared__ double scale;
-    if (threadIdx.x == 0) { flags[0] = 0; flags[1] = 0; flags[2] = 0; }
-#pragma unroll
-    for (int j = 0; j < 7; ++j) red[j][threadIdx.x] = s[j];
-    __syncthreads();
-    if (bad_nf) atomicOr(&flags[0], 1);
-    if (bad_ph) atomicOr(&flags[1], 1);
-    // sum j over the block by warp j (independent FP64 chains on different schedulers)
-    if (wid < 7) {
-        double v = 0.0;
-#pragma unroll
-        for (int q = 0; q < RT / 32; ++q) v += red[wid][q * 32 + lane];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) tot[wid] = v;
-    }
-    __syncthreads();
-    // the four terms of the residual on four warps
-    if (lane == 0 && wid < 4)
-        term[wid] = wid == 0 ? sqrt(tot[0] / tot[1]) : (wid == 1 ? sqrt(tot[2] / tot[3]) : sqrt(tot[wid + 2]));
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = fmax(fmax(term[0], term[1]), fmax(term[2], term[3]));
-        *I.steps += 1;
-        I.misc[M_RESID] = r;
-        resid_all[idx] = r;
-        const bool fp32 = I.precision == FDLB_FP32_STORAGE;
-        if (flags[0]) *I.status = FDLB_FAILED_NONFINITE;
-        else if (flags[1]) *I.status = FDLB_FAILED_UNPHYSICAL;
-        else if (fp32 && r == 0.0 && I.two_phase) flags[2] = 1;   // FP32 f stopped changing
-        else if (fp32 && r == 0.0 && tol > 0.0) *I.status = FDLB_STAGNATED;
-        else if (tol > 0.0 && r < tol) *I.status = FDLB_CONVERGED;
-        else if (I.two_phase && fp32) flags[2] = stagnated(I, r, (double)*I.steps);
-        scale = I.misc[M_MASS0] / tot[6];
-    }
-    __syncthreads();
-    if (!flags[2]) return;
-    // Up-cast f: floats of F -> doubles in the stage buffer A, then back into F (which holds
-    // K ld doubles in a two-phase instance; A is free between steps), times the factor that
-    // restores the channel mass of the last anchor.  The discrete scheme conserves mass, but
-    // FP32 rounding near stagnation drops the same small updates step after step and lets the
-    // mass drift, which would move the FP64 steady state.  The node rows are rescaled alike
-    // (extensive rows by the factor, ln n and ln chi(eta0 n) anew; u and T are unchanged),
-    // so the next stage sees the moments of the rescaled f.
-    const double c = scale;
-    const size_t nf = (size_t)I.K * ld;
-    const float* src = static_cast<const float*>(I.f[0]);
-    double* tmp = static_cast<double*>(I.f[1]);
-    for (size_t e = threadIdx.x; e < nf; e += blockDim.x) tmp[e] = (double)src[e] * c;
-    __syncthreads();
-    double* dst = static_cast<double*>(I.f[0]);
-    for (size_t e = threadIdx.x; e < nf; e += blockDim.x) dst[e] = tmp[e];
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const double n = nd[R_N * ld + i] * c;
-        nd[R_N * ld + i] = n;
-        nd[R_PREV_N * ld + i] *= c;
-        nd[R_QX * ld + i] *= c;
-        nd[R_QY * ld + i] *= c;
-        nd[R_PXX * ld + i] *= c;
-        nd[R_PXY * ld + i] *= c;
-        nd[R_SNEG * ld + i] *= c;
-        nd[R_SPOS * ld + i] *= c;
-        nd[R_LNN * ld + i] = log(n);
-        nd[R_LNCHI * ld + i] = log(chi_cs(I.eta0 * n));
-    }
-    if (threadIdx.x == 0) {
-        I.precision = FDLB_FP64;
-        I.misc[M_SWITCH] = (double)*I.steps;
-    }
-}
-
-
 __global__ void __launch_bounds__(256) k_resid(Inst* insts, int anchor, double tol, double* resid_all) {
     pdl_wait();
     Inst& I = insts[blockIdx.x];
@@ -1256,7 +1269,8 @@ __global__ void __launch_bounds__(256) k_resid(Inst* insts, int anchor, double t
         return;
     }
     if (*I.status != FDLB_ACTIVE || I.smem_res) return;
-    resid_item(I, blockIdx.x, tol, resid_all);
+    __shared__ double buf[7 * 256];
+    resid_item(I, blockIdx.x, tol, resid_all, buf);
 }
 
 // ---------------------------------------------------------------------------
@@ -2006,7 +2020,7 @@ __device__ void res_step(Inst& I, int idx, double tol, double* resid_all, int ra
         cl.sync();
         if (nch > 1) res_final<S>(I, rank, CS, sm, cl);
     }
-    if (rank == 0) resid_item(I, idx, tol, resid_all);
+    if (rank == 0) resid_item(I, idx, tol, resid_all, reinterpret_cast<double*>(sm));
 }
 
 // Cluster c of the grid advances instance list[c] by up to nsteps steps (it stops early when
@@ -2066,7 +2080,7 @@ __device__ void smem_step(Inst& I, int idx, double tol, double* resid_all, unsig
             __syncthreads();
         }
     }
-    resid_item(I, idx, tol, resid_all);
+    resid_item(I, idx, tol, resid_all, reinterpret_cast<double*>(sm));
     __syncthreads();
 }
 
@@ -2228,10 +2242,13 @@ static cudaError_t set_smem(DevAttr* A, size_t smem64, size_t smem32) {
     return e;
 }
 
-cudaError_t launch_nodal(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, cudaStream_t s) {
+cudaError_t launch_nodal(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, int n_resid, double freeze_tol,
+                         double* d_resid_all, cudaStream_t s) {
     const size_t smem = (size_t)nodal_smem_doubles(qmax) * sizeof(double);
-    if (qmax <= 8) return launch_pdl(k_nodal<8>, (unsigned)n_nod, dim3(TILE * NOD_WARPS), smem, s, d_inst, d_nod);
-    return launch_pdl(k_nodal<QMAX>, (unsigned)n_nod, dim3(TILE * NOD_WARPS), smem, s, d_inst, d_nod);
+    const unsigned grid = (unsigned)(n_nod + n_resid);
+    Inst* in = const_cast<Inst*>(d_inst);
+    if (qmax <= 8) return launch_pdl(k_nodal<8>, grid, dim3(TILE * NOD_WARPS), smem, s, in, d_nod, n_nod, freeze_tol, d_resid_all);
+    return launch_pdl(k_nodal<QMAX>, grid, dim3(TILE * NOD_WARPS), smem, s, in, d_nod, n_nod, freeze_tol, d_resid_all);
 }
 
 cudaError_t prepare_kernels(size_t smem64, size_t smem32, int qmax) {
