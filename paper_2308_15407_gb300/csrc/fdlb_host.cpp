@@ -41,6 +41,7 @@ struct fdlb_ctx {
     Work* d_upd = nullptr;
     Work* d_nod = nullptr;
     int n_upd = 0, n_nod = 0, qmax = 1;
+    int xparts = 1;                   // blocks per x projection (choose_parts)
     int* d_list = nullptr;            // count ints: instances in resident-cluster order
     int* d_status_all = nullptr;      // count ints (Inst::status points here)
     long long* d_steps_all = nullptr;
@@ -100,6 +101,7 @@ struct fdlb_ctx {
 static void choose_cluster(fdlb_ctx* c);
 static void choose_smem_resident(fdlb_ctx* c);
 static void choose_update_width(fdlb_ctx* c, const int* st);
+static void choose_parts(fdlb_ctx* c);
 
 // Record a start/stop event pair around one launch of class `kind` when profiling is on.
 static cudaError_t prof_mark(fdlb_ctx* c, int kind) {
@@ -130,7 +132,7 @@ static cudaError_t step_many(fdlb_ctx* c, int64_t nsteps, double freeze_tol) {
     for (int64_t s = 0; s < nsteps && e == cudaSuccess; ++s) {
         for (int stage = 1; stage <= 3; ++stage) {
             const int n_resid = fold && s > 0 && stage == 1 ? c->count : 0;
-            guard(KK_NODAL, [&] { return launch_nodal(c->d_inst, c->d_nod, c->n_nod, c->qmax, n_resid, freeze_tol, c->d_resid_all, c->stream); });
+            guard(KK_NODAL, [&] { return launch_nodal(c->d_inst, c->d_nod, c->n_nod, c->qmax, c->xparts, n_resid, freeze_tol, c->d_resid_all, c->stream); });
             guard(KK_UPDATE, [&] { return launch_update(c->d_inst, c->d_upd, c->n_upd, stage, c->smem_upd_f64, c->smem_upd_f32,
                                                         c->any_fp64, c->any_fp32, c->upd_wide, c->stream); });
         }
@@ -895,6 +897,7 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
         }
         choose_update_width(c, nullptr);
         c->upd_wide_all = c->upd_wide;
+        choose_parts(c);
     }
     c->smem_upd_f64 = max_smem64;
     c->smem_upd_f32 = max_smem32;
@@ -1098,6 +1101,18 @@ static bool ensure_graph(fdlb_ctx* c, double tol) {
     c->graph_tol = tol;
     c->graph_wide = c->upd_wide;
     return true;
+}
+
+// Blocks per x projection.  A projection of n polynomials takes n^2 products per node beside the sums
+// that every block repeats, and its block fills an SM, so above 32 polynomials a batch whose tiles
+// leave SMs idle shares each projection's nodes between up to 8 blocks, one warp's nodes at least
+// 4 (three instances of full-range order 200 on 18 tiles, FP64: 250 us per launch with one block,
+// 77 with 6; lower orders take less than the launch).
+static void choose_parts(fdlb_ctx* c) {
+    const int tiles = c->n_nod / NODAL_ROLES;
+    c->xparts = 1;
+    if (c->qmax <= 32 || c->n_sms <= 0) return;
+    c->xparts = std::max(1, std::min({8, c->n_sms / std::max(1, tiles) - 1, c->qmax / 32}));
 }
 
 // Update width from the instances still active (st: statuses, null = all active).

@@ -430,7 +430,7 @@ __device__ void moments_final_tile(const Inst& I, int i0, double* ss, int tid, i
 // 4) 18.8 -> 12.6, six of order 100 per side 1079 -> 711, three of full-range order 200 in FP64
 // 2581 -> 248.
 // Shared doubles: role 0 (half): [NOD_WARPS + 1][2 nl + 6][32] sums, [4][32] node scalars, beyond
-//                 QMAX polynomials [M][2][32] recurrence states; (full): [Lx + 4][32];
+//                 QMAX polynomials [M][2][32] recurrence states; (full): [3 Lx + 4][32];
 //                 role 1: CL_ROWS rows + Py [4 QYMAX] + Pz [2 QZMAX] + A [8 QYMAX] + moments.
 constexpr int CL_ROWS = 5 + 8 + 14;                       // gradients, scalars, coefficients and n
 constexpr int CL_MOM = (QYMAX + 4) + (QZMAX + 4) + 1;     // m_l and T_a of y and z, T
@@ -441,11 +441,14 @@ __host__ __device__ inline int nodal_smem_doubles(int qmax) {
     const int qb = qmax > QMAX ? QMAX : qmax;
     const int mst = qmax > QMAX ? aux_points_half(qmax > QX_HALF_MAX ? QX_HALF_MAX : qmax) : 0;
     const int rh = ((NOD_WARPS + 1) * (2 * qb + 6) + 4 + 2 * mst) * TILE;
-    const int rf = (qmax + 4) * TILE;
+    const int rf = (3 * qmax + 4) * TILE;
     const int rc = (CL_ROWS + 4 * QYMAX + 2 * QZMAX + 8 * QYMAX + CL_MOM) * TILE;
     const int m = rh > rf ? rh : rf;
     return m > rc ? m : rc;
 }
+
+constexpr int XQ_DF = 32;           // half-range double-float projections: unscaled up to this order
+constexpr float XQ_TMAX = 1.8f;     // e^((T - 1) q^2/4) < 1e25 at q = 17, the outermost point of order 100
 
 // 1/j as float pairs, j = 0..16 (set by prepare_kernels)
 constexpr int NINV2 = 17;
@@ -544,6 +547,26 @@ __device__ __forceinline__ void put_powers(O* out, int Q, int k, R p, R u, R d, 
 __device__ __forceinline__ float to_float(double x) { return (float)x; }
 __device__ __forceinline__ float to_float(df x) { return x.hi; }
 
+// A share of a tile's x projection (tiles of high orders are split over several blocks when the
+// batch has few of them): nodes k = NOD_WARPS (i + n j) + 0 .. NOD_WARPS - 1.
+struct Part {
+    int i, n;
+};
+
+// Weight W and first polynomial h of an auxiliary point, scaled by 2^e and 2^-e so that both stay in
+// the float range: W falls like e^(-q^2/2) and the polynomials grow like e^(x^2/4), x = sqrt(T) q;
+// with 2^e ~ W^(-1/2) both run between e^(-q^2/4) and e^((T - 1) q^2/4).  (Exact powers of two; the
+// tail of h underflows only at points that do not contribute.)
+__device__ __forceinline__ void scale_point(double W, df& w, df& h) {
+    const int e = (1023 - ((__double2hiint(W) >> 20) & 0x7ff)) / 2;
+    const double s = __hiloint2double(__double2hiint(W) + (e << 20), __double2loint(W));
+    w.hi = (float)s;
+    w.lo = (float)(s - (double)w.hi);
+    const float f = __uint_as_float((uint32_t)(127 - e) << 23);
+    h = {h.hi * f, h.lo * f};
+}
+__device__ __forceinline__ void scale_point(double, double&, double&) {}
+
 // Half-range x projection of a tile (Sec. III A 2), both half-axes: the auxiliary points
 // x = sqrt(T) q and the polynomials there do not depend on the sign of u, so one recurrence
 // serves both.  With |v| < 0.02 and Q <= 12 the 8-point auxiliary rule is used.  It is exact for
@@ -553,7 +576,7 @@ __device__ __forceinline__ float to_float(df x) { return x.hi; }
 // takes auxiliary points w, w + 8, ...  R: double, or double-float for FP32 storage; out: the
 // table written (FP32 storage's tab32 also from double).
 template <int QB, typename R, typename O>
-__device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out) {
+__device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out, Part pt) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int i = i0 + lane, N = I.N, ld = I.ld, Q = I.Q;
     const bool valid = i < N;
@@ -587,6 +610,7 @@ __device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out) {
     const double *xa = I.xa, *xb = I.xb, *xib = I.xib, *xH = I.xH, *px = I.px;
     const float2 *xa2 = I.xa2, *xb2 = I.xb2, *xib2 = I.xib2, *xH2 = I.xH2, *px2 = I.px2;
     const R h0 = r_pair(I.x_h0, I.x_h02, R{});
+    const bool scaled = QB > 8 && sizeof(O) == 4 && Q > XQ_DF;      // (R = double-float: see nodal_item)
     const R sT = xs[lane], u = xs[TILE + lane], v = xs[2 * TILE + lane], d = xs[3 * TILE + lane];
     // blocks of QB polynomials: per block the sums over the auxiliary points (the recurrence
     // continued from the previous block's state), then the H products, whose chain continues
@@ -601,14 +625,16 @@ __device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) Tp[a] = Tm[a] = zero;
         for (int m = wid; m < M; m += NOD_WARPS) {
-            const R q = r_tab(xq, xq2, m, zero), W = r_tab(xw, xw2, m, zero);
+            const R q = r_tab(xq, xq2, m, zero);
+            R W = r_tab(xw, xw2, m, zero), hs = h0;
+            if (scaled) scale_point(xw[m], W, hs);
             R ep, em;
             if (short_rule) exp_pair_short(q * v, d, ep, em);
             else exp_pair(q * v, d, ep, em);
             ep = W * ep;
             em = W * em;
             const R x = sT * q;
-            R hm = zero, h = h0;
+            R hm = zero, h = hs;
             if (lb > 0) {
                 hm = hst[(2 * m) * TILE + lane];
                 h = hst[(2 * m + 1) * TILE + lane];
@@ -662,7 +688,7 @@ __device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out) {
         }
         __syncthreads();
         R* chain = reinterpret_cast<R*>(I.tab) + tab_col(I, i0, lane);
-        for (int k = wid; k < Q; k += NOD_WARPS) {
+        for (int k = pt.i * NOD_WARPS + wid; k < Q; k += NOD_WARPS * pt.n) {
             R sp = zero, sm = zero;
             if (lb > 0 && valid) {
                 sp = chain[k * TILE];
@@ -696,7 +722,7 @@ __device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out) {
 // recurrence (warp 0), then the sums over l, the even and the odd part once for both signs of
 // the node.
 template <typename R, typename O>
-__device__ void xproj_full(const Inst& I, int i0, double* nsm, O* out) {
+__device__ void xproj_full(const Inst& I, int i0, double* nsm, O* out, Part pt) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int i = i0 + lane, N = I.N, ld = I.ld, Q = I.Q, Lx = I.Lx;
     const bool valid = i < N;
@@ -704,13 +730,35 @@ __device__ void xproj_full(const Inst& I, int i0, double* nsm, O* out) {
     const R zero = r_of(0.0, R{});
     R* ml = reinterpret_cast<R*>(nsm);                               // [Lx + 1][32] m_l
     R* ts = ml + (Lx + 1) * TILE;                                    // [3][32] T_a
+    R* ca = ts + 3 * TILE;                                           // [Lx][32] u/sqrt(l + 1)
+    R* cb = ca + Lx * TILE;                                          // [Lx][32] (T - 1) sqrt(l/(l + 1))
     const double *xb = I.xb, *xib = I.xib, *xH = I.xH, *px = I.px;
     const float2 *xb2 = I.xb2, *xib2 = I.xib2, *xH2 = I.xH2, *px2 = I.px2;
-    const double T = I.node[R_T * ld + ic];
-    const R u = r_of(I.node[R_UX * ld + ic], R{});
-    if (wid == 0) hermite_moments(u, r_of(T, zero), Lx, xb, xb2, xib, xib2, ml + lane, ts + lane);
+    const R T = r_of(I.node[R_T * ld + ic], zero), u = r_of(I.node[R_UX * ld + ic], zero), t1 = T - r_c(1.0, zero);
+    // the recurrence's factors by all warps, then the chain (a product and an FMA per step) by warp 0
+    for (int l = wid; l < Lx; l += NOD_WARPS) {
+        const R il = r_tab(xib, xib2, l + 1, zero);
+        ca[l * TILE + lane] = u * il;
+        cb[l * TILE + lane] = t1 * (r_tab(xb, xb2, l, zero) * il);
+    }
     __syncthreads();
-    for (int k = wid; k < Q; k += NOD_WARPS) {
+    if (wid == 0) {
+        R mp = zero, m = r_c(1.0, zero), mm = zero;
+        ml[lane] = m;
+        for (int l = 0; l < Lx; ++l) {
+            const R mn = ca[l * TILE + lane] * m + cb[l * TILE + lane] * mp;
+            mm = mp;
+            mp = m;
+            m = mn;
+            ml[(l + 1) * TILE + lane] = m;
+        }
+        const R bn = r_tab(xb, xb2, Lx, zero);
+        ts[lane] = m;
+        ts[TILE + lane] = T * (bn * mp);
+        ts[2 * TILE + lane] = T * m + (T * bn) * ((T * r_tab(xb, xb2, Lx - 1, zero)) * mm);
+    }
+    __syncthreads();
+    for (int k = pt.i * NOD_WARPS + wid; k < Q; k += NOD_WARPS * pt.n) {
         R e = zero, o = zero;
         for (int l = 0; l < Lx; l += 2) {
             e = acc(e, r_tab(xH, xH2, l * Q + k, zero), ml[l * TILE + lane]);
@@ -1004,7 +1052,7 @@ __device__ __forceinline__ void warm_tables(const Inst& I, int role, int tid, in
 // One (tile, role) item by a block of NOD_WARPS warps; nsm holds nodal_smem_doubles(max Lx)
 // doubles; fp32: the instance stores f in FP32 (tables go to tab32).
 template <int QB>
-__device__ void nodal_item(const Inst& I, int i0, int role, double* nsm, bool fp32) {
+__device__ void nodal_item(const Inst& I, int i0, int role, double* nsm, bool fp32, Part pt = {0, 1}) {
     const int lane = threadIdx.x & 31;
     __syncthreads();                      // the previous item's readers of nsm are done
     if (role == 1) {
@@ -1015,18 +1063,27 @@ __device__ void nodal_item(const Inst& I, int i0, int role, double* nsm, bool fp
     if (I.xfull) {
         // the coefficients m_l and w_k h_l(p_k) stay small at every order: double-float for FP32
         // storage up to order 200
-        if (fp32) xproj_full<df>(I, i0, nsm, r_out(I, i0, lane, df{}));
-        else xproj_full<double>(I, i0, nsm, r_out(I, i0, lane, 0.0));
+        if (fp32) xproj_full<df>(I, i0, nsm, r_out(I, i0, lane, df{}), pt);
+        else xproj_full<double>(I, i0, nsm, r_out(I, i0, lane, 0.0), pt);
         return;
     }
-    // FP32 storage: double-float up to 32 polynomials.  Larger half-range orders sum in FP64
-    // (writing the FP32 table): the orthonormal polynomials grow to ~e^(x^2/4) at the auxiliary
-    // points x = sqrt(T) q, beyond the float range (3e38) once x > ~18.8 -- the aux rule of order
-    // 100 has q up to ~17 (overflow from T ~ 1.2); at 32 polynomials it ends near q = 11, which
-    // would need T > 3.
-    if (!fp32) xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, 0.0));
-    else if (I.Lx <= 32) xproj_half<QB, df>(I, i0, nsm, r_out(I, i0, lane, df{}));
-    else xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, df{}));
+    if (!fp32) {
+        xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, 0.0), pt);
+        return;
+    }
+    // FP32 storage: double-float.  Above XQ_DF polynomials the points are scaled (scale_point), which
+    // holds to T = XQ_TMAX at the largest order; a hotter tile sums in FP64 (708 us per launch for
+    // six instances of order 100, against 212 in double-float).
+    if constexpr (QB > 8) {               // (QB = 8: no order above 8 in the batch)
+        if (I.Lx > XQ_DF) {
+            const float T = (float)I.node[R_T * I.ld + min(i0 + lane, I.N - 1)];
+            if (__any_sync(0xffffffffu, !(T < XQ_TMAX))) {         // (the same in every warp)
+                xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, df{}), pt);
+                return;
+            }
+        }
+    }
+    xproj_half<QB, df>(I, i0, nsm, r_out(I, i0, lane, df{}), pt);
 }
 
 // ---------------------------------------------------------------------------
@@ -1161,12 +1218,14 @@ __global__ void __launch_bounds__(TILE * NOD_WARPS, QB == 8 ? 3 : 1) k_nodal(Ins
     extern __shared__ __align__(16) double nsm[];
     __shared__ Inst I;
     if ((int)blockIdx.x >= n_nod) {
+        if (blockIdx.y) return;
         pdl_wait();
         Inst& g = insts[blockIdx.x - n_nod];
         if (*(volatile int*)g.status == FDLB_ACTIVE && !g.smem_res) resid_item(g, blockIdx.x - n_nod, tol, resid_all, nsm);
         return;
     }
     const Work w = work[blockIdx.x];
+    if (blockIdx.y && w.k0 != 0) return;                // the x projections alone are split
     load_inst(insts + w.inst, &I, threadIdx.x, TILE * NOD_WARPS);
     warm_tables(I, w.k0, threadIdx.x, TILE * NOD_WARPS);
     pdl_wait();
@@ -1174,7 +1233,7 @@ __global__ void __launch_bounds__(TILE * NOD_WARPS, QB == 8 ? 3 : 1) k_nodal(Ins
     const int st = *(volatile int*)I.status, res = *(const volatile int*)&g.smem_res, pr = *(const volatile int*)&g.precision;
     // (one decision for the block: the residual block of this launch may change the status meanwhile)
     if (__syncthreads_or(st != FDLB_ACTIVE || res)) return;
-    nodal_item<QB>(I, w.i0, w.k0, nsm, pr == FDLB_FP32_STORAGE);
+    nodal_item<QB>(I, w.i0, w.k0, nsm, pr == FDLB_FP32_STORAGE, {(int)blockIdx.y, (int)gridDim.y});
 }
 
 // Projected local equilibrium of the profile rows (n, u_x = 0, u_y, T) into F: one block per tile of
@@ -1196,8 +1255,8 @@ __global__ void __launch_bounds__(TILE * NOD_WARPS) k_profiles(Inst* insts, cons
     const int ic = valid ? i : I.N - 1;
     const bool fp32 = I.two_phase || I.precision == FDLB_FP32_STORAGE;
     double* col = I.tab + tab_col(I, i0, lane);
-    if (I.xfull) xproj_full<double>(I, i0, nsm, col);
-    else xproj_half<QB, double>(I, i0, nsm, col);
+    if (I.xfull) xproj_full<double>(I, i0, nsm, col, Part{0, 1});
+    else xproj_half<QB, double>(I, i0, nsm, col, Part{0, 1});
     const double n = I.node[R_N * ld + ic], T = I.node[R_T * ld + ic];
     const int form = I.form, Qy = I.Qy, Qz = form == FORM_UNREDUCED ? I.Qz : 0;
     double* mz = Yz + (QYMAX + 4) * TILE;
@@ -2121,12 +2180,12 @@ __global__ void __launch_bounds__(RES_THREADS, 1) k_smemres(Inst* insts, const i
 // The stepping kernels (closure, update, residual) are launched with programmatic stream
 // serialization: the next kernel of a step is set up while the previous one finishes.
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+static cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -2221,7 +2280,7 @@ cudaError_t launch_resid(const Inst* d_inst, int count, int anchor_inst, double 
         k_resid<<<count, 256, 0, s>>>(const_cast<Inst*>(d_inst), anchor_inst, freeze_tol, d_resid_all);
         return cudaGetLastError();
     }
-    return launch_pdl(k_resid, (unsigned)count, dim3(256), 0, s, const_cast<Inst*>(d_inst), anchor_inst, freeze_tol, d_resid_all);
+    return launch_pdl(k_resid, dim3(count), dim3(256), 0, s, const_cast<Inst*>(d_inst), anchor_inst, freeze_tol, d_resid_all);
 }
 
 // (the caller holds g_attr_mu)
@@ -2242,10 +2301,10 @@ static cudaError_t set_smem(DevAttr* A, size_t smem64, size_t smem32) {
     return e;
 }
 
-cudaError_t launch_nodal(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, int n_resid, double freeze_tol,
-                         double* d_resid_all, cudaStream_t s) {
+cudaError_t launch_nodal(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, int xparts, int n_resid,
+                         double freeze_tol, double* d_resid_all, cudaStream_t s) {
     const size_t smem = (size_t)nodal_smem_doubles(qmax) * sizeof(double);
-    const unsigned grid = (unsigned)(n_nod + n_resid);
+    const dim3 grid(n_nod + n_resid, xparts);
     Inst* in = const_cast<Inst*>(d_inst);
     if (qmax <= 8) return launch_pdl(k_nodal<8>, grid, dim3(TILE * NOD_WARPS), smem, s, in, d_nod, n_nod, freeze_tol, d_resid_all);
     return launch_pdl(k_nodal<QMAX>, grid, dim3(TILE * NOD_WARPS), smem, s, in, d_nod, n_nod, freeze_tol, d_resid_all);
@@ -2404,13 +2463,13 @@ cudaError_t launch_update(const Inst* d_inst, const Work* d_upd, int n_upd, int 
     cudaError_t e = cudaSuccess;
     if (wide) {
         const dim3 blk(TILE, UPD_WARPS_WIDE);
-        if (f64) e = launch_pdl(k_update<double, UPD_WARPS_WIDE>, (unsigned)n_upd, blk, smem64, s, d_inst, d_upd, stage);
+        if (f64) e = launch_pdl(k_update<double, UPD_WARPS_WIDE>, dim3(n_upd), blk, smem64, s, d_inst, d_upd, stage);
         if (e == cudaSuccess && f32)
-            e = launch_pdl(k_update<float, UPD_WARPS_WIDE>, (unsigned)n_upd, blk, smem32, s, d_inst, d_upd, stage);
+            e = launch_pdl(k_update<float, UPD_WARPS_WIDE>, dim3(n_upd), blk, smem32, s, d_inst, d_upd, stage);
     } else {
         const dim3 blk(TILE, UPD_WARPS);
-        if (f64) e = launch_pdl(k_update<double, UPD_WARPS>, (unsigned)n_upd, blk, smem64, s, d_inst, d_upd, stage);
-        if (e == cudaSuccess && f32) e = launch_pdl(k_update<float, UPD_WARPS>, (unsigned)n_upd, blk, smem32, s, d_inst, d_upd, stage);
+        if (f64) e = launch_pdl(k_update<double, UPD_WARPS>, dim3(n_upd), blk, smem64, s, d_inst, d_upd, stage);
+        if (e == cudaSuccess && f32) e = launch_pdl(k_update<float, UPD_WARPS>, dim3(n_upd), blk, smem32, s, d_inst, d_upd, stage);
     }
     return e;
 }

@@ -35,3 +35,20 @@ def test_projection_edges_match_oracle(batch, precision, tol):
         compare(s.moments(i), Mo, tol, f"instance {i} ({precision})")
         if d["nx"] == WAVE["nx"]:
             assert np.max(np.abs(Mo["ux"]) / np.sqrt(Mo["T"])) > 0.02     # the long rule was in use
+
+
+# FP32 storage above 32 polynomials: double-float with scaled points up to T = 1.8, FP64 in hotter
+# tiles; an instance below and one whose tiles differ (x projections split over blocks)
+HOT = [dict(nx=40, kn=0.3, eta0=0.05, qx_half=40, qy=0, qz=0, T_left=1.5, T_right=1.7),
+       dict(nx=70, kn=0.3, eta0=0.05, qx_half=36, qy=3, qz=0, T_left=1.0, T_right=2.4, T_init=1.7)]
+
+
+def test_hot_high_orders_match_oracle():
+    F = lib()
+    s = F.Solver([F.Params(**d, precision="fp32") for d in HOT])
+    s.set_schedule("tiled")
+    s.step(10)
+    for i, d in enumerate(HOT):
+        o = oracle_for(F.Params(**d))
+        o.step(10)
+        compare(s.moments(i), o.moments(), 1e-5, f"instance {i}")
