@@ -285,54 +285,73 @@ __device__ __forceinline__ R chi_of(R eta) {
     return r_div(r_c(2.0, R{}) - eta, r_c(2.0, R{}) * om * om * om);
 }
 
-// Moments of the nodes of tile i0 from the raw sums ss[MOM_SUMS][TILE], by 128 threads: warp 0
-// writes the primitive rows, warps 1..3 ln n, ln T and ln chi(eta0 n) (independent chains on
-// different schedulers).  FP32 storage finalises its double-float sums in double-float: in FP64
+// Moments of the nodes of tile i0 from the raw sums ss[MOM_SUMS][TILE], by nw warps: independent
+// chains, one per warp (n, u, T and the stresses; ln n; ln T; ln chi(eta0 n); q_x; q_y).  SPLIT: six
+// chains, for the last block of a split tile, which everything waits for (one Couette instance:
+// update 18.1 -> 16.4 us per launch); else the heat fluxes with the first, which shares its
+// quotients (2048 mixed instances: 756 us per launch with six chains, 705 with four).  FP32 storage finalises its double-float sums in double-float: in FP64
 // this took 362 FP64 instructions per tile, 45 % of the FP64 pipe's time on large batches.
+// Heat fluxes from the raw sums s[j TILE]: third-order sums about the mean, s8 - 3 ux s4 + 2 n ux^3 and
+// so on.
 template <typename R>
-__device__ void finalize_tile(const Inst& I, int i0, const R* ss, int tid) {
-    const int lane = tid & 31, g = tid >> 5, i = i0 + lane;
+__device__ __forceinline__ R heat_flux_x(const R* s, R n, R ux, R uy) {
+    const R two = r_c(2.0, R{}), n2 = two * n;
+    const R cx3 = s[8 * TILE] + ux * (n2 * (ux * ux) - r_c(3.0, R{}) * s[4 * TILE]);
+    const R cxyy = s[9 * TILE] - two * (uy * s[5 * TILE]) + ux * (n2 * (uy * uy) - s[6 * TILE]);
+    return r_c(0.5, R{}) * (cx3 + cxyy) + (s[12 * TILE] - ux * s[7 * TILE]);
+}
+template <typename R>
+__device__ __forceinline__ R heat_flux_y(const R* s, R n, R ux, R uy) {
+    const R two = r_c(2.0, R{}), n2 = two * n;
+    const R cxxy = s[10 * TILE] - two * (ux * s[5 * TILE]) + uy * (n2 * (ux * ux) - s[4 * TILE]);
+    const R cy3 = s[11 * TILE] + uy * (n2 * (uy * uy) - r_c(3.0, R{}) * s[6 * TILE]);
+    return r_c(0.5, R{}) * (cy3 + cxxy) + (s[13 * TILE] - uy * s[7 * TILE]);
+}
+
+template <bool SPLIT, typename R>
+__device__ __forceinline__ void finalize_chain(const Inst& I, int i0, const R* ss, int lane, int g) {
+    const int i = i0 + lane, ld = I.ld;
     if (i >= I.N) return;
-    const int ld = I.ld;
     double* nd = I.node;
-    R s[MOM_SUMS];
-#pragma unroll
-    for (int j = 0; j < MOM_SUMS; ++j) s[j] = ss[j * TILE + lane];
-    const R n = s[0], half = r_c(0.5, R{}), two = r_c(2.0, R{}), three = r_c(3.0, R{});
+    const R* s = ss + lane;                        // raw sum j at s[j TILE]
+    const R n = s[0], half = r_c(0.5, R{});
     if (g == 1) {
         nd[R_LNN * ld + i] = r_dbl(r_log(n));
     } else if (g == 3) {
         nd[R_LNCHI * ld + i] = r_dbl(r_log(chi_of(r_of(I.eta0, R{}) * n)));
-    } else {
+    } else if (g == 0 || g == 2) {
         // n times the thermal energy, without a division: T = (n E)/(1.5 n^2)
-        const R sx = s[1] + s[2];
-        const R nE = half * ((n * s[4] - sx * sx) + (n * s[6] - s[3] * s[3])) + n * s[7];
+        const R s1 = s[1 * TILE], s2 = s[2 * TILE], s3 = s[3 * TILE], s4 = s[4 * TILE];
+        const R sx = s1 + s2;
+        const R nE = half * ((n * s4 - sx * sx) + (n * s[6 * TILE] - s3 * s3)) + n * s[7 * TILE];
         const R T = r_div(nE, r_c(1.5, R{}) * (n * n));
         if (g == 2) {
             nd[R_LNT * ld + i] = r_dbl(r_log(T));
             return;
         }
-        const R ux = r_div(sx, n), uy = r_div(s[3], n);
-        const R ux2 = ux * ux, uy2 = uy * uy, n2 = two * n;
-        const R Pxx = s[4] - n * ux2, Pxy = s[5] - n * (ux * uy);
-        // third-order sums about the mean: s8 - 3 ux s4 + 2 n ux^3 and so on
-        const R cx3 = s[8] + ux * (n2 * ux2 - three * s[4]);
-        const R cxyy = s[9] - two * (uy * s[5]) + ux * (n2 * uy2 - s[6]);
-        const R cxxy = s[10] - two * (ux * s[5]) + uy * (n2 * ux2 - s[4]);
-        const R cy3 = s[11] + uy * (n2 * uy2 - three * s[6]);
-        const R qx = half * (cx3 + cxyy) + (s[12] - ux * s[7]);
-        const R qy = half * (cy3 + cxxy) + (s[13] - uy * s[7]);
+        const R ux = r_div(sx, n), uy = r_div(s3, n), nux = n * ux;
         nd[R_N * ld + i] = r_dbl(n);
         nd[R_UX * ld + i] = r_dbl(ux);
         nd[R_UY * ld + i] = r_dbl(uy);
         nd[R_T * ld + i] = r_dbl(T);
-        nd[R_QX * ld + i] = r_dbl(qx);
-        nd[R_QY * ld + i] = r_dbl(qy);
-        nd[R_PXX * ld + i] = r_dbl(Pxx);
-        nd[R_PXY * ld + i] = r_dbl(Pxy);
-        nd[R_SNEG * ld + i] = r_dbl(s[1]);
-        nd[R_SPOS * ld + i] = r_dbl(s[2]);
+        nd[R_PXX * ld + i] = r_dbl(s4 - nux * ux);
+        nd[R_PXY * ld + i] = r_dbl(s[5 * TILE] - nux * uy);
+        nd[R_SNEG * ld + i] = r_dbl(s1);
+        nd[R_SPOS * ld + i] = r_dbl(s2);
+        if (!SPLIT) {
+            nd[R_QX * ld + i] = r_dbl(heat_flux_x(s, n, ux, uy));
+            nd[R_QY * ld + i] = r_dbl(heat_flux_y(s, n, ux, uy));
+        }
+    } else {
+        const R ux = r_div(s[1 * TILE] + s[2 * TILE], n), uy = r_div(s[3 * TILE], n);
+        if (g == 4) nd[R_QX * ld + i] = r_dbl(heat_flux_x(s, n, ux, uy));
+        else nd[R_QY * ld + i] = r_dbl(heat_flux_y(s, n, ux, uy));
     }
+}
+template <bool SPLIT, typename R>
+__device__ __forceinline__ void finalize_tile(const Inst& I, int i0, const R* ss, int lane, int wy, int nw) {
+#pragma unroll 1
+    for (int g = wy; g < (SPLIT ? 6 : 4); g += nw) finalize_chain<SPLIT>(I, i0, ss, lane, g);
 }
 
 // Programmatic dependent launch: a stepping kernel launched with programmatic stream
@@ -402,7 +421,7 @@ __device__ void moments_final_tile(const Inst& I, int i0, double* ss, int tid, i
         rs[j * TILE + lane] = a;
     }
     named_sync(bar, 32 * nw);
-    if (tid < 128) finalize_tile<R>(I, i0, rs, tid);
+    finalize_tile<true>(I, i0, rs, lane, g, nw);
 }
 
 // ---------------------------------------------------------------------------
@@ -477,6 +496,7 @@ __device__ __forceinline__ void hermite_moments(R u, R T, int n, const double* b
     const R zero = r_c(0.0, R{}), one = r_c(1.0, R{}), t1 = T - one;
     R mp = zero, m = one, mm = zero;                // m_{l-1}, m_l, m_{l-2}
     ml[0] = m;
+#pragma unroll 1
     for (int l = 0; l < n; ++l) {
         const R il = r_tab(ib, ib2, l + 1, zero);
         // off the chain: the factor of m_{l-1}; on it: one product and sum
@@ -895,7 +915,7 @@ __device__ void closure_item(const Inst& I, int i0, double* nsm) {
             const R* m = ydir ? my : mz;
             const R* ts = m + (ydir ? QYMAX + 1 : QZMAX + 1) * TILE;
             R P = z;
-#pragma unroll
+#pragma unroll 1
             for (int l = 0; l < QYMAX; ++l)
                 if (l < Qn) P = acc(P, r_tab(H, H2, l * Qn + k, z), m[l * TILE + lane]);
             P = fin(P);
@@ -1212,8 +1232,8 @@ __device__ void resid_item(Inst& I, int idx, double tol, double* resid_all, doub
 // instance 74 -> 69 us per step).  Whether the instance goes on is decided by the status that the
 // update kernels read; a closure block that still saw ACTIVE has only written tables that nothing
 // reads.  Not with two-phase instances, whose residual pass may rewrite f and the moments.
-template <int QB>
-__global__ void __launch_bounds__(TILE * NOD_WARPS, QB == 8 ? 3 : 1) k_nodal(Inst* __restrict__ insts, const Work* __restrict__ work,
+template <int QB, int MB>
+__global__ void __launch_bounds__(TILE * NOD_WARPS, MB) k_nodal(Inst* __restrict__ insts, const Work* __restrict__ work,
                                                                            int n_nod, double tol, double* resid_all) {
     extern __shared__ __align__(16) double nsm[];
     __shared__ Inst I;
@@ -1236,9 +1256,8 @@ __global__ void __launch_bounds__(TILE * NOD_WARPS, QB == 8 ? 3 : 1) k_nodal(Ins
     nodal_item<QB>(I, w.i0, w.k0, nsm, pr == FDLB_FP32_STORAGE, {(int)blockIdx.y, (int)gridDim.y});
 }
 
-// Projected local equilibrium of the profile rows (n, u_x = 0, u_y, T) into F: one block per tile of
-// the work list's x-projection items (the other items leave at once), with the x projection of
-// the closure and the zeroth y and z projections, in FP64 for either storage; then a warp per
+// Projected local equilibrium of the profile rows (n, u_x = 0, u_y, T) into F: one block per tile (the
+// work list's x-projection items), with the x projection of the closure and the zeroth y and z projections, in FP64 for either storage; then a warp per
 // velocity writes f, whole lines at a time.  (One block per instance with a thread per node took
 // 1.0 ms for a 200-node instance of 288 velocities; this takes 20 us.)  A two-phase instance
 // restarts in its FP32 phase.
@@ -1248,7 +1267,6 @@ __global__ void __launch_bounds__(TILE * NOD_WARPS) k_profiles(Inst* insts, cons
     __shared__ double Yz[(QYMAX + 4 + QZMAX + 4) * TILE];            // m_l and T_a of y, then of z
     __shared__ double Yt[(QYMAX + QZMAX) * TILE];                    // P_0 of y, then of z
     const Work w = work[blockIdx.x];
-    if (w.k0 != 0) return;
     Inst& I = insts[w.inst];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, i0 = w.i0, i = i0 + lane, ld = I.ld, Q = I.Q, Tc = I.Tc;
     const bool valid = i < I.N;
@@ -1620,8 +1638,7 @@ __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, co
     }
     if (G > 1) return;
     __syncthreads();
-    const int tid = wy * TILE + lane;
-    if (tid < 128) finalize_tile<R>(I, i0, ss, tid);
+    finalize_tile<false>(I, i0, ss, lane, wy, UPD_WARPS);
 }
 
 // Tiled schedule, tiles split into several chunks: the last chunk block of the tile to arrive
@@ -1824,6 +1841,15 @@ struct Force {
 // n velocities t, t + 1, ... of one x-velocity; POS: p_x > 0.
 template <typename S, bool POS, bool FORCE>
 __device__ __forceinline__ void update_run(const Stage& g, Lane<S>& c, const Force<S>& fc, int t, int n) {
+    const S *Kr = fc.K, *q0 = fc.f;              // FORCE: row p_y of the kernel, first of the p_y values
+    int kz = 0;
+    if (FORCE) {
+        const int ky = t / fc.Tz;
+        kz = t - ky * fc.Tz;
+        Kr += ky * fc.Qy;
+        q0 += (size_t)kz * fc.stride;
+    }
+    const size_t qs = FORCE ? (size_t)fc.Tz * fc.stride : 0;
     for (int m = 0; m < n; ++m) {
         // right face (i + 1/2) from the five upwind nodes
         const S* r = c.row;
@@ -1837,11 +1863,15 @@ __device__ __forceinline__ void update_run(const Stage& g, Lane<S>& c, const For
         for (int a = 1; a < 4; ++a) tgt += c.Px[a] * c.Y[a * c.TcS];
         S inc = c.xp * (fr - fl) + (tgt - fi) * c.invtau;
         if (FORCE) {
-            const int ky = (t + m) / fc.Tz, kz = (t + m) - ky * fc.Tz;
-            const S* Kr = fc.K + ky * fc.Qy;
-            const S* q = fc.f + (size_t)kz * fc.stride;
+            const S* q = q0;
             S d = (S)0;
-            for (int kp = 0; kp < fc.Qy; ++kp, q += (size_t)fc.Tz * fc.stride) d += Kr[kp] * *q;
+            for (int kp = 0; kp < fc.Qy; ++kp, q += qs) d += Kr[kp] * *q;
+            q0 += fc.stride;
+            if (++kz == fc.Tz) {
+                kz = 0;
+                q0 = fc.f;
+                Kr += fc.Qy;
+            }
             inc -= fc.ay * d;
         }
         const S out = rk_combine(g, fi, g.first ? (S)0 : *c.fo, inc, c.elem);
@@ -2301,13 +2331,19 @@ static cudaError_t set_smem(DevAttr* A, size_t smem64, size_t smem32) {
     return e;
 }
 
-cudaError_t launch_nodal(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, int xparts, int n_resid,
+cudaError_t launch_nodal(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, int xparts, bool one_wave, int n_resid,
                          double freeze_tol, double* d_resid_all, cudaStream_t s) {
     const size_t smem = (size_t)nodal_smem_doubles(qmax) * sizeof(double);
     const dim3 grid(n_nod + n_resid, xparts);
     Inst* in = const_cast<Inst*>(d_inst);
-    if (qmax <= 8) return launch_pdl(k_nodal<8>, grid, dim3(TILE * NOD_WARPS), smem, s, in, d_nod, n_nod, freeze_tol, d_resid_all);
-    return launch_pdl(k_nodal<QMAX>, grid, dim3(TILE * NOD_WARPS), smem, s, in, d_nod, n_nod, freeze_tol, d_resid_all);
+    if (qmax <= 8) {
+        // three blocks per SM (80 registers, a few spilled) where blocks queue: 2048 mixed instances
+        // 790 -> 720 us per launch against two; unconstrained (150 registers) when each block has an
+        // SM to itself: one Couette instance 13.5 -> 12.2 us (and 12 instances 15.3 -> 20.3, so not there)
+        auto k = one_wave ? k_nodal<8, 1> : k_nodal<8, 3>;
+        return launch_pdl(k, grid, dim3(TILE * NOD_WARPS), smem, s, in, d_nod, n_nod, freeze_tol, d_resid_all);
+    }
+    return launch_pdl(k_nodal<QMAX, 1>, grid, dim3(TILE * NOD_WARPS), smem, s, in, d_nod, n_nod, freeze_tol, d_resid_all);
 }
 
 cudaError_t prepare_kernels(size_t smem64, size_t smem32, int qmax) {
@@ -2330,8 +2366,9 @@ cudaError_t prepare_kernels(size_t smem64, size_t smem32, int qmax) {
     }
     const int smem = nodal_smem_doubles(qmax) * (int)sizeof(double);
     if ((size_t)smem > SMEM_OPTIN && smem > A->nodal) {
-        cudaError_t e = cudaFuncSetAttribute(k_nodal<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_nodal<QMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(k_nodal<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_nodal<8, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_nodal<QMAX, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k_profiles<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k_profiles<QMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;

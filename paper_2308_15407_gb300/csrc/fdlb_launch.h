@@ -26,14 +26,14 @@ cudaError_t launch_resid(const Inst* d_inst, int count, int anchor_inst, double 
                          cudaStream_t s);
 
 // Projected local equilibrium from the profile rows (n, u_x = 0, u_y, T) into F, for the tiles of
-// the closure items d_nod[0..n_nod); qmax as for launch_nodal.
+// the x-projection items d_nod[0..n_nod); qmax as for launch_nodal.
 cudaError_t launch_profiles(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, cudaStream_t s);
 
 // Per-node closure (chi, Pr, tau, gradients, projection tables, wall densities), the x projection of
-// a tile by xparts blocks; with n_resid = the
+// a tile by xparts blocks; one_wave: every block has an SM to itself; with n_resid = the
 // number of instances also the residual / status pass of the step before (not with two-phase
 // instances), else 0.
-cudaError_t launch_nodal(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, int xparts, int n_resid,
+cudaError_t launch_nodal(const Inst* d_inst, const Work* d_nod, int n_nod, int qmax, int xparts, bool one_wave, int n_resid,
                          double freeze_tol, double* d_resid_all, cudaStream_t s);
 
 // RK stage `stage` (1..3) update of every ACTIVE instance; wide: blocks of 16 warps instead of
