@@ -889,9 +889,15 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
         if (p.precision != FDLB_FP32_STORAGE) max_smem64 = std::max(max_smem64, update_smem_bytes(L.trows, L.ukc, 8)), c->any_fp64 = true;
         if (p.precision != FDLB_FP64) max_smem32 = std::max(max_smem32, update_smem_bytes(L.trows, L.ukc, 4)), c->any_fp32 = true;
     }
-    // by role, so that the blocks on an SM run the same code (their instructions do not fit the cache
-    // together: 2048 mixed instances 725 -> 624 us per closure launch)
-    for (auto& f : c->nod_first) f += (int)wn.size();
+    // by role and, within one, by form and force, so that the blocks on an SM run the same code (their
+    // instructions do not fit the cache together: 2048 mixed instances 725 -> 624 us per closure
+    // launch, 705 -> 650 per update launch); the 1D form first, whose blocks are the shortest and
+    // share their SM with the launch's last ones
+    const auto kind = [&](const Work& w) { return (FORM_REDUCED1D - c->inst[w.inst].form) * 2 + (c->inst[w.inst].accel_y != 0.0 ? 1 : 0); };
+    const auto by_kind = [&](const Work& a, const Work& b) { return kind(a) < kind(b); };
+    for (auto* v : {&wu, &wn, &wx}) std::stable_sort(v->begin(), v->end(), by_kind);
+    for (size_t j = wu.size(); j-- > 0;) c->upd_first[wu[j].inst] = (int)j;
+    for (size_t j = wx.size(); j-- > 0;) c->nod_first[wx[j].inst] = (int)(wn.size() + j);
     wn.insert(wn.end(), wx.begin(), wx.end());
     if (off > need) { delete c; return fail(nullptr, FDLB_EINVAL, "internal: workspace layout overflow"); }
     {
@@ -939,7 +945,7 @@ extern "C" int fdlb_create(fdlb_ctx** out, const fdlb_params* params, int32_t co
     if (!rc) rc = cuda_check(c, prepare_kernels(c->smem_upd_f64, c->smem_upd_f32, c->qmax), "kernel attributes");
     if (!rc) choose_cluster(c);
     if (!rc) rc = cuda_check(c, launch_setup(c->d_inst, count, s), "setup kernel");
-    if (!rc) rc = cuda_check(c, launch_profiles(c->d_inst, c->d_nod + c->nod_first[0], n_nod / NODAL_ROLES, c->qmax, s), "setup kernel");
+    if (!rc) rc = cuda_check(c, launch_profiles(c->d_inst, c->d_nod + n_nod / NODAL_ROLES, n_nod / NODAL_ROLES, c->qmax, s), "setup kernel");
     if (!rc) rc = cuda_check(c, launch_moments(c->d_inst, c->d_upd, n_upd, 0, c->ukc_max, c->any_fp64, c->any_fp32, s), "moments kernel");
     if (!rc) rc = cuda_check(c, launch_resid(c->d_inst, count, -1, 0.0, c->d_resid_all, s), "residual kernel");
     if (!rc) rc = cuda_check(c, cudaStreamSynchronize(s), "fdlb_create synchronize");
