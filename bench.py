@@ -53,7 +53,7 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12      # 80.5
 FP64_PEAK_TFLOPS = 1.25                                # recipe nominal (measured FMA probe: 1.22)
 HBM_FALLBACK_GBS = 6800.0                              # recipe fallback when no measured copy rate exists
 KERNEL_SRC = os.path.join(ROOT, "paper_2308_15407_gb300", "csrc", "fdlb_kernels.cu")
-# ncu DRAM bytes (read + write) per k_update<float,float> launch on the 12-instance sweep,
+# ncu DRAM bytes (read + write) per k_update<float> launch on the 12-instance sweep,
 # cold cache, mean over the three stages of one capture, with the SHA-256 prefix of the
 # kernel source it was taken on; the bench reports it only while the source is unchanged.
 UPDATE_TRAFFIC = {"bytes": 6691499, "kernel_src_sha16": "37dfbdfebdbecda5"}
@@ -394,7 +394,7 @@ def run_fdlb(args):
     total_kernel_ms = sum(v[0] for v in prof.values())
     dom = max(prof, key=lambda k: prof[k][0])
     dom_ms, dom_launches = prof[dom]
-    kname = {"update": "k_update<float,float>", "moments": "k_moments<float>", "nodal": "k_nodal<8>", "resid": "k_resid"}
+    kname = {"update": "k_update<float>", "moments": "k_moments<float>", "nodal": "k_nodal<8>", "resid": "k_resid"}
     upd_ms, upd_launches = prof["update"]
     # algorithmic work over the profiled steps: per instance, its steps done x per-step work
     upd_bytes = float(sum(update_bytes_per_step(params[i], nx[i], s.nvel[i]) * int(pdone[i]) for i in range(s.count)))

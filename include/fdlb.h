@@ -65,8 +65,9 @@ extern "C" {
 
 /* Storage precision of f. */
 #define FDLB_FP64          0   /* everything in FP64 */
-#define FDLB_FP32_STORAGE  1   /* f stored, advected and combined in FP32; moments, gradients,
-                                  projections and the residual in FP64 */
+#define FDLB_FP32_STORAGE  1   /* f stored, advected and combined in FP32; moments, projections and
+                                  closure in double-float (float pairs, ~1e-14), gradients and
+                                  the residual in FP64 */
 #define FDLB_FP32_THEN_FP64 2  /* two phases: FDLB_FP32_STORAGE until the per-step residual
                                   stagnates, then FDLB_FP64 for the rest of the solve.  f is
                                   up-cast exactly on the device at the end of the step that
