@@ -1,15 +1,19 @@
 // WENO-5 face values (Sec. III B 2) of the update kernel, in the differences of the stencil.
 //
 // With the first differences d1..d4 and second differences e1..e3 of the five upwind nodes
-// (a, b, c, d, e) the candidates differ from the middle one by third differences,
-//   F1 = F2 - (e2 - e1)/3,   F2 = c + (d2 + 2 d3)/6,   F3 = F2 - (e3 - e2)/6,
-// and the indicators are 13/12 e_q^2 + 1/4 q_q^2 with q1 = e1 + 2 d2, q2 = d2 + d3,
-// q3 = e3 - 2 d3.  With m_1 = (s2 s3)^2 and so on (omega~_q = delta_q/s_q^2 times a common factor)
-//   face = c + (d2 + 2 d3 - (2 m1 (e2 - e1) + 3 m3 (e3 - e2))/(m1 + 6 m2 + 3 m3))/6.
+// (a, b, c, d, e) the indicators are 13/12 e_q^2 + 1/4 q_q^2 with q1 = e1 + 2 d2, q2 = d2 + d3,
+// q3 = e3 - 2 d3, and the candidates are offsets from c,
+//   F1 = c + (5 d2 - 2 d1)/6,   F2 = c + (d2 + 2 d3)/6,   F3 = c + (4 d3 - d4)/6,
+// which differ by third differences: F2 - F1 = (e2 - e1)/3, F3 - F2 = -(e3 - e2)/6.  With
+// m_1 = (s2 s3)^2 and so on (omega~_q = delta_q/s_q^2 times a common factor, delta_q = 1 : 6 : 3)
+//   face = c + (m1 (5 d2 - 2 d1) + 6 m2 (d2 + 2 d3) + 3 m3 (4 d3 - d4))/(6 (m1 + 6 m2 + 3 m3))
+//        = c + (d2 + 2 d3 - (2 m1 (e2 - e1) + 3 m3 (e3 - e2))/(m1 + 6 m2 + 3 m3))/6.
 // No epsilon; a vanishing indicator takes the weight in the limit.
 //
-// FP32: 42 instructions against 61 of the three candidates and normalised weights, and the large
-// part of the value, c, is never multiplied.
+// FP32: the first form, 45 instructions against 61 of the candidates and normalised weights.  Each
+// offset carries its own weight, so next to a front, where d2 + 2 d3 holds a jump, no two terms of the
+// jump's size cancel: 6e-8 of the face for jumps of 1e2 between neighbouring nodes (the second form, 42
+// instructions: 1e-5, and no digit from jumps of 1e7 on; the sum of weighted candidates: 5e-7).
 //
 // FP64: the pipe issues one warp instruction per 64 to 76 cycles and scheduler on this GPU, so only
 // what carries the value is FP64: the differences (exact cancellation), F2 and the final sum, 11
@@ -33,7 +37,7 @@ __device__ __forceinline__ float weno_face(float a, float b, float c, float d, f
     const float a1 = s1 * r, a2 = s2 * r, a3 = s3 * r;
     const float p1 = a1 * a1, p2 = a2 * a2, p3 = a3 * a3;
     float m1 = p2 * p3, m2 = p1 * p3, m3 = p1 * p2;
-    float sum = fmaf(6.0f, m2, fmaf(3.0f, m3, m1));
+    float w2 = 6.0f * m2, w3 = 3.0f * m3, sum = (m1 + w2) + w3;
     if (sum < 1e-30f) {
         if (smax < 4e-30f) {
             // uniform to FP32 resolution: the candidates agree, the ideal weights are the limit
@@ -45,10 +49,13 @@ __device__ __forceinline__ float weno_face(float a, float b, float c, float d, f
             m2 = s2 == smin ? 1.0f : 0.0f;
             m3 = s3 == smin ? 1.0f : 0.0f;
         }
-        sum = fmaf(6.0f, m2, fmaf(3.0f, m3, m1));
+        w2 = 6.0f * m2;
+        w3 = 3.0f * m3;
+        sum = (m1 + w2) + w3;
     }
-    const float num = fmaf(3.0f * m3, e3 - e2, (m1 + m1) * (e2 - e1));
-    return fmaf(fmaf(-num, rcp_approx(sum), fmaf(2.0f, d3, d2)), 1.0f / 6.0f, c);
+    // six times the candidates' offsets from c, each times its own weight
+    const float o1 = fmaf(-2.0f, d1, 5.0f * d2), o2 = fmaf(2.0f, d3, d2), o3 = fmaf(4.0f, d3, -d4);
+    return fmaf(fmaf(m1, o1, fmaf(w2, o2, w3 * o3)), rcp_approx(sum) * (1.0f / 6.0f), c);
 }
 
 __device__ __forceinline__ double weno_face(double a, double b, double c, double d, double e) {
