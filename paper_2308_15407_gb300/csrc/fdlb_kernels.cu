@@ -1823,7 +1823,7 @@ __device__ __forceinline__ float rk_combine(const Stage& g, float fi, float F, f
 // velocity to the next.
 template <typename S>
 struct Lane {
-    bool valid, at_wall;
+    bool valid, at_wall, inner;    // inner: its right face is neither the wall's nor padding
     int lane, ld, TcS;
     S xp, invtau, Px[4];       // -cb dt p/(x' ds), cb dt/tau, the x projections of this p
     const S* row;              // staged row at this node
@@ -1841,6 +1841,74 @@ struct Force {
     S ay;
 };
 
+// Position of the k-th set bit (k from 0) of a mask with more than k.
+__device__ __forceinline__ int nth_bit(unsigned mask, int k) {
+    int at = 0;
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) {
+        const int n = __popc(mask & ((1u << w) - 1u));
+        if (k >= n) {
+            k -= n;
+            mask >>= w;
+            at += w;
+        }
+    }
+    return at;
+}
+
+// Right faces of nb <= FACE_BATCH velocities (one in FP32) from the staged rows r, r + SW, ...  FP64: the
+// nodes whose stencil is rough (fdlb_weno.cuh: three to five next to a wall at start-up, rarely more) of all
+// the batch's velocities are dealt out to the lanes, so that their 40 FP64 instructions run once a batch and
+// not once a velocity.  Twelve Couette instances: update 96 us per launch, 104 with batches of two, 121
+// one velocity at a time (93 with double-float weights everywhere); 900 nodes: 56, 56 and 65 (56).  A
+// batch of four spills 296 bytes at the 80 registers of three blocks per SM; two blocks: 97 and 55, but
+// full-range order 200 138 against 128.
+constexpr int FACE_BATCH = 4;
+
+template <bool POS>
+__device__ __forceinline__ void upwind_faces(const float* r, int, const Lane<float>&, float* fb) {
+    fb[0] = POS ? weno_face(r[-2], r[-1], r[0], r[1], r[2]) : weno_face(r[3], r[2], r[1], r[0], r[-1]);
+}
+template <bool POS>
+__device__ __forceinline__ void upwind_faces(const double* r, int nb, const Lane<double>& c, double* fb) {
+    unsigned mask[FACE_BATCH];
+    int total = 0;
+#pragma unroll
+    for (int b = 0; b < FACE_BATCH; ++b) {
+        bool rough = false;
+        if (b < nb) {
+            const double* q = r + b * SW;
+            fb[b] = POS ? weno_face_smooth(q[-2], q[-1], q[0], q[1], q[2], rough)
+                        : weno_face_smooth(q[3], q[2], q[1], q[0], q[-1], rough);
+        }
+        mask[b] = __ballot_sync(0xffffffffu, rough && c.inner);
+        total += __popc(mask[b]);
+    }
+    // the rough ones, one per lane whichever velocity and node they belong to
+    for (int base = 0; base < total; base += 32) {
+        int k = base + c.lane, at = -1;
+#pragma unroll
+        for (int b = 0; b < FACE_BATCH; ++b) {
+            const int nm = __popc(mask[b]);
+            if (k >= 0 && k < nm) at = b * SW + 4 + nth_bit(mask[b], k);
+            k -= nm;
+        }
+        double v = 0.0;
+        if (base + c.lane < total) {
+            const double* q = c.wall + at;
+            v = POS ? weno_face_rough(q[-2], q[-1], q[0], q[1], q[2]) : weno_face_rough(q[3], q[2], q[1], q[0], q[-1]);
+        }
+        int first = -base;
+#pragma unroll
+        for (int b = 0; b < FACE_BATCH; ++b) {
+            const int rank = first + __popc(mask[b] & ((1u << c.lane) - 1u));
+            const double x = __shfl_sync(0xffffffffu, v, rank & 31);
+            if ((mask[b] >> c.lane & 1) && rank >= 0 && rank < 32) fb[b] = x;
+            first += __popc(mask[b]);
+        }
+    }
+}
+
 // n velocities t, t + 1, ... of one x-velocity; POS: p_x > 0.
 template <typename S, bool POS, bool FORCE>
 __device__ __forceinline__ void update_run(const Stage& g, Lane<S>& c, const Force<S>& fc, int t, int n) {
@@ -1853,11 +1921,16 @@ __device__ __forceinline__ void update_run(const Stage& g, Lane<S>& c, const For
         q0 += (size_t)kz * fc.stride;
     }
     const size_t qs = FORCE ? (size_t)fc.Tz * fc.stride : 0;
+    constexpr int B = sizeof(S) == 8 ? FACE_BATCH : 1;
+    S fb[B];
     for (int m = 0; m < n; ++m) {
-        // right face (i + 1/2) from the five upwind nodes
+        // right faces (i + 1/2) from the five upwind nodes, of B velocities at a time
         const S* r = c.row;
+        if (m % B == 0) upwind_faces<POS>(r, min(B, n - m), c, fb);
         const S fi = r[0];
-        S fr = POS ? weno_face(r[-2], r[-1], fi, r[1], r[2]) : weno_face(r[3], r[2], r[1], fi, r[-1]);
+        S fr = fb[0];
+#pragma unroll
+        for (int b = 1; b < B; ++b) fr = m % B == b ? fb[b] : fr;
         if (c.at_wall) fr = c.wall[SW - 1];
         S fl = __shfl_up_sync(0xffffffffu, fr, 1);
         if (c.lane == 0) fl = c.wall[0];
@@ -1900,7 +1973,7 @@ __device__ __forceinline__ void update_run(const Stage& g, Lane<S>& c, const For
 // computes the moments of the new values (chunk_moments).  Returns false when the staging copies
 // failed.
 // What bounds it: FP64 storage, the FP64 pipe (21 FP64 instructions per node-velocity and stage
-// before the moments, from ~170: the first node's left face had cost a second whole face
+// before the moments where the solution is smooth, from ~170: the first node's left face had cost a second whole face
 // evaluation per warp, now one per 32 velocities, and see fdlb_weno.cuh); FP32 storage, the
 // instructions issued.
 template <typename S, bool BULK, int W = UPD_WARPS>
@@ -1992,6 +2065,7 @@ __device__ bool update_item(const Inst& I, int i0, int k0, int k1, int stage, un
     Lane<S> c;
     c.valid = valid;
     c.at_wall = i + 1 == N;
+    c.inner = i + 1 < N;
     c.lane = lane;
     c.ld = ld;
     c.TcS = Tc * TILE;

@@ -58,13 +58,25 @@ def fronts(jump, falling, dtype, seed=0):
 JUMPS = [1.0, 3.0, 1e2, 1e3, 1e4, 1e6, 1e8, 1e12]
 
 
+# A candidate is a sum of three products whose coefficients add up to 10/3 at most: up to seven roundings of
+# the face with those of the coefficients themselves; the weighted mean adds the weights' products, their
+# sum and a quotient (in FP32 an approximate reciprocal of two units, but of the offset from c only).
+BARS = [(np.float32, 10 * 2.0 ** -24), (np.float64, 12 * 2.0 ** -53)]
+
+
 @pytest.mark.parametrize("falling", [False, True], ids=["rising", "falling"])
 @pytest.mark.parametrize("jump", JUMPS)
-# A candidate is a sum of three products whose coefficients add up to 10/3 at most, in three roundings, and
-# the weighted mean adds the weights' products, their sum and a quotient: about eight roundings of the
-# face.  (A quotient is an approximate reciprocal of two units in FP32, two more.)
-@pytest.mark.parametrize("dtype,tol", [(np.float32, 10 * 2.0 ** -24)], ids=["fp32"])
+@pytest.mark.parametrize("dtype,tol", BARS, ids=["fp32", "fp64"])
 def test_faces_at_fronts(dev, dtype, tol, jump, falling):
     v = fronts(jump, falling, dtype)
+    ref = faces_wide(v)
+    assert np.max(np.abs(faces(dev, v) / ref - 1)) <= tol
+
+
+# FP64 takes its weights in double-float up to third differences of 2^-7 of the value
+@pytest.mark.parametrize("noise", [1e-4, 1e-3, 2e-3, 4e-3, 0.03, 0.3])
+@pytest.mark.parametrize("dtype,tol", BARS, ids=["fp32", "fp64"])
+def test_faces_across_the_smoothness_line(dev, dtype, tol, noise):
+    v = (1 + noise * np.random.default_rng(3).uniform(-1, 1, (20000, 5))).astype(dtype)
     ref = faces_wide(v)
     assert np.max(np.abs(faces(dev, v) / ref - 1)) <= tol
