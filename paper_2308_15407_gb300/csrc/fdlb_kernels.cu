@@ -25,6 +25,7 @@
 // pairs) and keep the gradients and the residual in double.
 #include "fdlb_internal.h"
 #include "fdlb_launch.h"
+#include "fdlb_round.cuh"
 #include "fdlb_weno.cuh"
 #include "../../include/fdlb.h"
 
@@ -1369,7 +1370,7 @@ constexpr int UPD_WARPS_WIDE = 16;    // wide update blocks: the velocity loop o
 // over the channel, which drifts the mass.  Rounding base + inc up or down at random, with the
 // probabilities that make the expected stored value the exact sum (Connolly, Higham & Mary,
 // SIAM J. Sci. Comput. 43, 2021), keeps small changes in expectation: no stall, and a mass
-// error that only random-walks.  The random bits come from a counter-based hash of (the
+// error that only random-walks (sr_add, fdlb_round.cuh).  The random bits come from a counter-based hash of (the
 // instance's parameters, step, stage, velocity, node), so runs are reproducible, both schedules
 // round alike, and an instance rounds the same way whatever batch it is in.
 
@@ -1387,23 +1388,6 @@ __device__ __forceinline__ uint32_t fmix32(uint32_t h) {
 __device__ __forceinline__ uint32_t sr_seed(const Inst& I, int stage) {
     const unsigned long long step = (unsigned long long)*(volatile long long*)I.steps;
     return fmix32((uint32_t)(step * 3ull + (unsigned long long)stage) ^ fmix32(I.sr_key));
-}
-
-// base + inc stored as a float: the exact sum s + err (TwoSum) goes to its round-to-nearest
-// value s, or to the neighbouring float on the side of err with probability |err| / gap, so
-// that its expectation is the exact sum: err plus a uniform number of (-gap/2, gap/2) added to s
-// rounds to the neighbour exactly with that probability (gap = the last place of s; at a power of
-// two the finer grid below takes part of it, and below 2^-103 the sum is rounded to nearest).
-// 15 instructions, no branch and no integer-to-float conversion, against 25 for comparing a
-// uniform number with |err| / gap.
-__device__ __forceinline__ float sr_add(float base, float inc, uint32_t bits) {
-    const float s = __fadd_rn(base, inc);
-    const float bb = __fsub_rn(s, base);
-    const float err = __fadd_rn(__fsub_rn(base, __fsub_rn(s, bb)), __fsub_rn(inc, bb));
-    const float gap = __int_as_float(max((int)(__float_as_uint(s) & 0x7f800000u) - (23 << 23), 0));
-    // uniform on [-1/2, 1/2), shifted by half a step so that it is symmetric
-    const float u = __fadd_rn(__uint_as_float(0x3f800000u | (bits >> 9)), -1.49999994f);
-    return __fadd_rn(s, err == 0.0f ? 0.0f : __fmaf_rn(u, gap, err));
 }
 
 // Tables read by the update kernel in its compute type (FP32 copies for FP32 storage).

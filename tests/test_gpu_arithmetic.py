@@ -80,3 +80,48 @@ def test_faces_across_the_smoothness_line(dev, dtype, tol, noise):
     v = (1 + noise * np.random.default_rng(3).uniform(-1, 1, (20000, 5))).astype(dtype)
     ref = faces_wide(v)
     assert np.max(np.abs(faces(dev, v) / ref - 1)) <= tol
+
+
+def rounding(dev, base, inc, lo, hi):
+    """Of all 2^24 random numbers, how many round base + inc to lo, to hi, and to neither."""
+    import torch
+    n = torch.zeros(3, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    assert dev.rounding(C.c_float(base), C.c_float(inc), C.c_float(lo), C.c_float(hi), C.c_void_p(n.data_ptr())) == 0
+    return n.cpu().tolist()
+
+
+# base, exponent of the last place there, increment in units of it
+ROUNDINGS = [(1.5, -23, 0.25), (1.5, -23, 0.75), (1.25, -23, 1e-3), (1.0, -23, 0.125),      # inside a binade
+             (1.0, -24, -1e-3), (1.0, -24, -0.5), (1.0, -24, -0.875),                     # down from a power of two
+             (1.0 - 2.0 ** -24, -24, 0.999), (1.0 - 2.0 ** -24, -24, 1e-3),                # up to one
+             (2.0 ** -110, -133, 0.25), (2.0 ** -110, -134, -0.25), (2.0 ** -126, -149, 0.0),   # 2^-103 and below
+             (3.0 * 2.0 ** -120, -142, 0.375), (1.5, -23, 0.0), (0.0, -23, 1.0), (1.75, -23, 2.0 ** -20)]
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0], ids=["plus", "minus"])
+@pytest.mark.parametrize("case", ROUNDINGS, ids=str)
+def test_rounding_is_exact_in_expectation(dev, case, sign):
+    """A sum goes to one of its two neighbouring floats, to each as often as the other is near: of the 2^24
+    random numbers to within one (half a step of the comparison, half a unit of the remainder)."""
+    base, e, units = case
+    inc = np.float32(units * 2.0 ** e)
+    s = np.float64(base) + np.float64(inc)                   # exact: at most 47 bits apart
+    lo = np.float32(s)
+    if lo > s:
+        lo = np.nextafter(lo, np.float32(-np.inf))
+    hi = lo if lo == s else np.nextafter(lo, np.float32(np.inf))
+    up = 0.0 if lo == s else float((s - np.float64(lo)) / (np.float64(hi) - np.float64(lo)))
+    n = rounding(dev, sign * base, sign * float(inc), sign * float(lo), sign * float(hi))
+    assert n[2] == 0
+    assert abs(n[1] - up * 2 ** 24) <= 1
+    if sign < 0:
+        assert n == rounding(dev, base, float(inc), float(lo), float(hi))
+
+
+def test_rounding_keeps_what_is_not_finite(dev):
+    inf, big = float("inf"), float(np.finfo(np.float32).max)
+    assert rounding(dev, inf, 1.0, inf, 0.0)[0] == 2 ** 24
+    assert rounding(dev, 1.0, -inf, -inf, 0.0)[0] == 2 ** 24
+    assert rounding(dev, float("nan"), 1.0, 1.0, inf)[2] == 2 ** 24
+    assert rounding(dev, big, 0.0, big, inf)[0] == 2 ** 24
