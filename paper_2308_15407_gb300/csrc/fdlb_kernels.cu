@@ -377,11 +377,13 @@ __device__ __forceinline__ void load_inst(const Inst* src, Inst* dst, int tid, i
 }
 
 // After the predecessor: does this launch step the instance (active, of this storage, not with the
-// shared-memory-resident kernel)?  g: the record in global memory, I: its copy.
+// shared-memory-resident kernel)?  g: the record in global memory, I: its copy.  One decision for the
+// block: another block of the launch may set FDLB_FAILED_COPY between two threads' reads, and the threads
+// that went on would miss the others' copies and barrier.
 __device__ __forceinline__ bool runs_now(const Inst& g, const Inst& I, bool fp64) {
     pdl_wait();
     const int st = *(volatile int*)I.status, res = *(const volatile int*)&g.smem_res, pr = *(const volatile int*)&g.precision;
-    return st == FDLB_ACTIVE && !res && (pr == FDLB_FP64) == fp64;
+    return !__syncthreads_or(st != FDLB_ACTIVE || res || (pr == FDLB_FP64) != fp64);
 }
 
 // Named barrier over `n` threads (moment finalisation runs on 128-thread parts of a block).
