@@ -1513,6 +1513,8 @@ extern "C" int fdlb_set_state(fdlb_ctx* c, int32_t inst, const void* host, size_
         if (!rc) rc = cuda_check(c, cudaMemcpyAsync(I.misc + M_SWITCH, &swd, sizeof(swd), cudaMemcpyHostToDevice, c->stream), "state upload");
     }
     if (!rc) rc = cuda_check(c, cudaMemcpyAsync(I.f[0], static_cast<const char*>(host) + 24 + ph, need - 24 - ph, cudaMemcpyHostToDevice, c->stream), "state upload");
+    // (tickets of a tile whose update gave up)
+    if (!rc) rc = cuda_check(c, cudaMemsetAsync(I.mcnt, 0, sizeof(int) * (I.ld / TILE), c->stream), "clear counters");
     if (!rc) rc = moments_of(c, inst);
     if (!rc) rc = cuda_check(c, launch_resid(c->d_inst, c->count, inst, 0.0, c->d_resid_all, c->stream), "residual kernel");
     if (!rc) rc = cuda_check(c, cudaMemcpyAsync(I.steps, &st, sizeof(st), cudaMemcpyHostToDevice, c->stream), "state upload");

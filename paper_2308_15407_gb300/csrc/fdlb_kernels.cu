@@ -1311,6 +1311,7 @@ __global__ void __launch_bounds__(TILE * NOD_WARPS) k_profiles(Inst* insts, cons
             else static_cast<double*>(I.f[0])[e] = v;
         }
     }
+    if (threadIdx.x == 0) I.mcnt[i0 / TILE] = 0;
     if (threadIdx.x == 0 && i0 == 0) {
         if (I.two_phase) {
             I.precision = FDLB_FP32_STORAGE;
@@ -1632,7 +1633,8 @@ __device__ void chunk_moments(const Inst& I, int i0, int k0, int k1, int grp, co
 
 // Tiled schedule, tiles split into several chunks: the last chunk block of the tile to arrive
 // (ticket) adds the chunks' partial sums in chunk order -- the result does not depend on the
-// arrival order -- and resets the ticket.  ss: MOM_SUMS x TILE shared doubles.
+// arrival order -- and resets the ticket.  (A chunk whose copies failed takes none; the tile's count then
+// stays short until new profiles or a loaded state clear it.)  ss: MOM_SUMS x TILE shared doubles.
 template <typename S>
 __device__ void chunk_ticket_final(const Inst& I, int i0, double* ss, int nwb = UPD_WARPS) {
     __shared__ int last;
