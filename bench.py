@@ -85,7 +85,7 @@ def couette_params(F, precision="fp32"):
 def kernel_flops(kind, p, nx, nvel):
     """Arithmetic per launch of one instance from the kernels' operation counts (FP64 flops;
     FP32 flops for the update of an FP32-storage instance).  The closure assumes the 8-point
-    auxiliary rule, which the kernel uses whenever |u_x|/sqrt(T) < 0.02 and Q <= 12 (all
+    auxiliary rule, which the kernel uses whenever |u_x|/sqrt(T) < 0.02 and Q <= 8 (all
     nodes of these wall-bounded flows once the start-up transient has passed)."""
     Q, Qy, Qz = p.qx_half, p.qy, p.qz
     Tc = Qy * Qz if Qz else (2 * Qy if Qy else 2)
@@ -95,7 +95,7 @@ def kernel_flops(kind, p, nx, nvel):
         per_node = 60 * Q + 120 if p.precision == "fp32" else 12 * nvel + 60 * Q + 120
         return per_node * nx
     if kind == "nodal":
-        M = 8 if Q <= 12 else 16
+        M = 8 if Q <= 8 else 16
         My = (Qy + 5) // 2 if Qy else 0
         Mz = (Qz + 5) // 2 if Qz else 0
         closure = 235

@@ -595,10 +595,10 @@ __device__ __forceinline__ void scale_point(double, double&, double&) {}
 
 // Half-range x projection of a tile (Sec. III A 2), both half-axes: the auxiliary points
 // x = sqrt(T) q and the polynomials there do not depend on the sign of u, so one recurrence
-// serves both.  With |v| < 0.02 and Q <= 12 the 8-point auxiliary rule is used.  It is exact for
-// v = 0 (degree 15 >= Q + 2); what it misses of exp(q v) at |v| = 0.02 is 3e-13 of the largest
-// value at Q = 8 and below that for smaller orders, but 7e-11 at Q = 9 and grows to 1e-4 at
-// Q = 12 (at |v| = 0.002: 2e-15 and 1e-6).  Warp w
+// serves both.  With |v| < 0.02 and Q <= MX8 the 8-point auxiliary rule is used: it is exact for v = 0
+// (degree 15 >= Q + 2), and what it misses of exp(q v) at |v| = 0.02 is 3e-13 of the largest value at
+// Q = 8 and less at smaller orders (7e-11 at Q = 9, 1e-4 at Q = 12: those take the 16-point rule, 41 us
+// per launch for twelve Couette instances of order 9 in FP64 against 31).  Warp w
 // takes auxiliary points w, w + 8, ...  R: double, or double-float for FP32 storage; out: the
 // table written (FP32 storage's tab32 also from double).
 template <int QB, typename R, typename O>
@@ -627,7 +627,7 @@ __device__ void xproj_half(const Inst& I, int i0, double* nsm, O* out, Part pt) 
         if (lane == 0) use_short = av < 0.02f ? 1 : 0;
     }
     __syncthreads();
-    const bool short_rule = use_short && Q <= 12;
+    const bool short_rule = use_short && Q <= MX8;
     const int M = short_rule ? MX8 : I.Mx;
     const double* xq = short_rule ? I.xq8 : I.xq;
     const double* xw = short_rule ? I.xw8 : I.xw;
