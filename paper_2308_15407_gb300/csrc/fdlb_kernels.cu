@@ -473,7 +473,18 @@ __host__ __device__ inline int nodal_smem_doubles(int qmax) {
 }
 
 constexpr int XQ_DF = 32;           // half-range double-float projections: unscaled up to this order
-constexpr float XQ_TMAX = 1.8f;     // e^((T - 1) q^2/4) < 1e25 at q = 17, the outermost point of order 100
+
+// Do the x projections of the tile's nodes stay in the double-float range at every order?  T < XQ_TMAX
+// and |u| < sqrt(T) (the same answer in every warp; NaN: no).  Half range, scaled points: e^((T - 1)
+// q^2/4) < 1e25 at q = 17, the outermost point of order 100, and exponents q |u|/sqrt(T) below 17.  Full range: the
+// coefficients m_l are at most 17 up to order 200; beyond, they grow like |T - 1|^(l/2), 2e7 at T =
+// 2.2 and out of the float range at T = 3.3.
+constexpr float XQ_TMAX = 1.8f;
+__device__ __forceinline__ bool in_df_range(const Inst& I, int i0, int lane) {
+    const int i = min(i0 + lane, I.N - 1);
+    const float T = (float)I.node[R_T * I.ld + i], u = (float)I.node[R_UX * I.ld + i];
+    return __all_sync(0xffffffffu, T < XQ_TMAX && u * u < T);
+}
 
 // 1/j as float pairs, j = 0..16 (set by prepare_kernels)
 constexpr int NINV2 = 17;
@@ -1086,27 +1097,23 @@ __device__ void nodal_item(const Inst& I, int i0, int role, double* nsm, bool fp
         else closure_item<double>(I, i0, nsm);
         return;
     }
+    // FP32 storage: double-float, FP64 in tiles beyond its range (708 us per launch for six instances of order
+    // 100, against 212 in double-float)
     if (I.xfull) {
-        // the coefficients m_l and w_k h_l(p_k) stay small at every order: double-float for FP32
-        // storage up to order 200
-        if (fp32) xproj_full<df>(I, i0, nsm, r_out(I, i0, lane, df{}), pt);
-        else xproj_full<double>(I, i0, nsm, r_out(I, i0, lane, 0.0), pt);
+        if (!fp32) xproj_full<double>(I, i0, nsm, r_out(I, i0, lane, 0.0), pt);
+        else if (in_df_range(I, i0, lane)) xproj_full<df>(I, i0, nsm, r_out(I, i0, lane, df{}), pt);
+        else xproj_full<double>(I, i0, nsm, r_out(I, i0, lane, df{}), pt);
         return;
     }
     if (!fp32) {
         xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, 0.0), pt);
         return;
     }
-    // FP32 storage: double-float.  Above XQ_DF polynomials the points are scaled (scale_point), which
-    // holds to T = XQ_TMAX at the largest order; a hotter tile sums in FP64 (708 us per launch for
-    // six instances of order 100, against 212 in double-float).
     if constexpr (QB > 8) {               // (QB = 8: no order above 8 in the batch)
-        if (I.Lx > XQ_DF) {
-            const float T = (float)I.node[R_T * I.ld + min(i0 + lane, I.N - 1)];
-            if (__any_sync(0xffffffffu, !(T < XQ_TMAX))) {         // (the same in every warp)
-                xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, df{}), pt);
-                return;
-            }
+        // above XQ_DF polynomials the points are scaled (scale_point)
+        if (I.Lx > XQ_DF && !in_df_range(I, i0, lane)) {
+            xproj_half<QB, double>(I, i0, nsm, r_out(I, i0, lane, df{}), pt);
+            return;
         }
     }
     xproj_half<QB, df>(I, i0, nsm, r_out(I, i0, lane, df{}), pt);
