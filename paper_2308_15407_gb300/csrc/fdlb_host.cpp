@@ -33,6 +33,14 @@ using namespace fdlb;
 // ---------------------------------------------------------------------------
 static thread_local std::string g_err;
 
+// For its lifetime the calling thread may free page-locked memory while it or another thread captures a
+// graph (of other streams), which the call would else break.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 struct fdlb_ctx {
     int count = 0;
     std::vector<fdlb_params> prm;
@@ -94,7 +102,10 @@ struct fdlb_ctx {
         if (ev_fork) cudaEventDestroy(ev_fork);
         if (ev_join) cudaEventDestroy(ev_join);
         if (stream2) cudaStreamDestroy(stream2);
-        if (pin) cudaFreeHost(pin);
+        if (pin) {
+            RelaxedCapture relaxed;
+            cudaFreeHost(pin);
+        }
     }
 };
 
