@@ -64,9 +64,11 @@ extern "C" {
 #define FDLB_GRID_TANH    1    /* x = tanh(A s)/(2 tanh A), A = stretch (nodes crowd at the walls) */
 
 /* Storage precision of f. */
-#define FDLB_FP64          0   /* everything in FP64 */
+#define FDLB_FP64          0   /* FP64; the WENO-5 weights of smooth stencils, which multiply third
+                                  differences below 2^-6 of the value, in double-float (the
+                                  faces stay as accurate as with FP64 weights) */
 #define FDLB_FP32_STORAGE  1   /* f stored, advected and combined in FP32; moments, projections and
-                                  closure in double-float (float pairs, ~1e-14), gradients and
+                                  closure in double-float (float pairs, ~3e-14), gradients and
                                   the residual in FP64 */
 #define FDLB_FP32_THEN_FP64 2  /* two phases: FDLB_FP32_STORAGE until the per-step residual
                                   stagnates, then FDLB_FP64 for the rest of the solve.  f is

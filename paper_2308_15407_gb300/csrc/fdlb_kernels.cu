@@ -20,7 +20,7 @@
 //
 // Storage type S (double | float) holds f; compute type C of the per-velocity work is
 // double for FDLB_FP64 and float for FDLB_FP32_STORAGE.  FP64 instances do all the rest in
-// double (but for the WENO weights, fdlb_weno.cuh); FP32-storage instances run the moment sums
+// double (but for the WENO weights of smooth stencils, fdlb_weno.cuh); FP32-storage instances run the moment sums
 // and their finalisation, the velocity projections and the closure chain in double-float (float
 // pairs) and keep the gradients and the residual in double.
 #include "fdlb_internal.h"
@@ -276,23 +276,14 @@ __device__ __forceinline__ float* r_out(const Inst& I, int i0, int lane, df) { r
 
 constexpr int NTW = 6;     // transverse weights: mt, mt py, mt py^2, mt py^3, et, et py
 
-// Per node: the 14 raw sums over all velocities, factorised as sum_kx px^a (sum_t w_j(t) f),
-// and the moments they give.
-
 template <typename R>
 __device__ __forceinline__ R chi_of(R eta) {
     const R om = r_c(1.0, R{}) - eta;
     return r_div(r_c(2.0, R{}) - eta, r_c(2.0, R{}) * om * om * om);
 }
 
-// Moments of the nodes of tile i0 from the raw sums ss[MOM_SUMS][TILE], by nw warps: independent
-// chains, one per warp (n, u, T and the stresses; ln n; ln T; ln chi(eta0 n); q_x; q_y).  SPLIT: six
-// chains, for the last block of a split tile, which everything waits for (one Couette instance:
-// update 18.1 -> 16.4 us per launch); else the heat fluxes with the first, which shares its
-// quotients (2048 mixed instances: 756 us per launch with six chains, 705 with four).  FP32 storage finalises its double-float sums in double-float: in FP64
-// this took 362 FP64 instructions per tile, 45 % of the FP64 pipe's time on large batches.
-// Heat fluxes from the raw sums s[j TILE]: third-order sums about the mean, s8 - 3 ux s4 + 2 n ux^3 and
-// so on.
+// Heat fluxes from the raw sums s[j TILE] (each sum_kx px^a (sum_t w_j(t) f)): third-order sums about the
+// mean, s8 - 3 ux s4 + 2 n ux^3 and so on.
 template <typename R>
 __device__ __forceinline__ R heat_flux_x(const R* s, R n, R ux, R uy) {
     const R two = r_c(2.0, R{}), n2 = two * n;
@@ -308,6 +299,13 @@ __device__ __forceinline__ R heat_flux_y(const R* s, R n, R ux, R uy) {
     return r_c(0.5, R{}) * (cy3 + cxxy) + (s[13 * TILE] - uy * s[7 * TILE]);
 }
 
+// Moments of the nodes of tile i0 from the 14 raw sums ss[MOM_SUMS][TILE], by nw warps: independent
+// chains, one per warp (n, u, T and the stresses; ln n; ln T; ln chi(eta0 n); q_x; q_y).  SPLIT: six
+// chains, for the last block of a split tile, which everything waits for (one Couette instance:
+// update 18.1 -> 16.4 us per launch); else the heat fluxes with the first, which shares its
+// quotients (2048 mixed instances: 756 us per launch with six chains, 705 with four).  FP32 storage
+// finalises its double-float sums in double-float: in FP64 this took 362 FP64 instructions per tile,
+// 45 % of the FP64 pipe's time on large batches.
 template <bool SPLIT, typename R>
 __device__ __forceinline__ void finalize_chain(const Inst& I, int i0, const R* ss, int lane, int g) {
     const int i = i0 + lane, ld = I.ld;
