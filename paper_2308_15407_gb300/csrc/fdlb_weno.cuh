@@ -66,13 +66,15 @@ __device__ __forceinline__ float weno_face(float a, float b, float c, float d, f
 constexpr int WENO_SMOOTH = 6;
 
 // The face of a stencil that is not smooth, the first form, all of it in FP64, from the differences.  (The
-// offsets' weights are eighth powers of differences: those beyond 2^-100 .. 2^100 are scaled first.)
+// offsets' weights are eighth powers of differences, those beyond 2^-60 .. 2^100 are scaled first: with the
+// largest at 2^-t and the smooth side at 2^-(t + r), the numerator is 2^-(9 t + 5 r), and a full number for all
+// jumps up to 2^96.)
 __device__ __forceinline__ double weno_face_rough(double a, double b, double c, double d, double e) {
     double d1 = b - a, d2 = c - b, d3 = d - c, d4 = e - d;
     const int top = max(max(__double2hiint(d1) & 0x7fffffff, __double2hiint(d2) & 0x7fffffff),
                         max(__double2hiint(d3) & 0x7fffffff, __double2hiint(d4) & 0x7fffffff));
     const double o1 = fma(-2.0, d1, 5.0 * d2), o2 = fma(2.0, d3, d2), o3 = fma(4.0, d3, -d4);
-    if ((unsigned)(top - (923 << 20)) > (200u << 20)) {
+    if ((unsigned)(top - (963 << 20)) > (160u << 20)) {
         const double sc = __hiloint2double(max((2045 << 20) - (top & 0x7ff00000), 1 << 20), 0);
         d1 *= sc;
         d2 *= sc;

@@ -73,6 +73,16 @@ def test_faces_at_fronts(dev, dtype, tol, jump, falling):
     assert np.max(np.abs(faces(dev, v) / ref - 1)) <= tol
 
 
+# The velocity tails: the same stencils, smaller by powers of two.
+@pytest.mark.parametrize("falling", [False, True], ids=["rising", "falling"])
+@pytest.mark.parametrize("jump", [*JUMPS, 3e4, 1e5, 2e5])
+@pytest.mark.parametrize("dtype,tol,e", [(np.float64, BARS[1][1], e) for e in (-60, -80, -99, -130, -400)])
+def test_small_faces_at_fronts(dev, dtype, tol, e, jump, falling):
+    v = np.ldexp(fronts(jump, falling, dtype), e)
+    ref = faces_wide(np.ldexp(v, -e))
+    assert np.max(np.abs(np.ldexp(faces(dev, v), -e) / ref - 1)) <= tol
+
+
 # FP64 takes its weights in double-float up to third differences of 2^-7 of the value
 @pytest.mark.parametrize("noise", [1e-4, 1e-3, 2e-3, 4e-3, 0.03, 0.3])
 @pytest.mark.parametrize("dtype,tol", BARS, ids=["fp32", "fp64"])
