@@ -10,7 +10,7 @@
 //        = c + (d2 + 2 d3 - (2 m1 (e2 - e1) + 3 m3 (e3 - e2))/(m1 + 6 m2 + 3 m3))/6.
 // No epsilon; a vanishing indicator takes the weight in the limit.
 //
-// FP32: the first form, 45 instructions against 61 of the candidates and normalised weights.  Each
+// FP32: the first form, 47 instructions against 61 of the candidates and normalised weights.  Each
 // offset carries its own weight, so next to a front, where d2 + 2 d3 holds a jump, no two terms of the
 // jump's size cancel: 6e-8 of the face for jumps of 1e2 between neighbouring nodes (the second form, 42
 // instructions: 1e-5, and no digit from jumps of 1e7 on; the sum of weighted candidates: 5e-7).
@@ -58,9 +58,11 @@ __device__ __forceinline__ float weno_face(float a, float b, float c, float d, f
         w3 = 3.0f * m3;
         sum = (m1 + w2) + w3;
     }
-    // six times the candidates' offsets from c, each times its own weight
+    // six times the candidates' offsets from c, each times its own weight.  The weights are normalised first:
+    // next to a front they are as small as 1e-30, and times the offsets of a velocity tail no normal numbers.
     const float o1 = fmaf(-2.0f, d1, 5.0f * d2), o2 = fmaf(2.0f, d3, d2), o3 = fmaf(4.0f, d3, -d4);
-    return fmaf(fmaf(m1, o1, fmaf(w2, o2, w3 * o3)), rcp_approx(sum) * (1.0f / 6.0f), c);
+    const float rs = rcp_approx(sum) * (1.0f / 6.0f);
+    return fmaf(m1 * rs, o1, fmaf(w2 * rs, o2, (w3 * rs) * o3)) + c;
 }
 
 constexpr int WENO_SMOOTH = 6;

@@ -76,7 +76,8 @@ def test_faces_at_fronts(dev, dtype, tol, jump, falling):
 # The velocity tails: the same stencils, smaller by powers of two.
 @pytest.mark.parametrize("falling", [False, True], ids=["rising", "falling"])
 @pytest.mark.parametrize("jump", [*JUMPS, 3e4, 1e5, 2e5])
-@pytest.mark.parametrize("dtype,tol,e", [(np.float64, BARS[1][1], e) for e in (-60, -80, -99, -130, -400)])
+@pytest.mark.parametrize("dtype,tol,e", [(np.float32, BARS[0][1], e) for e in (0, -20, -30, -36, -45)] +
+                         [(np.float64, BARS[1][1], e) for e in (-60, -80, -99, -130, -400)])
 def test_small_faces_at_fronts(dev, dtype, tol, e, jump, falling):
     v = np.ldexp(fronts(jump, falling, dtype), e)
     ref = faces_wide(np.ldexp(v, -e))
