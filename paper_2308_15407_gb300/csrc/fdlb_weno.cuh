@@ -10,7 +10,7 @@
 //        = c + (d2 + 2 d3 - (2 m1 (e2 - e1) + 3 m3 (e3 - e2))/(m1 + 6 m2 + 3 m3))/6.
 // No epsilon; a vanishing indicator takes the weight in the limit.
 //
-// FP32: the first form, 47 instructions against 61 of the candidates and normalised weights.  Each
+// FP32: the first form, 46 instructions against 61 of the candidates and normalised weights.  Each
 // offset carries its own weight, so next to a front, where d2 + 2 d3 holds a jump, no two terms of the
 // jump's size cancel: 6e-8 of the face for jumps of 1e2 between neighbouring nodes (the second form, 42
 // instructions: 1e-5, and no digit from jumps of 1e7 on; the sum of weighted candidates: 5e-7).
@@ -36,14 +36,15 @@ __device__ __forceinline__ float weno_face(float a, float b, float c, float d, f
     const float q1 = fmaf(2.0f, d2, e1), q2 = d2 + d3, q3 = fmaf(-2.0f, d3, e3);
     const float k = 13.0f / 3.0f;
     const float s1 = fmaf(k * e1, e1, q1 * q1), s2 = fmaf(k * e2, e2, q2 * q2), s3 = fmaf(k * e3, e3, q3 * q3);
-    // scaled by the largest, so that the fourth powers stay in range
+    // scaled by the largest, so that the fourth powers stay in range: up to 2^60, since next to a front the
+    // largest is 1e-30 of that, and times the offsets of a velocity tail it has to stay a normal number
     const float smax = fmaxf(s1, fmaxf(s2, s3));
-    const float r = rcp_approx(fmaxf(smax, 4e-30f));
+    const float r = rcp_approx(fmaxf(smax, 4e-30f)) * 0x1p15f;
     const float a1 = s1 * r, a2 = s2 * r, a3 = s3 * r;
     const float p1 = a1 * a1, p2 = a2 * a2, p3 = a3 * a3;
     float m1 = p2 * p3, m2 = p1 * p3, m3 = p1 * p2;
     float w2 = 6.0f * m2, w3 = 3.0f * m3, sum = (m1 + w2) + w3;
-    if (sum < 1e-30f) {
+    if (sum < 0x1p60f * 1e-30f) {
         if (smax < 4e-30f) {
             // uniform to FP32 resolution: the candidates agree, the ideal weights are the limit
             m1 = m2 = m3 = 1.0f;
@@ -58,11 +59,9 @@ __device__ __forceinline__ float weno_face(float a, float b, float c, float d, f
         w3 = 3.0f * m3;
         sum = (m1 + w2) + w3;
     }
-    // six times the candidates' offsets from c, each times its own weight.  The weights are normalised first:
-    // next to a front they are as small as 1e-30, and times the offsets of a velocity tail no normal numbers.
+    // six times the candidates' offsets from c, each times its own weight
     const float o1 = fmaf(-2.0f, d1, 5.0f * d2), o2 = fmaf(2.0f, d3, d2), o3 = fmaf(4.0f, d3, -d4);
-    const float rs = rcp_approx(sum) * (1.0f / 6.0f);
-    return fmaf(m1 * rs, o1, fmaf(w2 * rs, o2, (w3 * rs) * o3)) + c;
+    return fmaf(fmaf(m1, o1, fmaf(w2, o2, w3 * o3)), rcp_approx(sum) * (1.0f / 6.0f), c);
 }
 
 constexpr int WENO_SMOOTH = 6;
