@@ -58,7 +58,7 @@ KERNEL_SRC = [os.path.join(ROOT, "paper_2308_15407_gb300", "csrc", f)
 # ncu DRAM bytes (read + write) per k_update<float> launch on the 12-instance sweep,
 # cold cache, mean over the three stages of one capture, with the SHA-256 prefix of the
 # sources it was taken on; the bench reports it only while they are unchanged.
-UPDATE_TRAFFIC = {"bytes": 6698240, "kernel_src_sha16": "6d7ec876b9d0f9e7"}
+UPDATE_TRAFFIC = {"bytes": 6698112, "kernel_src_sha16": "c75b30f367e97327"}
 
 
 def kernel_src_sha16():
